@@ -447,8 +447,6 @@ struct Solver final : SolverBase {
     double* khr_dev = nullptr;  // layered media: k h per grid row (device), else null
     CT* RT = nullptr;
     CT* dlt = nullptr;          // the level-1 update of the current step (leaf precision)
-    CT* AC0 = nullptr;          // A~_0 C_0: the root's operator on its basis (column-major)
-    CT* RP = nullptr;           // r' of the current step (the root's input residual)
     c128* partial = nullptr;
     double *npart = nullptr, *dnorm = nullptr;
     int* derr = nullptr;
@@ -463,7 +461,6 @@ struct Solver final : SolverBase {
     bool pre_direct = false;    // its leaf sweeps write the owned rows into the parents
     const int* step_gate = nullptr;   // gate of the launches of the step being enqueued
     std::vector<const void*> view_key, eview_key;
-    std::vector<EigTask> h_pre;   // host copy of the preconditioner's leaf tasks (batched solves)
     // eigenbasis leaf path
     bool eig = false;
     int eig_fused = 0;          // cluster size of the one-launch single-vector sweep (0: off)
@@ -473,6 +470,30 @@ struct Solver final : SolverBase {
     bool tc = false;
     std::vector<void*> EVT, EVN;
     EigTask *d_etasks_view = nullptr, *d_etasks_own = nullptr, *d_etask_one = nullptr, *d_etasks_pre = nullptr;
+    // iteration on the cut rows (k_cut.cu)
+    bool cut = false;
+    CutProb cp{};               // host copy of the problem's descriptor (d_cut on the device)
+    CutProb* d_cut = nullptr;
+    size_t cut_smem = 0;        // shared memory of a step block
+    CutCtl* cctl = nullptr;     // its control words, behind the norms (dnorm + 10)
+    CutUpdJob* d_upd = nullptr; // update jobs: [0] u -> ut, [1] ut -> u
+    unsigned* cbar = nullptr;
+    EigTask *d_etasks_cin = nullptr, *d_etasks_cout = nullptr;   // full residual in, every row out
+    std::vector<CT*> EF0;       // the round's transformed residual
+    CT *cut_Cp = nullptr, *cut_Ep = nullptr, *cut_MT = nullptr;
+    c128 *cut_E64 = nullptr, *cut_G = nullptr, *cut_M64 = nullptr, *cut_part = nullptr;
+    unsigned char* d_cut_tab = nullptr;
+    size_t cut_tab_bytes = 0, cut_pairs_max = 0;
+    struct CutLevel {           // the panel and product entries of one level's nodes (device)
+        CutCpEntry* cpe;
+        CutEpEntry* epe;
+        CutGramPair* prs;
+        CutGramDest* dst;
+        CutMinv* minv;
+        int ncp, nep, nprs, ndst, nminv;
+    };
+    std::vector<CutLevel> clev;
+    std::vector<EigTask> h_cin, h_cout;   // host copies of the transform tasks (batched solves)
     // flexible GMRES
     int mk = 0;                                   // restart length
     c128 *Vb = nullptr, *Zb = nullptr, *gw = nullptr, *gv = nullptr, *gz = nullptr, *gdots = nullptr,
@@ -549,6 +570,217 @@ struct Solver final : SolverBase {
         eig = (Sx > 1 && P.leaf_solver == HH_LEAF_EIGEN);
         tc = eig && sizeof(CT) == sizeof(c64) && !(P.flags & HH_FLAG_CUDA_CORE_SWEEPS);
         mk = P.outer == HH_OUTER_GMRES ? P.restart : 0;
+        cut = false;
+        cp = CutProb{};
+        const int D = 2 * r * ((1 << L) - 1);
+        if (eig && P.n_inner == 1 && L <= CUT_MAXL && D <= CUT_MAXD) {
+            cp.Sx = Sx;
+            cp.L = L;
+            cp.r = r;
+            cp.ncut = (1 << L) - 1;
+            cp.D = D;
+            cp.q1 = q1();
+            cp.kh = kh;
+            cut_smem = cut_plan<T>(cp, b_max);
+            cut = cut_smem > 0;
+        }
+    }
+
+    // ------------------------------------------- the iteration on the cut rows: tables
+    // Level and position of the node whose cut is c (between leaves c and c + 1).
+    int cut_lev(int c) const { return L - __builtin_ffs(c + 1); }
+    // The group of node `id` (level l) among the E columns of cut c: the own node's two
+    // children, the ancestors from the nearest up, then the nodes ending (0) or beginning (1)
+    // at the cut, level by level.
+    int ep_group(int c, int id, int side) const {
+        const int lc = cut_lev(c), l = nodes[id].level;
+        if (l == lc) return side;
+        return l < lc ? 2 + (lc - 1 - l) : 2 + lc + 2 * (l - lc - 1) + side;
+    }
+    // Offsets of the panels in elements; returns the elements of Cp and Ep.
+    void cut_panel_sizes(size_t& ncp, size_t& nep) {
+        ncp = nep = 0;
+        for (int c = 0; c < cp.ncut; ++c) {
+            cp.cp_off[c] = ncp;
+            cp.ep_off[c] = nep;
+            ncp += 2 * (size_t)Sx * (cut_lev(c) + 1) * r;
+            nep += 2 * (size_t)Sx * (2 * L - cut_lev(c)) * r;
+        }
+    }
+    // The device tables (leaves, nodes, panel and product entries), built with the arena's
+    // addresses; upload = false only counts their bytes.
+    size_t cut_tables(bool upload) {
+        std::vector<unsigned char> blob;
+        auto put = [&](const void* src, size_t bytes) {
+            const size_t off = align_up(blob.size(), 16);
+            blob.resize(off + bytes);
+            if (bytes) std::memcpy(blob.data() + off, src, bytes);
+            return d_cut_tab + off;
+        };
+        std::vector<CutLeaf> lf;
+        for (int i = 0; i <= cp.ncut; ++i) {
+            const Node& nd = nodes[lev[L][i]];
+            CutLeaf f{};
+            f.V = EV[nd.id];
+            f.xi = EXI[nd.id];
+            f.sc = ESC[nd.id];
+            f.fh0 = EF0[nd.id];
+            f.fh = EFh[nd.id];
+            f.b = nd.b();
+            const int up = nd.oa - nd.ra, dn = nd.ob - nd.ra;   // local rows below the two cuts
+            for (int k = 0; k < 2; ++k) {
+                f.rin[k] = i > 0 ? up - 1 + k : -1;
+                f.rin[2 + k] = i < cp.ncut ? dn - 1 + k : -1;
+                f.rout[k] = i > 0 ? up + k : -1;
+                f.rout[2 + k] = i < cp.ncut ? dn - 2 + k : -1;
+            }
+            lf.push_back(f);
+            if (i < cp.ncut) cp.mid[i] = nd.ob;
+        }
+        std::vector<CutNode> nv;
+        for (int id = 0; id < cp.ncut; ++id) nv.push_back({C[id], pts(id), nodes[id].ra});
+        cp.leaf = (const CutLeaf*)put(lf.data(), sizeof(CutLeaf) * lf.size());
+        cp.node = (const CutNode*)put(nv.data(), sizeof(CutNode) * nv.size());
+        clev.assign(L, CutLevel{});
+        cut_pairs_max = 0;
+        const size_t Nx = (size_t)Sx;
+        for (int l = 0; l < L; ++l) {
+            std::vector<CutCpEntry> ce;
+            std::vector<CutEpEntry> ee;
+            std::map<std::tuple<int, int, int, int>, std::vector<CutGramPair>> by_dest;   // (p, kp, q, kq)
+            std::vector<CutMinv> mv;
+            const int span = 1 << (L - l);
+            for (int p : lev[l]) {
+                const int t = p + 1 - (1 << l), own = t * span + span / 2 - 1;
+                const CT* Cb = C[p];
+                const size_t N = pts(p);
+                auto row = [&](int k, int grow) { return Cb + (long long)(k * r) * (long long)N + (long long)(grow - nodes[p].ra) * (long long)Nx; };
+                auto add_e = [&](int c, int k, int side, int ml, int mr) {
+                    const int g = ep_group(c, p, side), Ke = (2 * L - cut_lev(c)) * r;
+                    const size_t o = cp.ep_off[c] + (size_t)g * r * Nx;
+                    ee.push_back({row(k, cp.mid[c] - 2), cut_Ep + o, cut_E64 + o, N, Ke, ml, mr});
+                    cp.yidx[c * 2 * CUT_MAXL + g] = (unsigned short)(p * 2 * r + k * r);
+                };
+                for (int c = t * span; c < (t + 1) * span - 1; ++c) {
+                    const int lc = cut_lev(c), K = (lc + 1) * r;
+                    CT* base = cut_Cp + cp.cp_off[c];
+                    const int kin = c < own ? 0 : 1;
+                    for (int rw = 0; rw < 2; ++rw)
+                        ce.push_back({row(c == own ? rw : kin, cp.mid[c] - 1 + rw), base + rw * Nx * K + l * r, N, K});
+                    if (c == own) {
+                        add_e(c, 0, 0, 1, 1);
+                        add_e(c, 1, 1, 1, 1);
+                    } else {
+                        add_e(c, kin, 0, 1, 1);
+                    }
+                    // products with every node at or below p that has columns at this cut
+                    auto add_p = [&](int q, int kq, int side) {
+                        const CutGramPair pr{base + l * r, cut_E64 + cp.ep_off[c] + (size_t)ep_group(c, q, side) * r * Nx,
+                                             K, (2 * L - lc) * r, 0};
+                        for (int rw = 0; rw < 2; ++rw) {
+                            CutGramPair x = pr;
+                            if (c != own) {
+                                if (rw) break;
+                                x.rows = 3;
+                                by_dest[{p, kin, q, kq}].push_back(x);
+                            } else {
+                                x.rows = 1 << rw;
+                                by_dest[{p, rw, q, kq}].push_back(x);
+                            }
+                        }
+                    };
+                    const int tc = (c + 1) >> (L - lc), oid = (1 << lc) - 1 + tc;   // the cut's own node
+                    add_p(oid, 0, 0);
+                    add_p(oid, 1, 1);
+                    for (int q = oid; q != p;) {
+                        const int up = (q - 1) >> 1;
+                        add_p(up, q == 2 * up + 2, 0);
+                        q = up;
+                    }
+                    for (int lb = lc + 1; lb < L; ++lb) {
+                        const int tr = (c + 1) >> (L - lb);   // the node beginning at the cut
+                        add_p((1 << lb) - 1 + tr - 1, 1, 0);
+                        add_p((1 << lb) - 1 + tr, 0, 1);
+                    }
+                }
+                if (t > 0) add_e(t * span - 1, 0, 1, 0, 1);
+                if (t < (1 << l) - 1) add_e((t + 1) * span - 1, 1, 0, 1, 0);
+                mv.push_back({p, p, Ainv[p]});
+            }
+            // the diagonal blocks first, then the others of the same rows (one launch each)
+            const int ndiag = (int)mv.size();
+            for (int p : lev[l])
+                for (int ls = l + 1; ls < L; ++ls)
+                    for (int s2 : lev[ls])
+                        if (((s2 + 1) >> (ls - l)) - 1 == p) mv.push_back({p, s2, Ainv[p]});
+            std::vector<CutGramPair> pr;
+            std::vector<CutGramDest> ds;
+            for (auto& kv : by_dest) {
+                const auto [p, kp, q, kq] = kv.first;
+                if (p == q) continue;
+                CutGramDest d;
+                d.out = cut_G + ((size_t)p * 2 * r + kp * r) * cp.D + (size_t)q * 2 * r + kq * r;
+                d.ld = cp.D;
+                d.first = (int)pr.size();
+                d.count = (int)kv.second.size();
+                ds.push_back(d);
+                pr.insert(pr.end(), kv.second.begin(), kv.second.end());
+            }
+            (void)ndiag;
+            CutLevel& cl = clev[l];
+            cl.ncp = (int)ce.size(); cl.nep = (int)ee.size(); cl.nprs = (int)pr.size(); cl.ndst = (int)ds.size();
+            cl.nminv = (int)mv.size();
+            cl.cpe = (CutCpEntry*)put(ce.data(), sizeof(CutCpEntry) * ce.size());
+            cl.epe = (CutEpEntry*)put(ee.data(), sizeof(CutEpEntry) * ee.size());
+            cl.prs = (CutGramPair*)put(pr.data(), sizeof(CutGramPair) * pr.size());
+            cl.dst = (CutGramDest*)put(ds.data(), sizeof(CutGramDest) * ds.size());
+            cl.minv = (CutMinv*)put(mv.data(), sizeof(CutMinv) * mv.size());
+            cut_pairs_max = std::max(cut_pairs_max, pr.size());
+        }
+        std::vector<EigTask> tin, tout;
+        for (int id : lev[L]) {
+            const Node& nd = nodes[id];
+            EigTask k = eig_task(id, RT + row_off(0, nd.ra, 1), nullptr);
+            k.Fh = EF0[id];
+            tin.push_back(k);
+            EigTask o = eig_task(id, nullptr, dlt + row_off(0, nd.oa, 1));
+            o.w0 = nd.oa - nd.ra;
+            o.w1 = nd.ob - nd.ra;
+            tout.push_back(o);
+        }
+        h_cin = tin;
+        h_cout = tout;
+        d_etasks_cin = (EigTask*)put(tin.data(), sizeof(EigTask) * tin.size());
+        d_etasks_cout = (EigTask*)put(tout.data(), sizeof(EigTask) * tout.size());
+        CutUpdJob uj[2] = {{d_cut, u, ut, dlt, Sy}, {d_cut, ut, u, dlt, Sy}};
+        d_upd = (CutUpdJob*)put(uj, sizeof(uj));
+        cp.Cp = cut_Cp;
+        cp.Ep = cut_Ep;
+        cp.M = cut_MT;
+        cp.rt = RT;
+        cp.nrm = dnorm;
+        cp.b2 = dnorm + 2;
+        cp.ctl = cctl;
+        cp.max_iter = P.max_iter;
+        cp.stall = 0;
+        // squares of the FP64 test's window and of the reduction after which a round starts
+        // anew (see loop_cut)
+        cp.test2 = 1.05 * 1.05 * P.tol * P.tol;
+        cp.anchor2 = CUT_ANCHOR_RED * CUT_ANCHOR_RED;
+        if (upload) {
+            ck(cudaMemcpyAsync(d_cut_tab, blob.data(), blob.size(), cudaMemcpyHostToDevice, stream), cerr);
+            ck(cudaMemcpyAsync(d_cut, &cp, sizeof(cp), cudaMemcpyHostToDevice, stream), cerr);
+        }
+        return blob.size();
+    }
+    static constexpr double CUT_ANCHOR_RED = sizeof(T) == sizeof(float) ? 1e-2 : 1e-8;
+
+    // Rows, products and G blocks of level l's nodes (their bases and A_c^{-1} are done).
+    void cut_level_setup(int l) {
+        const CutLevel& cl = clev[l];
+        launch_cut_panels<T>(cl.cpe, cl.ncp, cl.epe, cl.nep, Sx, r, geom(0), stream);
+        if (cl.nprs) launch_cut_gram<T>(cl.prs, cl.nprs, cl.dst, cl.ndst, Sx, r, cut_part, stream);
+        launch_cut_minv<T>(cl.minv, cl.nminv, cp.D, L, 2 * r, cut_G, cut_M64, cut_MT, cp.cl, stream);
     }
 
     size_t plan(char* base) override {
@@ -565,10 +797,6 @@ struct Solver final : SolverBase {
         const size_t N = (size_t)Sy * Sx;
         u = a.take<c128>(N); ut = a.take<c128>(N); bvec = a.take<c128>(N); res = a.take<c128>(N);
         dlt = a.take<CT>(N);
-        if (recur_possible()) {
-            AC0 = a.take<CT>(N * 2 * (size_t)r);
-            RP = a.take<CT>(N);
-        }
         gbuf = a.take<c128>(4 * (size_t)S);
         khr_dev = P.k_rows ? a.take<double>(S) : nullptr;
         RT = a.take<CT>(N * nmax);
@@ -616,7 +844,9 @@ struct Solver final : SolverBase {
         npart = a.take<double>(2048);
         // [0] ||r||^2 (FP64 residual), [1] ||r||^2 (recursive residual), [2..4) ||b||^2,
         // [4..6) the device status words, [6..10) the device-tested loop's control words
-        dnorm = a.take<double>(10);
+        // and the cut-row iteration's control words from 10 on
+        dnorm = a.take<double>(10 + sizeof(CutCtl) / sizeof(double));
+        cctl = (CutCtl*)(dnorm + 10);
         derr = (int*)(dnorm + 4);
         dcounter = a.take<unsigned>(4);
         const int nleaf = 1 << L;
@@ -644,6 +874,33 @@ struct Solver final : SolverBase {
             gls.st = a.take<GmresState>(1);
         }
         d_ptrs = a.take<void*>(3 * 64);
+        if (cut) {
+            size_t ncp = 0, nep = 0;
+            cut_panel_sizes(ncp, nep);
+            EF0.assign(nn, nullptr);
+            for (int id : lev[L]) EF0[id] = a.take<CT>(pts(id));
+            cut_Cp = a.take<CT>(ncp);
+            cut_Ep = a.take<CT>(nep);
+            cut_E64 = a.take<c128>(nep);
+            cut_G = a.take<c128>((size_t)cp.D * cp.D);
+            cut_M64 = a.take<c128>((size_t)cp.D * cp.D);
+            cut_MT = a.take<CT>(cut_m_packed(L, r));
+            const size_t row = 2 * (size_t)cp.ncut * Sx;
+            cp.v = a.take<CT>(row);
+            cp.vsum = a.take<CT>(row);
+            cp.res0 = a.take<CT>(row);
+            cp.prow = a.take<CT>((size_t)cp.nA * 4 * Sx);
+            cp.pd = a.take<CT>((size_t)cp.nB * (L + 1) * r);
+            cp.d = a.take<CT>(cp.D);
+            cp.y = a.take<CT>(cp.D);
+            cp.yacc = a.take<CT>(cp.D);
+            cp.npart = a.take<float>((size_t)cp.nB * 8);
+            cbar = a.take<unsigned>(2);
+            d_cut = a.take<CutProb>(1);
+            if (!base) cut_tab_bytes = cut_tables(false);   // also sets cut_pairs_max
+            d_cut_tab = a.take<unsigned char>(cut_tab_bytes);
+            cut_part = (c128*)a.take<unsigned char>(cut_gram_scratch((int)cut_pairs_max));
+        }
         return align_up(a.off, 256);
     }
 
@@ -757,19 +1014,30 @@ struct Solver final : SolverBase {
             if (c) launch_tc_transform(stg == 0 ? 0 : 1, tasks, ntasks, b_max, Sx, nc, derr, stream, step_gate);
             else launch_eig_sweep_stage<T>(stg, tasks, ntasks, b_max, Sx, nc, stream, step_gate);
         };
+        run(tune_transform(stg, ntasks, nc, run));   // the outputs are those of the chosen candidate
+    }
+    template <class F> int tune_transform(int stg, int ntasks, int nc, F run) {
+        if (P.flags & HH_FLAG_TENSOR_CORE_SWEEPS) return 1;
         const TuneKey key{current_device(), 0, stg, b_max, Sx, nc * 64 + std::min(ntasks, 63)};
         int choice = 1;
-        if (P.flags & HH_FLAG_TENSOR_CORE_SWEEPS) choice = 1;
-        else if (!tune_find(key, choice)) {
-            if (stream_capturing(stream)) choice = 1;
-            else {
-                TuneEntry e{};
-                e.choice = tune_pair(stream, run, e.ms);
-                tune_store(key, e);
-                choice = e.choice;
-            }
+        if (!tune_find(key, choice) && !stream_capturing(stream)) {
+            TuneEntry e{};
+            e.choice = tune_pair(stream, run, e.ms);
+            tune_store(key, e);
+            choice = e.choice;
         }
-        run(choice);   // the outputs are those of the chosen candidate
+        return choice;
+    }
+    // The transform kernel of a round's full residual (stage 0) and summed result (stage 2);
+    // a shape's first use times both on this handle's own buffers (scratch between rounds).
+    int cut_choice(int stg) {
+        if (!tc) return 0;
+        const EigTask* t = stg == 0 ? d_etasks_cin : d_etasks_cout;
+        const int nl = (int)lev[L].size();
+        return tune_transform(stg, nl, 1, [&](int c) {
+            if (c) launch_tc_transform(stg == 0 ? 0 : 1, t, nl, b_max, Sx, 1, derr, stream);
+            else launch_eig_sweep_stage<T>(stg, t, nl, b_max, Sx, 1, stream);
+        });
     }
     void upload_eig_view_tasks(int nc) {
         std::vector<EigTask> t;
@@ -816,7 +1084,6 @@ struct Solver final : SolverBase {
             }
         }
         if (eig) {
-            h_pre = et;
             ck(cudaMemcpyAsync(d_etasks_pre, et.data(), sizeof(EigTask) * et.size(), cudaMemcpyHostToDevice, stream),
                cerr);
         }
@@ -1115,6 +1382,7 @@ struct Solver final : SolverBase {
             bt.AT[cnt++] = c64 ? (void*)AinvT[p] : nullptr;
         }
         launch_gj_inverse(bt, cnt, coarse_fp32(), stream);
+        if (cut) cut_level_setup(l - 1);
     }
 
     hh_status setup() override {
@@ -1142,6 +1410,10 @@ struct Solver final : SolverBase {
                                stream),
                cerr);
         }
+        if (cut) {
+            cut_tables(true);
+            zero(cut_G, sizeof(c128) * (size_t)cp.D * cp.D);
+        }
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
@@ -1154,7 +1426,6 @@ struct Solver final : SolverBase {
         for (int l = L; l >= 1; --l) sketch_level(l);
         upload_pre_tasks();
         tune_fused_cluster();
-        if (device_test_path() && recur_possible()) launch_apply_cols<T>(C[0], AC0, geom(0), 2 * r, stream);
         cudaEventRecord(e1, stream);
         hh_status st;
         const bool ok = sync_check(st);
@@ -1186,9 +1457,7 @@ struct Solver final : SolverBase {
     // RT, the leaf precision, when rt_ready):
     // out = base + sum_c P_c M_c R_c res (base null: zero; base may be out), then
     // out += C A_c^{-1} C^H (rhs - A out).
-    // recur: the root's extras forming the next residual recursively (null: none)
-    void oras_step(const c128* base, const c128* rhs, c128* out, bool rt_ready = false, const int* gate = nullptr,
-                   const CoarseRecur* recur = nullptr) {
+    void oras_step(const c128* base, const c128* rhs, c128* out, bool rt_ready = false, const int* gate = nullptr) {
         const size_t N = (size_t)Sy * Sx;
         step_gate = gate;
         if (!rt_ready) launch_copy<double, T>(res, RT, N, false, false, stream);
@@ -1216,12 +1485,9 @@ struct Solver final : SolverBase {
             // precision) less A applied to the update the level-1 kernel kept in dlt.
             // Both terms are in the leaf precision, like the correction computed from them;
             // the FP64 residual of the new iterate is formed afterwards as before.
-            // with the recursive residual also r' kept, the r columns of A C_0 at each point
-            // read and the next residual written; r complex multiply-adds per point
-            pjoin(PC_COARSE, coarse_bytes(0), 2.0 * 8.0 * 2 * r * N + (recur ? 8.0 * r * N : 0.0));
+            pjoin(PC_COARSE, coarse_bytes(0), 2.0 * 8.0 * 2 * r * N);
             CoarseBatch rb = one_job(0, RT, dlt, out, true);
             rb.gate = gate;
-            if (recur) rb.rr = *recur;
             launch_coarse_batch<T, T, T, double>(rb, 2 * r, partial, dcounter + 2, derr, stream);
         } else {
             pjoin(PC_COARSE, coarse_bytes(0), 2.0 * 8.0 * 2 * r * N);
@@ -1412,15 +1678,15 @@ struct Solver final : SolverBase {
 
     // residual b - A u into RT (the step's input; the FP64 vector itself is not kept), its
     // norm and the device stopping test (ctl), one launch; dcounter[0] is its ticket
-    void gated_residual(int* ctl, const int* need = nullptr, const int* anchor = nullptr) {
+    void gated_residual(int* ctl) {
         pbeg(PC_SPMV, 48.0 * (double)Sy * Sx);
-        launch_residual_stop<T>(u, bvec, nullptr, RT, geom(0), npart, dnorm, ctl, dcounter, P.tol, stream, need, anchor);
+        launch_residual_stop<T>(u, bvec, nullptr, RT, geom(0), npart, dnorm, ctl, dcounter, P.tol, stream);
         pend(PC_SPMV);
     }
 
     // the norms, the status words and the stop words (dnorm[0..8)) to the host
     bool read_norms(hh_status& st) {
-        ck(cudaMemcpyAsync(h_norm, dnorm, 10 * sizeof(double), cudaMemcpyDeviceToHost, stream), cerr);
+        ck(cudaMemcpyAsync(h_norm, dnorm, 10 * sizeof(double) + sizeof(CutCtl), cudaMemcpyDeviceToHost, stream), cerr);
         ck(cudaGetLastError(), cerr);
         ck(cudaStreamSynchronize(stream), cerr);
         if (cerr != cudaSuccess) { st = HH_ECUDA; return false; }
@@ -1436,28 +1702,8 @@ struct Solver final : SolverBase {
     // queued after the test passed does nothing, and u, the iteration count and the
     // final residual are those of the loop that tests after every step.  The number of
     // steps queued follows the contraction observed so far.
-    //
-    // In the complex64 form the residual that drives the steps is formed recursively by
-    // the root's correction, r_{k+1} = (r_k - A delta_1) - (A C_0) y_0 in the leaf
-    // precision, and replaced by the FP64 residual b - A u every RECUR_ANCHOR steps.  The FP64 residual is formed at those
-    // steps and wherever the recursive one comes within 2 tol: the stopping test always
-    // takes the FP64 residual, and the anchors depend on the step count only, so the
-    // iterates do not depend on when the test ran.
-    static constexpr int RECUR_ANCHOR = 8;
-    // The recursive residual serves the complex64 form: the FP64 form's residual is already
-    // in its working precision, and there the recursion's extra FP64 work costs more than
-    // the residual launch it saves.
-    // It reads the root's A~_0 C_0 (r columns at each point) in every step: worth it while
-    // that stays in the L2, not when it is read from HBM, where it costs about as much as the
-    // FP64 residual it replaces.
-    bool recur_possible() const {
-        const size_t ac_bytes = 2 * (size_t)r * Sy * Sx * sizeof(CT);
-        return sizeof(T) == sizeof(float) && eig && L >= 2 && P.n_inner == 1 && P.outer == HH_OUTER_ORAS &&
-               ac_bytes <= ((size_t)64 << 20) && !q1();
-    }
     hh_status loop_oras_device_test(int& it, double& rel) {
-        // [0] stop (1 converged, 2 not finite), [1] FP64 tests run, [2] FP64 residual due,
-        // [3] steps done, [4] anchor step
+        // [0] stop (1 converged, 2 not finite), [1] FP64 tests run
         int* ctl = (int*)(dnorm + 6);
         const int* hctl = (const int*)(h_norm + 6);
         hh_status st = HH_OK;
@@ -1465,17 +1711,6 @@ struct Solver final : SolverBase {
         zero(dcounter, 2 * sizeof(unsigned));   // the residual's and the root's tickets
         gated_residual(ctl);
         if (!read_norms(st)) return st;
-        const bool recur = recur_possible();
-        CoarseRecur rr{};
-        rr.AC = recur ? AC0 : nullptr;
-        rr.rp = RP;
-        rr.rt = RT;
-        rr.part = npart;
-        rr.ticket = dcounter + 1;
-        rr.nrm = dnorm;
-        rr.ctl = ctl;
-        rr.tol = P.tol;
-        rr.anchor = RECUR_ANCHOR;
         double rel_prev = -1.0;
         int it_prev = 0, chunks = 0;
         for (;;) {
@@ -1489,35 +1724,29 @@ struct Solver final : SolverBase {
                 rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;
                 return hctl[0] == 1 ? HH_OK : HH_ENOCONV;
             }
-            // the current residual: the recursive one once steps have run
-            const double relc =
-                (it == 0 || !recur) ? rel : (h_norm[2] > 0 ? std::sqrt(h_norm[1] / h_norm[2]) : 0.0);
             // Two chunks of 8 first: the residual of the first steps may grow before it
             // settles into its asymptotic rate, so a rate measured from step 0 overshoots.
             // Then the steps still needed at the rate of the last chunk, none to spare (a
             // short estimate costs one more synchronisation, a long one gated steps).
             int chunk = 8;
-            if (chunks >= 2 && it > it_prev && relc < rel_prev && relc > 0) {
-                const double rho = std::pow(relc / rel_prev, 1.0 / (it - it_prev));
-                const double need = std::log(P.tol / relc) / std::log(rho);
+            if (chunks >= 2 && it > it_prev && rel < rel_prev && rel > 0) {
+                const double rho = std::pow(rel / rel_prev, 1.0 / (it - it_prev));
+                const double need = std::log(P.tol / rel) / std::log(rho);
                 chunk = need < 64.0 ? std::max(1, (int)std::ceil(need)) : 64;
             }
             ++chunks;
-            rel_prev = relc;
+            rel_prev = rel;
             it_prev = it;
             const int n = std::max(1, std::min(chunk, P.max_iter - it));
-            // steps done: counted by the root's correction (recursive residual), else by
-            // the FP64 tests, one per step
-            const int count0 = recur ? hctl[3] : hctl[1];
+            const int count0 = hctl[1];   // steps done: one FP64 test per step
             const bool fresh = graphs[2].exec == nullptr;
             for (int k = 0; k < n; ++k)
                 replay_fresh(2, [&] {
-                    oras_step(u, bvec, u, true, ctl, recur ? &rr : nullptr);
-                    if (recur) gated_residual(ctl, ctl + 2, ctl + 4);
-                    else gated_residual(ctl);
+                    oras_step(u, bvec, u, true, ctl);
+                    gated_residual(ctl);
                 });
             const bool ok = read_norms(st);
-            const int ran = (recur ? hctl[3] : hctl[1]) - count0;
+            const int ran = hctl[1] - count0;
             // the first step of a new handle ran directly (its pairs are pending); the
             // replays that did work are the next ran - 1
             runs_release(graphs[2], (size_t)std::max(0, ran - (fresh ? 1 : 0)));
@@ -1526,8 +1755,99 @@ struct Solver final : SolverBase {
         }
     }
 
+    // The stationary iteration on the cut rows (k_cut.cu), in rounds.  A round starts from
+    // the FP64 residual of u, steps on the cut rows in the leaf precision until the residual
+    // there has fallen by CUT_ANCHOR_RED (an anchor), comes within 5% of tol |b| (a test is
+    // due), or the step limit, and then forms ut = u + M (the sum of the step inputs) and
+    // its FP64 residual.  The stopping test always takes that residual.  An anchor makes ut
+    // the next round's u; after a test that failed the steps go on where they stopped.  The
+    // anchors depend on the step residuals alone, so the iterates do not depend on tol.
+    hh_status loop_cut(int& it, double& rel) {
+        int* ctl = (int*)(dnorm + 6);
+        const CutCtl* hc = (const CutCtl*)(h_norm + 10);
+        hh_status st = HH_OK;
+        zero(ctl, 4 * sizeof(double) + sizeof(CutCtl));   // the residual's words and the steps'
+        zero(dcounter, 2 * sizeof(unsigned));
+        auto resid = [&](const c128* x) {
+            pbeg(PC_SPMV, 48.0 * (double)Sy * Sx);
+            // the steps' own residuals are counted, and the first
+            if (it > 0 && prof_cat(PC_SPMV)) prof_pending.back().nl = 0;
+            launch_residual_stop<T>(x, bvec, nullptr, RT, geom(0), npart, dnorm, ctl, dcounter, P.tol, stream);
+            pend(PC_SPMV);
+        };
+        resid(u);
+        int mode = 1;
+        bool cand = false;   // a candidate stands in ut
+        for (;;) {
+            if (!read_norms(st)) return st;
+            it = hc->it;
+            rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;
+            if (cand && (!std::isfinite(rel) || rel < P.tol || it >= P.max_iter || hc->reason != CUT_TEST)) {
+                std::swap(u, ut);
+                cut_flip ^= 1;
+                mode = 1;
+            } else if (cand) {
+                mode = 2;
+            }
+            if (!std::isfinite(rel)) return HH_ENOCONV;
+            if (rel < P.tol) return HH_OK;
+            if (it >= P.max_iter) return HH_ENOCONV;
+            const int nl = (int)lev[L].size();
+            if (mode == 1) eig_stage_prof(0, d_etasks_cin);
+            if (!launch_cut_steps<T>(d_cut, 1, cut_group(), cp.cl, cut_smem, nullptr, mode, cbar, 1, derr, prof_on, stream))
+                return HH_ECUDA;
+            launch_cut_lines<T>(d_cut, 1, nullptr, nl, b_max, Sx, stream);
+            eig_stage_prof(2, d_etasks_cout);
+            launch_cut_update<T>(d_upd + cut_flip, 1, Sy, Sx, stream);
+            it = 1;   // residual launches from here on belong to steps already counted
+            resid(ut);
+            cand = true;
+        }
+    }
+    int cut_flip = 0;
+    // blocks of the steps' group: one per item of the larger phase, at most one per SM
+    int cut_group() const { return std::min(148, std::max(cp.nA, cp.nB)); }
+    void eig_stage_prof(int stg, const EigTask* tasks) {
+        double by = 0.0, fl = 0.0;
+        for (int id : lev[L]) {
+            const double b = nodes[id].b(), sx = Sx;
+            fl += 8.0 * b * b * sx;
+            by += sizeof(CT) * (b * b + 2.0 * b * sx);
+        }
+        // time of the single-vector sweeps (the steps are the counted ones)
+        pbeg(PC_SWEEP, by, fl);
+        if (prof_cat(PC_SWEEP)) prof_pending.back().nl = 0;
+        eig_sweep_stage(stg, tasks, (int)lev[L].size(), 1);
+        pend(PC_SWEEP);
+    }
+    // The steps' phases to the profiler: the kernel's own clock (one leaf sweep, L coarse
+    // corrections and one residual per step).
+    void cut_prof(int steps) {
+        const CutCtl* hc = (const CutCtl*)(h_norm + 10);
+        size_t ncp = 0, nep = 0;
+        cut_panel_sizes(ncp, nep);
+        double lines = 0.0;
+        for (int id : lev[L]) lines += (double)nodes[id].b() * Sx;
+        const struct { int cat, n, ph; double by, fl; } c[3] = {
+            {PC_SWEEP, 1, 0, sizeof(CT) * lines, (8.0 * 8 + 28.0) * lines},
+            {PC_COARSE, L, 1, (double)sizeof(CT) * ncp, 8.0 * ncp},
+            {PC_SPMV, 1, 2, (double)sizeof(CT) * nep, 8.0 * nep}};
+        for (auto& x : c) {
+            if (!prof_cat(x.cat)) continue;
+            prof_ms[x.cat] += hc->ns[x.ph] * 1e-6;
+            prof_n[x.cat] += (long long)x.n * steps;
+            prof_bytes[x.cat] += x.by * steps;
+            prof_flops[x.cat] += x.fl * steps;
+        }
+    }
+
     // Stationary iteration u <- u + M (b - A u)  (Eqs. (2)-(3)).
     hh_status loop_oras(int& it, double& rel) {
+        if (cut) {
+            const hh_status cs = loop_cut(it, rel);
+            if (prof_on) cut_prof(it);
+            return cs;
+        }
         if (device_test_path()) return loop_oras_device_test(it, rel);
         hh_status st = HH_OK;
         for (;;) {
@@ -1825,382 +2145,269 @@ static hh_status setup_one(const hh_params* p, cudaStream_t s, SolverBase** out,
 }
 
 // ------------------------------------------------------------------ batched solves
-// Several set-up problems solved together in lockstep (the batching form): per iteration
-// one residual launch and one norm launch for all of them, one one-launch leaf sweep over
-// all their leaves, one cooperative coarse launch per height of the hierarchy over all
-// their nodes, and one for all roots; a problem leaves the batch when it converges.
-// Requires the stationary outer iteration, n_i = 1, the eigenbasis leaf path with the
-// one-launch sweep and at least two levels, for every problem, in one precision.
+// Several set-up problems solved together (the batching form).  Requires the stationary
+// iteration on the cut rows (n_i = 1, eigenbasis leaves) of the 5-point rows with leaves that
+// fit the one-launch sweep, for every problem, in one precision.
 template <typename T>
 static bool batchable(const Solver<T>* p) {
-    return p->eig && p->eig_fused && p->pre_direct && p->P.n_inner == 1 && p->P.outer == HH_OUTER_ORAS && p->L >= 2 &&
-           !p->q1();
+    return p->cut && p->eig_fused && p->pre_direct && p->P.outer == HH_OUTER_ORAS && !p->q1();
 }
 
-// Lockstep iteration of several set-up problems: the engine of the batching and serving
+// Iteration of several set-up problems together: the engine of the batching and serving
 // forms.  Problems are added with their right-hand sides and leave when they converge (or
-// when the stationary iteration stops contracting for them); each step() is one
-// iteration for all current problems: one residual launch and one norm launch, one
-// one-launch leaf sweep over all their leaves, one cooperative coarse launch per
-// hierarchy height and one for the roots.
+// when the stationary iteration stops contracting for them).  Each step() is one round
+// (see Solver::loop_cut) of every current problem: one transform launch per problem shape,
+// one launch in which the problems' clusters (or grid groups) run their steps to their next
+// stop side by side, and one launch each for the lines, the update and the residual.  A
+// problem's arithmetic is that of its own solve, whatever shares the launches.
 template <typename T>
 struct BatchEngine {
     struct Prob {
         Solver<T>* p = nullptr;
         c128* uo = nullptr;          // where the solution goes when the problem leaves
         void* tag = nullptr;
-        unsigned long long serial = 0;   // unique per add(): the key of the task upload
-        int it = 0, chk_it = 0;
-        double rel = 0.0, best = 0.0, chk = 0.0;
+        int slot = 0, it = 0;
+        int mode = 0;                // of the next round; 0: its first residual is due
+        double rel = 0.0;
         hh_status st = HH_OK;
-        bool live = true;                // false once it has left (its jobs gated off)
     };
     cudaStream_t stream = nullptr;
     int cap_probs = 0, cap_tasks = 0;
     AllocHook hook;
     char* base = nullptr;
     size_t bytes = 0;
+    CutProb* d_probs = nullptr;      // by slot
+    int* d_modes = nullptr;          // by slot: cluster problems, then grid problems
+    CutUpdJob* d_jobs = nullptr;
     EigTask* d_tasks = nullptr;
     double* part = nullptr;
-    double* norms = nullptr;
-    c128* cpart = nullptr;
-    unsigned* bar = nullptr;
+    double* norms = nullptr;         // by slot; then the status word and the control words
+    CutCtl* d_ctl = nullptr;
     int* berr = nullptr;
-    double* h_norms = nullptr;       // pinned
+    unsigned* bars = nullptr;
+    char *h_up = nullptr, *h_dn = nullptr;   // pinned: uploads, read-back
+    size_t up_bytes = 0, dn_bytes = 0;
     int part_cap = RB_MAX_JOBS * 304;
+    static constexpr int MAX_GROUPS = 64;
     std::vector<Prob> act;
-    // serials of the problems whose leaf tasks are in d_tasks (a freed solver's address
-    // can come back for a new problem, so addresses are no key)
-    std::vector<unsigned long long> uploaded;
-    unsigned long long next_serial = 1;
-    int cl = 0, bmax = 0, sxmax = 0;
+    std::vector<char> used;
     cudaError_t cerr = cudaSuccess;
-    // One lockstep iteration after the first (the preconditioner step of every current
-    // problem, then their residuals for the next test) is a CUDA graph, captured on a
-    // private stream for the current set of problems and replayed while the set stays.
-    cudaStream_t cap_stream = nullptr;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t gexec = nullptr;
-    std::vector<unsigned long long> graph_key;
-    bool resid_pending = false;   // the current problems' residuals are already enqueued
-    unsigned long long replays = 0, captures = 0;
-    // Gate word per position of act: a problem that leaves keeps its place in the captured
-    // graph with its word set, so that its jobs return at once; the set is compacted (and
-    // the graph captured again) when a quarter of it has left or a problem joins.
-    int* gates = nullptr;
-    bool joined = false;
 
     hh_status init(cudaStream_t s, int probs, int tasks, const AllocHook& h) {
         stream = s;
         cap_probs = std::max(probs, 1);
         cap_tasks = std::max(tasks, 1);
         hook = h;
-        bytes = align_up(sizeof(EigTask) * cap_tasks, 256) + align_up(sizeof(double) * part_cap, 256) +
-                align_up(sizeof(double) * (cap_probs + 8), 256) + align_up(sizeof(c128) * 304 * 64, 256) + 256 +
-                align_up(sizeof(int) * cap_probs, 256);
+        used.assign(cap_probs, 0);
+        auto lay = [&](char* b0) {
+            size_t off = 0;
+            auto take = [&](size_t b) { char* q = b0 + off; off += align_up(b, 256); return q; };
+            d_probs = (CutProb*)take(sizeof(CutProb) * cap_probs);
+            // one upload: modes, jobs, tasks
+            d_modes = (int*)take(sizeof(int) * 2 * cap_probs);
+            d_jobs = (CutUpdJob*)take(sizeof(CutUpdJob) * cap_probs);
+            d_tasks = (EigTask*)take(sizeof(EigTask) * 2 * cap_tasks);
+            up_bytes = (size_t)((char*)d_tasks - (char*)d_modes) + sizeof(EigTask) * 2 * cap_tasks;
+            // one read-back: norms, control words, status
+            norms = (double*)take(sizeof(double) * cap_probs);
+            d_ctl = (CutCtl*)take(sizeof(CutCtl) * cap_probs);
+            berr = (int*)take(256);
+            dn_bytes = (size_t)((char*)berr - (char*)norms) + sizeof(int);
+            part = (double*)take(sizeof(double) * part_cap);
+            bars = (unsigned*)take(sizeof(unsigned) * MAX_GROUPS);
+            return off;
+        };
+        bytes = lay(nullptr);
         base = (char*)dev_alloc(bytes, stream, hook);
         if (!base) return HH_ENOMEM;
-        size_t off = 0;
-        auto take = [&](size_t b) { char* q = base + off; off += align_up(b, 256); return q; };
-        d_tasks = (EigTask*)take(sizeof(EigTask) * cap_tasks);
-        part = (double*)take(sizeof(double) * part_cap);
-        norms = (double*)take(sizeof(double) * (cap_probs + 8));
-        cpart = (c128*)take(sizeof(c128) * 304 * 64);
-        bar = (unsigned*)take(256);
-        berr = (int*)(bar + 4);
-        gates = (int*)take(sizeof(int) * cap_probs);
-        ck(cudaMemsetAsync(gates, 0, sizeof(int) * cap_probs, stream), cerr);
-        ck(cudaMallocHost(&h_norms, sizeof(double) * (cap_probs + 8)), cerr);
-        ck(cudaMemsetAsync(bar, 0, 256, stream), cerr);
+        lay(base);
+        ck(cudaMallocHost(&h_up, up_bytes + sizeof(CutProb) * cap_probs), cerr);
+        ck(cudaMallocHost(&h_dn, dn_bytes), cerr);
+        ck(cudaMemsetAsync(berr, 0, sizeof(int), stream), cerr);
         return cerr == cudaSuccess ? HH_OK : HH_ECUDA;
     }
-    void drop_graph() {
-        if (gexec) cudaGraphExecDestroy(gexec);
-        if (graph) cudaGraphDestroy(graph);
-        gexec = nullptr;
-        graph = nullptr;
-        graph_key.clear();
-    }
     void release() {
-        drop_graph();
-        if (cap_stream) cudaStreamDestroy(cap_stream);
-        cap_stream = nullptr;
-        if (h_norms) cudaFreeHost(h_norms);
-        h_norms = nullptr;
+        if (h_up) cudaFreeHost(h_up);
+        if (h_dn) cudaFreeHost(h_dn);
+        h_up = h_dn = nullptr;
         if (base) dev_free(base, bytes, stream, hook);
         base = nullptr;
     }
+    void clear() {
+        act.clear();
+        std::fill(used.begin(), used.end(), 0);
+    }
     int tasks_in_use() const {
         int n = 0;
-        for (auto& q : act)
-            if (q.live) n += (int)q.p->h_pre.size();
+        for (auto& q : act) n += 1 << q.p->L;
         return n;
     }
-    int live_count() const {
-        int n = 0;
-        for (auto& q : act) n += q.live;
-        return n;
-    }
-    // whether p can join: lockstep-able, room left, and a fused-sweep cluster size that
-    // serves every member
+    // whether p can join: taken by the iteration on the cut rows, and room left
     bool can_add(Solver<T>* p) const {
-        if (!batchable(p) || live_count() >= cap_probs) return false;
-        if (tasks_in_use() + (int)p->h_pre.size() > cap_tasks) return false;
-        int bm = p->b_max, sx = p->Sx, smin = p->Sx;
-        for (auto& q : act) {
-            if (!q.live) continue;
-            bm = std::max(bm, q.p->b_max);
-            sx = std::max(sx, q.p->Sx);
-            smin = std::min(smin, q.p->Sx);
-        }
-        const int c = eig_sweep_fused_ready<T>(bm, sx);
-        return c && c <= smin;
+        return batchable(p) && (int)act.size() < cap_probs && tasks_in_use() + (1 << p->L) <= cap_tasks &&
+               (!p->cp.cl || cut_cluster_ready(p->cut_smem));
     }
     // enqueue the right-hand side, ||b||^2 and u = 0 of a problem that joins
     void add(Solver<T>* p, const c128* f, const c128* g, c128* uo, void* tag) {
         p->stream = stream;
-        p->zero(p->derr, sizeof(int) * 4);
-        launch_rhs(f, g, p->bvec, p->P.dim, p->S, p->h, stream, p->q1());
-        p->norm_sq(p->bvec, p->dnorm + 2);
-        ck(cudaMemcpyAsync(p->h_norm + 2, p->dnorm + 2, sizeof(double), cudaMemcpyDeviceToHost, stream), cerr);
-        p->zero(p->u, sizeof(c128) * (size_t)p->Sy * p->Sx);
         Prob q;
         q.p = p;
         q.uo = uo;
         q.tag = tag;
-        q.serial = next_serial++;
-        q.it = -1;   // the first step reads ||b||^2
-        compact();   // a joining problem takes its place in a set without departed ones
+        while (used[q.slot]) ++q.slot;
+        used[q.slot] = 1;
+        launch_rhs(f, g, p->bvec, p->P.dim, p->S, p->h, stream, p->q1());
+        p->norm_sq(p->bvec, p->dnorm + 2);
+        ck(cudaMemcpyAsync(p->h_norm + 2, p->dnorm + 2, sizeof(double), cudaMemcpyDeviceToHost, stream), cerr);
+        p->zero(p->u, sizeof(c128) * (size_t)p->Sy * p->Sx);
+        CutProb* hp = (CutProb*)(h_up + up_bytes) + q.slot;   // read by the copy before the slot's next use
+        *hp = p->cp;
+        hp->nrm = norms + q.slot;
+        hp->b2 = p->dnorm + 2;
+        hp->ctl = d_ctl + q.slot;
+        hp->stall = 1;
+        ck(cudaMemcpyAsync(d_probs + q.slot, hp, sizeof(CutProb), cudaMemcpyHostToDevice, stream), cerr);
+        ck(cudaMemsetAsync(d_ctl + q.slot, 0, sizeof(CutCtl), stream), cerr);
         act.push_back(q);
-        ck(cudaMemsetAsync(gates, 0, sizeof(int) * act.size(), stream), cerr);
-        resid_pending = false;   // the next step enqueues every current problem's residual
-        joined = true;
     }
-    // drop the departed problems from the set (positions change: the gate words are reset)
-    void compact() {
-        std::vector<Prob> keep;
-        for (auto& q : act)
-            if (q.live) keep.push_back(q);
-        if (keep.size() == act.size()) return;
-        act.swap(keep);
-        ck(cudaMemsetAsync(gates, 0, sizeof(int) * std::max<size_t>(act.size(), 1), stream), cerr);
-    }
-    // One iteration for every current problem; problems that leave are appended to `done`
-    // (their solution already copied to uo, the copy complete).
-    // Residuals of every current problem (norms[k] for act[k]), enqueued on `stream`.
-    void enqueue_residuals() {
-        const int na = (int)act.size();
-        for (int c0 = 0; c0 < na; c0 += RB_MAX_JOBS) {
-            ResidBatch rb{};
-            for (int k = c0; k < na && k < c0 + RB_MAX_JOBS; ++k) {
-                Solver<T>* p = act[k].p;
-                ResidJob& j = rb.job[rb.njobs++];
-                j.x = p->u;
-                j.v = p->bvec;
-                j.y = p->res;
-                j.yt = p->RT;
-                j.g = p->geom(0);
-                j.gate = gates + k;
+    // FP64 residuals of the problems sel (their u, or ut): norms[slot]
+    template <class Sel, class X> void residuals(Sel sel, X x) {
+        ResidBatch rb{};
+        for (auto& q : act) {
+            if (!sel(q)) continue;
+            ResidJob& j = rb.job[rb.njobs++];
+            j.x = x(q);
+            j.v = q.p->bvec;
+            j.yt = q.p->RT;
+            j.g = q.p->geom(0);
+            j.norm = norms + q.slot;
+            if (rb.njobs == RB_MAX_JOBS) {
+                launch_residual_batch<T>(rb, part, part_cap, stream);
+                rb = ResidBatch{};
             }
-            launch_residual_batch<T>(rb, part, part_cap, norms + c0, stream);
         }
+        launch_residual_batch<T>(rb, part, part_cap, stream);
     }
-    hh_status step(std::vector<Prob>& done) {
-        if (act.empty()) return HH_OK;
-        const int na = (int)act.size();
-        if (!resid_pending) enqueue_residuals();
-        resid_pending = false;
-        ck(cudaMemcpyAsync(h_norms, norms, sizeof(double) * na, cudaMemcpyDeviceToHost, stream), cerr);
-        ck(cudaMemcpyAsync(h_norms + cap_probs, berr, sizeof(int), cudaMemcpyDeviceToHost, stream), cerr);
+    hh_status read_back() {
+        ck(cudaMemcpyAsync(h_dn, norms, dn_bytes, cudaMemcpyDeviceToHost, stream), cerr);
+        ck(cudaGetLastError(), cerr);
         ck(cudaStreamSynchronize(stream), cerr);
         if (cerr != cudaSuccess) return HH_ECUDA;
-        if (*(const int*)(h_norms + cap_probs) == DEV_TIMEOUT) return HH_ETIMEOUT;
-        bool left = false;
-        for (int k = 0; k < na; ++k) {
-            Prob& q = act[k];
-            if (!q.live) continue;
-            if (q.it < 0) q.it = 0;
-            const double b2 = q.p->h_norm[2];
-            q.rel = b2 > 0 ? std::sqrt(h_norms[k] / b2) : 0.0;
-            if (q.it == 0) q.best = q.chk = q.rel;
-            q.best = std::min(q.best, q.rel);
-            // the stationary iteration is not a contraction for every problem: one whose
-            // residual has grown a hundredfold past its best, or fell less than tenfold over
-            // the last 25 steps, leaves early (its owner solves it by GMRES)
-            bool slow = false;
-            if (q.it - q.chk_it >= 25) {
-                slow = q.rel > 0.1 * q.chk;
-                q.chk = q.rel;
-                q.chk_it = q.it;
-            }
-            bool out = true;
-            if (!std::isfinite(q.rel) || q.rel > 100.0 * q.best || (slow && q.rel >= q.p->P.tol)) q.st = HH_ENOCONV;
-            else if (q.rel < q.p->P.tol) q.st = HH_OK;
-            else if (q.it >= q.p->P.max_iter) q.st = HH_ENOCONV;
-            else out = false;
-            if (out) {
-                ck(cudaMemcpyAsync(q.uo, q.p->u, sizeof(c128) * (size_t)q.p->Sy * q.p->Sx, cudaMemcpyDeviceToDevice,
-                                   stream),
-                   cerr);
-                // its jobs in the captured graph return at once from now on
-                const int one = 1;
-                ck(cudaMemcpyAsync(gates + k, &one, sizeof(int), cudaMemcpyHostToDevice, stream), cerr);
-                q.live = false;
-                done.push_back(q);
-                left = true;
-            }
-        }
-        if (left) ck(cudaStreamSynchronize(stream), cerr);
-        const int nl = live_count();
-        if (nl == 0) {
-            act.clear();
-            drop_graph();
-            return cerr == cudaSuccess ? HH_OK : HH_ECUDA;
-        }
-        // compact once a quarter of the set has left (the graph is captured again)
-        if (4 * (na - nl) >= na) compact();
-        joined = false;
-        // one preconditioner step for every current problem
-        std::vector<Solver<T>*> ids;
-        std::vector<unsigned long long> key;
-        for (auto& q : act) {
-            ids.push_back(q.p);
-            key.push_back(q.serial);
-        }
-        if (key != uploaded) {
-            std::vector<EigTask> tk;
-            bmax = sxmax = 0;
-            int smin = 1 << 30;
-            for (size_t k = 0; k < ids.size(); ++k) {
-                Solver<T>* p = ids[k];
-                for (EigTask t : p->h_pre) {
-                    t.gate = gates + k;
-                    tk.push_back(t);
-                }
-                bmax = std::max(bmax, p->b_max);
-                sxmax = std::max(sxmax, p->Sx);
-                smin = std::min(smin, p->Sx);
-            }
-            cl = eig_sweep_fused_ready<T>(bmax, sxmax);
-            if (!cl || cl > smin) return HH_ENOTIMPL;
-            ck(cudaMemcpyAsync(d_tasks, tk.data(), sizeof(EigTask) * tk.size(), cudaMemcpyHostToDevice, stream),
-               cerr);
-            // the pageable source must stay alive until the copy has read it
-            ck(cudaStreamSynchronize(stream), cerr);
-            uploaded = key;
-        }
-        if (key != graph_key) {
-            // capture the iteration for this set of problems: the preconditioner step and
-            // the residuals of the next test (launches only: no host synchronisation inside)
-            drop_graph();
-            if (!cap_stream) ck(cudaStreamCreateWithFlags(&cap_stream, cudaStreamNonBlocking), cerr);
-            cudaStream_t user = stream;
-            bool ok = cerr == cudaSuccess &&
-                      cudaStreamBeginCapture(cap_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-            if (ok) {
-                stream = cap_stream;
-                enqueue_precond(ids);
-                enqueue_residuals();
-                stream = user;
-                ok = cudaStreamEndCapture(cap_stream, &graph) == cudaSuccess && graph &&
-                     cudaGraphInstantiate(&gexec, graph, 0) == cudaSuccess;
-            }
-            stream = user;
-            if (!ok) {
-                cudaGetLastError();
-                drop_graph();
-                return HH_ECUDA;
-            }
-            graph_key = key;
-            ++captures;
-        }
-        ck(cudaGraphLaunch(gexec, stream), cerr);
-        ++replays;
-        resid_pending = true;
-        for (auto& q : act)
-            if (q.live) ++q.it;
-        ck(cudaGetLastError(), cerr);
-        return cerr == cudaSuccess ? HH_OK : HH_ECUDA;
+        const int e = *(const int*)(h_dn + ((char*)berr - (char*)norms));
+        return e == DEV_TIMEOUT ? HH_ETIMEOUT : e != DEV_OK ? HH_ECUDA : HH_OK;
     }
-
-    // One preconditioner step for the problems `ids` (the current set, in order).
-    void enqueue_precond(const std::vector<Solver<T>*>& ids) {
-        int nt = 0, lmax = 0;
-        for (auto* p : ids) {
-            nt += (int)p->h_pre.size();
-            lmax = std::max(lmax, p->L);
+    const CutCtl& ctl_of(const Prob& q) const { return ((const CutCtl*)(h_dn + ((char*)d_ctl - (char*)norms)))[q.slot]; }
+    double rel_of(const Prob& q) const {
+        const double b2 = q.p->h_norm[2], r2 = ((const double*)h_dn)[q.slot];
+        return b2 > 0 ? std::sqrt(r2 / b2) : 0.0;
+    }
+    // the problem leaves with the solution in x (the copy is complete after `settle`)
+    void leave(Prob& q, hh_status st, const c128* x, std::vector<Prob>& done) {
+        ck(cudaMemcpyAsync(q.uo, x, sizeof(c128) * (size_t)q.p->Sy * q.p->Sx, cudaMemcpyDeviceToDevice, stream), cerr);
+        q.st = st;
+        used[q.slot] = 0;
+        done.push_back(q);
+        q.p = nullptr;
+    }
+    void settle() {
+        const size_t n0 = act.size();
+        act.erase(std::remove_if(act.begin(), act.end(), [](const Prob& q) { return !q.p; }), act.end());
+        if (act.size() != n0) ck(cudaStreamSynchronize(stream), cerr);
+    }
+    // One round of every current problem; problems that leave are appended to `done`
+    // (their solution already copied to uo, the copy complete).
+    hh_status step(std::vector<Prob>& done) {
+        if (act.empty()) return HH_OK;
+        bool fresh = false;
+        for (auto& q : act) fresh |= q.mode == 0;
+        if (fresh) {
+            residuals([](const Prob& q) { return q.mode == 0; }, [](const Prob& q) { return q.p->u; });
+            const hh_status st = read_back();
+            if (st != HH_OK) return st;
+            for (auto& q : act) {
+                if (q.mode) continue;
+                q.mode = 1;
+                q.rel = rel_of(q);
+                if (!std::isfinite(q.rel)) leave(q, HH_ENOCONV, q.p->u, done);
+                else if (q.rel < q.p->P.tol) leave(q, HH_OK, q.p->u, done);
+            }
+            settle();
+            if (act.empty()) return cerr == cudaSuccess ? HH_OK : HH_ECUDA;
         }
-        launch_eig_sweep_fused<T>(cl, d_tasks, nt, bmax, sxmax, stream);
-        // internal nodes, deepest first: height = L - level; level 1 writes into u (FP64)
-        for (int hgt = 1; hgt < lmax; ++hgt) {
-            for (int to64 = 0; to64 < 2; ++to64) {
-                struct NodeJob {
-                    Solver<T>* p;
-                    int id, k;   // node, position of the problem in the set
-                };
-                std::vector<NodeJob> jobs;
-                for (size_t k = 0; k < ids.size(); ++k) {
-                    Solver<T>* p = ids[k];
-                    const int l = p->L - hgt;
-                    if (l < 1 || (l == 1) != (to64 == 1)) continue;
-                    for (int id : p->lev[l]) jobs.push_back({p, id, (int)k});
+        // the round's tables
+        int* modes = (int*)h_up;
+        CutUpdJob* jobs = (CutUpdJob*)(h_up + ((char*)d_jobs - (char*)d_modes));
+        EigTask* tasks = (EigTask*)(h_up + ((char*)d_tasks - (char*)d_modes));
+        std::fill(modes, modes + 2 * cap_probs, 0);
+        struct Shape { int b_max, Sx, in, out; };
+        std::map<std::tuple<int, int, int, int>, std::vector<Prob*>> shapes;   // (b_max, Sx, choices in and out)
+        int top = 0, ncl = 0, ngr = 0, group = 1, nleaf = 1, bm = 0, sx = 0;
+        size_t sm_cl = 0, sm_gr = 0;
+        for (auto& q : act) {
+            Solver<T>* p = q.p;
+            top = std::max(top, q.slot + 1);
+            modes[(p->cp.cl ? 0 : cap_probs) + q.slot] = q.mode;
+            if (p->cp.cl) { ++ncl; sm_cl = std::max(sm_cl, p->cut_smem); }
+            else { ++ngr; sm_gr = std::max(sm_gr, p->cut_smem); group = std::max(group, p->cut_group()); }
+            nleaf = std::max(nleaf, 1 << p->L);
+            bm = std::max(bm, p->b_max);
+            sx = std::max(sx, p->Sx);
+            shapes[{p->b_max, p->Sx, p->cut_choice(0), p->cut_choice(2)}].push_back(&q);
+        }
+        int nj = 0, nt = 0;
+        struct Run { int first, n, b_max, Sx, choice, stage; };
+        std::vector<Run> runs;
+        for (auto& q : act) jobs[nj++] = {d_probs + q.slot, q.p->u, q.p->ut, q.p->dlt, q.p->Sy};
+        for (int stage = 0; stage <= 2; stage += 2)
+            for (auto& kv : shapes) {
+                const auto [b, x, ci, co] = kv.first;
+                Run r{nt, 0, b, x, stage == 0 ? ci : co, stage};
+                for (Prob* q : kv.second) {
+                    if (stage == 0 && q->mode != 1) continue;
+                    for (const EigTask& t : stage == 0 ? q->p->h_cin : q->p->h_cout) tasks[nt++] = t;
                 }
-                std::vector<int> widths;   // one launch per basis width and per CB_MAX_JOBS nodes
-                for (auto& jn : jobs)
-                    if (std::find(widths.begin(), widths.end(), 2 * jn.p->r) == widths.end())
-                        widths.push_back(2 * jn.p->r);
-                for (int w : widths) {
-                    CoarseBatch bt{};
-                    auto flush = [&]() {
-                        if (!bt.njobs) return;
-                        if (to64) launch_coarse_batch<T, T, T, double>(bt, w, cpart, bar, berr, stream);
-                        else launch_coarse_batch<T, T, T, T>(bt, w, cpart, bar, berr, stream);
-                        bt = CoarseBatch{};
-                    };
-                    for (auto& jn : jobs) {
-                        Solver<T>* p = jn.p;
-                        if (2 * p->r != w) continue;
-                        const int id = jn.id;
-                        const Node& nd = p->nodes[id];
-                        CoarseJob& j = bt.job[bt.njobs++];
-                        j.C = p->C[id];
-                        j.v = p->RT + p->row_off(0, nd.ra, 1);
-                        j.w_in = p->W[id];
-                        j.out = to64 ? (void*)(p->u + p->row_off(0, nd.own_a, 1))
-                                     : (void*)(p->W[nd.parent] + p->row_off(nd.parent, nd.own_a, 1));
-                        j.Minv = p->AinvT[id];
-                        j.y = p->ycoef[id];
-                        j.g = p->geom(id);
-                        j.r0 = nd.own_a - nd.ra;
-                        j.r1 = nd.own_b - nd.ra;
-                        j.acc_out = to64;
-                        j.add_w = 1;
-                        j.split = p->split_row(id);
-                        j.gate = gates + jn.k;
-                        if (bt.njobs == CB_MAX_JOBS) flush();
-                    }
-                    flush();
-                }
+                r.n = nt - r.first;
+                if (r.n) runs.push_back(r);
+            }
+        ck(cudaMemcpyAsync(d_modes, h_up, (size_t)((char*)(tasks + nt) - h_up), cudaMemcpyHostToDevice, stream), cerr);
+        auto transforms = [&](int stage) {
+            for (const Run& r : runs) {
+                if (r.stage != stage) continue;
+                if (r.choice) launch_tc_transform(stage == 0 ? 0 : 1, d_tasks + r.first, r.n, r.b_max, r.Sx, 1, berr, stream);
+                else launch_eig_sweep_stage<T>(stage, d_tasks + r.first, r.n, r.b_max, r.Sx, 1, stream);
+            }
+        };
+        transforms(0);
+        bool ok = true;
+        if (ncl) ok = launch_cut_steps<T>(d_probs, top, 0, true, sm_cl, d_modes, 0, bars, MAX_GROUPS, berr, 0, stream);
+        // grid groups: a quarter of the SMs each when several problems run side by side
+        if (ok && ngr)
+            ok = launch_cut_steps<T>(d_probs, top, std::max(16, ngr >= 4 ? group / 4 : ngr >= 2 ? group / 2 : group), false,
+                                     sm_gr, d_modes + cap_probs, 0, bars, MAX_GROUPS, berr, 0, stream);
+        if (!ok) return HH_ECUDA;
+        // (a slot without a problem has both its modes zero)
+        if (ncl) launch_cut_lines<T>(d_probs, top, d_modes, nleaf, bm, sx, stream);
+        if (ngr) launch_cut_lines<T>(d_probs, top, d_modes + cap_probs, nleaf, bm, sx, stream);
+        transforms(2);
+        launch_cut_update<T>(d_jobs, nj, sx, sx, stream);
+        residuals([](const Prob&) { return true; }, [](const Prob& q) { return q.p->ut; });
+        const hh_status st = read_back();
+        if (st != HH_OK) return st;
+        for (auto& q : act) {
+            const CutCtl& c = ctl_of(q);
+            q.it = c.it;
+            q.rel = rel_of(q);
+            if (!std::isfinite(q.rel)) leave(q, HH_ENOCONV, q.p->ut, done);
+            else if (q.rel < q.p->P.tol) leave(q, HH_OK, q.p->ut, done);
+            else if (c.reason == CUT_STALL || q.it >= q.p->P.max_iter) leave(q, HH_ENOCONV, q.p->ut, done);
+            else if (c.reason == CUT_TEST) q.mode = 2;
+            else {
+                std::swap(q.p->u, q.p->ut);
+                q.mode = 1;
             }
         }
-        // the roots: u += C A_c^{-1} C^H (b - A u)
-        std::vector<int> widths;
-        for (auto* p : ids)
-            if (std::find(widths.begin(), widths.end(), 2 * p->r) == widths.end()) widths.push_back(2 * p->r);
-        for (int w : widths) {
-            CoarseBatch bt{};
-            for (size_t k = 0; k < ids.size(); ++k) {
-                Solver<T>* p = ids[k];
-                if (2 * p->r != w) continue;
-                bt.job[bt.njobs] = p->one_job(0, p->bvec, p->u, p->u, true).job[0];
-                bt.job[bt.njobs++].gate = gates + k;
-                if (bt.njobs == CB_MAX_JOBS) {
-                    launch_coarse_batch<T, double, double, double>(bt, w, cpart, bar, berr, stream);
-                    bt = CoarseBatch{};
-                }
-            }
-            if (bt.njobs) launch_coarse_batch<T, double, double, double>(bt, w, cpart, bar, berr, stream);
-        }
+        settle();
+        return cerr == cudaSuccess ? HH_OK : HH_ECUDA;
     }
 };
 
@@ -2209,13 +2416,13 @@ static hh_status batch_solve(std::vector<Solver<T>*>& ps, const c128* const* f, 
                              c128* const* uo, cudaStream_t stream, hh_stats* stats, std::vector<hh_status>& res) {
     const int np = (int)ps.size();
     int nleaf = 0;
-    for (auto* p : ps) nleaf += (int)p->h_pre.size();
+    for (auto* p : ps) nleaf += 1 << p->L;
     BatchEngine<T> eng;
     eng.cap_probs = np;
     eng.cap_tasks = nleaf;
     for (auto* p : ps) {
         if (!eng.can_add(p)) return HH_ENOTIMPL;
-        eng.act.push_back({});   // capacity and cluster checks against the members so far
+        eng.act.push_back({});   // capacity checks against the members so far
         eng.act.back().p = p;
     }
     eng.act.clear();
@@ -2569,24 +2776,17 @@ struct Server {
             hh_status st64 = e64.step(d64);
             retire(e64, d64);
             if (st32 != HH_OK) {
-                for (auto& q : e32.act)
-                    if (q.live) complete((ServerReq*)q.tag, st32, es);
-                e32.act.clear();
-                e32.uploaded.clear();
+                for (auto& q : e32.act) complete((ServerReq*)q.tag, st32, es);
+                e32.clear();
             }
             if (st64 != HH_OK) {
-                for (auto& q : e64.act)
-                    if (q.live) complete((ServerReq*)q.tag, st64, es);
-                e64.act.clear();
-                e64.uploaded.clear();
+                for (auto& q : e64.act) complete((ServerReq*)q.tag, st64, es);
+                e64.clear();
             }
         }
-        // shutting down: requests still iterating are dropped (their handles freed); the
-        // entries that have left were completed when they left
-        for (auto& q : e32.act)
-            if (q.live) complete((ServerReq*)q.tag, HH_ECUDA, es);
-        for (auto& q : e64.act)
-            if (q.live) complete((ServerReq*)q.tag, HH_ECUDA, es);
+        // shutting down: requests still iterating are dropped (their handles freed)
+        for (auto& q : e32.act) complete((ServerReq*)q.tag, HH_ECUDA, es);
+        for (auto& q : e64.act) complete((ServerReq*)q.tag, HH_ECUDA, es);
         cudaStreamSynchronize(es);
         e32.release();
         e64.release();

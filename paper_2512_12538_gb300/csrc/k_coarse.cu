@@ -82,46 +82,6 @@ __device__ bool grid_barrier(unsigned* bar, int* err, long long limit) {
     return s_ok != 0;
 }
 
-// CoarseRecur's end of phase 3: the block's |next residual|^2, then in the last block to
-// finish the fixed-order sum and the control words.  The norm only decides when the FP64
-// residual is formed, so it is summed in FP32 (the FP64 pipe is slow here).
-__device__ __forceinline__ void coarse_recur_tail(const CoarseRecur& R, float rr2, unsigned lb, unsigned nblk) {
-    __shared__ float rred[8];
-    __shared__ unsigned s_last;
-    rr2 = warp_sum(rr2);
-    if ((threadIdx.x & 31) == 0) rred[threadIdx.x >> 5] = rr2;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += rred[w];
-        ((float*)R.part)[lb] = t;
-        __threadfence();
-        s_last = atomicAdd(R.ticket, 1u) == nblk - 1;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    float a = 0.f;
-    for (unsigned k = threadIdx.x; k < nblk; k += blockDim.x) a += __ldcg((const float*)R.part + k);
-    a = warp_sum(a);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) rred[threadIdx.x >> 5] = a;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += rred[w];
-        *R.ticket = 0u;
-        R.nrm[1] = (double)t;
-        const int steps = R.ctl[3] + 1;
-        R.ctl[3] = steps;
-        const int anchor = (steps % R.anchor) == 0;
-        const float b2 = (float)R.nrm[2];
-        const float rel = b2 > 0.f ? sqrtf(t / b2) : 0.f;
-        R.ctl[4] = anchor;
-        R.ctl[2] = (anchor || !isfinite(rel) || rel < 2.f * (float)R.tol) ? 1 : 0;
-    }
-}
-
 // One-column coarse corrections of several nodes (Eq. (3)) in one cooperative launch;
 // job k owns blocks [blk0, blk0 + nblk).  A node's basis has p = 2r columns: those of its
 // first child [0, p/2) vanish on the rows at and below `split`, the second child's
@@ -167,12 +127,6 @@ __global__ void __launch_bounds__(256, sizeof(TC) == 4 ? 2 : 1) k_coarse_batch(C
     const unsigned N = (unsigned)g.b * (unsigned)g.Sx;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ph = p >> 1, G = J.ngrp;
-    // a job of a problem that has left (the same word for all its blocks): its blocks take
-    // part in the grid barrier only, touching none of its buffers
-    if (J.gate && *J.gate) {
-        grid_barrier(bar, err, bt.wait_polls);
-        return;
-    }
     {
         const int chunks = (int)(sizeof(CA) * p * p / 16);
         for (int t = threadIdx.x; t < chunks; t += blockDim.x)
@@ -212,9 +166,7 @@ __global__ void __launch_bounds__(256, sizeof(TC) == 4 ? 2 : 1) k_coarse_batch(C
             if (jr < g.b - 1) ax = ax - wi * cvt<R>(w_in[pt + g.Sx]);
             rv = rv - ax;
         }
-        const CA ra = cvt<TC>(rv);
-        if (bt.rr.AC && gi == 0) ((CA*)bt.rr.rp)[pt] = ra;   // r' for the next residual
-        return ra;
+        return cvt<TC>(rv);
     };
     // When the launch's basis exceeds the L2, the lines phase 1 reads last are kept for
     // phase 3 (which reads them first): the first (1 - keep) of each sweep is loaded with
@@ -325,7 +277,6 @@ __global__ void __launch_bounds__(256, sizeof(TC) == 4 ? 2 : 1) k_coarse_batch(C
     const unsigned n0 = J.split < 0 ? N : nsplit;
     const unsigned nc0 = (n0 + 255u) / 256u, nc1 = (N - n0 + 255u) / 256u;
     const unsigned ncm = min(nc0, nc1), nct = nc0 + nc1;
-    float rr2 = 0.f;   // |next residual|^2 of the thread's points (CoarseRecur)
     for (unsigned c = lb; c < nct; c += nblk) {
         unsigned hh, k;
         if (c < 2u * ncm) {
@@ -374,30 +325,7 @@ __global__ void __launch_bounds__(256, sizeof(TC) == 4 ? 2 : 1) k_coarse_batch(C
         if (J.dout) ((cplx<TC>*)J.dout)[pt - lo] = J.add_w ? a + cvt<TC>(w_in[pt]) : a;
         cplx<TO>& o = out[pt - lo];
         o = J.acc_out ? o + val : val;
-        if (bt.rr.AC) {
-            // the next residual r' - (A C) y; A C's columns of one child reach one row into
-            // the other child's rows (the stencil), so both halves count next to the split
-            const int jr = (int)(pt / (unsigned)g.Sx);
-            int k0 = 0, k1 = p;
-            if (J.split >= 0) {
-                if (jr < J.split - 1) k1 = p >> 1;
-                else if (jr > J.split) k0 = p >> 1;
-            }
-            const CA* AC = (const CA*)bt.rr.AC;
-            CA rn = ((const CA*)bt.rr.rp)[pt];
-            for (; k0 + 8 <= k1; k0 += 8) {
-                CA av[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) av[u] = AC[(size_t)(k0 + u) * N + pt];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) rn = rn - av[u] * s_y[k0 + u];
-            }
-            for (; k0 < k1; ++k0) rn = rn - AC[(size_t)k0 * N + pt] * s_y[k0];
-            ((CA*)bt.rr.rt)[pt] = rn;
-            rr2 += (float)abs2(rn);
-        }
     }
-    if (bt.rr.AC) coarse_recur_tail(bt.rr, rr2, lb, nblk);
 }
 
 template <typename TC, typename TV, typename TW, typename TO>

@@ -1,0 +1,1396 @@
+// k_cut.cu -- the stationary iteration on the rows next to the leaf cuts.
+//
+// One coarse-corrected ORAS step (Eqs. (2)-(3), n_i = 1) leaves a residual that vanishes off
+// the two rows at each cut between neighbouring leaves: inside a leaf's owned rows the leaf
+// solve satisfies A~ w = v exactly, and every basis column is extended from an artificial
+// boundary outside the owned rows, so A~_p C_p is zero there as well.  For L levels that is
+// 2 (2^L - 1) of S rows (14 of 1025 for eight leaves).  The iteration
+//     u <- u + M r,  r <- r - A M r
+// can therefore be run on those rows alone, and by linearity the iterate after K steps is
+//     u_K = u_0 + M (r_0 + r_1 + ... + r_{K-1}),
+// one application of M to the summed inputs.  Per step that leaves, for each leaf, the
+// scalar recursions of its b modes with a right-hand side on at most four rows and four rows
+// of the result, and for each node p the products of its basis with the residual on its
+// cuts: instead of 2 passes over every basis (HBM) and two dense transforms per leaf.
+// In exact arithmetic the iterates are those of the full iteration; the rows left out carry
+// the leaf solves' rounding, which the FP64 residual at the end of each round brings back
+// (the driver in hh_solver.cu starts a new round from it).
+//
+// Corrections of all levels at once: with t the composition of the leaf solutions and
+// res0 = v - A t, d_p = C_p^H res0 and E_q = A C_q on the cut rows (C_q restricted to the
+// rows q owns), the corrections y of Eq. (3) solve the block triangular system
+//     A_p y_p + sum_{q below p} (C_p^H E_q) y_q = d_p,
+// so y = M d with M its explicit inverse (k_cut_minv), and r <- res0 - sum_q E_q y_q.
+#include <algorithm>
+#include <atomic>
+
+#include <cooperative_groups.h>
+
+#include "k_line.cuh"
+#include "kernels.h"
+
+namespace cg = cooperative_groups;
+
+namespace hh {
+
+// ---------------------------------------------------------------- tree arithmetic
+// Cut c (0-based) lies between leaves c and c + 1; its node has level l and position t.
+__device__ __forceinline__ int cut_level(int c, int L) { return L - __ffs(c + 1); }
+
+// Barrier over the n co-resident blocks of a group (cooperative launch), bounded: the polls
+// run out after `limit` (0: at once, the testing form), DEV_TIMEOUT is recorded and false
+// returned.  A release-add on a counter that only grows and acquire loads of it: 1.2 us over
+// 152 blocks (a counter that is reset and a generation word behind full fences: 2.2 us).
+struct GroupBar {
+    unsigned* ctr;
+    unsigned n, target;
+    int* err;
+    long long limit;
+    __device__ bool operator()() {
+        __syncthreads();
+        bool ok = true;
+        target += n;
+        if (threadIdx.x == 0) {
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr) : "memory");
+            ok = false;
+            for (long long it = 0; it < limit && !ok; ++it) {
+                unsigned v;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
+                ok = (int)(v - target) >= 0;
+                if (it > 4096) __nanosleep(64);
+            }
+            if (!ok) atomicExch(err, DEV_TIMEOUT);
+        }
+        return __syncthreads_and(ok);
+    }
+};
+
+__device__ __forceinline__ c64 ldcg(const c64* p) {
+    const float2 v = __ldcg((const float2*)p);
+    return {v.x, v.y};
+}
+__device__ __forceinline__ c128 ldcg(const c128* p) {
+    const double2 v = __ldcg((const double2*)p);
+    return {v.x, v.y};
+}
+__device__ __forceinline__ unsigned long long gtime() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+}
+
+// The tests after a step: |v|^2 relative to the round's start, n2, against the thresholds,
+// and (P.stall) whether the steps still contract: a residual a hundred times its smallest, or
+// one that fell less than tenfold over the last 25 steps, stops the problem (its owner solves
+// it by GMRES).
+struct StepWatch {
+    float best, chk;
+    int chk_it;
+    __device__ StepWatch(const CutCtl& c, double n0) {
+        best = c.it ? (float)(c.best / n0) : 1.f;
+        chk = c.it ? (float)(c.chk / n0) : 1.f;
+        chk_it = c.chk_it;
+    }
+    __device__ int test(float n2, int it, const CutProb& P, float anchor, float due) {
+        if (!isfinite(n2)) return CUT_NONFINITE;
+        best = fminf(best, n2);
+        bool slow = n2 > 1e4f * best;
+        if (it - chk_it >= 25) {
+            slow = slow || n2 > 0.01f * chk;
+            chk = n2;
+            chk_it = it;
+        }
+        if (P.stall && slow && n2 >= due) return CUT_STALL;
+        if (n2 <= anchor) return CUT_ANCHOR;
+        if (n2 < due) return CUT_TEST;
+        return it >= P.max_iter ? CUT_LIMIT : 0;
+    }
+    __device__ void store(CutCtl& c, double n0) const {
+        c.best = best * n0;
+        c.chk = chk * n0;
+        c.chk_it = chk_it;
+    }
+};
+
+// ------------------------------------------------------------------- the cut rows
+// Rows of the bases at the cuts.  Cp: [row 0/1][x][K] per cut, K = (level + 1) r: the r
+// columns of each ancestor's child that holds the cut, then the own node's (row 0, above
+// the cut, its first child's columns, row 1 its second child's).  One block per entry and
+// 32 columns of the grid, transposed through shared memory.
+template <typename T>
+__global__ void __launch_bounds__(256) k_cut_cp(const CutCpEntry* __restrict__ ent, int Sx, int r) {
+    using C = cplx<T>;
+    __shared__ C tile[32][33];
+    const CutCpEntry e = ent[blockIdx.y];
+    const int x0 = blockIdx.x * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const C* src = (const C*)e.src;
+    C* dst = (C*)e.dst;
+    for (int j = ty; j < r; j += 8)
+        if (x0 + tx < Sx) tile[j][tx] = src[(size_t)j * e.ldc + x0 + tx];
+    __syncthreads();
+    for (int x = ty; x < 32; x += 8)
+        if (x0 + x < Sx && tx < r) dst[(size_t)(x0 + x) * e.K + tx] = tile[tx][x];
+}
+
+// E = A C on the cut rows, in FP64 products of the stored basis (e64, for the Galerkin
+// sums) and rounded to the basis precision (the iteration): [row][column][x].  maskl/maskr:
+// whether the rows above / below the cut belong to the rows the node owns.
+template <typename T>
+__global__ void __launch_bounds__(256) k_cut_ep(const CutEpEntry* __restrict__ ent, int Sx, int r, OpGeom g) {
+    using C = cplx<T>;
+    const CutEpEntry e = ent[blockIdx.y];
+    const int x = blockIdx.x * 256 + threadIdx.x, j = blockIdx.z;
+    if (x >= Sx || j >= r) return;
+    const C* src = (const C*)e.src + (size_t)j * e.ldc;   // row mid - 2 of column j
+    auto at = [&](int a, int xx) -> c128 {                // row mid - 2 + a
+        const bool in = a < 2 ? e.maskl : e.maskr;
+        return in && xx >= 0 && xx < Sx ? cvt<double>(src[(size_t)a * Sx + xx]) : c128{0, 0};
+    };
+#pragma unroll
+    for (int row = 0; row < 2; ++row) {
+        c128 s;
+        const int a0 = 1 + row;
+        if (g.q1) {
+            s = q1_row<double>(1, x, g, [&](int dj, int di) { return at(a0 + dj, x + di); });
+        } else {
+            s = op_diag(1, x, g) * at(a0, x);
+            s = s - at(a0, x - 1) - at(a0, x + 1) - wcol(x, Sx) * (at(a0 - 1, x) + at(a0 + 1, x));
+        }
+        const size_t o = ((size_t)row * e.Ke + j) * Sx + x;
+        ((c128*)e.d64)[o] = s;
+        ((C*)e.dst)[o] = cvt<T>(s);
+    }
+}
+
+// Partial sums of C_p^H E_q over the cut rows of one (cut, group of p, group of q) pair and
+// one share of the columns x: r x r FP64 products of the stored rows.  Two by two outputs
+// per thread, tiles of 16 x staged in FP64.
+static constexpr int GRAM_SPLIT = 8;
+template <typename T>
+__global__ void __launch_bounds__(256) k_cut_gram(const CutGramPair* __restrict__ prs, int Sx, int r, c128* part) {
+    using C = cplx<T>;
+    __shared__ c128 cs[16][33], es[16][33];
+    const CutGramPair p = prs[blockIdx.x];
+    const int ti = threadIdx.x >> 4, tj = threadIdx.x & 15;
+    const int xs = (Sx + GRAM_SPLIT - 1) / GRAM_SPLIT;
+    const int xa = blockIdx.y * xs, xb = min(Sx, xa + xs);
+    c128 acc[2][2] = {{{0, 0}, {0, 0}}, {{0, 0}, {0, 0}}};
+    for (int row = 0; row < 2; ++row) {
+        if (!((p.rows >> row) & 1)) continue;
+        const C* cp = (const C*)p.cp + (size_t)row * Sx * p.K;
+        const c128* ep = (const c128*)p.ep + (size_t)row * p.Ke * Sx;
+        for (int x0 = xa; x0 < xb; x0 += 16) {
+            for (int t = threadIdx.x; t < 16 * 32; t += 256) {
+                const int x = t >> 5, j = t & 31, x2 = t & 15, j2 = t >> 4;
+                cs[x][j] = x0 + x < xb && j < r ? cvt<double>(cp[(size_t)(x0 + x) * p.K + j]) : c128{0, 0};
+                es[x2][j2] = x0 + x2 < xb && j2 < r ? ep[(size_t)j2 * Sx + x0 + x2] : c128{0, 0};
+            }
+            __syncthreads();
+#pragma unroll 4
+            for (int x = 0; x < 16; ++x) {
+                const c128 a0 = cs[x][ti], a1 = cs[x][ti + 16], b0 = es[x][tj], b1 = es[x][tj + 16];
+                cfma_cj(acc[0][0], a0, b0);
+                cfma_cj(acc[0][1], a0, b1);
+                cfma_cj(acc[1][0], a1, b0);
+                cfma_cj(acc[1][1], a1, b1);
+            }
+            __syncthreads();
+        }
+    }
+    c128* o = part + ((size_t)blockIdx.x * GRAM_SPLIT + blockIdx.y) * 1024;
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int v = 0; v < 2; ++v) o[(ti + 16 * u) * 32 + tj + 16 * v] = acc[u][v];
+}
+__global__ void __launch_bounds__(256) k_cut_gram_red(const CutGramDest* __restrict__ ds, int r, const c128* part) {
+    const CutGramDest d = ds[blockIdx.x];
+    for (int t = threadIdx.x; t < r * r; t += 256) {
+        const int i = t / r, j = t - i * r;
+        c128 s = {0, 0};
+        for (int k = d.first * GRAM_SPLIT; k < (d.first + d.count) * GRAM_SPLIT; ++k)
+            s = s + part[(size_t)k * 1024 + i * 32 + j];
+        d.out[(size_t)i * d.ld + j] = s;
+    }
+}
+
+// Row e of the packed M (node p of level l at position t): its offset and its length, the
+// corrections of p's subtree level by level.
+__device__ __forceinline__ int cut_m_row(int e, int L, int r, int& l, int& t) {
+    const int p2 = 2 * r, p = e / p2;
+    l = 31 - __clz(p + 1);
+    t = p + 1 - (1 << l);
+    int o = 0;
+    for (int q = 0; q < l; ++q) o += (1 << q) * p2 * p2 * ((1 << (L - q)) - 1);
+    const int len = p2 * ((1 << (L - l)) - 1);
+    return o + (t * p2 + (e - p * p2)) * len;
+}
+
+// M_ps for one pair (p, s below or equal p): Ainv_p if s = p, else
+// -Ainv_p sum_{s <= q < p} G_pq M_qs, FP64, the sum first in shared memory.
+template <typename T>
+__global__ void __launch_bounds__(256) k_cut_minv(const CutMinv* __restrict__ prs, int D, int L, int p2,
+                                                  const c128* __restrict__ G, c128* M, cplx<T>* MT, int tr) {
+    using C = cplx<T>;
+    extern __shared__ __align__(16) unsigned char msm[];
+    c128* xs = (c128*)msm;                 // [p2][p2]
+    const CutMinv e = prs[blockIdx.x];
+    const size_t rp = (size_t)e.p * p2, cs = (size_t)e.s * p2;
+    // M in the basis precision is packed: rows of p's subtree level by level
+    int l, t;
+    C* mt = MT + cut_m_row(e.p * p2, L, p2 / 2, l, t);
+    const int len = p2 * ((1 << (L - l)) - 1), ls = 31 - __clz(e.s + 1);
+    const int k0 = p2 * ((1 << (ls - l)) - 1 + (e.s + 1 - (1 << ls)) - (t << (ls - l)));
+    // (tr: the cluster form's order, transposed within the node's rows)
+    auto put = [&](int i, int j, c128 v) { mt[tr ? (size_t)(k0 + j) * p2 + i : (size_t)i * len + k0 + j] = cvt<T>(v); };
+    if (e.p == e.s) {
+        for (int q = threadIdx.x; q < p2 * p2; q += 256) {
+            const int i = q / p2, j = q - i * p2;
+            const c128 v = e.Ainv[q];
+            M[(rp + i) * D + cs + j] = v;
+            put(i, j, v);
+        }
+        return;
+    }
+    for (int t = threadIdx.x; t < p2 * p2; t += 256) {
+        const int i = t / p2, j = t - i * p2;
+        c128 a = {0, 0};
+        for (int q = e.s; q != e.p; q = (q - 1) >> 1)   // s and its ancestors below p
+            for (int k = 0; k < p2; ++k) cfma(a, G[(rp + i) * D + (size_t)q * p2 + k], M[((size_t)q * p2 + k) * D + cs + j]);
+        xs[t] = a;
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < p2 * p2; t += 256) {
+        const int i = t / p2, j = t - i * p2;
+        c128 a = {0, 0};
+        for (int k = 0; k < p2; ++k) cfma(a, e.Ainv[i * p2 + k], xs[k * p2 + j]);
+        M[(rp + i) * D + cs + j] = -a;
+        put(i, j, -a);
+    }
+}
+
+// ------------------------------------------------------------------- the iteration
+// Shared memory of a step block, in elements: the xi lines and their lane products, the
+// lines of one item, the input rows; M where every block forms y itself; the panels of the
+// block's items where they fit (res); and the small arrays of phases B, Y and C.
+struct CutSmem {
+    int xi, pr, ln, v, m, ce, t, rs, red, d, y, ya, up, own, total;
+};
+HH_HD int cut_m_elems(int L, int r) {
+    int n = 0;
+    for (int l = 0; l < L; ++l) n += (1 << l) * (2 * r) * (2 * r) * ((1 << (L - l)) - 1);
+    return n;
+}
+HH_HD CutSmem cut_smem_layout(const CutProb& P, int nw) {
+    CutSmem s;
+    const int kmax = P.L * P.r;
+    int o = 0;
+    s.xi = o; o += P.MG * P.Sx;
+    s.pr = o; o += P.MG * 64;
+    s.ln = o; o += P.MG * P.Sx;
+    s.v = o; o += 4 * P.Sx;
+    s.m = o; o += P.dist ? 0 : cut_m_elems(P.L, P.r);
+    s.ce = o; o += P.res ? P.nbi * 2 * P.XC * (3 * P.L) * P.r : 0;
+    s.t = o; o += 4 * (P.XC + 2);
+    s.rs = o; o += 2 * P.XC;
+    s.red = o; o += nw * 2 * kmax;
+    s.d = o; o += P.D;
+    s.y = o; o += P.D;
+    s.ya = o; o += P.D;
+    s.up = o; o += CUT_KG * 2 * P.XC;
+    s.own = o; o += 4 * P.XC;
+    s.total = o;
+    return s;
+}
+
+// One group of co-resident blocks per problem runs its steps until the next test,
+// anchor or limit; a launch's groups take the problems in turn.  The work is cut into
+// items that depend on the problem alone, so the group's size changes no sum.
+//   A: item (leaf, MG modes), one warp per mode: f^ = sum of at most four rows (the first
+//      step of a round: the transformed full residual), both recursions, and the item's
+//      share of the four rows of the result;
+//   B: item (cut, XC columns): the rows' sums over the items, res0 = v - A t, and its
+//      products with the basis rows of the cut's ancestors;
+//   Y: d and y = M d, in every block, or (dist) one entry per warp and a barrier each;
+//   C: the items of B again: v = res0 - sum E y, and its norm.
+// What bounds it is latency: a barrier and a first load from the L2 per phase.
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ probs, int nprob, int gsz,
+                                                  const int* modes, int mode_all, unsigned* bars, int* err,
+                                                  long long limit, int prof) {
+    using C = cplx<T>;
+    constexpr int NW = NT / 32;
+    extern __shared__ __align__(16) unsigned char csm[];
+    __shared__ C s_vin[4][CUT_MGMAX], s_vout[4][CUT_MGMAX], s_sc[CUT_MGMAX];
+    __shared__ float s_red[NW];
+    // the descriptors in shared memory: the barriers' acquires drop the L1, so that every
+    // phase would fetch them from the L2 again, one dependent load after another
+    __shared__ CutProb P;
+    __shared__ CutLeaf F;
+    const int ngroups = gridDim.x / gsz, group = blockIdx.x / gsz, rank = blockIdx.x - group * gsz;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    GroupBar bar{bars + group, (unsigned)gsz, 0u, err, limit};
+    bool ok = true;
+    for (int pi = group; ok && pi < nprob; pi += ngroups) {
+        const int mode = modes ? modes[pi] : mode_all;
+        if (!mode) continue;
+        __syncthreads();   // the previous problem's arrays are no longer read
+        for (int q = tid; q < (int)(sizeof(CutProb) / 4); q += NT) ((int*)&P)[q] = ((const int*)(probs + pi))[q];
+        __syncthreads();
+        const int Sx = P.Sx, r = P.r, L = P.L, nch = P.nch, XC = P.XC, D = P.D, MG = P.MG;
+        const int kmax = L * r;
+        const bool dist = P.dist, res = P.res && P.nB <= P.nbi * gsz;
+        const bool one = P.nB <= gsz;   // at most one item of phases B and C a block: its rows stay here
+        CutCtl* ctl = P.ctl;
+        const CutSmem lay = cut_smem_layout(P, NW);
+        C* const sm = (C*)csm;
+        C* s_xi = sm + lay.xi;
+        C* s_pr = sm + lay.pr;
+        C* s_ln = sm + lay.ln;
+        C* s_v = sm + lay.v;
+        C* s_m = sm + lay.m;
+        C* s_ce = sm + lay.ce;
+        C* s_t = sm + lay.t;
+        C* s_rs = sm + lay.rs;
+        C* s_pd = sm + lay.red;
+        C* s_d = sm + lay.d;
+        C* s_y = sm + lay.y;
+        C* s_up = sm + lay.up;
+        C* s_own = sm + lay.own;
+        C* s_vs = s_own + 2 * XC;
+        C* s_ya = sm + lay.ya;
+        C* v = (C*)P.v;
+        C* vsum = (C*)P.vsum;
+        C* res0 = (C*)P.res0;
+        C* prow = (C*)P.prow;
+        C* pd = (C*)P.pd;
+        C* gd = (C*)P.d;
+        C* gy = (C*)P.y;
+        C* yacc = (C*)P.yacc;
+        const C* Mt = (const C*)P.M;
+        OpGeom g;
+        g.b = 3;
+        g.Sx = Sx;
+        g.kh = P.kh;
+        g.khr = nullptr;
+        g.q1 = P.q1;
+        // thresholds of this launch (the FP64 norms of the round's start)
+        bool first = mode == 1;
+        const double b2 = *P.b2, n0 = first ? *P.nrm : ctl->n0;
+        // |v|^2 relative to the round's start, in single precision (an FP64 chain costs more
+        // than a phase; the value only decides when the FP64 residual is formed)
+        const float thr_test = (float)(P.test2 * b2 / n0), thr_anchor = (float)P.anchor2;
+        const T inv0 = (T)(1.0 / sqrt(n0));
+        int it = ctl->it, in_round = first ? 0 : ctl->in_round, reason = 0;
+        StepWatch watch(*ctl, n0);
+        float n2 = 0.f;
+        int xi_item = -1;
+        bool stepped = false;   // a step of this launch is done
+        unsigned long long t0 = 0, tA = 0, tB = 0, tC = 0;
+        const bool timing = prof && rank == 0 && tid == 0;
+        if (!dist)
+            for (int q = tid; q < cut_m_elems(L, r); q += NT) s_m[q] = Mt[q];
+        // the panels of the block's items: C as [row][x][K], then E as [row][k][x]
+        if (res) {
+            for (int q = 0, e = rank; e < P.nB; ++q, e += gsz) {
+                const int c = e / nch, x0 = (e - c * nch) * XC, xn = min(XC, Sx - x0);
+                const int lev = cut_level(c, L), K = (lev + 1) * r, Ke = (2 * L - lev) * r;
+                C* dc = s_ce + (size_t)q * 2 * XC * 3 * L * r;
+                C* de = dc + 2 * XC * K;
+                for (int row = 0; row < 2; ++row) {
+                    const C* sc = (const C*)P.Cp + P.cp_off[c] + ((size_t)row * Sx + x0) * K;
+                    for (int u = tid; u < xn * K; u += NT) dc[row * XC * K + u] = sc[u];
+                    const C* se = (const C*)P.Ep + P.ep_off[c] + (size_t)row * Ke * Sx + x0;
+                    for (int u = tid; u < Ke * xn; u += NT) {
+                        const int k = u / xn, x = u - k * xn;
+                        de[(row * Ke + k) * XC + x] = se[(size_t)k * Sx + x];
+                    }
+                }
+            }
+        }
+        for (;;) {
+            if (timing) t0 = gtime();
+            // ------------------------------------------------------------------ A
+            for (int a = rank; a < P.nA; a += gsz) {
+                const int lf = a / P.ngrp, m0 = (a - lf * P.ngrp) * MG;
+                if (xi_item != a) {
+                    __syncthreads();
+                    if (tid < (int)(sizeof(CutLeaf) / 4)) ((int*)&F)[tid] = ((const int*)(P.leaf + lf))[tid];
+                }
+                __syncthreads();
+                const int b = F.b, nm = min(MG, b - m0);
+                if (xi_item != a && nm > 0) {
+                    const C* V = (const C*)F.V;
+                    for (int q = tid; q < 4 * nm; q += NT) {
+                        const int k = q / nm, w = q - k * nm;
+                        const C sc = F.sc ? ((const C*)F.sc)[m0 + w] : C{1, 0};
+                        s_vout[k][w] = F.rout[k] >= 0 ? V[(size_t)F.rout[k] * b + m0 + w] : C{0, 0};
+                        const C vi = F.rin[k] >= 0 ? V[(size_t)F.rin[k] * b + m0 + w] : C{0, 0};
+                        s_vin[k][w] = F.sc ? sc * vi : vi;
+                        if (k == 0) s_sc[w] = sc;
+                    }
+                    for (int w = warp; w < nm; w += NW) {
+                        const C* xi = (const C*)F.xi + (size_t)(m0 + w) * Sx;
+                        for (int i = lane; i < Sx; i += 32) s_xi[w * Sx + i] = xi[i];
+                        __syncwarp();
+                        line_products(s_xi + w * Sx, Sx, lane, s_pr[w * 64 + lane], s_pr[w * 64 + 32 + lane]);
+                    }
+                }
+                xi_item = a;
+                if (nm <= 0) continue;
+                if (!first) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const C* src = v + ((size_t)(lf - (k < 2)) * 2 + (k & 1)) * Sx;
+                        for (int i = tid; i < Sx; i += NT) s_v[k * Sx + i] = F.rin[k] >= 0 ? ldcg(src + i) : C{0, 0};
+                    }
+                }
+                __syncthreads();
+                // the lines' right-hand sides, then the recursions, one warp a line
+                if (first) {
+                    for (int w = warp; w < nm; w += NW) {
+                        const C* f0 = (const C*)F.fh0 + (size_t)(m0 + w) * Sx;
+                        const C sc = s_sc[w];
+                        for (int i = lane; i < Sx; i += 32) s_ln[w * Sx + i] = F.sc ? sc * f0[i] : f0[i];
+                    }
+                } else {
+                    for (int i = tid; i < Sx; i += NT) {
+                        const C v0 = s_v[i], v1 = s_v[Sx + i], v2 = s_v[2 * Sx + i], v3 = s_v[3 * Sx + i];
+                        for (int w = 0; w < nm; ++w) {
+                            C f = {0, 0};
+                            cfma(f, s_vin[0][w], v0);
+                            cfma(f, s_vin[1][w], v1);
+                            cfma(f, s_vin[2][w], v2);
+                            cfma(f, s_vin[3][w], v3);
+                            s_ln[w * Sx + i] = f;
+                        }
+                    }
+                }
+                __syncthreads();
+                for (int w = warp; w < nm; w += NW)
+                    line_solve(s_xi + w * Sx, s_ln + w * Sx, Sx, lane, s_pr[w * 64 + lane], s_pr[w * 64 + 32 + lane]);
+                __syncthreads();
+                for (int i = tid; i < Sx; i += NT) {
+                    C o[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+                    for (int w = 0; w < nm; ++w) {
+                        const C f = s_ln[w * Sx + i];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) cfma(o[k], s_vout[k][w], f);
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (F.rout[k] >= 0) prow[((size_t)a * 4 + k) * Sx + i] = o[k];
+                }
+            }
+            if (!(ok = bar())) break;
+            if (timing) { const unsigned long long t = gtime(); tA += t - t0; t0 = t; }
+            // ------------------------------------------------------------------ B
+            for (int e = rank, q0 = 0; e < P.nB; e += gsz, ++q0) {
+                const int c = e / nch, x0 = (e - c * nch) * XC, xn = min(XC, Sx - x0);
+                const int lev = cut_level(c, L), K = (lev + 1) * r;
+                // the four rows next to the cut, halo of one column
+                for (int q = tid; q < 4 * (xn + 2); q += NT) {
+                    const int row = q / (xn + 2), il = q - row * (xn + 2), i = x0 - 1 + il;
+                    C s = {0, 0};
+                    if (i >= 0 && i < Sx) {
+                        const int lf = c + (row >> 1), k = row < 2 ? row + 2 : row - 2;
+                        const int ng = (P.leaf[lf].b + MG - 1) / MG;
+                        const C* src = prow + ((size_t)lf * P.ngrp * 4 + k) * Sx + i;
+                        for (int u0 = 0; u0 < ng; u0 += 12) {
+                            C a[12];
+#pragma unroll
+                            for (int u = 0; u < 12; ++u)
+                                a[u] = u0 + u < ng ? ldcg(src + (size_t)(u0 + u) * 4 * Sx) : C{0, 0};
+#pragma unroll
+                            for (int u = 0; u < 12; ++u) s = s + a[u];
+                        }
+                    }
+                    s_t[row * (XC + 2) + il] = s;
+                }
+                __syncthreads();
+                for (int q = tid; q < 2 * xn; q += NT) {
+                    const int row = q / xn, il = q - row * xn, i = x0 + il;
+                    const size_t o = ((size_t)c * 2 + row) * Sx + i;
+                    const C vv = first ? ((const C*)P.rt)[(size_t)(P.mid[c] - 1 + row) * Sx + i]
+                                       : (one && stepped ? s_own[row * XC + il] : ldcg(v + o));
+                    if (one) s_vs[row * XC + il] = first ? C{0, 0} : (stepped ? s_vs[row * XC + il] : vsum[o]) + vv;
+                    else vsum[o] = first ? C{0, 0} : vsum[o] + vv;
+                    const C* tc = s_t + (row + 1) * (XC + 2) + il + 1;
+                    C at;
+                    if (P.q1) {
+                        at = q1_row<T>(1, i, g, [&](int dj, int di) { return tc[dj * (XC + 2) + di]; });
+                    } else {
+                        at = op_diag_t<T>(1, i, g) * tc[0] - tc[-1] - tc[1] -
+                             (T)wcol(i, Sx) * (tc[-(XC + 2)] + tc[XC + 2]);
+                    }
+                    const C rs = vv - at;
+                    s_rs[row * XC + il] = rs;
+                    if (!one) res0[o] = rs;
+                }
+                __syncthreads();
+                {
+                    const C* c0 = res ? s_ce + (size_t)q0 * 2 * XC * 3 * L * r
+                                      : (const C*)P.Cp + P.cp_off[c] + (size_t)x0 * K;
+                    const C* c1 = c0 + (size_t)(res ? XC : Sx) * K;
+                    for (int k0 = 0; k0 < K; k0 += 32) {
+                        const int k = k0 + lane;
+                        C a0 = {0, 0}, a1 = {0, 0};
+                        if (k < K) {
+#pragma unroll 4
+                            for (int il = warp; il < xn; il += NW) {
+                                cfma_cj(a0, c0[(size_t)il * K + k], s_rs[il]);
+                                cfma_cj(a1, c1[(size_t)il * K + k], s_rs[XC + il]);
+                            }
+                            s_pd[(warp * 2) * kmax + k] = a0;
+                            s_pd[(warp * 2 + 1) * kmax + k] = a1;
+                        }
+                    }
+                }
+                __syncthreads();
+                // slots: the ancestors' columns (both rows), the own node's first and second child
+                for (int s = tid; s < (lev + 2) * r; s += NT) {
+                    const bool own1 = s >= (lev + 1) * r;
+                    const int k = own1 ? s - r : s;
+                    C t = {0, 0};
+#pragma unroll
+                    for (int w = 0; w < NW; ++w) {
+                        if (!own1) t = t + s_pd[(w * 2) * kmax + k];
+                        if (own1 || s < lev * r) t = t + s_pd[(w * 2 + 1) * kmax + k];
+                    }
+                    pd[(size_t)e * (L + 1) * r + s] = t;
+                }
+                __syncthreads();
+            }
+            if (!(ok = bar())) break;
+            // ------------------------------------------------------------------ Y
+            // d[e]: the partials of the cuts under the entry's child and of the own cut, by
+            // eight lanes in a fixed order
+            {
+                constexpr int EB = NT / 8;
+                const int sub = tid & 7;
+                for (int eb = dist ? rank * EB : 0; eb < D; eb += dist ? gsz * EB : EB) {
+                    const int e = eb + (tid >> 3);
+                    C s = {0, 0};
+                    if (e < D) {
+                        const int p = e / (2 * r), j = e - p * 2 * r, k = j >= r, jr = j - k * r;
+                        const int l = 31 - __clz(p + 1), t = p + 1 - (1 << l);
+                        const int span = 1 << (L - l), ca = t * span + k * (span / 2);
+                        const int own = t * span + span / 2 - 1;
+                        const int nin = span / 2 - 1;    // cuts inside the child
+#pragma unroll 4
+                        for (int q = sub; q < (nin + 1) * nch; q += 8) {
+                            const int cc = q / nch, ch = q - cc * nch;
+                            const int cut = cc < nin ? ca + cc : own;
+                            const int slot = (cc < nin ? l : l + k) * r + jr;
+                            s = s + ldcg(pd + ((size_t)cut * nch + ch) * (L + 1) * r + slot);
+                        }
+                    }
+                    for (int o = 4; o > 0; o >>= 1) {
+                        s.re += __shfl_xor_sync(0xffffffffu, s.re, o);
+                        s.im += __shfl_xor_sync(0xffffffffu, s.im, o);
+                    }
+                    if (sub == 0 && e < D) {
+                        if (dist) gd[e] = s;
+                        else s_d[e] = s;
+                    }
+                }
+            }
+            if (dist) {
+                if (!(ok = bar())) break;
+                for (int e = tid; e < D; e += NT) s_d[e] = ldcg(gd + e);
+            }
+            __syncthreads();
+            for (int e = dist ? rank * NW + warp : warp; e < D; e += dist ? gsz * NW : NW) {
+                int l, t;
+                const int mo = cut_m_row(e, L, r, l, t);
+                const C* mr = dist ? Mt + mo : s_m + mo;
+                C s = {0, 0};
+                for (int lv = l, k0 = 0; lv < L; ++lv) {
+                    const int q0 = ((1 << lv) - 1 + (t << (lv - l))) * 2 * r, n = 2 * r << (lv - l);
+#pragma unroll 4
+                    for (int k = lane; k < n; k += 32) cfma(s, mr[k0 + k], s_d[q0 + k]);
+                    k0 += n;
+                }
+                s = warp_sum(s);
+                if (lane == 0) {
+                    if (dist) gy[e] = s;
+                    else s_y[e] = s;
+                }
+            }
+            if (dist) {
+                if (!(ok = bar())) break;
+                for (int e = tid; e < D; e += NT) s_y[e] = ldcg(gy + e);
+            }
+            __syncthreads();
+            if (rank == 0)
+                for (int e = tid; e < D; e += NT)
+                    s_ya[e] = first ? s_y[e] : (stepped ? s_ya[e] : yacc[e]) + s_y[e];
+            if (timing) { const unsigned long long t = gtime(); tB += t - t0; t0 = t; }
+            // ------------------------------------------------------------------ C
+            for (int e = rank, q0 = 0; e < P.nB; e += gsz, ++q0) {
+                const int c = e / nch, x0 = (e - c * nch) * XC, xn = min(XC, Sx - x0);
+                const int lev = cut_level(c, L), ne = 2 * L - lev, Ke = ne * r;
+                const C* E = res ? s_ce + (size_t)q0 * 2 * XC * 3 * L * r + 2 * XC * (lev + 1) * r
+                                 : (const C*)P.Ep + P.ep_off[c] + x0;
+                const int ldx = res ? XC : Sx;
+                const unsigned short* yi = P.yidx + c * 2 * CUT_MAXL;
+                // (row, x) pairs times shares of the columns; a share's partial per pair
+                const int np = 2 * xn, kg = min(CUT_KG, max(1, NT / np));
+                for (int q = tid; q < np * kg; q += NT) {
+                    const int kk = q / np, pr = q - kk * np, row = pr / xn, il = pr - row * xn;
+                    const C* er = E + (size_t)row * Ke * ldx + il;
+                    C s = {0, 0};
+                    for (int gq = 0; gq < ne; ++gq) {
+                        const C* yg = s_y + yi[gq];
+                        const C* eg = er + (size_t)gq * r * ldx;
+#pragma unroll 8
+                        for (int j = kk; j < r; j += kg) cfma(s, eg[(size_t)j * ldx], yg[j]);
+                    }
+                    s_up[kk * 2 * XC + row * XC + il] = s;
+                }
+                __syncthreads();
+                float nn = 0.f;   // |v|^2, one partial a warp
+                for (int q = tid; q < np; q += NT) {
+                    const int row = q / xn, il = q - row * xn;
+                    const size_t o = ((size_t)c * 2 + row) * Sx + x0 + il;
+                    C s = one ? s_rs[row * XC + il] : res0[o];
+                    for (int w = 0; w < kg; ++w) s = s - s_up[w * 2 * XC + row * XC + il];
+                    v[o] = s;
+                    if (one) s_own[row * XC + il] = s;
+                    nn += (float)abs2(inv0 * s);
+                }
+                nn = warp_sum(nn);
+                if (lane == 0) P.npart[e * NW + warp] = nn;
+            }
+            stepped = true;
+            if (!(ok = bar())) break;
+            // the norm, in the same order in every block; then the tests
+            {
+                float t = 0.f;
+                for (int e = tid; e < P.nB * NW; e += NT) t += __ldcg(P.npart + e);
+                t = warp_sum(t);
+                if (lane == 0) s_red[warp] = t;
+                __syncthreads();
+                n2 = 0.f;
+#pragma unroll
+                for (int w = 0; w < NW; ++w) n2 += s_red[w];
+            }
+            if (timing) { const unsigned long long t = gtime(); tC += t - t0; t0 = t; }
+            first = false;
+            ++it;
+            ++in_round;
+            reason = watch.test(n2, it, P, thr_anchor, thr_test);
+            if (reason) break;
+        }
+        if (ok && one && rank < P.nB) {
+            const int c = rank / nch, x0 = (rank - c * nch) * XC, xn = min(XC, Sx - x0);
+            for (int q = tid; q < 2 * xn; q += NT) {
+                const int row = q / xn, il = q - row * xn;
+                vsum[((size_t)c * 2 + row) * Sx + x0 + il] = s_vs[row * XC + il];
+            }
+        }
+        if (ok && rank == 0)
+            for (int e = tid; e < D; e += NT) yacc[e] = s_ya[e];
+        if (ok && rank == 0 && tid == 0) {
+            ctl->it = it;
+            ctl->in_round = in_round;
+            ctl->reason = reason;
+            ctl->n2 = (double)n2 * n0;
+            ctl->n0 = n0;
+            watch.store(*ctl, n0);
+            ctl->ns[0] += (double)tA;
+            ctl->ns[1] += (double)tB;
+            ctl->ns[2] += (double)tC;
+        }
+    }
+}
+
+// ------------------------------------------------- the iteration on one cluster
+// The complex64 problems whose data fits sixteen blocks' shared memory (255 columns at
+// r = 16: 205 KB a block) run on a cluster of sixteen with everything on chip.  The phases
+// are those above with one item a block, and what they exchange goes straight into the
+// consumers' shared memory (st.async, counted by the consumer's mbarrier), so that a phase
+// waits for one remote store instead of draining its stores, a barrier and a load from the
+// L2 (each 0.4 to 0.7 us):
+//   1: rows of the leaf items to the blocks of their cuts (with the halo columns);
+//   2: the products with the basis rows to every block, which forms y itself;
+//   3: v to the blocks of the two leaves at the cut, and |v|^2 to every block.
+// One buffer each is enough: 2 and 3 go from every block to every block (a word where there
+// is nothing to tell), so a block that is a phase ahead has heard from all others that they
+// are done with the buffer, and the mbarrier's phase, it writes next.
+static constexpr int CC_CL = 16, CC_NT = 544, CC_NW = CC_NT / 32;
+struct CcSmem {
+    int xi, ln, v, m, c, e, t, red, up, rs, d, y, ya, own, vs, bx, bd, total;
+};
+HH_HD CcSmem cc_layout(const CutProb& P) {
+    CcSmem s;
+    const int r = P.r, L = P.L, D = P.D, XC = P.XC;
+    int o = 0;
+    s.xi = o; o += P.MG * P.Sx;
+    s.ln = o;                       // the lines; phases B, Y and C: the rows and partial sums
+    s.t = o;
+    s.red = s.t + 4 * (XC + 2);
+    s.up = s.red + CC_NW * 2 * L * r;
+    const int tmp = 4 * (XC + 2) + CC_NW * 2 * L * r + (CUT_KG * 2 * XC > 5 * D ? CUT_KG * 2 * XC : 5 * D);
+    o += P.MG * P.Sx > tmp ? P.MG * P.Sx : tmp;
+    s.v = o; o += 4 * P.Sx;
+    s.m = o; o += cut_m_elems(L, r);
+    s.c = o; o += 2 * XC * (2 * L + 1) * r;
+    s.e = s.c;                      // E follows the block's C panel
+    s.rs = o; o += 2 * XC;
+    s.d = o; o += D;
+    s.y = o; o += D;
+    s.ya = o; o += D;
+    s.own = o; o += 2 * XC;
+    s.vs = o; o += 2 * XC;
+    s.bx = o; o += 4 * P.ngrp * (XC + 2);
+    s.bd = o; o += P.nB * (L + 1) * r;
+    s.total = o;
+    return s;
+}
+__device__ __forceinline__ uint32_t mapa(uint32_t a, int rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+// 8 or 4 bytes into another block's shared memory, counted on that block's mbarrier
+__device__ __forceinline__ void st_async(uint32_t dst, c64 v, uint32_t mbar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(dst),
+                 "f"(v.re), "f"(v.im), "r"(mbar)
+                 : "memory");
+}
+__device__ __forceinline__ void st_async(uint32_t dst, float v, uint32_t mbar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(dst), "f"(v),
+                 "r"(mbar)
+                 : "memory");
+}
+
+__global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restrict__ probs, int nprob,
+                                                          const int* modes, int mode_all, int* err, long long limit,
+                                                          int prof) {
+    using C = c64;
+    constexpr int NT = CC_NT, NW = CC_NW;
+    extern __shared__ __align__(16) unsigned char csm[];
+    __shared__ C s_vin[4][CUT_MGMAX], s_vout[4][CUT_MGMAX], s_sc[CUT_MGMAX];
+    __shared__ float s_nrm[CC_CL][4], s_word[CC_CL];
+    __shared__ unsigned short s_yi[CUT_KMAX * 2];
+    __shared__ __align__(8) uint64_t s_mb[3];
+    __shared__ CutProb P;
+    __shared__ CutLeaf F;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), ngroups = gridDim.x / CC_CL, group = blockIdx.x / CC_CL;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) {
+        for (int k = 0; k < 3; ++k) mbar_init(&s_mb[k], 1);
+        fence_barrier_init();
+    }
+    cluster.sync();
+    const uint32_t mb = smem_u32(s_mb);
+    unsigned phase = 0;   // steps this block has done: the mbarriers' parity
+    bool ok = true;
+    // wait for `bytes` of exchange k; bounded
+    auto wait = [&](int k, unsigned bytes) -> bool {
+        if (tid == 0) mbar_arrive_expect_tx(&s_mb[k], bytes);
+        bool got = false;
+        for (long long q = 0; q < limit && !got; ++q) {
+            uint32_t d;
+            asm volatile(
+                "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+                " selp.u32 %0, 1, 0, p;\n}\n"
+                : "=r"(d) : "r"(mb + 8 * k), "r"(phase & 1u) : "memory");
+            got = d != 0;
+        }
+        if (!got) atomicExch(err, DEV_TIMEOUT);
+        return __syncthreads_and(got);
+    };
+    for (int pi = group; pi < nprob; pi += ngroups) {
+        const int mode = modes ? modes[pi] : mode_all;
+        if (!mode) continue;
+        if (!ok) {
+            // a wait gave up: only keep the cluster's barriers in step with the blocks that go on
+            cluster.sync();
+            continue;
+        }
+        __syncthreads();
+        for (int q = tid; q < (int)(sizeof(CutProb) / 4); q += NT) ((int*)&P)[q] = ((const int*)(probs + pi))[q];
+        __syncthreads();
+        const int Sx = P.Sx, r = P.r, L = P.L, nch = P.nch, XC = P.XC, D = P.D, MG = P.MG, ngrp = P.ngrp;
+        const CcSmem lay = cc_layout(P);
+        C* const sm = (C*)csm;
+        C *s_xi = sm + lay.xi, *s_ln = sm + lay.ln, *s_v = sm + lay.v, *s_m = sm + lay.m, *s_t = sm + lay.t,
+          *s_red = sm + lay.red, *s_up = sm + lay.up, *s_rs = sm + lay.rs, *s_d = sm + lay.d, *s_y = sm + lay.y,
+          *s_ya = sm + lay.ya, *s_own = sm + lay.own, *s_vs = sm + lay.vs, *s_bx = sm + lay.bx, *s_bd = sm + lay.bd;
+        CutCtl* ctl = P.ctl;
+        OpGeom g;
+        g.b = 3;
+        g.Sx = Sx;
+        g.kh = P.kh;
+        g.khr = nullptr;
+        g.q1 = P.q1;
+        // the block's leaf item and cut item
+        const int lf = min(rank / ngrp, P.ncut), m0 = (rank - lf * ngrp) * MG;
+        if (tid < (int)(sizeof(CutLeaf) / 4)) ((int*)&F)[tid] = ((const int*)(P.leaf + lf))[tid];
+        const bool has_b = rank < P.nB;
+        const int c = has_b ? rank / nch : 0, ch = rank - c * nch, x0 = has_b ? ch * XC : 0;
+        const int xn = has_b ? min(XC, Sx - x0) : 0;   // at least one column by the plan's choice of XC
+        const int lev = cut_level(c, L), K = (lev + 1) * r, Ke = (2 * L - lev) * r;
+        C* s_c = sm + lay.c;
+        C* s_e = s_c + 2 * XC * K;
+        const int ng0 = has_b ? (P.leaf[c].b + MG - 1) / MG : 0, ng1 = has_b ? (P.leaf[c + 1].b + MG - 1) / MG : 0;
+        __syncthreads();
+        const int b = F.b, nm = rank < P.nA ? max(0, min(MG, b - m0)) : 0;
+        bool first = mode == 1;
+        const double n0 = first ? *P.nrm : ctl->n0;
+        const float thr_test = (float)(P.test2 * *P.b2 / n0), thr_anchor = (float)P.anchor2;
+        const float inv0 = (float)(1.0 / sqrt(n0));
+        int it = ctl->it, in_round = first ? 0 : ctl->in_round, reason = 0;
+        StepWatch watch(*ctl, n0);
+        float n2 = 0.f;
+        // resident data: V entries, xi and its lane products, M, the panels, the state
+        for (int q = tid; q < 4 * nm; q += NT) {
+            const C* V = (const C*)F.V;
+            const int k = q / nm, w = q - k * nm;
+            const C sc = F.sc ? ((const C*)F.sc)[m0 + w] : C{1, 0};
+            s_vout[k][w] = F.rout[k] >= 0 ? V[(size_t)F.rout[k] * b + m0 + w] : C{0, 0};
+            const C vi = F.rin[k] >= 0 ? V[(size_t)F.rin[k] * b + m0 + w] : C{0, 0};
+            s_vin[k][w] = F.sc ? sc * vi : vi;
+            if (k == 0) s_sc[w] = sc;
+        }
+        C pf[2], pb[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int w = warp + u * NW;
+            if (w < nm) {
+                const C* xi = (const C*)F.xi + (size_t)(m0 + w) * Sx;
+                for (int i = lane; i < Sx; i += 32) s_xi[w * Sx + i] = xi[i];
+                __syncwarp();
+                line_products(s_xi + w * Sx, Sx, lane, pf[u], pb[u]);
+            }
+        }
+        for (int q = tid; q < cut_m_elems(L, r); q += NT) s_m[q] = ((const C*)P.M)[q];
+        if (has_b) {
+            for (int row = 0; row < 2; ++row) {
+                const C* sc = (const C*)P.Cp + P.cp_off[c] + ((size_t)row * Sx + x0) * K;
+                for (int u = tid; u < xn * K; u += NT) s_c[row * XC * K + u] = sc[u];
+                const C* se = (const C*)P.Ep + P.ep_off[c] + (size_t)row * Ke * Sx + x0;
+                for (int u = tid; u < Ke * xn; u += NT) {
+                    const int k = u / xn, x = u - k * xn;
+                    s_e[(row * Ke + k) * XC + x] = se[(size_t)k * Sx + x];
+                }
+            }
+            for (int k = tid; k < Ke; k += NT) s_yi[k] = (unsigned short)(P.yidx[c * 2 * CUT_MAXL + k / r] + k % r);
+            for (int q = tid; q < 2 * xn; q += NT) {
+                const int row = q / xn, il = q - row * xn;
+                const size_t o = ((size_t)c * 2 + row) * Sx + x0 + il;
+                s_own[row * XC + il] =
+                    first ? ((const C*)P.rt)[(size_t)(P.mid[c] - 1 + row) * Sx + x0 + il] : ((const C*)P.v)[o];
+                s_vs[row * XC + il] = first ? C{0, 0} : ((const C*)P.vsum)[o];
+            }
+        }
+        for (int q = tid; q < 4 * ngrp * (XC + 2); q += NT) s_bx[q] = C{0, 0};
+        for (int e = tid; e < D; e += NT) s_ya[e] = first ? C{0, 0} : ((const C*)P.yacc)[e];
+        for (int q = tid; q < 4 * Sx; q += NT) {
+            const int k = q / Sx, i = q - k * Sx;
+            s_v[q] = !first && F.rin[k] >= 0 ? ((const C*)P.v)[((size_t)(lf - (k < 2)) * 2 + (k & 1)) * Sx + i] : C{0, 0};
+        }
+        // bytes of the three exchanges
+        const int xw = min(Sx, x0 + xn + 1) - max(0, x0 - 1);   // columns with the halo
+        const unsigned by1 = has_b ? 8u * 2u * (unsigned)xw * (unsigned)(ng0 + ng1) : 0u;
+        unsigned by2 = 4u * (unsigned)(CC_CL - P.nB);
+        for (int q = 0; q < P.ncut; ++q) by2 += 8u * (unsigned)(nch * (cut_level(q, L) + 2) * r);
+        const unsigned by3 = 4u * 4u * CC_CL + (nm > 0 ? 8u * 2u * (unsigned)Sx * ((F.rin[0] >= 0) + (F.rin[2] >= 0)) : 0u);
+        unsigned long long t0 = 0, tA = 0, tB = 0, tC = 0;
+        const bool timing = prof && rank == 0 && tid == 0;
+        cluster.sync();   // every block's buffers are ready
+        for (;;) {
+            if (timing) t0 = gtime();
+            // ------------------------------------------------------------------ A
+            for (int u = 0; u < 2; ++u) {
+                const int w = warp + u * NW;
+                if (w >= nm) break;
+                C* fs = s_ln + w * Sx;
+                if (first) {
+                    const C* f0 = (const C*)F.fh0 + (size_t)(m0 + w) * Sx;
+                    const C sc = s_sc[w];
+                    for (int i = lane; i < Sx; i += 32) fs[i] = F.sc ? sc * f0[i] : f0[i];
+                } else {
+                    const C a0 = s_vin[0][w], a1 = s_vin[1][w], a2 = s_vin[2][w], a3 = s_vin[3][w];
+                    for (int i = lane; i < Sx; i += 32) {
+                        C f = a0 * s_v[i];
+                        cfma(f, a1, s_v[Sx + i]);
+                        cfma(f, a2, s_v[2 * Sx + i]);
+                        cfma(f, a3, s_v[3 * Sx + i]);
+                        fs[i] = f;
+                    }
+                }
+                __syncwarp();
+                line_solve(s_xi + w * Sx, fs, Sx, lane, u ? pf[1] : pf[0], u ? pb[1] : pb[0]);
+            }
+            __syncthreads();
+            // rows of the result: up (to the cut above) and down, one thread a column and pair
+            if (nm > 0)
+                for (int q = tid; q < 2 * Sx; q += NT) {
+                    const int h = q >= Sx, i = q - h * Sx;
+                    if (F.rout[2 * h] < 0) continue;
+                    C o0 = {0, 0}, o1 = {0, 0};
+                    for (int w = 0; w < nm; ++w) {
+                        const C f = s_ln[w * Sx + i];
+                        cfma(o0, s_vout[2 * h][w], f);
+                        cfma(o1, s_vout[2 * h + 1][w], f);
+                    }
+                    // h = 0: rows 2, 3 of cut lf - 1; h = 1: rows 0, 1 of cut lf
+                    const int cc = lf - 1 + h, row = h ? 0 : 2, grp = rank - lf * ngrp;
+                    const int k = i / XC;
+                    const int ka = (i - k * XC == 0 && k > 0) ? k - 1 : k;
+                    const int kb = (i - k * XC == XC - 1 && k + 1 < nch) ? k + 1 : k;
+                    for (int kk = ka; kk <= kb; ++kk) {
+                        const int dst = cc * nch + kk, il = i - kk * XC + 1;
+                        const uint32_t rm = mapa(mb, dst);
+                        const uint32_t ra = mapa(smem_u32(s_bx + (row * ngrp + grp) * (XC + 2) + il), dst);
+                        st_async(ra, o0, rm);
+                        st_async(ra + 8u * ngrp * (XC + 2), o1, rm);
+                    }
+                }
+            if (!(ok = wait(0, by1))) break;
+            if (timing) { const unsigned long long t = gtime(); tA += t - t0; t0 = t; }
+            // ------------------------------------------------------------------ B
+            if (has_b) {
+                for (int q = tid; q < 4 * (XC + 2); q += NT) {
+                    const int row = q / (XC + 2), il = q - row * (XC + 2);
+                    C s = {0, 0};
+                    for (int u = 0; u < ngrp; ++u) s = s + s_bx[(row * ngrp + u) * (XC + 2) + il];
+                    s_t[q] = s;
+                }
+                __syncthreads();
+                for (int q = tid; q < 2 * xn; q += NT) {
+                    const int row = q / xn, il = q - row * xn, i = x0 + il;
+                    const C vv = s_own[row * XC + il];
+                    if (!first) s_vs[row * XC + il] = s_vs[row * XC + il] + vv;
+                    const C* tc = s_t + (row + 1) * (XC + 2) + il + 1;
+                    C at;
+                    if (P.q1) {
+                        at = q1_row<float>(1, i, g, [&](int dj, int di) { return tc[dj * (XC + 2) + di]; });
+                    } else {
+                        at = op_diag_t<float>(1, i, g) * tc[0] - tc[-1] - tc[1] -
+                             (float)wcol(i, Sx) * (tc[-(XC + 2)] + tc[XC + 2]);
+                    }
+                    s_rs[row * XC + il] = vv - at;
+                }
+                __syncthreads();
+                for (int k0 = 0; k0 < K; k0 += 32) {
+                    const int k = k0 + lane;
+                    if (k < K) {
+                        C a0 = {0, 0}, a1 = {0, 0};
+                        for (int il = warp; il < xn; il += NW) {
+                            cfma_cj(a0, s_c[il * K + k], s_rs[il]);
+                            cfma_cj(a1, s_c[(XC + il) * K + k], s_rs[XC + il]);
+                        }
+                        s_red[(warp * 2) * L * r + k] = a0;
+                        s_red[(warp * 2 + 1) * L * r + k] = a1;
+                    }
+                }
+                __syncthreads();
+                // slots (the ancestors' columns, the own node's first and second child), four
+                // lanes a slot, each sending to four blocks
+                const int ns = (lev + 2) * r;
+                for (int q = tid; q < (ns * 4 + 31) / 32 * 32; q += NT) {
+                    const int s = q >> 2, sub = q & 3;
+                    C t = {0, 0};
+                    if (s < ns) {
+                        const bool own1 = s >= (lev + 1) * r;
+                        const int k = own1 ? s - r : s;
+                        for (int w = sub; w < NW; w += 4) {
+                            if (!own1) t = t + s_red[(w * 2) * L * r + k];
+                            if (own1 || s < lev * r) t = t + s_red[(w * 2 + 1) * L * r + k];
+                        }
+                    }
+#pragma unroll
+                    for (int o = 1; o < 4; o <<= 1) {
+                        t.re += __shfl_xor_sync(0xffffffffu, t.re, o);
+                        t.im += __shfl_xor_sync(0xffffffffu, t.im, o);
+                    }
+                    if (s < ns) {
+                        const uint32_t la = smem_u32(s_bd + rank * (L + 1) * r + s);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int dst = 4 * sub + u;
+                            st_async(mapa(la, dst), t, mapa(mb + 8, dst));
+                        }
+                    }
+                }
+            }
+            else if (tid < CC_CL) st_async(mapa(smem_u32(&s_word[rank]), tid), 0.f, mapa(mb + 8, tid));
+            if (!(ok = wait(1, by2))) break;
+            // ------------------------------------------------------------------ Y
+            for (int q = tid; q < D * 4; q += NT) {
+                const int e = q >> 2, sub = q & 3;
+                const int p = e / (2 * r), j = e - p * 2 * r, k = j >= r, jr = j - k * r;
+                const int l = 31 - __clz(p + 1), t = p + 1 - (1 << l);
+                const int span = 1 << (L - l), ca = t * span + k * (span / 2), own = t * span + span / 2 - 1;
+                const int nin = span / 2 - 1;
+                C s = {0, 0};
+                for (int u = sub; u < (nin + 1) * nch; u += 4) {
+                    const int cc = u / nch, cu = cc < nin ? ca + cc : own;
+                    s = s + s_bd[(cu * nch + u - cc * nch) * (L + 1) * r + (cc < nin ? l : l + k) * r + jr];
+                }
+#pragma unroll
+                for (int o = 1; o < 4; o <<= 1) {
+                    s.re += __shfl_xor_sync(__activemask(), s.re, o);
+                    s.im += __shfl_xor_sync(__activemask(), s.im, o);
+                }
+                if (sub == 0) s_d[e] = s;
+            }
+            __syncthreads();
+            // y = M d: M transposed within a node's rows, so that the lanes' reads are
+            // consecutive; a row's columns shared out over NT / D threads
+            const int ks = min(5, NT / D);
+            for (int q = tid; q < D * ks; q += NT) {
+                const int sub = q / D, e = q - sub * D;
+                const int p = e / (2 * r), i = e - p * 2 * r;
+                int l, t;
+                const int mo = cut_m_row(p * 2 * r, L, r, l, t);
+                C s = {0, 0};
+                for (int lv = l, k0 = 0; lv < L; ++lv) {   // the subtree's columns, level by level
+                    const C* dl = s_d + ((1 << lv) - 1 + (t << (lv - l))) * 2 * r;
+                    const C* ml = s_m + mo + k0 * 2 * r + i;
+                    const int n = 2 * r << (lv - l);
+#pragma unroll 4
+                    for (int k = sub; k < n; k += ks) cfma(s, ml[k * 2 * r], dl[k]);
+                    k0 += n;
+                }
+                s_up[sub * D + e] = s;
+            }
+            __syncthreads();
+            for (int e = tid; e < D; e += NT) {
+                C s = s_up[e];
+                for (int u = 1; u < ks; ++u) s = s + s_up[u * D + e];
+                s_y[e] = s;
+                if (rank == 0) s_ya[e] = s_ya[e] + s;
+            }
+            __syncthreads();
+            if (timing) { const unsigned long long t = gtime(); tB += t - t0; t0 = t; }
+            // ------------------------------------------------------------------ C
+            float nn = 0.f;
+            if (has_b) {
+                const int np = 2 * xn, kg = min(CUT_KG, max(1, NT / np));
+                for (int q = tid; q < np * kg; q += NT) {
+                    const int kk = q / np, pr = q - kk * np, row = pr >= xn, il = pr - row * xn;
+                    const C* er = s_e + (size_t)row * Ke * XC + il;
+                    C s = {0, 0};
+#pragma unroll 4
+                    for (int k = kk; k < Ke; k += kg) cfma(s, er[k * XC], s_y[s_yi[k]]);
+                    s_up[kk * 2 * XC + row * XC + il] = s;
+                }
+                __syncthreads();
+                for (int q = tid; q < np; q += NT) {
+                    const int row = q >= xn, il = q - row * xn;
+                    C s = s_rs[row * XC + il];
+                    for (int w = 0; w < kg; ++w) s = s - s_up[w * 2 * XC + row * XC + il];
+                    s_own[row * XC + il] = s;
+                    nn += abs2(inv0 * s);
+                }
+                __syncthreads();
+                const int nd = ng0 + ng1;
+                for (int q = tid; q < np * nd; q += NT) {
+                    const int dq = q / np, pr = q - dq * np, row = pr >= xn, il = pr - row * xn;
+                    // leaf c (its cut below: input rows 2, 3), then leaf c + 1 (rows 0, 1)
+                    const bool up = dq < ng0;
+                    const int dst = up ? c * ngrp + dq : (c + 1) * ngrp + dq - ng0;
+                    const uint32_t la = smem_u32(s_v + ((up ? 2 : 0) + row) * Sx + x0 + il);
+                    st_async(mapa(la, dst), s_own[row * XC + il], mapa(mb + 16, dst));
+                }
+            }
+            // |v|^2: one partial of the first four warps to every block
+            nn = warp_sum(nn);
+            if (warp < 4 && lane < CC_CL) st_async(mapa(smem_u32(&s_nrm[rank][warp]), lane), nn, mapa(mb + 16, lane));
+            if (!(ok = wait(2, by3))) break;
+            n2 = 0.f;
+            for (int q = 0; q < CC_CL; ++q) n2 += (s_nrm[q][0] + s_nrm[q][1]) + (s_nrm[q][2] + s_nrm[q][3]);
+            if (timing) { const unsigned long long t = gtime(); tC += t - t0; t0 = t; }
+            first = false;
+            ++it;
+            ++in_round;
+            ++phase;
+            reason = watch.test(n2, it, P, thr_anchor, thr_test);
+            if (reason) break;
+        }
+        if (ok && has_b)
+            for (int q = tid; q < 2 * xn; q += NT) {
+                const int row = q / xn, il = q - row * xn;
+                const size_t o = ((size_t)c * 2 + row) * Sx + x0 + il;
+                ((C*)P.vsum)[o] = s_vs[row * XC + il];
+                ((C*)P.v)[o] = s_own[row * XC + il];
+            }
+        if (ok && rank == 0) {
+            for (int e = tid; e < D; e += NT) ((C*)P.yacc)[e] = s_ya[e];
+            if (tid == 0) {
+                ctl->it = it;
+                ctl->in_round = in_round;
+                ctl->reason = reason;
+                ctl->n2 = (double)n2 * n0;
+                ctl->n0 = n0;
+                watch.store(*ctl, n0);
+                ctl->ns[0] += (double)tA;
+                ctl->ns[1] += (double)tB;
+                ctl->ns[2] += (double)tC;
+            }
+        }
+    }
+    // no block leaves while another's stores may still arrive (after a wait that gave up,
+    // also those nobody waited for)
+    cluster.sync();
+    if (!ok) __nanosleep(20000);
+    cluster.sync();
+}
+
+// The round's summed inputs through the leaves: Fh = the recursions of f^_0 + V^T (the cut
+// rows' sums), one warp per mode, for the transform back of every row.
+template <typename T>
+__global__ void __launch_bounds__(256) k_cut_lines(const CutProb* __restrict__ probs, const int* modes, int wpb) {
+    using C = cplx<T>;
+    if (modes && !modes[blockIdx.z]) return;
+    const CutProb& P = probs[blockIdx.z];
+    if ((int)blockIdx.y >= P.ncut + 1) return;
+    const int Sx = P.Sx, lf = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const CutLeaf& F = P.leaf[lf];
+    const int m = blockIdx.x * wpb + warp;
+    if (warp >= wpb || m >= F.b) return;
+    extern __shared__ __align__(16) unsigned char lsm[];
+    C* as = (C*)lsm + (size_t)warp * 2 * Sx;
+    C* fs = as + Sx;
+    const C* xi = (const C*)F.xi + (size_t)m * Sx;
+    const C* f0 = (const C*)F.fh0 + (size_t)m * Sx;
+    const C sc = F.sc ? ((const C*)F.sc)[m] : C{1, 0};
+    C vin[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) vin[k] = F.rin[k] >= 0 ? ((const C*)F.V)[(size_t)F.rin[k] * F.b + m] : C{0, 0};
+    for (int i = lane; i < Sx; i += 32) {
+        C f = f0[i];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (F.rin[k] >= 0)
+                cfma(f, vin[k], ((const C*)P.vsum)[((size_t)(lf - (k < 2)) * 2 + (k & 1)) * Sx + i]);
+        as[i] = xi[i];
+        fs[i] = F.sc ? sc * f : f;
+    }
+    __syncwarp();
+    warp_line_solve(as, fs, Sx, lane);
+    C* fh = (C*)F.fh + (size_t)m * Sx;
+    for (int i = lane; i < Sx; i += 32) fh[i] = fs[i];
+}
+
+// ut = u + w + sum over the levels of C_p y_p at every grid point (w: the composed leaf
+// solutions; y: the round's summed corrections).  HBM-bound: each level's basis read once,
+// L r values a point.  One block per row and 256 columns; rows of one leaf share the nodes.
+template <typename T>
+__global__ void __launch_bounds__(256) k_cut_update(const CutUpdJob* __restrict__ jobs) {
+    using C = cplx<T>;
+    __shared__ C sy[CUT_KMAX];
+    const CutUpdJob& J = jobs[blockIdx.z];
+    const CutProb& P = *J.prob;
+    const int Sx = P.Sx, r = P.r, L = P.L, row = blockIdx.y;
+    if (row >= J.Sy || (int)blockIdx.x * 256 >= Sx) return;
+    int lf = 0;
+    while (lf < P.ncut && row >= P.mid[lf]) ++lf;
+    for (int t = threadIdx.x; t < L * r; t += 256) {
+        const int l = t / r, j = t - l * r;
+        const int p = (1 << l) - 1 + (lf >> (L - l)), k = (lf >> (L - l - 1)) & 1;
+        sy[t] = ((const C*)P.yacc)[(size_t)p * 2 * r + k * r + j];
+    }
+    __syncthreads();
+    const int x = blockIdx.x * 256 + threadIdx.x;
+    if (x >= Sx) return;
+    const size_t o = (size_t)row * Sx + x;
+    C acc = ((const C*)J.w)[o];
+    for (int l = 0; l < L; ++l) {
+        const int p = (1 << l) - 1 + (lf >> (L - l)), k = (lf >> (L - l - 1)) & 1;
+        const CutNode& nd = P.node[p];
+        const C* c = (const C*)nd.C + (size_t)(k * r) * nd.N + (size_t)(row - nd.ra) * Sx + x;
+#pragma unroll 16
+        for (int j = 0; j < r; ++j) cfma(acc, c[(size_t)j * nd.N], sy[l * r + j]);
+    }
+    const c128 u = J.u[o];
+    J.ut[o] = u + cvt<double>(acc);
+}
+
+// ---------------------------------------------------------------------- launchers
+template <typename T>
+void launch_cut_panels(const CutCpEntry* cp, int ncp, const CutEpEntry* ep, int nep, int Sx, int r, OpGeom g,
+                       cudaStream_t s) {
+    g.b = 3;
+    k_cut_cp<T><<<dim3((Sx + 31) / 32, ncp), 256, 0, s>>>(cp, Sx, r);
+    note_launch();
+    k_cut_ep<T><<<dim3((Sx + 255) / 256, nep, r), 256, 0, s>>>(ep, Sx, r, g);
+    note_launch();
+}
+size_t cut_gram_scratch(int npairs) { return (size_t)npairs * GRAM_SPLIT * 1024 * sizeof(c128); }
+template <typename T>
+void launch_cut_gram(const CutGramPair* prs, int npairs, const CutGramDest* ds, int ndest, int Sx, int r, c128* part,
+                     cudaStream_t s) {
+    k_cut_gram<T><<<dim3(npairs, GRAM_SPLIT), 256, 0, s>>>(prs, Sx, r, part);
+    note_launch();
+    k_cut_gram_red<<<ndest, 256, 0, s>>>(ds, r, part);
+    note_launch();
+}
+template <typename T>
+void launch_cut_minv(const CutMinv* prs, int n, int D, int L, int p2, const c128* G, c128* M, cplx<T>* MT, int tr,
+                     cudaStream_t s) {
+    static std::atomic<unsigned long long> attr{0};
+    smem_limit_once(attr, k_cut_minv<T>, 64 * 64 * sizeof(c128));
+    k_cut_minv<T><<<n, 256, sizeof(c128) * p2 * p2, s>>>(prs, D, L, p2, G, M, MT, tr);
+    note_launch();
+}
+
+size_t cut_m_packed(int L, int r) { return (size_t)cut_m_elems(L, r); }
+
+// Items of a problem and the shared memory of its steps; 0 bytes when the lines do not fit.
+// Two forms, by what bounds them:
+//  * the complex64 problems whose lines, panels and M fit sixteen blocks' shared memory run
+//    on one cluster of sixteen (k_cut_cluster), bound by latency alone;
+//  * the others on a grid group of up to one block per SM (k_cut_steps): there the lines
+//    (FP64: the pipe, four warps fill it) and the panels' bytes want every SM.
+static constexpr int CUT_NT = 256, CUT_SMEM = 216 * 1024;
+static bool cluster_form(CutProb& P, int b_max) {
+    const int NL = P.ncut + 1;
+    if (P.D > 128 || NL > CC_CL) return false;
+    P.MG = (b_max + CC_CL / NL - 1) / (CC_CL / NL);
+    P.ngrp = (b_max + P.MG - 1) / P.MG;
+    P.nA = NL * P.ngrp;
+    P.XC = (P.Sx + CC_CL / P.ncut - 1) / (CC_CL / P.ncut);
+    P.nch = (P.Sx + P.XC - 1) / P.XC;
+    P.nB = P.ncut * P.nch;
+    // two lines a warp; |v|^2 comes from the first four warps; the halo is one neighbour's
+    return P.MG <= 2 * CC_NW && P.MG <= CUT_MGMAX && 2 * P.XC <= 128 && P.XC >= 2 &&
+           (2 * P.L) * P.r <= 2 * CUT_KMAX && sizeof(c64) * cc_layout(P).total <= (size_t)CUT_SMEM;
+}
+template <typename T>
+size_t cut_plan(CutProb& P, int b_max) {
+    const size_t c = sizeof(cplx<T>), cap = CUT_SMEM;
+    const int NL = P.ncut + 1;
+    P.res = P.dist = 0;
+    P.nbi = 1;
+    P.cl = sizeof(T) == 4 && cluster_form(P, b_max);
+    if (P.cl) return c * cc_layout(P).total;
+    P.XC = std::min(64, std::max(8, (P.ncut * P.Sx + 147) / 148));
+    P.nch = (P.Sx + P.XC - 1) / P.XC;
+    P.nB = P.ncut * P.nch;
+    P.nbi = (P.nB + 147) / 148;
+    for (int mg = std::min(8, std::max(2, (NL * b_max + 147) / 148)); mg >= 1; --mg) {
+        P.MG = mg;
+        // every block's y = M d while D is small (FP64: its products cost more than the two
+        // barriers); the panels kept where there is room
+        for (int o = P.D > (sizeof(T) == 4 ? 128 : 32) ? 2 : 0; o < 4; ++o) {
+            P.dist = o >> 1;
+            P.res = !(o & 1);
+            const size_t b = c * cut_smem_layout(P, CUT_NT / 32).total;
+            if (b > cap) continue;
+            P.ngrp = (b_max + mg - 1) / mg;
+            P.nA = NL * P.ngrp;
+            return b;
+        }
+    }
+    return 0;
+}
+// Clusters of CC_CL blocks with this much shared memory that run at once (0: none).
+static int cluster_count(size_t smem) {
+    static std::atomic<unsigned long long> attr{0};
+    if (!once_per_device(attr, [] {
+            return cudaFuncSetAttribute(k_cut_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, CUT_SMEM) ==
+                       cudaSuccess &&
+                   cudaFuncSetAttribute(k_cut_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+                       cudaSuccess;
+        })) {
+        cudaGetLastError();
+        return 0;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    cfg.gridDim = dim3(CC_CL);
+    cfg.blockDim = dim3(CC_NT);
+    cfg.dynamicSmemBytes = smem;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CC_CL;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_cut_cluster, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+    }
+    return n;
+}
+bool cut_cluster_ready(size_t smem) { return cluster_count(smem) > 0; }
+template <typename T>
+bool launch_cut_steps(const CutProb* probs, int nprob, int group, bool cl, size_t smem, const int* modes, int mode_all,
+                      unsigned* bars, int max_groups, int* err, int prof, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaError_t e;
+    const long long polls = wait_polls(1ll << 24);
+    if (cl) {
+        const int nmax = cluster_count(smem);
+        if (nmax < 1) return false;
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = CC_CL;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(CC_CL * std::min(nprob, nmax));
+        cfg.blockDim = dim3(CC_NT);
+        // (a try_wait suspends for up to microseconds: fewer of them make about a second)
+        e = cudaLaunchKernelEx(&cfg, k_cut_cluster, probs, nprob, modes, mode_all, err, std::min(polls, 1ll << 20),
+                               prof);
+    } else {
+        static std::atomic<unsigned long long> attr{0};
+        smem_limit_once(attr, k_cut_steps<T, CUT_NT>, CUT_SMEM);
+        int sms = 0, nb = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, current_device());
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cut_steps<T, CUT_NT>, CUT_NT, smem) != cudaSuccess ||
+            nb < 1) {
+            cudaGetLastError();
+            return false;
+        }
+        const int gsz = std::min(group, sms * nb), ng = std::max(1, std::min({nprob, sms * nb / gsz, max_groups}));
+        cudaMemsetAsync(bars, 0, sizeof(unsigned) * ng, s);
+        at[0].id = cudaLaunchAttributeCooperative;
+        at[0].val.cooperative = 1;
+        cfg.gridDim = dim3(gsz * ng);
+        cfg.blockDim = dim3(CUT_NT);
+        e = cudaLaunchKernelEx(&cfg, k_cut_steps<T, CUT_NT>, probs, nprob, gsz, modes, mode_all, bars, err, polls,
+                               prof);
+    }
+    note_launch();
+    return e == cudaSuccess;
+}
+template <typename T>
+void launch_cut_lines(const CutProb* probs, int nprob, const int* modes, int nleaf_max, int b_max, int Sx_max,
+                      cudaStream_t s) {
+    static std::atomic<unsigned long long> attr{0};
+    smem_limit_once(attr, k_cut_lines<T>, 200 * 1024);
+    const size_t per = 2 * sizeof(cplx<T>) * (size_t)Sx_max;
+    const int wpb = (int)std::max<size_t>(1, std::min<size_t>(8, (200u << 10) / per));
+    k_cut_lines<T><<<dim3((b_max + wpb - 1) / wpb, nleaf_max, nprob), 256, per * wpb, s>>>(probs, modes, wpb);
+    note_launch();
+}
+template <typename T>
+void launch_cut_update(const CutUpdJob* jobs, int njobs, int Sy_max, int Sx_max, cudaStream_t s) {
+    k_cut_update<T><<<dim3((Sx_max + 255) / 256, Sy_max, njobs), 256, 0, s>>>(jobs);
+    note_launch();
+}
+
+#define HH_CUT_INST(T)                                                                                             \
+    template void launch_cut_panels<T>(const CutCpEntry*, int, const CutEpEntry*, int, int, int, OpGeom, cudaStream_t); \
+    template void launch_cut_gram<T>(const CutGramPair*, int, const CutGramDest*, int, int, int, c128*, cudaStream_t); \
+    template void launch_cut_minv<T>(const CutMinv*, int, int, int, int, const c128*, c128*, cplx<T>*, int, cudaStream_t); \
+    template size_t cut_plan<T>(CutProb&, int);                                                                       \
+    template bool launch_cut_steps<T>(const CutProb*, int, int, bool, size_t, const int*, int, unsigned*, int, int*, int,   \
+                                      cudaStream_t);                                                                  \
+    template void launch_cut_lines<T>(const CutProb*, int, const int*, int, int, int, cudaStream_t);                  \
+    template void launch_cut_update<T>(const CutUpdJob*, int, int, int, cudaStream_t);
+HH_CUT_INST(float)
+HH_CUT_INST(double)
+
+}  // namespace hh

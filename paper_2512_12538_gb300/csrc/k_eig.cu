@@ -40,6 +40,7 @@
 
 #include <cooperative_groups.h>
 
+#include "k_line.cuh"
 #include "kernels.h"
 
 namespace cg = cooperative_groups;
@@ -563,67 +564,7 @@ __global__ void __launch_bounds__(256) k_eig_gemm2(const EigTask* __restrict__ t
 }
 
 // Scalar recursions along each line, in place on Fh[m][c][i]: one warp per line (mode m,
-// right-hand side c).  Both recursions are affine, y_i = xi_i y_{i-1} + xi_i f_i and
-// x_i = xi_i x_{i+1} + y_i (with x_{n-1} = y_{n-1}), so each lane composes the maps of a
-// contiguous chunk of the line, a warp scan (shuffles) composes the chunks, and each lane
-// then replays its chunk from its entering value.  The line is staged in shared memory.
-template <typename T>
-__device__ __forceinline__ void affine_shfl(cplx<T>& A, cplx<T>& B, int d, bool up, cplx<T>& A2, cplx<T>& B2) {
-    if (up) {
-        A2.re = __shfl_up_sync(0xffffffffu, A.re, d); A2.im = __shfl_up_sync(0xffffffffu, A.im, d);
-        B2.re = __shfl_up_sync(0xffffffffu, B.re, d); B2.im = __shfl_up_sync(0xffffffffu, B.im, d);
-    } else {
-        A2.re = __shfl_down_sync(0xffffffffu, A.re, d); A2.im = __shfl_down_sync(0xffffffffu, A.im, d);
-        B2.re = __shfl_down_sync(0xffffffffu, B.re, d); B2.im = __shfl_down_sync(0xffffffffu, B.im, d);
-    }
-}
-
-// Both recursions of one line, in place: on entry fs = f^ (Sx values) and as = xi; on
-// exit fs = x^.  One warp; lane l owns the contiguous chunk [l L, (l + 1) L).
-template <typename T>
-__device__ __forceinline__ void warp_line_solve(const cplx<T>* as, cplx<T>* fs, int Sx, int lane) {
-    using C = cplx<T>;
-    const int L = (Sx + 31) / 32;
-    const int s = lane * L, e = min(Sx, s + L);
-    // forward: y_i = a_i (y_{i-1} + f_i)
-    C A = {1, 0}, B = {0, 0};
-    for (int i = s; i < e; ++i) { A = as[i] * A; B = as[i] * (B + fs[i]); }
-    for (int d = 1; d < 32; d <<= 1) {
-        C A2, B2;
-        affine_shfl(A, B, d, true, A2, B2);
-        if (lane >= d) { B = A * B2 + B; A = A * A2; }
-    }
-    C y;
-    y.re = __shfl_up_sync(0xffffffffu, B.re, 1);
-    y.im = __shfl_up_sync(0xffffffffu, B.im, 1);
-    if (lane == 0) y = {0, 0};
-    for (int i = s; i < e; ++i) { y = as[i] * (fs[i] + y); fs[i] = y; }
-    __syncwarp();
-    // backward: x_i = y_i + a'_i x_{i+1}, a'_{n-1} = 0
-    A = {1, 0};
-    B = {0, 0};
-    for (int i = e - 1; i >= s; --i) {
-        const C ap = (i == Sx - 1) ? C{0, 0} : as[i];
-        B = ap * B + fs[i];
-        A = ap * A;
-    }
-    for (int d = 1; d < 32; d <<= 1) {
-        C A2, B2;
-        affine_shfl(A, B, d, false, A2, B2);
-        if (lane + d < 32) { B = A * B2 + B; A = A * A2; }
-    }
-    C x;
-    x.re = __shfl_down_sync(0xffffffffu, B.re, 1);
-    x.im = __shfl_down_sync(0xffffffffu, B.im, 1);
-    if (lane == 31) x = {0, 0};
-    for (int i = e - 1; i >= s; --i) {
-        const C ap = (i == Sx - 1) ? C{0, 0} : as[i];
-        x = fs[i] + ap * x;
-        fs[i] = x;
-    }
-    __syncwarp();
-}
-
+// right-hand side c), by warp_line_solve; the line is staged in shared memory.
 template <typename T>
 __global__ void __launch_bounds__(256) k_eig_recur(const EigTask* __restrict__ tasks, int Sx, int nrhs, int wpb,
                                                    const int* gate) {
@@ -868,9 +809,6 @@ __global__ void __launch_bounds__(FS_THREADS) k_eig_sweep_fused(const EigTask* _
     const int q = (int)cluster.block_rank();
     const int cl = (int)cluster.num_blocks();
     const EigTask tk = tasks[blockIdx.y];
-    // a task of a problem that has left (the same word for the whole cluster): return before
-    // any cluster barrier and any access to its buffers
-    if (tk.gate && *tk.gate) return;
     const int b = tk.b;
     const int Sx = tk.Sx;
     const FsGeom G = fs_geom(b, Sx, cl);

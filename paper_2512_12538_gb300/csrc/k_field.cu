@@ -98,15 +98,11 @@ struct ResidStop {
     int* ctl;
     unsigned* ticket;
     double tol;
-    const int* need;     // may be null: else the launch does nothing while *need is zero
-    const int* anchor;   // may be null: else yt is written only while *anchor is nonzero
 };
 template <typename T, bool Q1>
 __global__ void k_residual_cast(const c128* __restrict__ x, const c128* __restrict__ v, c128* __restrict__ y,
                                 cplx<T>* __restrict__ yt, OpGeom g, double* part, const int* gate, ResidStop stop) {
     if (gate && *gate) return;
-    if (stop.need && !*stop.need) return;
-    const bool wt = !stop.anchor || *stop.anchor;
     const size_t total = (size_t)g.b * g.Sx;
     // interior points of a 2D band with one k: the row is (4 - (kh)^2) x minus the four
     // neighbours, formed as v - (4 - (kh)^2) x (one FMA) plus the neighbours' sum, without
@@ -143,7 +139,7 @@ __global__ void k_residual_cast(const c128* __restrict__ x, const c128* __restri
             out = v[t] - ax;
         }
         if (y) y[t] = out;
-        if (wt) yt[t] = cvt<T>(out);
+        yt[t] = cvt<T>(out);
         acc2 = fma(out.re, out.re, acc2);
         acc2 = fma(out.im, out.im, acc2);
         i += step_r;
@@ -216,7 +212,7 @@ void launch_residual_cast(const c128* x, const c128* v, c128* y, cplx<T>* yt, Op
                           cudaStream_t s, const int* gate) {
     const size_t total = (size_t)g.b * g.Sx;
     const int grid = g.q1 ? resid_grid<T, true>(total) : resid_grid<T, false>(total);
-    const ResidStop none{nullptr, nullptr, nullptr, 0.0, nullptr, nullptr};
+    const ResidStop none{nullptr, nullptr, nullptr, 0.0};
     if (g.q1) k_residual_cast<T, true><<<grid, 256, 0, s>>>(x, v, y, yt, g, part, gate, none);
     else k_residual_cast<T, false><<<grid, 256, 0, s>>>(x, v, y, yt, g, part, gate, none);
     note_launch();
@@ -224,52 +220,18 @@ void launch_residual_cast(const c128* x, const c128* v, c128* y, cplx<T>* yt, Op
 }
 template <typename T>
 void launch_residual_stop(const c128* x, const c128* v, c128* y, cplx<T>* yt, OpGeom g, double* part, double* nrm,
-                          int* ctl, unsigned* ticket, double tol, cudaStream_t s, const int* need,
-                          const int* anchor) {
+                          int* ctl, unsigned* ticket, double tol, cudaStream_t s) {
     const size_t total = (size_t)g.b * g.Sx;
     const int grid = g.q1 ? resid_grid<T, true>(total) : resid_grid<T, false>(total);
-    const ResidStop st{nrm, ctl, ticket, tol, need, anchor};
+    const ResidStop st{nrm, ctl, ticket, tol};
     if (g.q1) k_residual_cast<T, true><<<grid, 256, 0, s>>>(x, v, y, yt, g, part, ctl, st);
     else k_residual_cast<T, false><<<grid, 256, 0, s>>>(x, v, y, yt, g, part, ctl, st);
     note_launch();
 }
 template void launch_residual_stop<float>(const c128*, const c128*, c128*, c64*, OpGeom, double*, double*, int*,
-                                          unsigned*, double, cudaStream_t, const int*, const int*);
+                                          unsigned*, double, cudaStream_t);
 template void launch_residual_stop<double>(const c128*, const c128*, c128*, c128*, OpGeom, double*, double*, int*,
-                                           unsigned*, double, cudaStream_t, const int*, const int*);
-
-// y[j N + pt] = (A~ x_j)[pt] for p column-major columns (one thread per (column, point))
-template <typename T>
-__global__ void k_apply_cols(const cplx<T>* __restrict__ x, cplx<T>* __restrict__ y, OpGeom g, int p) {
-    const size_t N = (size_t)g.b * g.Sx, total = N * p;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-        const size_t pt = t % N;
-        const int i = (int)(pt % g.Sx), j = (int)(pt / g.Sx);
-        cplx<T> ax;
-        if (g.q1) {
-            ax = q1_row<T>(j, i, g, [&](int dj, int di) { return x[(size_t)((long long)t + (long long)dj * g.Sx + di)]; });
-        } else {
-            ax = op_diag_t<T>(j, i, g) * x[t];
-            const T wj = (j == 0 || j == g.b - 1) ? (T)0.5 : (T)1;
-            const T wi = g.Sx == 1 ? (T)1 : ((i == 0 || i == g.Sx - 1) ? (T)0.5 : (T)1);
-            if (g.Sx > 1) {
-                if (i > 0) ax = ax - wj * x[t - 1];
-                if (i < g.Sx - 1) ax = ax - wj * x[t + 1];
-            }
-            if (j > 0) ax = ax - wi * x[t - g.Sx];
-            if (j < g.b - 1) ax = ax - wi * x[t + g.Sx];
-        }
-        y[t] = ax;
-    }
-}
-template <typename T>
-void launch_apply_cols(const cplx<T>* x, cplx<T>* y, OpGeom g, int p, cudaStream_t s) {
-    const size_t total = (size_t)g.b * g.Sx * p;
-    k_apply_cols<T><<<grid_for(total, 256), 256, 0, s>>>(x, y, g, p);
-    note_launch();
-}
-template void launch_apply_cols<float>(const c64*, c64*, OpGeom, int, cudaStream_t);
-template void launch_apply_cols<double>(const c128*, c128*, OpGeom, int, cudaStream_t);
+                                           unsigned*, double, cudaStream_t);
 template void launch_residual_cast<float>(const c128*, const c128*, c128*, c64*, OpGeom, double*, int*, cudaStream_t,
                                           const int*);
 template void launch_residual_cast<double>(const c128*, const c128*, c128*, c128*, OpGeom, double*, int*,
@@ -283,7 +245,6 @@ __global__ void k_residual_batch(ResidBatch bt, double* part) {
     int jb = 0;
     while (jb + 1 < bt.njobs && blockIdx.x >= bt.job[jb + 1].blk0) ++jb;
     const ResidJob& J = bt.job[jb];
-    if (J.gate && *J.gate) return;   // a problem that has left: nothing of it is touched
     const OpGeom g = J.g;
     const size_t total = (size_t)g.b * g.Sx;
     const unsigned lb = blockIdx.x - J.blk0;
@@ -305,7 +266,6 @@ __global__ void k_residual_batch(ResidBatch bt, double* part) {
             if (j < g.b - 1) ax = ax - wi * J.x[t + g.Sx];
         }
         const c128 out = J.v[t] - ax;
-        J.y[t] = out;
         ((cplx<T>*)J.yt)[t] = cvt<T>(out);
         acc2 += abs2(out);
     }
@@ -319,9 +279,8 @@ __global__ void k_residual_batch(ResidBatch bt, double* part) {
         if (threadIdx.x == 0) part[blockIdx.x] = s2;
     }
 }
-__global__ void k_sum_batch(ResidBatch bt, const double* part, double* norms) {
+__global__ void k_sum_batch(ResidBatch bt, const double* part) {
     const ResidJob& J = bt.job[blockIdx.x];
-    if (J.gate && *J.gate) return;
     double a = 0.0;
     for (unsigned i = threadIdx.x; i < J.nblk; i += blockDim.x) a += part[J.blk0 + i];
     __shared__ double red[32];
@@ -331,11 +290,11 @@ __global__ void k_sum_batch(ResidBatch bt, const double* part, double* norms) {
     if (threadIdx.x < 32) {
         double s2 = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
         s2 = warp_sum(s2);
-        if (threadIdx.x == 0) norms[blockIdx.x] = s2;
+        if (threadIdx.x == 0) *J.norm = s2;
     }
 }
 template <typename T>
-void launch_residual_batch(ResidBatch bt, double* part, int part_cap, double* norms, cudaStream_t s) {
+void launch_residual_batch(ResidBatch bt, double* part, int part_cap, cudaStream_t s) {
     if (bt.njobs < 1) return;
     const int cap = std::max(1, std::min(152 * 2, part_cap / bt.njobs));
     unsigned blk = 0;
@@ -347,11 +306,11 @@ void launch_residual_batch(ResidBatch bt, double* part, int part_cap, double* no
     }
     k_residual_batch<T><<<blk, 256, 0, s>>>(bt, part);
     note_launch();
-    k_sum_batch<<<bt.njobs, 256, 0, s>>>(bt, part, norms);
+    k_sum_batch<<<bt.njobs, 256, 0, s>>>(bt, part);
     note_launch();
 }
-template void launch_residual_batch<float>(ResidBatch, double*, int, double*, cudaStream_t);
-template void launch_residual_batch<double>(ResidBatch, double*, int, double*, cudaStream_t);
+template void launch_residual_batch<float>(ResidBatch, double*, int, cudaStream_t);
+template void launch_residual_batch<double>(ResidBatch, double*, int, cudaStream_t);
 
 __global__ void k_sum(const double* part, int n, double* out) {
     double a = 0.0;

@@ -22,43 +22,35 @@ template <typename T>
 void launch_residual_cast(const c128* x, const c128* v, c128* y, cplx<T>* yt, OpGeom g, double* part, int* nblk_out,
                           cudaStream_t s, const int* gate = nullptr);
 
-// Residuals of up to RB_MAX_JOBS problems in one launch: per job y = v - A x (FP64) and
-// yt = y in T; norms[k] = ||y_k||^2 (fixed-order sums).  part: scratch of part_cap doubles.
+// Residuals of up to RB_MAX_JOBS problems in one launch: per job yt = v - A x (FP64) rounded
+// to T and *norm = ||v - A x||^2 (fixed-order sums).  part: scratch of part_cap doubles.
 constexpr int RB_MAX_JOBS = 32;
 struct ResidJob {
     const c128* x;
     const c128* v;
-    c128* y;
     void* yt;
+    double* norm;
     OpGeom g;
     unsigned blk0, nblk;   // set by the launcher
-    const int* gate;       // may be null: while the word is nonzero the job touches nothing
 };
 struct ResidBatch {
     ResidJob job[RB_MAX_JOBS];
     int njobs;
 };
 template <typename T>
-void launch_residual_batch(ResidBatch bt, double* part, int part_cap, double* norms, cudaStream_t s);
+void launch_residual_batch(ResidBatch bt, double* part, int part_cap, cudaStream_t s);
 
 // out = sum of n doubles (deterministic single-block reduction)
 void launch_sum(const double* part, int n, double* out, cudaStream_t s);
-// A~ applied to p column-major columns of a node's band: y[j N + pt] = (A~ x_j)[pt].
-template <typename T>
-void launch_apply_cols(const cplx<T>* x, cplx<T>* y, OpGeom g, int p, cudaStream_t s);
-
 // launch_residual_cast with the stopping test of the stationary iteration kept on the
-// device, in the same launch.  Unless ctl[0] is already set, or need is given and zero
-// (then nothing is done); yt is written only when anchor is null or nonzero:
+// device, in the same launch.  Unless ctl[0] is already set (then nothing is done):
 // y (may be null: not stored), yt and the partials as launch_residual_cast, then
-// nrm[0] = ||y||^2 (launch_sum's
-// order), ctl[1] += 1, and with rel = sqrt(nrm[0] / nrm[2]) (0 when nrm[2] <= 0)
+// nrm[0] = ||y||^2 (launch_sum's order), ctl[1] += 1, and with rel = sqrt(nrm[0] / nrm[2]) (0 when nrm[2] <= 0)
 // ctl[0] = 2 if rel is not finite, 1 if rel < tol.  ctl[0] is the gate of the next
 // step's launches; ticket is a device counter that is zero between launches.
 template <typename T>
 void launch_residual_stop(const c128* x, const c128* v, c128* y, cplx<T>* yt, OpGeom g, double* part, double* nrm,
-                          int* ctl, unsigned* ticket, double tol, cudaStream_t s, const int* need = nullptr,
-                          const int* anchor = nullptr);
+                          int* ctl, unsigned* ticket, double tol, cudaStream_t s);
 
 // b = h^2 w_i w_j f + h (w_j gx + w_i gy) for the global problem (q1: the bilinear
 // elements' load vector, h^2 M_y F M_x^T + h (edge masses) g).
@@ -120,34 +112,11 @@ struct CoarseJob {
                            // out's old value), in the basis precision, at out's index
     int ngrp;              // set by the launcher: column groups per half (p/2 / CB_COLS, rounded up)
     unsigned sb[5];        // set by the launcher: blocks of set s are [sb[s], sb[s + 1])
-    const int* gate;       // may be null: while the word is nonzero the job's blocks only take
-                           // part in the grid barrier and touch none of the job's buffers
-};
-// Optional extras of a one-job launch on the root in the device-tested stationary loop.
-// Phase 1 keeps r' = v - A~ w (the residual after the level-1 update) in rp; phase 3
-// forms the next residual r' - (A C) y (AC: A applied to the basis, laid out as C) into
-// rt, with its |.|^2 per block in part, and the last block to finish (ticket: zero
-// between launches) adds those in block order and sets the loop's control words:
-//   ctl[3] += 1 (steps done); ctl[4] = 1 when ctl[3] is a multiple of `anchor` (the FP64
-//   residual then replaces rt), else 0; ctl[2] = 1 when the FP64 residual must be formed
-//   (an anchor step, or sqrt(sum / nrm[2]) < 2 tol, or the sum not finite), else 0;
-//   nrm[1] = the sum.
-struct CoarseRecur {
-    const void* AC;        // null: none of this
-    void* rp;
-    void* rt;
-    double* part;
-    unsigned* ticket;
-    double* nrm;
-    int* ctl;
-    double tol;
-    int anchor;
 };
 struct CoarseBatch {
     CoarseJob job[CB_MAX_JOBS];
     int njobs;
     const int* gate;       // may be null: when the word is nonzero at launch, nothing is done
-    CoarseRecur rr;
     long long wait_polls;  // polls of the grid barrier's wait before it gives up (set by the launcher)
     float keep;            // set by the launcher: < 1 when the launch's basis exceeds the L2 (see the kernel)
 };
@@ -285,8 +254,6 @@ struct EigTask {
                       // (all rows: w0 = 0, w1 = b)
     const void* vt_emb;   // complex64 form: V^T and V as the tensor-core transforms' B operand
     const void* vn_emb;   // (tc_prepare_v layout; null where the transforms run on CUDA cores)
-    const int* gate;      // one-launch sweep: may be null; while the word is nonzero the task's
-                          // cluster returns at once, touching none of the task's buffers
     void* sc;             // bilinear elements: [b] per-mode scale of the recursions' input
                           // (null: the 5-point rows, scale 1)
 };
@@ -339,5 +306,89 @@ template <typename T>
 void launch_eig_sweep_stage(int stage, const EigTask* d_tasks, int ntasks, int b_max, int Sx, int nrhs,
                             cudaStream_t s, const int* gate = nullptr);
 int eig_bmax();
+
+// ---- the iteration on the cut rows (k_cut.cu) ---------------------------------------
+constexpr int CUT_MAXL = 6;               // levels of the hierarchy it takes
+constexpr int CUT_KMAX = 32 * CUT_MAXL;   // basis columns at one cut row (r <= 32 per level)
+constexpr int CUT_MGMAX = 40;             // modes of one item
+constexpr int CUT_KG = 8;                 // shares of the columns in the update
+constexpr int CUT_MAXD = 4096;            // corrections of one problem, 2 r (2^L - 1)
+constexpr int CUT_NCUT = (1 << CUT_MAXL) - 1;
+// why the steps stopped: the FP64 test is due, a new round is due, the step limit, not
+// finite, no longer contracting (where that is asked for)
+enum CutReason : int { CUT_TEST = 1, CUT_ANCHOR = 2, CUT_LIMIT = 3, CUT_NONFINITE = 4, CUT_STALL = 5 };
+struct CutCtl {
+    int it, in_round, reason, chk_it;
+    double n2, n0;        // |v|^2 after the last step; the FP64 |r|^2 the round started from
+    double best, chk;     // smallest |v|^2 so far, and that at step chk_it
+    double ns[3];         // profiled phases (ns): leaf lines, projections and y, update
+};
+struct CutLeaf {
+    const void *V, *xi, *sc;   // as EigTask
+    const void* fh0;           // [b][Sx] the round's transformed residual
+    void* fh;                  // [b][Sx] the recursions of the round's summed inputs
+    int b;
+    int rin[4], rout[4];       // local rows at the cut above (0, 1) and below (2, 3), -1: none
+};
+struct CutNode {
+    const void* C;             // basis [2 r][N]
+    size_t N;
+    int ra;
+};
+struct CutProb {
+    int Sx, L, r, ncut, D, q1;
+    int MG, ngrp, nA, XC, nch, nB;    // items of the phases (cut_plan)
+    int cl, dist, res, nbi;           // cluster form; y shared out; panels in shared memory, items a block
+    int max_iter, stall;              // stall: stop when the steps no longer contract
+    double kh, test2, anchor2;        // squares of the test and anchor factors (of |b|, |r_0|)
+    int mid[CUT_NCUT];                // grid row below each cut
+    size_t cp_off[CUT_NCUT], ep_off[CUT_NCUT];
+    unsigned short yidx[CUT_NCUT * 2 * CUT_MAXL];   // first y index of each E group of a cut
+    const CutLeaf* leaf;
+    const CutNode* node;
+    const void *Cp, *Ep, *M;
+    const void* rt;                   // [Sy][Sx] the round's residual
+    void *v, *vsum, *res0;            // [ncut][2][Sx]
+    void *prow, *pd, *d, *y, *yacc;   // [nA][4][Sx], [nB][(L + 1) r], [D] each
+    float* npart;                     // [nB][8] partial |v|^2
+    const double *nrm, *b2;           // |r|^2 and |b|^2 (FP64)
+    CutCtl* ctl;
+};
+// panel entries (one group of r basis columns at one cut row / cut)
+struct CutCpEntry { const void* src; void* dst; size_t ldc; int K; };
+struct CutEpEntry { const void* src; void* dst; c128* d64; size_t ldc; int Ke, maskl, maskr; };
+struct CutGramPair { const void* cp; const c128* ep; int K, Ke, rows; };
+struct CutGramDest { c128* out; int ld, first, count; };
+struct CutMinv { int p, s; const c128* Ainv; };
+struct CutUpdJob { const CutProb* prob; const c128* u; c128* ut; const void* w; int Sy; };
+template <typename T>
+void launch_cut_panels(const CutCpEntry* cp, int ncp, const CutEpEntry* ep, int nep, int Sx, int r, OpGeom g,
+                       cudaStream_t s);
+size_t cut_gram_scratch(int npairs);
+// sums of C_p^H E_q per pair into the destinations (pairs [first, first + count) each)
+template <typename T>
+void launch_cut_gram(const CutGramPair* prs, int npairs, const CutGramDest* ds, int ndest, int Sx, int r, c128* part,
+                     cudaStream_t s);
+// blocks of the inverse of the corrections' triangular system (children before parents);
+// MT: packed (cut_m_packed entries), row-major or (tr) transposed within a node's rows
+size_t cut_m_packed(int L, int r);
+template <typename T>
+void launch_cut_minv(const CutMinv* prs, int n, int D, int L, int p2, const c128* G, c128* M, cplx<T>* MT, int tr,
+                     cudaStream_t s);
+// whether the cluster form can run with this much shared memory on the current device
+bool cut_cluster_ready(size_t smem);
+// fills the items of P; returns the steps' shared memory, 0 if the lines do not fit
+template <typename T>
+size_t cut_plan(CutProb& P, int b_max);
+// runs every problem with a nonzero mode (1: new round, 2: go on) until its next stop;
+// group: blocks per problem of a grid group (cl: one cluster); bars: a word per group; false if it cannot be launched
+template <typename T>
+bool launch_cut_steps(const CutProb* probs, int nprob, int group, bool cl, size_t smem, const int* modes, int mode_all,
+                      unsigned* bars, int max_groups, int* err, int prof, cudaStream_t s);
+template <typename T>
+void launch_cut_lines(const CutProb* probs, int nprob, const int* modes, int nleaf_max, int b_max, int Sx_max,
+                      cudaStream_t s);
+template <typename T>
+void launch_cut_update(const CutUpdJob* jobs, int njobs, int Sy_max, int Sx_max, cudaStream_t s);
 
 }  // namespace hh

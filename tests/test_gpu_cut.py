@@ -1,0 +1,61 @@
+"""The stationary iteration on the cut rows against the oracle's iterates on every row.
+
+A few steps are run (HH_ENOCONV at max_iter, the last iterate returned) and u_K is compared
+with the oracle's u_K.  The sizes sit at the edges of the kernels' items: one column per
+lane and one past it, the smallest bands, one basis column and the most, one level to five,
+bands of unequal height, corrections formed by every block (up to 128 of them) or shared
+out, the cluster form and the grid form.  Tolerances are those of one step (FP64 1e-8,
+complex64 1e-3, test_gpu_parity.py): K steps of a contraction or near it add up no more
+than K of its errors, each relative to a residual of the size of the first."""
+import numpy as np
+import pytest
+
+from oracle.method import OMethod
+from oracle.problem import Problem
+from workloads import random_complex
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # n, k, levels, overlap, rank, oversample, scheme
+    (6, 2.0, 1, 2, 1, 0, "fd"),          # two bands of 5 rows, 8 columns
+    (14, 4.0, 2, 2, 3, 2, "fd"),         # the smallest bands
+    (30, 8.0, 2, 2, 4, 4, "fd"),         # 32 columns: one a lane
+    (31, 8.0, 2, 4, 5, 3, "q1"),         # 33 columns
+    (62, 14.0, 3, 2, 16, 6, "fd"),       # 112 corrections
+    (63, 14.0, 3, 4, 17, 6, "fd"),       # 238: shared out; 17 columns
+    (78, 30.0, 2, 2, 32, 16, "fd"),      # the most columns
+    (101, 18.0, 4, 2, 4, 4, "q1"),       # 16 bands of unequal height
+    (127, 20.0, 5, 2, 2, 2, "fd"),       # 32 bands: more leaves than a cluster's blocks
+    (200, 40.0, 1, 6, 12, 4, "fd"),      # two tall bands
+]
+
+
+@pytest.fixture(scope="module")
+def hh():
+    from paper_2512_12538_gb300 import build
+    build.build()
+    import paper_2512_12538_gb300 as m
+    return m
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: f"n{c[0]}L{c[2]}r{c[4]}{c[6]}")
+def test_iterates_match_the_oracle(hh, case):
+    n, k, levels, overlap, rank, over, scheme = case
+    P = Problem(2, n, k, scheme=scheme)
+    O = OMethod(P, levels, overlap, rank, over, seed=3)
+    f = random_complex((P.S, P.S), 11)
+    g = random_complex((4, P.S), 12)
+    K = 3
+    want, _, _ = O.solve(P.rhs(f, g), tol=0.0, maxit=K)
+    flags = hh.HH_FLAG_BILINEAR if scheme == "q1" else 0
+    for prec, tol in (("fp64", 1e-8), ("mixed", 1e-3)):
+        s = hh.Solver(2, n, k, levels, overlap, rank, over, tol=1e-300, max_iter=K, precision=prec, seed=3,
+                      flags=flags)
+        u, st = s.solve(torch.from_numpy(f).cuda(), torch.from_numpy(g).cuda(), allow_noconv=True)
+        s.close()
+        assert st["iters"] == K
+        err = np.linalg.norm(u.cpu().numpy().reshape(-1) - want) / np.linalg.norm(want)
+        print(f"{prec}: err {err:.2e}")
+        assert err < tol, prec
