@@ -493,6 +493,14 @@ struct Solver final : SolverBase {
         int ncp, nep, nprs, ndst, nminv;
     };
     std::vector<CutLevel> clev;
+    // the set-up's sub-level solves from the interface rows (k_edge.cu): tasks per level
+    bool edge = false;
+    std::vector<EdgeTask*> d_edge;
+    std::vector<EigTask*> d_edge_out;         // the extension's transforms back
+    std::vector<std::vector<EdgeTask>> h_edge;
+    std::vector<CT*> Erows, Evin, Epd;
+    std::vector<c128*> Ey;
+    c128* edge_part = nullptr;
     std::vector<EigTask> h_cin, h_cout;   // host copies of the transform tasks (batched solves)
     // flexible GMRES
     int mk = 0;                                   // restart length
@@ -584,6 +592,81 @@ struct Solver final : SolverBase {
             cut_smem = cut_plan<T>(cp, b_max);
             cut = cut_smem > 0;
         }
+        edge = cut && edge_rows_fit<T>(Sx);
+    }
+
+    // Tasks of the children of level l (edge leaf, rows, path), addresses from the arena.
+    std::vector<EdgeTask> edge_tasks(int l) const {
+        std::vector<EdgeTask> out;
+        for (int c : lev[l]) {
+            const Node& cn = nodes[c];
+            const Node& sn = nodes[cn.sib];
+            const bool first = c & 1;                  // the edge is at its last row
+            int lf = c;
+            EdgeTask t{};
+            t.npath = L - l;
+            for (int u = 0; u < t.npath; ++u) {
+                EdgePath& q = t.path[t.npath - 1 - u];
+                q.id = lf;
+                q.ra = nodes[lf].ra;
+                q.kin = q.kedge = first ? 1 : 0;
+                q.C = C[lf];
+                q.N = pts(lf);
+                lf = nodes[lf].child[first ? 1 : 0];
+            }
+            const Node& ln = nodes[lf];
+            t.V = EV[lf];
+            t.xi = EXI[lf];
+            t.sc = ESC[lf];
+            t.b = ln.b();
+            t.node = c;
+            t.g_if = cn.ifrow;
+            t.g_sif = sn.ifrow;
+            t.g_sin = sn.inward;
+            t.a_if = t.g_if - ln.ra;
+            t.a_sif = t.g_sif - ln.ra;
+            t.a_sin = t.g_sin - ln.ra;
+            t.below = first;
+            t.lev = l;
+            t.o0 = t.npath ? (first ? ln.oa : ln.ob - 2) - ln.ra : -1;
+            t.o1 = t.npath ? t.o0 + 1 : -1;
+            t.K = L * r;
+            const int leaf_pos = lf + 1 - (1 << L), cutc = first ? leaf_pos - 1 : leaf_pos;
+            t.cp = t.npath ? cut_Cp + cp.cp_off[cutc] : nullptr;
+            t.sb = sn.b();
+            t.Om = Om[c];
+            t.Z = Z[c];
+            t.Vc = Vc[c];
+            t.rows = Erows[c];
+            t.vin = Evin[c];
+            t.pd = Epd[c];
+            t.y = Ey[c];
+            t.Fh = EFh[lf];
+            t.Gm = Gm[c];
+            t.U = U[c];
+            t.lam = lam[c];
+            const Node& pn = nodes[cn.parent];
+            t.W = W[c] + (size_t)(cn.own_a - cn.ra) * Sx * r;
+            t.Np = pts(pn.id);
+            t.Cout = C[pn.id] + (size_t)(first ? 0 : r) * t.Np;
+            t.dst0 = (long long)(cn.own_a - pn.ra) * Sx;
+            t.npts = (long long)(cn.own_b - cn.own_a) * Sx;
+            out.push_back(t);
+        }
+        return out;
+    }
+    // The edge leaves' transforms back: their owned rows into the children's solutions.
+    std::vector<EigTask> edge_out_tasks(int l) const {
+        std::vector<EigTask> out;
+        for (int c : lev[l]) {
+            int lf = c;
+            while (!nodes[lf].leaf()) lf = nodes[lf].child[(c & 1) ? 1 : 0];
+            EigTask k = eig_task(lf, nullptr, W[c] + row_off(c, nodes[lf].own_a, r));
+            k.w0 = nodes[lf].own_a - nodes[lf].ra;
+            k.w1 = nodes[lf].own_b - nodes[lf].ra;
+            out.push_back(k);
+        }
+        return out;
     }
 
     // ------------------------------------------- the iteration on the cut rows: tables
@@ -676,7 +759,7 @@ struct Solver final : SolverBase {
                     // products with every node at or below p that has columns at this cut
                     auto add_p = [&](int q, int kq, int side) {
                         const CutGramPair pr{base + l * r, cut_E64 + cp.ep_off[c] + (size_t)ep_group(c, q, side) * r * Nx,
-                                             K, (2 * L - lc) * r, 0};
+                                             K, (2 * L - lc) * r, 0, 0};
                         for (int rw = 0; rw < 2; ++rw) {
                             CutGramPair x = pr;
                             if (c != own) {
@@ -717,14 +800,25 @@ struct Solver final : SolverBase {
             std::vector<CutGramDest> ds;
             for (auto& kv : by_dest) {
                 const auto [p, kp, q, kq] = kv.first;
-                if (p == q) continue;
+                if (p == q && coarse_fp32()) continue;   // that variant's FP32 products: the full kernel
                 CutGramDest d;
                 d.out = cut_G + ((size_t)p * 2 * r + kp * r) * cp.D + (size_t)q * 2 * r + kq * r;
                 d.ld = cp.D;
+                if (p == q) {
+                    d.out = Ainv[p] + (size_t)kp * r * 2 * r + kq * r;
+                    d.ld = 2 * r;
+                }
                 d.first = (int)pr.size();
                 d.count = (int)kv.second.size();
                 ds.push_back(d);
-                pr.insert(pr.end(), kv.second.begin(), kv.second.end());
+                // A_c in FP64 products; the blocks below it only enter M, in the basis precision
+                for (CutGramPair x : kv.second) {
+                    if (p != q && sizeof(CT) != sizeof(c128)) {
+                        x.ep = cut_Ep + ((const c128*)x.ep - cut_E64);
+                        x.low = 1;
+                    }
+                    pr.push_back(x);
+                }
             }
             (void)ndiag;
             CutLevel& cl = clev[l];
@@ -737,6 +831,16 @@ struct Solver final : SolverBase {
             cl.minv = (CutMinv*)put(mv.data(), sizeof(CutMinv) * mv.size());
             cut_pairs_max = std::max(cut_pairs_max, pr.size());
         }
+        d_edge.assign(L + 1, nullptr);
+        d_edge_out.assign(L + 1, nullptr);
+        h_edge.assign(L + 1, {});
+        if (edge)
+            for (int l = 1; l <= L; ++l) {
+                h_edge[l] = edge_tasks(l);
+                const std::vector<EigTask> eo = edge_out_tasks(l);
+                d_edge[l] = (EdgeTask*)put(h_edge[l].data(), sizeof(EdgeTask) * h_edge[l].size());
+                d_edge_out[l] = (EigTask*)put(eo.data(), sizeof(EigTask) * eo.size());
+            }
         std::vector<EigTask> tin, tout;
         for (int id : lev[L]) {
             const Node& nd = nodes[id];
@@ -775,11 +879,16 @@ struct Solver final : SolverBase {
     }
     static constexpr double CUT_ANCHOR_RED = sizeof(T) == sizeof(float) ? 1e-2 : 1e-8;
 
-    // Rows, products and G blocks of level l's nodes (their bases and A_c^{-1} are done).
-    void cut_level_setup(int l) {
+    // Rows and products of level l's nodes (their bases are done): A_c = C^H A~ C, which is
+    // the sum over the cut rows alone, and the blocks of the nodes below.  Then, with A_c
+    // inverted, the rows of M.
+    void cut_level_products(int l) {
         const CutLevel& cl = clev[l];
         launch_cut_panels<T>(cl.cpe, cl.ncp, cl.epe, cl.nep, Sx, r, geom(0), stream);
         if (cl.nprs) launch_cut_gram<T>(cl.prs, cl.nprs, cl.dst, cl.ndst, Sx, r, cut_part, stream);
+    }
+    void cut_level_minv(int l) {
+        const CutLevel& cl = clev[l];
         launch_cut_minv<T>(cl.minv, cl.nminv, cp.D, L, 2 * r, cut_G, cut_M64, cut_MT, cp.cl, stream);
     }
 
@@ -896,6 +1005,17 @@ struct Solver final : SolverBase {
             cp.yacc = a.take<CT>(cp.D);
             cp.npart = a.take<float>((size_t)cp.nB * 8);
             cbar = a.take<unsigned>(2);
+            Erows.assign(nn, nullptr); Evin.assign(nn, nullptr); Epd.assign(nn, nullptr); Ey.assign(nn, nullptr);
+            if (edge) {
+                for (int id = 1; id < nn; ++id) {
+                    const int np = L - nodes[id].level;
+                    Erows[id] = a.take<CT>(4 * (size_t)Sx * m);
+                    Evin[id] = a.take<CT>(2 * (size_t)Sx * m);
+                    Epd[id] = a.take<CT>(edge_pd_elems(np, r, m));
+                    Ey[id] = a.take<c128>((size_t)np * 2 * r * m);
+                }
+                edge_part = (c128*)a.take<unsigned char>(edge_gram_scratch(1 << L));
+            }
             d_cut = a.take<CutProb>(1);
             if (!base) cut_tab_bytes = cut_tables(false);   // also sets cut_pairs_max
             d_cut_tab = a.take<unsigned char>(cut_tab_bytes);
@@ -1278,11 +1398,145 @@ struct Solver final : SolverBase {
                                                        stream, (long long)split_row(p) * Sx);
         pend(PC_COARSE_MC);
         launch_ip_reduce(partial, nb, 2 * r, nc, nullptr, Ainv[p], ycoef[p], stream);
-        launch_coarse_updn<T, T>(C[p], ycoef[p], W[p], pts(p), 2 * r, nc, stream, (long long)split_row(p) * Sx);
+        launch_coarse_updn<T, T>(C[p], pts(p), ycoef[p], W[p], pts(p), 2 * r, nc, stream, (long long)split_row(p) * Sx);
     }
 
     // ------------------------------------------------------------------ set-up
+    // Profiler count of a stage that runs inside another's launch.
+    void prof_count(int cat, double bytes, double flops) {
+        if (!prof_cat(cat)) return;
+        prof_n[cat] += 1;
+        prof_bytes[cat] += bytes;
+        prof_flops[cat] += flops;
+    }
+    // One pass of M_c over nc columns from the interface rows: the rows of the result (see
+    // k_edge.cu), as the three stages of a leaf sweep to the profiler.
+    void edge_pass(int l, int adj) {
+        const int nch = (int)lev[l].size();
+        double lines = 0.0;
+        for (auto& t : h_edge[l]) lines += (double)t.b * Sx * m;
+        prof_count(PC_TIN, sizeof(CT) * 2.0 * Sx * m * nch, 8.0 * (adj ? 2 : 1) * lines);
+        prof_count(PC_TOUT, sizeof(CT) * 4.0 * Sx * m * nch, 8.0 * (l < L ? 4 : 2) * lines);
+        pbeg(PC_RECUR, sizeof(CT) * lines / m, 28.0 * lines);
+        launch_edge_rows<T>(d_edge[l], nch, Sx, m, adj, stream);
+        pend(PC_RECUR);
+        if (l < L) {
+            pbeg(PC_COARSE_MC);
+            launch_edge_path<T>(d_edge[l], nch, Sx, m, r, cp.D, cut_M64, geom(0), adj, true, stream);
+            pend(PC_COARSE_MC);
+        }
+    }
+    // The sketches and bases of level l (sketch_level) with M_c's structure used.
+    void edge_sketch_level(int l) {
+        const std::vector<int>& cs = lev[l];
+        const int nch = (int)cs.size();
+        launch_edge_sketch<T>(d_edge[l], nch, Sx, m, P.seed, stream);
+        edge_pass(l, 0);
+        launch_edge_robin<T>(d_edge[l], nch, Sx, m, kh, q1(), stream);
+        std::vector<CT*> ys;
+        std::vector<c128*> gs, us;
+        std::vector<double*> ls;
+        for (int c : cs) { ys.push_back(Om[c]); gs.push_back(Gm[c]); us.push_back(U[c]); ls.push_back(lam[c]); }
+        pbeg(PC_QR);
+        launch_qr<T>(ys.data(), nch, Sx, m, (CT**)d_ptrs, stream);
+        pend(PC_QR);
+        launch_edge_place<T>(d_edge[l], nch, Sx, m, kh, q1(), stream);
+        edge_pass(l, 1);
+        launch_edge_conj<T>(d_edge[l], nch, Sx, m, stream);
+        launch_edge_gram<T>(d_edge[l], nch, Sx, m, edge_part, stream);
+        pbeg(PC_JACOBI);
+        launch_heig(gs.data(), us.data(), ls.data(), nch, m, r, d_ptrs, stream);
+        pend(PC_JACOBI);
+        launch_edge_form_v<T>(d_edge[l], nch, Sx, m, r, stream);
+        // the extension C_c = P_c M_c B_c^T V_c: the edge leaf's rows, then the path's bases
+        double lines = 0.0, tr = 0.0;
+        for (auto& t : h_edge[l]) {
+            lines += (double)t.b * Sx * r;
+            tr += 8.0 * t.b * t.b * Sx * r;
+        }
+        prof_count(PC_TIN, sizeof(CT) * (double)Sx * r * nch, 8.0 * lines);
+        pbeg(PC_RECUR, 2.0 * sizeof(CT) * lines, 28.0 * lines);
+        launch_edge_basis_lines<T>(d_edge[l], nch, b_max, Sx, r, stream);
+        pend(PC_RECUR);
+        if (l < L) {
+            for (int c : cs) zero(W[c], sizeof(CT) * pts(c) * r);
+            // the leaf's rows at its inner cut, for the path's corrections
+            launch_edge_leaf_rows<T>(d_edge[l], nch, Sx, r, stream);
+        }
+        pbeg(PC_TOUT, 2.0 * sizeof(CT) * lines, tr);
+        eig_sweep_stage(2, d_edge_out[l], nch, r);
+        pend(PC_TOUT);
+        if (l < L) {
+            pbeg(PC_COARSE_MC);
+            launch_edge_path<T>(d_edge[l], nch, Sx, r, r, cp.D, cut_M64, geom(0), 0, false, stream);
+            for (auto& t : h_edge[l])
+                for (int u = 0; u < t.npath; ++u) {
+                    const Node& q = nodes[t.path[u].id];
+                    const bool top = q.id == t.node;
+                    const int lo = top ? q.ra : q.own_a, hi = top ? q.rb : q.own_b;
+                    launch_coarse_updn<T, T>(C[q.id] + (size_t)(lo - q.ra) * Sx, pts(q.id), t.y + (size_t)u * 2 * r * r,
+                                             W[t.node] + row_off(t.node, lo, r), (size_t)(hi - lo) * Sx, 2 * r, r,
+                                             stream, (long long)(split_row(q.id) + q.ra - lo) * Sx);
+                }
+            pend(PC_COARSE_MC);
+        }
+        size_t npm = 0;
+        for (auto& t : h_edge[l]) npm = std::max(npm, t.Np);
+        launch_edge_scatter<T>(d_edge[l], nch, npm, r, stream);
+    }
     void sketch_level(int l) {   // children at level l of the nodes at level l-1
+        if (edge) edge_sketch_level(l);
+        else dense_sketch_level(l);
+        if (cut) {
+            // A_c = C_p^H A~_p C_p over the cut rows (all nodes of the level together)
+            pbeg(PC_GALERKIN, 0.0, 0.0);
+            if (prof_cat(PC_GALERKIN)) prof_pending.back().nl = (int)lev[l - 1].size();
+            cut_level_products(l - 1);
+            pend(PC_GALERKIN);
+        }
+        for (int p : lev[l - 1]) {
+            if (cut && !coarse_fp32()) break;
+            // A_c = C_p^H A~_p C_p, then its inverse.  Algorithmic work: a point in one child's
+            // rows pairs that child's r columns of conj(C) with r columns of A~ C, complex
+            // products of 8 real flops: r^2 of them (the two rows next to the split pair r with
+            // 2r), or r (r + 1) / 2 in the Hermitian-packed form of the FP64 5-point products
+            // (the row before the split adds r^2)
+            const bool herm_form = !coarse_fp32() && !q1();
+            if (!cut) pbeg(PC_GALERKIN, (double)pts(p) * 2 * r * sizeof(CT),
+                 herm_form ? 8.0 * (0.5 * r * (r + 1.0) * pts(p) + (double)r * r * Sx)
+                           : 8.0 * r * r * (pts(p) + 2.0 * Sx));
+            const int split = nodes[nodes[p].child[1]].own_a - nodes[p].ra;
+            // FP64 products from the stored basis, or FP32 ones in the opt-in FP32 coarse
+            // variant of the mixed form
+            bool herm = false;
+            const int nb = coarse_fp32()
+                               ? launch_galerkin_partial<T, T>(C[p], geom(p), 2 * r, split, partial, MAX_PART_BLOCKS,
+                                                               stream)
+                               : launch_galerkin_partial<T, double>(C[p], geom(p), 2 * r, split, partial,
+                                                                    MAX_PART_BLOCKS, stream, &herm);
+            if (!cut) pend(PC_GALERKIN);
+            launch_ip_reduce(partial, nb, 2 * r, 2 * r, Ainv[p], nullptr, nullptr, stream);
+            if (herm) launch_herm_fill(Ainv[p], 2 * r, stream);
+        }
+        // the level's Galerkin matrices inverted together
+        GjBatch bt{};
+        bt.n = 2 * r;
+        bt.err = derr;
+        int cnt = 0;
+        // FP64 elimination in both forms (the opt-in FP32 coarse variant eliminates in
+        // FP32); the complex64 form also gets the inverse rounded to complex64 for its
+        // one-column corrections
+        const bool c64 = sizeof(CT) != sizeof(c128);
+        for (int p : lev[l - 1]) {
+            bt.A[cnt] = Ainv[p];
+            bt.AT[cnt++] = c64 ? (void*)AinvT[p] : nullptr;
+        }
+        launch_gj_inverse(bt, cnt, coarse_fp32(), stream);
+        if (cut) cut_level_minv(l - 1);
+    }
+    // The sketches and bases of level l by full sub-level solves (explicit-inverse leaves,
+    // 1D problems, n_i > 1).
+    void dense_sketch_level(int l) {
         const std::vector<int>& cs = lev[l];
         // Y = T_c Omega
         for (int c : cs) {
@@ -1346,43 +1600,7 @@ struct Solver final : SolverBase {
                                       (size_t)(cn.own_a - nodes[p].ra) * Sx, (size_t)(cn.own_b - cn.own_a) * Sx,
                                       stream);
             }
-            // A_c = C_p^H A~_p C_p, then its inverse.  Algorithmic work: a point in one child's
-            // rows pairs that child's r columns of conj(C) with r columns of A~ C, complex
-            // products of 8 real flops: r^2 of them (the two rows next to the split pair r with
-            // 2r), or r (r + 1) / 2 in the Hermitian-packed form of the FP64 5-point products
-            // (the row before the split adds r^2)
-            const bool herm_form = !coarse_fp32() && !q1();
-            pbeg(PC_GALERKIN, (double)pts(p) * 2 * r * sizeof(CT),
-                 herm_form ? 8.0 * (0.5 * r * (r + 1.0) * pts(p) + (double)r * r * Sx)
-                           : 8.0 * r * r * (pts(p) + 2.0 * Sx));
-            const int split = nodes[nodes[p].child[1]].own_a - nodes[p].ra;
-            // FP64 products from the stored basis, or FP32 ones in the opt-in FP32 coarse
-            // variant of the mixed form
-            bool herm = false;
-            const int nb = coarse_fp32()
-                               ? launch_galerkin_partial<T, T>(C[p], geom(p), 2 * r, split, partial, MAX_PART_BLOCKS,
-                                                               stream)
-                               : launch_galerkin_partial<T, double>(C[p], geom(p), 2 * r, split, partial,
-                                                                    MAX_PART_BLOCKS, stream, &herm);
-            pend(PC_GALERKIN);
-            launch_ip_reduce(partial, nb, 2 * r, 2 * r, Ainv[p], nullptr, nullptr, stream);
-            if (herm) launch_herm_fill(Ainv[p], 2 * r, stream);
         }
-        // the level's Galerkin matrices inverted together
-        GjBatch bt{};
-        bt.n = 2 * r;
-        bt.err = derr;
-        int cnt = 0;
-        // FP64 elimination in both forms (the opt-in FP32 coarse variant eliminates in
-        // FP32); the complex64 form also gets the inverse rounded to complex64 for its
-        // one-column corrections
-        const bool c64 = sizeof(CT) != sizeof(c128);
-        for (int p : lev[l - 1]) {
-            bt.A[cnt] = Ainv[p];
-            bt.AT[cnt++] = c64 ? (void*)AinvT[p] : nullptr;
-        }
-        launch_gj_inverse(bt, cnt, coarse_fp32(), stream);
-        if (cut) cut_level_setup(l - 1);
     }
 
     hh_status setup() override {
@@ -1397,7 +1615,8 @@ struct Solver final : SolverBase {
         if (tc && !tc_transform_ready()) return HH_ECUDA;
         zero(derr, sizeof(int) * 4);
         zero(dcounter, sizeof(unsigned) * 4);
-        for (int id = 1; id < nn; ++id) zero(Vs[id], sizeof(CT) * pts(id) * nmax);
+        if (!edge)
+            for (int id = 1; id < nn; ++id) zero(Vs[id], sizeof(CT) * pts(id) * nmax);
         if (eig) {
             std::vector<EigTask> own;
             for (int id : lev[L]) own.push_back(eig_task(id, Vs[id], W[id]));

@@ -422,13 +422,13 @@ void launch_coarse_batch(CoarseBatch bt, int p, void* partial, unsigned* bar, in
 // chunk (coalesced along the points) and used for all the chunk's columns; y staged in
 // shared memory in the basis precision.  The chunks in separate blocks keep several blocks
 // per SM in flight (the loop over j waits on L2 loads).
-// split_pt >= 0: the basis's first p/2 columns vanish from point split_pt on and the
+// The basis's first p/2 columns vanish from point split_pt on and the
 // others before it (a node's two children), so each point reads only its child's half.
 static constexpr int UPD_COLS = 16;
 template <typename TC, typename TW>
-__global__ void __launch_bounds__(256) k_coarse_updn(const cplx<TC>* __restrict__ C, const c128* __restrict__ y,
-                                                     cplx<TW>* __restrict__ W, size_t N, int p, int nc,
-                                                     long long split_pt) {
+__global__ void __launch_bounds__(256) k_coarse_updn(const cplx<TC>* __restrict__ C, size_t ldc,
+                                                     const c128* __restrict__ y, cplx<TW>* __restrict__ W, size_t N,
+                                                     int p, int nc, long long split_pt) {
     extern __shared__ __align__(16) unsigned char ysm[];
     cplx<TC>* ys = (cplx<TC>*)ysm;   // [p][UPD_COLS]: this chunk's columns of y
     const int c0 = blockIdx.y * UPD_COLS, cn = min(UPD_COLS, nc - c0);
@@ -442,12 +442,10 @@ __global__ void __launch_bounds__(256) k_coarse_updn(const cplx<TC>* __restrict_
 #pragma unroll
         for (int c = 0; c < UPD_COLS; ++c) acc[c] = {0, 0};
         int j = 0, je = p;
-        if (split_pt >= 0) {
-            if ((long long)pt < split_pt) je = p / 2;
-            else j = p / 2;
-        }
+        if ((long long)pt < split_pt) je = p / 2;
+        else j = p / 2;
         for (; j < je; ++j) {
-            const cplx<TC> cv = C[(size_t)j * N + pt];
+            const cplx<TC> cv = C[(size_t)j * ldc + pt];
             const cplx<TC>* yr = ys + j * UPD_COLS;
 #pragma unroll
             for (int c = 0; c < UPD_COLS; ++c) cfma(acc[c], cv, yr[c]);
@@ -468,9 +466,9 @@ __global__ void __launch_bounds__(256) k_coarse_updn(const cplx<TC>* __restrict_
 // the memory system wrote back several times over.)  A block whose points straddle the
 // split stages both halves in turn (the vanishing half is stored as zeros).
 static constexpr int UPD_SP = 64;
-__global__ void __launch_bounds__(UPD_SP * 4) k_coarse_updn_s(const c64* __restrict__ C, const c128* __restrict__ y,
-                                                              c64* __restrict__ W, size_t N, int p, int nc,
-                                                              long long split_pt) {
+__global__ void __launch_bounds__(UPD_SP * 4) k_coarse_updn_s(const c64* __restrict__ C, size_t ldc,
+                                                              const c128* __restrict__ y, c64* __restrict__ W,
+                                                              size_t N, int p, int nc, long long split_pt) {
     extern __shared__ __align__(16) unsigned char usm[];
     const int ncp = (nc + 15) / 16 * 16;        // right-hand sides padded to whole chunks
     c64* ys = (c64*)usm;                        // [p][ncp]
@@ -486,10 +484,8 @@ __global__ void __launch_bounds__(UPD_SP * 4) k_coarse_updn_s(const c64* __restr
         const int np = (int)min((size_t)UPD_SP, N - p0);
         const size_t plast = p0 + np - 1;
         int jlo = 0, jhi = p;
-        if (split_pt >= 0) {
-            if ((long long)plast < split_pt) jhi = p / 2;
-            else if ((long long)p0 >= split_pt) jlo = p / 2;
-        }
+        if ((long long)plast < split_pt) jhi = p / 2;
+        else if ((long long)p0 >= split_pt) jlo = p / 2;
         __syncthreads();   // the previous span's tile is written out
         for (int e = t; e < UPD_SP * ncp; e += nth) ot[e] = {0.f, 0.f};
         for (int g0 = jlo; g0 < jhi; g0 += 32) {
@@ -498,7 +494,7 @@ __global__ void __launch_bounds__(UPD_SP * 4) k_coarse_updn_s(const c64* __restr
             for (int e = t; e < gn * UPD_SP; e += nth) {
                 const int j = e / UPD_SP, k = e - j * UPD_SP;
                 const size_t x = p0 + k;
-                cp_async8_zfill(cs + e, C + (size_t)(g0 + j) * N + (x < N ? x : 0), x < N);
+                cp_async8_zfill(cs + e, C + (size_t)(g0 + j) * ldc + (x < N ? x : 0), x < N);
             }
             cp_async_commit();
             cp_async_wait_all();
@@ -533,8 +529,8 @@ __global__ void __launch_bounds__(UPD_SP * 4) k_coarse_updn_s(const c64* __restr
 }
 
 template <typename TC, typename TW>
-void launch_coarse_updn(const cplx<TC>* C, const c128* y, cplx<TW>* W, size_t N, int p, int nc, cudaStream_t s,
-                        long long split_pt) {
+void launch_coarse_updn(const cplx<TC>* C, size_t ldc, const c128* y, cplx<TW>* W, size_t N, int p, int nc,
+                        cudaStream_t s, long long split_pt) {
     if constexpr (sizeof(TC) == 4 && sizeof(TW) == 4) {
         const int ncp = (nc + 15) / 16 * 16;
         const size_t sm = sizeof(c64) * ((size_t)p * ncp + 32 * UPD_SP + (size_t)UPD_SP * ncp);
@@ -545,13 +541,13 @@ void launch_coarse_updn(const cplx<TC>* C, const c128* y, cplx<TW>* W, size_t N,
             // one group of UPD_SP threads per chunk of 16 right-hand sides (up to four), so
             // that every thread has the same number of chunks
             const int groups = std::min(4, ncp / 16);
-            k_coarse_updn_s<<<grid, UPD_SP * groups, sm, s>>>(C, y, W, N, p, nc, split_pt);
+            k_coarse_updn_s<<<grid, UPD_SP * groups, sm, s>>>(C, ldc, y, W, N, p, nc, split_pt);
             note_launch();
             return;
         }
     }
     const dim3 grid(blocks_for(N, 256, 152 * 8), (nc + UPD_COLS - 1) / UPD_COLS);
-    k_coarse_updn<TC, TW><<<grid, 256, sizeof(cplx<TC>) * p * UPD_COLS, s>>>(C, y, W, N, p, nc, split_pt);
+    k_coarse_updn<TC, TW><<<grid, 256, sizeof(cplx<TC>) * p * UPD_COLS, s>>>(C, ldc, y, W, N, p, nc, split_pt);
     note_launch();
 }
 
@@ -563,7 +559,7 @@ template void launch_coarse_batch<float, double, double, double>(CoarseBatch, in
                                                                  cudaStream_t);
 template void launch_coarse_batch<double, double, double, double>(CoarseBatch, int, void*, unsigned*, int*,
                                                                   cudaStream_t);
-template void launch_coarse_updn<float, float>(const c64*, const c128*, c64*, size_t, int, int, cudaStream_t, long long);
-template void launch_coarse_updn<double, double>(const c128*, const c128*, c128*, size_t, int, int, cudaStream_t, long long);
+template void launch_coarse_updn<float, float>(const c64*, size_t, const c128*, c64*, size_t, int, int, cudaStream_t, long long);
+template void launch_coarse_updn<double, double>(const c128*, size_t, const c128*, c128*, size_t, int, int, cudaStream_t, long long);
 
 }  // namespace hh

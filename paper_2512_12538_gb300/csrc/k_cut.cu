@@ -175,6 +175,39 @@ __global__ void __launch_bounds__(256) k_cut_gram(const CutGramPair* __restrict_
     const int xs = (Sx + GRAM_SPLIT - 1) / GRAM_SPLIT;
     const int xa = blockIdx.y * xs, xb = min(Sx, xa + xs);
     c128 acc[2][2] = {{{0, 0}, {0, 0}}, {{0, 0}, {0, 0}}};
+    if (p.low) {
+        // blocks that only enter M, which is kept in the basis precision
+        C* ct = (C*)&cs[0][0];
+        C* et = (C*)&es[0][0];
+        C lc[2][2] = {{{0, 0}, {0, 0}}, {{0, 0}, {0, 0}}};
+        for (int row = 0; row < 2; ++row) {
+            if (!((p.rows >> row) & 1)) continue;
+            const C* cp = (const C*)p.cp + (size_t)row * Sx * p.K;
+            const C* ep = (const C*)p.ep + (size_t)row * p.Ke * Sx;
+            for (int x0 = xa; x0 < xb; x0 += 16) {
+                for (int t = threadIdx.x; t < 16 * 32; t += 256) {
+                    const int x = t >> 5, j = t & 31, x2 = t & 15, j2 = t >> 4;
+                    ct[x * 33 + j] = x0 + x < xb && j < r ? cp[(size_t)(x0 + x) * p.K + j] : C{0, 0};
+                    et[x2 * 33 + j2] = x0 + x2 < xb && j2 < r ? ep[(size_t)j2 * Sx + x0 + x2] : C{0, 0};
+                }
+                __syncthreads();
+#pragma unroll 4
+                for (int x = 0; x < 16; ++x) {
+                    const C a0 = ct[x * 33 + ti], a1 = ct[x * 33 + ti + 16], b0 = et[x * 33 + tj],
+                            b1 = et[x * 33 + tj + 16];
+                    cfma_cj(lc[0][0], a0, b0);
+                    cfma_cj(lc[0][1], a0, b1);
+                    cfma_cj(lc[1][0], a1, b0);
+                    cfma_cj(lc[1][1], a1, b1);
+                }
+                __syncthreads();
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int v = 0; v < 2; ++v) acc[u][v] = cvt<double>(lc[u][v]);
+    } else
     for (int row = 0; row < 2; ++row) {
         if (!((p.rows >> row) & 1)) continue;
         const C* cp = (const C*)p.cp + (size_t)row * Sx * p.K;

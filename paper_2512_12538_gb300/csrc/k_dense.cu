@@ -1533,8 +1533,8 @@ void launch_heig(c128* const* G, c128* const* U, double* const* lam, int nq, int
 // each adding every eighth term, then a fixed shuffle tree (the FP64 products spread over
 // the SMs); the r scales 1 / sqrt(lam_j) formed once per block.
 template <typename T>
-__global__ void k_form_v(const cplx<T>* __restrict__ Z, const c128* __restrict__ U, const double* lam,
-                         cplx<T>* __restrict__ V, int Sx, int m, int r) {
+__device__ void form_v(const cplx<T>* __restrict__ Z, const c128* __restrict__ U, const double* lam,
+                       cplx<T>* __restrict__ V, int Sx, int m, int r) {
     __shared__ double sc[64];
     for (int j = threadIdx.x; j < r && j < 64; j += blockDim.x) {
         const double l = lam[j];
@@ -1559,6 +1559,22 @@ __global__ void k_form_v(const cplx<T>* __restrict__ Z, const c128* __restrict__
     }
     if (ok && sub == 0) V[t] = cvt<T>(sc[j] * a);
 }
+template <typename T>
+__global__ void k_form_v(const cplx<T>* Z, const c128* U, const double* lam, cplx<T>* V, int Sx, int m, int r) {
+    form_v<T>(Z, U, lam, V, Sx, m, r);
+}
+template <typename T>
+__global__ void k_edge_form_v(const EdgeTask* __restrict__ tasks, int Sx, int m, int r) {
+    const EdgeTask& E = tasks[blockIdx.y];
+    form_v<T>((const cplx<T>*)E.Z, E.U, E.lam, (cplx<T>*)E.Vc, Sx, m, r);
+}
+template <typename T>
+void launch_edge_form_v(const EdgeTask* tasks, int nchild, int Sx, int m, int r, cudaStream_t s) {
+    k_edge_form_v<T><<<dim3(((size_t)Sx * r * 8 + 255) / 256, nchild), 256, 0, s>>>(tasks, Sx, m, r);
+    note_launch();
+}
+template void launch_edge_form_v<float>(const EdgeTask*, int, int, int, int, cudaStream_t);
+template void launch_edge_form_v<double>(const EdgeTask*, int, int, int, int, cudaStream_t);
 template <typename T>
 void launch_form_v(const cplx<T>* Z, const c128* U, const double* lam, cplx<T>* V, int Sx, int m, int r,
                    cudaStream_t s) {

@@ -412,7 +412,7 @@ void launch_copy(const cplx<TS>* src, cplx<TD>* dst, size_t n, bool accumulate, 
 // the inward row, with q1_coef(0, 0, i, di) and q1_coef(0, 1, i, di) (the same for the last
 // row by symmetry).
 template <typename T>
-__global__ void k_robin_trace(const cplx<T>* __restrict__ uif, const cplx<T>* __restrict__ uin,
+__device__ void robin_trace(const cplx<T>* __restrict__ uif, const cplx<T>* __restrict__ uin,
                               cplx<T>* __restrict__ Y, int b_s, int Sx, int nc, double kh,
                               const double* khr_row, int q1) {
     const OpGeom g{b_s, Sx, kh, khr_row, q1};
@@ -441,6 +441,17 @@ __global__ void k_robin_trace(const cplx<T>* __restrict__ uif, const cplx<T>* __
     }
 }
 template <typename T>
+__global__ void k_robin_trace(const cplx<T>* uif, const cplx<T>* uin, cplx<T>* Y, int b_s, int Sx, int nc, double kh,
+                              const double* khr_row, int q1) {
+    robin_trace<T>(uif, uin, Y, b_s, Sx, nc, kh, khr_row, q1);
+}
+template <typename T>
+__global__ void k_edge_robin(const EdgeTask* __restrict__ tasks, int Sx, int nc, double kh, int q1) {
+    const EdgeTask& E = tasks[blockIdx.y];
+    const cplx<T>* rows = (const cplx<T>*)E.rows + 2 * (size_t)Sx * nc;
+    robin_trace<T>(rows, rows + (size_t)Sx * nc, (cplx<T>*)E.Om, E.sb, Sx, nc, kh, nullptr, q1);
+}
+template <typename T>
 void launch_robin_trace(const cplx<T>* u_if, const cplx<T>* u_in, cplx<T>* Y, int b_s, int Sx, int nc,
                         double kh, const double* khr_row, cudaStream_t s, int q1) {
     const size_t total = (size_t)Sx * nc;
@@ -449,7 +460,7 @@ void launch_robin_trace(const cplx<T>* u_if, const cplx<T>* u_in, cplx<T>* Y, in
 }
 
 template <typename T>
-__global__ void k_adjoint_place(const cplx<T>* __restrict__ Q, cplx<T>* __restrict__ vif,
+__device__ void adjoint_place(const cplx<T>* __restrict__ Q, cplx<T>* __restrict__ vif,
                                 cplx<T>* __restrict__ vin, int b_s, int Sx, int nc, double kh,
                                 const double* khr_row, int q1) {
     const OpGeom g{b_s, Sx, kh, khr_row, q1};
@@ -482,6 +493,23 @@ __global__ void k_adjoint_place(const cplx<T>* __restrict__ Q, cplx<T>* __restri
     }
 }
 template <typename T>
+__global__ void k_adjoint_place(const cplx<T>* Q, cplx<T>* vif, cplx<T>* vin, int b_s, int Sx, int nc, double kh,
+                                const double* khr_row, int q1) {
+    adjoint_place<T>(Q, vif, vin, b_s, Sx, nc, kh, khr_row, q1);
+}
+template <typename T>
+__global__ void k_edge_place(const EdgeTask* __restrict__ tasks, int Sx, int nc, double kh, int q1) {
+    const EdgeTask& E = tasks[blockIdx.y];
+    cplx<T>* v = (cplx<T>*)E.vin;
+    adjoint_place<T>((const cplx<T>*)E.Om, v, v + (size_t)Sx * nc, E.sb, Sx, nc, kh, nullptr, q1);
+}
+template <typename T>
+__global__ void k_edge_conj(const EdgeTask* __restrict__ tasks, int n) {
+    const EdgeTask& E = tasks[blockIdx.y];
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x)
+        ((cplx<T>*)E.Z)[t] = conj(((const cplx<T>*)E.rows)[(size_t)2 * n + t]);
+}
+template <typename T>
 void launch_adjoint_place(const cplx<T>* Q, cplx<T>* v_if, cplx<T>* v_in, int b_s, int Sx, int nc,
                           double kh, const double* khr_row, cudaStream_t s, int q1) {
     const size_t total = (size_t)Sx * nc;
@@ -499,7 +527,7 @@ __device__ __forceinline__ unsigned long long splitmix64_at(unsigned long long s
     return z ^ (z >> 31);
 }
 template <typename T>
-__global__ void k_sketch(cplx<T>* Om, int Sx, int m, int node, unsigned long long seed) {
+__device__ void sketch(cplx<T>* Om, int Sx, int m, int node, unsigned long long seed) {
     const size_t total = (size_t)Sx * m;
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
          t += (size_t)gridDim.x * blockDim.x) {
@@ -514,6 +542,14 @@ __global__ void k_sketch(cplx<T>* Om, int Sx, int m, int node, unsigned long lon
         sincospi(2.0 * u2, &sn, &cs);
         Om[t] = cplx<T>{(T)(rho * cs), (T)(rho * sn)};
     }
+}
+template <typename T>
+__global__ void k_sketch(cplx<T>* Om, int Sx, int m, int node, unsigned long long seed) {
+    sketch<T>(Om, Sx, m, node, seed);
+}
+template <typename T>
+__global__ void k_edge_sketch(const EdgeTask* __restrict__ tasks, int Sx, int m, unsigned long long seed) {
+    sketch<T>((cplx<T>*)tasks[blockIdx.y].Om, Sx, m, tasks[blockIdx.y].node, seed);
 }
 template <typename T>
 void launch_sketch(cplx<T>* Om, int Sx, int m, int node, unsigned long long seed, cudaStream_t s) {
@@ -722,5 +758,34 @@ template void launch_coarse_update<float, float>(const c64*, const c128*, c64*, 
 template void launch_coarse_update<float, double>(const c64*, const c128*, c128*, size_t, int, int, cudaStream_t);
 template void launch_coarse_update<double, double>(const c128*, const c128*, c128*, size_t, int, int,
                                                    cudaStream_t);
+
+// The sketches' row steps for all children of a level at once (EdgeTask).
+template <typename T>
+void launch_edge_sketch(const EdgeTask* tasks, int nchild, int Sx, int m, unsigned long long seed, cudaStream_t s) {
+    k_edge_sketch<T><<<dim3(grid_for((size_t)Sx * m, 256), nchild), 256, 0, s>>>(tasks, Sx, m, seed);
+    note_launch();
+}
+template <typename T>
+void launch_edge_robin(const EdgeTask* tasks, int nchild, int Sx, int nc, double kh, int q1, cudaStream_t s) {
+    k_edge_robin<T><<<dim3(grid_for((size_t)Sx * nc, 256), nchild), 256, 0, s>>>(tasks, Sx, nc, kh, q1);
+    note_launch();
+}
+template <typename T>
+void launch_edge_place(const EdgeTask* tasks, int nchild, int Sx, int nc, double kh, int q1, cudaStream_t s) {
+    k_edge_place<T><<<dim3(grid_for((size_t)Sx * nc, 256), nchild), 256, 0, s>>>(tasks, Sx, nc, kh, q1);
+    note_launch();
+}
+template <typename T>
+void launch_edge_conj(const EdgeTask* tasks, int nchild, int Sx, int nc, cudaStream_t s) {
+    k_edge_conj<T><<<dim3(grid_for((size_t)Sx * nc, 256), nchild), 256, 0, s>>>(tasks, Sx * nc);
+    note_launch();
+}
+#define HH_EDGE_FIELD(T)                                                                                              \
+    template void launch_edge_sketch<T>(const EdgeTask*, int, int, int, unsigned long long, cudaStream_t);            \
+    template void launch_edge_robin<T>(const EdgeTask*, int, int, int, double, int, cudaStream_t);                    \
+    template void launch_edge_place<T>(const EdgeTask*, int, int, int, double, int, cudaStream_t);                    \
+    template void launch_edge_conj<T>(const EdgeTask*, int, int, int, cudaStream_t);
+HH_EDGE_FIELD(float)
+HH_EDGE_FIELD(double)
 
 }  // namespace hh

@@ -130,10 +130,11 @@ void set_wait_polls(long long polls);
 long long wait_polls(long long dflt);
 template <typename TC, typename TV, typename TW, typename TO>
 void launch_coarse_batch(CoarseBatch bt, int p, void* partial, unsigned* bar, int* err, cudaStream_t s);
-// W[pt][c] += sum_j C[j][pt] y[j][c] (nc columns); split_pt as launch_ip_partial_colA
+// W[pt][c] += sum_j C[j ldc + pt] y[j][c] for N points (nc columns); split_pt as
+// launch_ip_partial_colA (it may be negative or past the end: one child's columns only)
 template <typename TC, typename TW>
-void launch_coarse_updn(const cplx<TC>* C, const c128* y, cplx<TW>* W, size_t N, int p, int nc, cudaStream_t s,
-                        long long split_pt = -1);
+void launch_coarse_updn(const cplx<TC>* C, size_t ldc, const c128* y, cplx<TW>* W, size_t N, int p, int nc,
+                        cudaStream_t s, long long split_pt);
 // tiled inner products with a column-major A (p x N); split_pt >= 0: A's first p/2
 // columns vanish from point split_pt on and the others before it (a node's coarse basis)
 template <typename TA, typename TB, typename ACC>
@@ -357,7 +358,7 @@ struct CutProb {
 // panel entries (one group of r basis columns at one cut row / cut)
 struct CutCpEntry { const void* src; void* dst; size_t ldc; int K; };
 struct CutEpEntry { const void* src; void* dst; c128* d64; size_t ldc; int Ke, maskl, maskr; };
-struct CutGramPair { const void* cp; const c128* ep; int K, Ke, rows; };
+struct CutGramPair { const void* cp; const void* ep; int K, Ke, rows, low; };   // low: products in the basis precision
 struct CutGramDest { c128* out; int ld, first, count; };
 struct CutMinv { int p, s; const c128* Ainv; };
 struct CutUpdJob { const CutProb* prob; const c128* u; c128* ut; const void* w; int Sy; };
@@ -390,5 +391,69 @@ void launch_cut_lines(const CutProb* probs, int nprob, const int* modes, int nle
                       cudaStream_t s);
 template <typename T>
 void launch_cut_update(const CutUpdJob* jobs, int njobs, int Sy_max, int Sx_max, cudaStream_t s);
+
+// ---- the set-up's sub-level solves from the interface rows (k_edge.cu) ---------------
+// A node on the path from a child's edge leaf up to the child: its basis, the child that
+// holds the inner cut and lies on the edge's side.
+struct EdgePath {
+    int id, ra, kin, kedge;
+    const void* C;
+    size_t N;
+};
+struct EdgeTask {
+    const void *V, *xi, *sc;          // edge leaf, as EigTask
+    int b, node;
+    int a_if, a_sif, a_sin;           // its local rows: the interface, the sibling's trace rows
+    int o0, o1;                       // its rows at the inner cut (-1: the child is a leaf)
+    int g_if, g_sif, g_sin;           // the grid rows of the first three
+    int below, lev, npath, K;         // the leaf lies below the cut; the child's level; path; panel width
+    int sb;                           // rows of the sibling's band
+    void *Om, *Z, *Vc;                // sketch / Y / Q, T^* Q, V_c
+    void *rows, *vin, *pd, *Fh;       // [4][Sx][nc], [2][Sx][nc], partial products, [b][Sx][r]
+    c128* y;                          // [npath][2r][nc]
+    const void* cp;                   // the cut's basis panel
+    c128 *Gm, *U;                     // Gram matrix, eigenvectors
+    double* lam;
+    const void* W;                    // the extension's first owned point [.][r]
+    void* Cout;                       // its columns of the parent's basis [r][Np]
+    size_t Np;
+    long long dst0, npts;             // the child's points in the parent
+    EdgePath path[CUT_MAXL];
+};
+template <typename T>
+bool edge_rows_fit(int Sx);
+size_t edge_pd_elems(int npath, int r, int nc);
+size_t edge_gram_scratch(int nchild);
+// the edge leaves' rows; then the path's corrections y of nc columns, added to the trace rows
+// (adj: the interface row) when rows_out
+template <typename T>
+void launch_edge_rows(const EdgeTask* tasks, int nchild, int Sx, int nc, int adj, cudaStream_t s);
+template <typename T>
+void launch_edge_path(const EdgeTask* tasks, int nchild, int Sx, int nc, int r, int D, const c128* M, OpGeom g, int adj,
+                      bool rows_out, cudaStream_t s);
+// recursions of the basis extension (into Fh, transformed layout of nc right-hand sides)
+template <typename T>
+void launch_edge_basis_lines(const EdgeTask* tasks, int nchild, int b_max, int Sx, int nc, cudaStream_t s);
+// the two rows at the inner cut of those (rows 0, 1)
+template <typename T>
+void launch_edge_leaf_rows(const EdgeTask* tasks, int nchild, int Sx, int nc, cudaStream_t s);
+// Gm = Z^H Z in FP64; part: edge_gram_scratch bytes
+template <typename T>
+void launch_edge_gram(const EdgeTask* tasks, int nchild, int Sx, int m, c128* part, cudaStream_t s);
+// the extensions into the parents' bases (the other child's rows zero)
+template <typename T>
+void launch_edge_scatter(const EdgeTask* tasks, int nchild, size_t np_max, int r, cudaStream_t s);
+// launch_sketch, launch_robin_trace (rows 2, 3 -> Om), launch_adjoint_place (Om -> vin), the
+// conjugate of row 2 into Z (k_field.cu) and launch_form_v (k_dense.cu), for all children
+template <typename T>
+void launch_edge_sketch(const EdgeTask* tasks, int nchild, int Sx, int m, unsigned long long seed, cudaStream_t s);
+template <typename T>
+void launch_edge_robin(const EdgeTask* tasks, int nchild, int Sx, int nc, double kh, int q1, cudaStream_t s);
+template <typename T>
+void launch_edge_place(const EdgeTask* tasks, int nchild, int Sx, int nc, double kh, int q1, cudaStream_t s);
+template <typename T>
+void launch_edge_conj(const EdgeTask* tasks, int nchild, int Sx, int nc, cudaStream_t s);
+template <typename T>
+void launch_edge_form_v(const EdgeTask* tasks, int nchild, int Sx, int m, int r, cudaStream_t s);
 
 }  // namespace hh

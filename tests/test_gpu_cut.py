@@ -27,7 +27,7 @@ CASES = [
     (63, 14.0, 3, 4, 17, 6, "fd"),       # 238: shared out; 17 columns
     (78, 30.0, 2, 2, 32, 16, "fd"),      # the most columns
     (101, 18.0, 4, 2, 4, 4, "q1"),       # 16 bands of unequal height
-    (127, 20.0, 5, 2, 2, 2, "fd"),       # 32 bands: more leaves than a cluster's blocks
+    (130, 20.0, 5, 2, 2, 2, "fd"),       # 32 bands: more leaves than a cluster's blocks
     (200, 40.0, 1, 6, 12, 4, "fd"),      # two tall bands
 ]
 
