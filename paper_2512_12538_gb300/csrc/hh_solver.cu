@@ -508,6 +508,7 @@ struct Solver final : SolverBase {
          *gy = nullptr;
     c128* h_dots = nullptr;                       // pinned host copy of the dot products
     GmresLs gls{};                                // the cycle's least-squares problem (device)
+    CutGmres cg{};                                // its vectors on the cut rows
     GmresState* h_gst = nullptr;                  // pinned snapshots of its state, GM_SLOTS
     static constexpr int GM_SLOTS = 4, GM_LAG = 2;
     cudaEvent_t gm_ev[GM_SLOTS] = {};
@@ -967,7 +968,19 @@ struct Solver final : SolverBase {
         d_etasks_view = a.take<EigTask>(nleaf);
         d_etasks_own = a.take<EigTask>(nleaf);
         d_etask_one = a.take<EigTask>(1);
-        if (mk > 0) {
+        if (mk > 0 && cut) {
+            const size_t nG = cut_ng(), nb = cut_gm_blocks((int)nG);
+            cg.V = a.take<c128>(nG * (mk + 1));
+            cg.alpha = a.take<c128>(mk + 1);
+            cg.v1 = a.take<c128>(nG);
+            cg.rG = a.take<c128>(nG);
+            cg.y0 = a.take<CT>(cp.D);
+            cg.part = a.take<c128>(2 * nb * 72);
+            cg.scale = a.take<c128>(1);
+            cg.rho2 = a.take<double>(1);
+            cg.npart = a.take<double>(nb);
+            cp.scale = cg.scale;
+        } else if (mk > 0) {
             Vb = a.take<c128>(N * (mk + 1));
             Zb = a.take<c128>(N * mk);
             gw = a.take<c128>(N);
@@ -975,12 +988,16 @@ struct Solver final : SolverBase {
             gz = a.take<c128>(N);
             gdots = a.take<c128>(4 * 80);
             gy = a.take<c128>(80);
+        }
+        if (mk > 0) {
             gls.mk = mk;
             gls.H = a.take<c128>((size_t)(mk + 1) * mk);
             gls.cs = a.take<double>(mk);
             gls.sn = a.take<c128>(mk);
             gls.g = a.take<c128>(mk + 1);
             gls.st = a.take<GmresState>(1);
+            cg.ls = gls;
+            cg.red = sizeof(T) == sizeof(float) ? 1e-4 : 1e-12;
         }
         d_ptrs = a.take<void*>(3 * 64);
         if (cut) {
@@ -2002,8 +2019,7 @@ struct Solver final : SolverBase {
             it = hc->it;
             rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;
             if (cand && (!std::isfinite(rel) || rel < P.tol || it >= P.max_iter || hc->reason != CUT_TEST)) {
-                std::swap(u, ut);
-                cut_flip ^= 1;
+                cut_swap();
                 mode = 1;
             } else if (cand) {
                 mode = 2;
@@ -2023,7 +2039,75 @@ struct Solver final : SolverBase {
             cand = true;
         }
     }
-    int cut_flip = 0;
+    int cut_flip = 0;   // which of the two update jobs has the current u as its source
+    void cut_swap() {
+        std::swap(u, ut);
+        cut_flip ^= 1;
+    }
+    int cut_ng() const { return 2 * cp.ncut * Sx; }   // entries on the cut rows
+
+    // Flexible GMRES (loop_gmres) with its Krylov space kept on the cut rows (k_cut.cu).  A
+    // cycle starts from the FP64 residual of u with one step on every row, which gives S r;
+    // each further Arnoldi step is one step on the cut rows and one launch.  It ends at the
+    // restart length, when the estimate is below tol / 2, or (complex64) when it has fallen by
+    // as much as the steps' rounding allows; u then takes one application of M, and the FP64
+    // residual decides.
+    hh_status loop_gmres_cut(int& it, double& rel) {
+        int* ctl = (int*)(dnorm + 6);
+        const int nG = cut_ng(), nl = (int)lev[L].size();
+        const int* gate = (const int*)gls.st;   // GmresState.stop
+        hh_status st = HH_OK;
+        auto resid = [&]() {
+            zero(ctl, 4 * sizeof(double) + sizeof(CutCtl));
+            zero(dcounter, 2 * sizeof(unsigned));
+            pbeg(PC_SPMV, 48.0 * (double)Sy * Sx);
+            launch_residual_stop<T>(u, bvec, nullptr, RT, geom(0), npart, dnorm, ctl, dcounter, P.tol, stream);
+            pend(PC_SPMV);
+        };
+        auto step = [&](int mode, const int* g) {
+            return launch_cut_steps<T>(d_cut, 1, cut_group(), cp.cl, cut_smem, nullptr, mode, cbar, 1, derr, 0, stream, 1, g);
+        };
+        resid();
+        for (;;) {
+            if (!read_norms(st)) return st;
+            rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;
+            if (!std::isfinite(rel)) return HH_ENOCONV;
+            if (rel < P.tol) return HH_OK;
+            if (it >= P.max_iter) return HH_ENOCONV;
+            eig_stage_prof(0, d_etasks_cin);
+            if (!step(1, nullptr)) return HH_ECUDA;
+            launch_cut_gm_start<T>(d_cut, cg, nG, stream);
+            const int nsteps = std::min(mk, P.max_iter - it);
+            int launched = 0;
+            for (int j = 0; j < nsteps; ++j) {
+                if (j >= GM_LAG) {
+                    const int sl = (j - GM_LAG) % GM_SLOTS;   // the state after step j - GM_LAG
+                    ck(cudaEventSynchronize(gm_ev[sl]), cerr);
+                    if (cerr != cudaSuccess) return HH_ECUDA;
+                    if (h_gst[sl].stop) break;
+                }
+                if (j > 0 && !step(2, gate)) return HH_ECUDA;
+                if (!launch_cut_arnoldi<T>(d_cut, cg, j, nG, P.tol, cbar, derr, stream)) return HH_ECUDA;
+                const int sl = j % GM_SLOTS;
+                ck(cudaMemcpyAsync(&h_gst[sl], gls.st, sizeof(GmresState), cudaMemcpyDeviceToHost, stream), cerr);
+                ck(cudaEventRecord(gm_ev[sl], stream), cerr);
+                ++launched;
+            }
+            const int last = (launched - 1) % GM_SLOTS;
+            if (!sync_check(st)) return st;
+            const GmresState fin = h_gst[last];   // of the last step queued: the cycle's end
+            if (fin.bad) return HH_ENOCONV;
+            const int jn = fin.stop ? fin.jstop : launched;
+            it += jn;
+            launch_cut_gm_combine<T>(d_cut, cg, jn, nG, stream);
+            if (!step(2, nullptr)) return HH_ECUDA;   // the corrections of the combined input
+            launch_cut_lines<T>(d_cut, 1, nullptr, nl, b_max, Sx, stream);
+            eig_stage_prof(2, d_etasks_cout);
+            launch_cut_update<T>(d_upd + cut_flip, 1, Sy, Sx, stream);
+            cut_swap();
+            resid();
+        }
+    }
     // blocks of the steps' group: one per item of the larger phase, at most one per SM
     int cut_group() const { return std::min(148, std::max(cp.nA, cp.nB)); }
     void eig_stage_prof(int stg, const EigTask* tasks) {
@@ -2091,6 +2175,7 @@ struct Solver final : SolverBase {
     // update reads (g and H up to the stopping column).  Convergence is confirmed on the
     // true residual at every restart.
     hh_status loop_gmres(int& it, double& rel) {
+        if (cut) return loop_gmres_cut(it, rel);
         const size_t N = (size_t)Sy * Sx;
         const int ld = mk + 1;
         hh_status st = HH_OK;
@@ -2621,7 +2706,7 @@ struct BatchEngine {
             else if (c.reason == CUT_STALL || q.it >= q.p->P.max_iter) leave(q, HH_ENOCONV, q.p->ut, done);
             else if (c.reason == CUT_TEST) q.mode = 2;
             else {
-                std::swap(q.p->u, q.p->ut);
+                q.p->cut_swap();
                 q.mode = 1;
             }
         }

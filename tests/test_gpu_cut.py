@@ -59,3 +59,47 @@ def test_iterates_match_the_oracle(hh, case):
         err = np.linalg.norm(u.cpu().numpy().reshape(-1) - want) / np.linalg.norm(want)
         print(f"{prec}: err {err:.2e}")
         assert err < tol, prec
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: f"n{c[0]}L{c[2]}r{c[4]}{c[6]}")
+def test_gmres_iterates_match_the_oracle(hh, case):
+    """Flexible GMRES with its vectors on the cut rows: five steps at restart 3 (a full cycle
+    and a cut one) are those of GMRES on the whole grid."""
+    n, k, levels, overlap, rank, over, scheme = case
+    P = Problem(2, n, k, scheme=scheme)
+    O = OMethod(P, levels, overlap, rank, over, seed=3)
+    f = random_complex((P.S, P.S), 13)
+    g = random_complex((4, P.S), 14)
+    K = 5
+    want, steps, _ = O.solve_gmres(P.rhs(f, g), tol=0.0, restart=3, maxit=K)
+    assert steps == K
+    flags = hh.HH_FLAG_BILINEAR if scheme == "q1" else 0
+    for prec, tol in (("fp64", 1e-8), ("mixed", 1e-3)):
+        s = hh.Solver(2, n, k, levels, overlap, rank, over, tol=1e-300, max_iter=K, precision=prec, seed=3,
+                      flags=flags, outer="gmres", restart=3)
+        u, st = s.solve(torch.from_numpy(f).cuda(), torch.from_numpy(g).cuda(), allow_noconv=True)
+        s.close()
+        err = np.linalg.norm(u.cpu().numpy().reshape(-1) - want) / np.linalg.norm(want)
+        print(f"{prec}: {st['iters']} steps, err {err:.2e}")
+        assert st["iters"] == K and err < tol, prec
+
+
+def test_a_handle_solves_alone_after_a_batch(hh):
+    """The rounds of a batch leave the iterate in either of a handle's two buffers."""
+    n, k = 63, 20.0
+    S = n + 2
+    ps = [hh.make_params(2, n, k, 2, 2, 8, 6, 1, 1e-10, 400, "mixed", 1 + i) for i in range(2)]
+    hs = hh.hh_setup_batch(ps)
+    try:
+        fs = [torch.from_numpy(random_complex((S, S), 15 + i)).cuda() for i in range(2)]
+        gs = [torch.zeros((4, S), dtype=torch.complex128, device="cuda")] * 2
+        for _ in range(2):
+            ub = [torch.empty_like(f) for f in fs]
+            hh.hh_solve_batch(hs, fs, gs, ub)
+            for h, f, g, u in zip(hs, fs, gs, ub):
+                alone = torch.empty_like(f)
+                hh.hh_solve(h, f, g, alone)
+                assert ((alone - u).norm() / u.norm()).item() < 1e-12
+    finally:
+        for h in hs:
+            hh.hh_destroy(h)
