@@ -2182,12 +2182,12 @@ struct Solver final : SolverBase {
         const c128 one = {1.0, 0.0};
         c128* gone = gdots + 3 * 80;
         ck(cudaMemcpyAsync(gone, &one, sizeof(c128), cudaMemcpyHostToDevice, stream), cerr);
-        const double nbv = std::sqrt(std::max(h_norm[2], 0.0));
         // with the profiler on, the captured preconditioner's events are read after every
         // step, which needs a synchronisation per step
         const int lag = prof_on ? 0 : GM_LAG;
         for (;;) {
             if (!true_residual(gw, st)) return st;
+            const double nbv = std::sqrt(std::max(h_norm[2], 0.0));
             const double beta = std::sqrt(std::max(h_norm[0], 0.0));
             rel = nbv > 0 ? beta / nbv : 0.0;
             if (!std::isfinite(rel)) return HH_ENOCONV;
@@ -2253,16 +2253,16 @@ struct Solver final : SolverBase {
         cudaEventRecord(e0, stream);
         launch_rhs(f, g, bvec, P.dim, S, h, stream, q1());
         norm_sq(bvec, dnorm + 2);   // dnorm[2..3] = ||b||^2 as a complex
-        ck(cudaMemcpyAsync(h_norm, dnorm, 4 * sizeof(double), cudaMemcpyDeviceToHost, stream), cerr);
         zero(u, sizeof(c128) * N);
         int it = 0;
         double rel = 0.0;
-        hh_status st = HH_OK;
-        if (sync_check(st)) st = mk > 0 ? loop_gmres(it, rel) : loop_oras(it, rel);
+        // (each loop reads the norms with its first residual and the status words with every one)
+        const hh_status st = mk > 0 ? loop_gmres(it, rel) : loop_oras(it, rel);
         d2d(uo, u, sizeof(c128) * N);
         cudaEventRecord(e1, stream);
-        hh_status st2;
-        sync_check(st2);
+        ck(cudaGetLastError(), cerr);
+        ck(cudaStreamSynchronize(stream), cerr);
+        const hh_status st2 = cerr == cudaSuccess ? HH_OK : HH_ECUDA;
         prof_collect();
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
