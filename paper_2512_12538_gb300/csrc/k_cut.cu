@@ -46,12 +46,18 @@ struct GroupBar {
     unsigned n, target;
     int* err;
     long long limit;
-    __device__ bool operator()() {
+    __device__ void arrive() {
         __syncthreads();
-        bool ok = true;
         target += n;
+        if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr) : "memory");
+    }
+    __device__ bool operator()() {
+        arrive();
+        return wait();
+    }
+    __device__ bool wait() {
+        bool ok = true;
         if (threadIdx.x == 0) {
-            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr) : "memory");
             ok = false;
             for (long long it = 0; it < limit && !ok; ++it) {
                 unsigned v;
@@ -73,6 +79,11 @@ __device__ __forceinline__ c128 ldcg(const c128* p) {
     const double2 v = __ldcg((const double2*)p);
     return {v.x, v.y};
 }
+// asynchronous copy of one element (the panels: written by earlier launches alone)
+__device__ __forceinline__ void cp_async_el(c64* s, const c64* g) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(s)), "l"(g) : "memory");
+}
+__device__ __forceinline__ void cp_async_el(c128* s, const c128* g) { cp_async16(s, g); }
 __device__ __forceinline__ unsigned long long gtime() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
@@ -307,7 +318,7 @@ __global__ void __launch_bounds__(256) k_cut_minv(const CutMinv* __restrict__ pr
 // lines of one item, the input rows; M where every block forms y itself; the panels of the
 // block's items where they fit (res); and the small arrays of phases B, Y and C.
 struct CutSmem {
-    int xi, pr, ln, v, m, ce, t, rs, red, d, y, ya, up, own, total;
+    int xi, ln, v, m, ce, t, rs, red, d, y, ya, up, own, total;
 };
 HH_HD int cut_m_elems(int L, int r) {
     int n = 0;
@@ -319,7 +330,6 @@ HH_HD CutSmem cut_smem_layout(const CutProb& P, int nw) {
     const int kmax = P.L * P.r;
     int o = 0;
     s.xi = o; o += P.MG * P.Sx;
-    s.pr = o; o += P.MG * 64;
     s.ln = o; o += P.MG * P.Sx;
     s.v = o; o += 4 * P.Sx;
     s.m = o; o += P.dist ? 0 : cut_m_elems(P.L, P.r);
@@ -355,7 +365,7 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
     using C = cplx<T>;
     constexpr int NW = NT / 32;
     extern __shared__ __align__(16) unsigned char csm[];
-    __shared__ C s_vin[4][CUT_MGMAX], s_vout[4][CUT_MGMAX], s_sc[CUT_MGMAX];
+    __shared__ __align__(32) C s_vin[CUT_MGMAX][4], s_vout[CUT_MGMAX][4], s_sc[CUT_MGMAX];
     __shared__ float s_red[NW];
     // the descriptors in shared memory: the barriers' acquires drop the L1, so that every
     // phase would fetch them from the L2 again, one dependent load after another
@@ -379,7 +389,6 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
         const CutSmem lay = cut_smem_layout(P, NW);
         C* const sm = (C*)csm;
         C* s_xi = sm + lay.xi;
-        C* s_pr = sm + lay.pr;
         C* s_ln = sm + lay.ln;
         C* s_v = sm + lay.v;
         C* s_m = sm + lay.m;
@@ -420,6 +429,7 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
         int done = 0;
         float n2 = 0.f;
         int xi_item = -1;
+        LineScan<T> scan;
         bool stepped = false;   // a step of this launch is done
         unsigned long long t0 = 0, tA = 0, tB = 0, tC = 0;
         const bool timing = prof && rank == 0 && tid == 0;
@@ -459,25 +469,31 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
                     for (int q = tid; q < 4 * nm; q += NT) {
                         const int k = q / nm, w = q - k * nm;
                         const C sc = F.sc ? ((const C*)F.sc)[m0 + w] : C{1, 0};
-                        s_vout[k][w] = F.rout[k] >= 0 ? V[(size_t)F.rout[k] * b + m0 + w] : C{0, 0};
+                        s_vout[w][k] = F.rout[k] >= 0 ? V[(size_t)F.rout[k] * b + m0 + w] : C{0, 0};
                         const C vi = F.rin[k] >= 0 ? V[(size_t)F.rin[k] * b + m0 + w] : C{0, 0};
-                        s_vin[k][w] = F.sc ? sc * vi : vi;
+                        s_vin[w][k] = F.sc ? sc * vi : vi;
                         if (k == 0) s_sc[w] = sc;
                     }
-                    for (int w = warp; w < nm; w += NW) {
-                        const C* xi = (const C*)F.xi + (size_t)(m0 + w) * Sx;
-                        for (int i = lane; i < Sx; i += 32) s_xi[w * Sx + i] = xi[i];
+                    if (warp < nm) {   // at most one mode a warp
+                        const C* xi = (const C*)F.xi + (size_t)(m0 + warp) * Sx;
+                        for (int i = lane; i < Sx; i += 32) s_xi[warp * Sx + i] = xi[i];
                         __syncwarp();
-                        line_products(s_xi + w * Sx, Sx, lane, s_pr[w * 64 + lane], s_pr[w * 64 + 32 + lane]);
+                        line_scan_init(s_xi + warp * Sx, Sx, lane, scan);
                     }
                 }
                 xi_item = a;
                 if (nm <= 0) continue;
                 if (!first) {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const C* src = v + ((size_t)(lf - (k < 2)) * 2 + (k & 1)) * Sx;
-                        for (int i = tid; i < Sx; i += NT) s_v[k * Sx + i] = F.rin[k] >= 0 ? ldcg(src + i) : C{0, 0};
+                    const C* src = v + (size_t)(lf - 1) * 2 * Sx;   // the cut above, then the cut below
+                    const bool up = F.rin[0] >= 0, dn = F.rin[2] >= 0;
+#pragma unroll 2
+                    for (int i = tid; i < Sx; i += NT) {
+                        const C a0 = up ? ldcg(src + i) : C{0, 0}, a1 = up ? ldcg(src + Sx + i) : C{0, 0};
+                        const C a2 = dn ? ldcg(src + 2 * Sx + i) : C{0, 0}, a3 = dn ? ldcg(src + 3 * Sx + i) : C{0, 0};
+                        s_v[i] = a0;
+                        s_v[Sx + i] = a1;
+                        s_v[2 * Sx + i] = a2;
+                        s_v[3 * Sx + i] = a3;
                     }
                 }
                 __syncthreads();
@@ -492,32 +508,50 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
                     for (int i = tid; i < Sx; i += NT) {
                         const C v0 = s_v[i], v1 = s_v[Sx + i], v2 = s_v[2 * Sx + i], v3 = s_v[3 * Sx + i];
                         for (int w = 0; w < nm; ++w) {
-                            C f = {0, 0};
-                            cfma(f, s_vin[0][w], v0);
-                            cfma(f, s_vin[1][w], v1);
-                            cfma(f, s_vin[2][w], v2);
-                            cfma(f, s_vin[3][w], v3);
+                            const cpair<T> p0 = *(const cpair<T>*)&s_vin[w][0], p1 = *(const cpair<T>*)&s_vin[w][2];
+                            C f = p0.x * v0;
+                            cfma(f, p0.y, v1);
+                            cfma(f, p1.x, v2);
+                            cfma(f, p1.y, v3);
                             s_ln[w * Sx + i] = f;
                         }
                     }
                 }
                 __syncthreads();
-                for (int w = warp; w < nm; w += NW)
-                    line_solve(s_xi + w * Sx, s_ln + w * Sx, Sx, lane, s_pr[w * 64 + lane], s_pr[w * 64 + 32 + lane]);
+                if (warp < nm) line_solve(s_xi + warp * Sx, s_ln + warp * Sx, Sx, lane, scan);
                 __syncthreads();
                 for (int i = tid; i < Sx; i += NT) {
                     C o[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
                     for (int w = 0; w < nm; ++w) {
                         const C f = s_ln[w * Sx + i];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) cfma(o[k], s_vout[k][w], f);
+                        const cpair<T> p0 = *(const cpair<T>*)&s_vout[w][0], p1 = *(const cpair<T>*)&s_vout[w][2];
+                        cfma(o[0], p0.x, f);
+                        cfma(o[1], p0.y, f);
+                        cfma(o[2], p1.x, f);
+                        cfma(o[3], p1.y, f);
                     }
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
                         if (F.rout[k] >= 0) prow[((size_t)a * 4 + k) * Sx + i] = o[k];
                 }
             }
-            if (!(ok = bar())) break;
+            bar.arrive();
+            // while the others arrive: the item's basis panel into the lines' place
+            const bool stage = !res && one && rank < P.nB;
+            const int sc_ = stage ? rank / nch : 0, sx0 = (rank - sc_ * nch) * XC, sxn = stage ? min(XC, Sx - sx0) : 0;
+            const int slev = cut_level(sc_, L), sK = (slev + 1) * r, sKe = (2 * L - slev) * r;
+            const int room = (MG + 4) * Sx;
+            const bool stage_c = stage && 2 * XC * sK <= room;
+            const int kfit = stage ? min(sKe, room / (2 * XC)) : 0;
+            if (stage_c) {
+                const C* src = (const C*)P.Cp + P.cp_off[sc_] + (size_t)sx0 * sK;
+                for (int q = tid; q < sxn * sK; q += NT) {
+                    cp_async_el(s_ln + q, src + q);
+                    cp_async_el(s_ln + XC * sK + q, src + (size_t)Sx * sK + q);
+                }
+                cp_async_commit();
+            }
+            if (!(ok = bar.wait())) break;
             if (timing) { const unsigned long long t = gtime(); tA += t - t0; t0 = t; }
             // ------------------------------------------------------------------ B
             for (int e = rank, q0 = 0; e < P.nB; e += gsz, ++q0) {
@@ -531,13 +565,13 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
                         const int lf = c + (row >> 1), k = row < 2 ? row + 2 : row - 2;
                         const int ng = (P.leaf[lf].b + MG - 1) / MG;
                         const C* src = prow + ((size_t)lf * P.ngrp * 4 + k) * Sx + i;
-                        for (int u0 = 0; u0 < ng; u0 += 12) {
-                            C a[12];
+                        for (int u0 = 0; u0 < ng; u0 += 18) {
+                            C a[18];
 #pragma unroll
-                            for (int u = 0; u < 12; ++u)
+                            for (int u = 0; u < 18; ++u)
                                 a[u] = u0 + u < ng ? ldcg(src + (size_t)(u0 + u) * 4 * Sx) : C{0, 0};
 #pragma unroll
-                            for (int u = 0; u < 12; ++u) s = s + a[u];
+                            for (int u = 0; u < 18; ++u) s = s + a[u];
                         }
                     }
                     s_t[row * (XC + 2) + il] = s;
@@ -563,15 +597,19 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
                     if (!one) res0[o] = rs;
                 }
                 __syncthreads();
+                if (stage_c) {
+                    cp_async_wait_all();
+                    __syncthreads();
+                }
                 {
                     const C* c0 = res ? s_ce + (size_t)q0 * 2 * XC * 3 * L * r
-                                      : (const C*)P.Cp + P.cp_off[c] + (size_t)x0 * K;
-                    const C* c1 = c0 + (size_t)(res ? XC : Sx) * K;
+                                      : stage_c ? s_ln : (const C*)P.Cp + P.cp_off[c] + (size_t)x0 * K;
+                    const C* c1 = c0 + (size_t)(res || stage_c ? XC : Sx) * K;
                     for (int k0 = 0; k0 < K; k0 += 32) {
                         const int k = k0 + lane;
                         C a0 = {0, 0}, a1 = {0, 0};
                         if (k < K) {
-#pragma unroll 4
+#pragma unroll 8
                             for (int il = warp; il < xn; il += NW) {
                                 cfma_cj(a0, c0[(size_t)il * K + k], s_rs[il]);
                                 cfma_cj(a1, c1[(size_t)il * K + k], s_rs[XC + il]);
@@ -596,15 +634,26 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
                 }
                 __syncthreads();
             }
-            if (!(ok = bar())) break;
+            bar.arrive();
+            if (kfit) {
+                // and as many columns of its E panel as fit there, for phase C: [row][k][XC]
+                const C* src = (const C*)P.Ep + P.ep_off[sc_] + sx0;
+                for (int k = warp; k < 2 * kfit; k += NW) {
+                    const int row = k >= kfit, kk = k - row * kfit;
+                    for (int x = lane; x < sxn; x += 32)
+                        cp_async_el(s_ln + (size_t)k * XC + x, src + ((size_t)row * sKe + kk) * Sx + x);
+                }
+                cp_async_commit();
+            }
+            if (!(ok = bar.wait())) break;
             // ------------------------------------------------------------------ Y
             // d[e]: the partials of the cuts under the entry's child and of the own cut, by
-            // eight lanes in a fixed order
+            // eight lanes (dist: a warp) in a fixed order
             {
-                constexpr int EB = NT / 8;
-                const int sub = tid & 7;
+                const int EL = dist ? 32 : 8, EB = NT / EL;
+                const int sub = tid & (EL - 1);
                 for (int eb = dist ? rank * EB : 0; eb < D; eb += dist ? gsz * EB : EB) {
-                    const int e = eb + (tid >> 3);
+                    const int e = eb + tid / EL;
                     C s = {0, 0};
                     if (e < D) {
                         const int p = e / (2 * r), j = e - p * 2 * r, k = j >= r, jr = j - k * r;
@@ -613,14 +662,14 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
                         const int own = t * span + span / 2 - 1;
                         const int nin = span / 2 - 1;    // cuts inside the child
 #pragma unroll 4
-                        for (int q = sub; q < (nin + 1) * nch; q += 8) {
+                        for (int q = sub; q < (nin + 1) * nch; q += EL) {
                             const int cc = q / nch, ch = q - cc * nch;
                             const int cut = cc < nin ? ca + cc : own;
                             const int slot = (cc < nin ? l : l + k) * r + jr;
                             s = s + ldcg(pd + ((size_t)cut * nch + ch) * (L + 1) * r + slot);
                         }
                     }
-                    for (int o = 4; o > 0; o >>= 1) {
+                    for (int o = EL / 2; o > 0; o >>= 1) {
                         s.re += __shfl_xor_sync(0xffffffffu, s.re, o);
                         s.im += __shfl_xor_sync(0xffffffffu, s.im, o);
                     }
@@ -642,7 +691,7 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
                 C s = {0, 0};
                 for (int lv = l, k0 = 0; lv < L; ++lv) {
                     const int q0 = ((1 << lv) - 1 + (t << (lv - l))) * 2 * r, n = 2 * r << (lv - l);
-#pragma unroll 4
+#pragma unroll 8
                     for (int k = lane; k < n; k += 32) cfma(s, mr[k0 + k], s_d[q0 + k]);
                     k0 += n;
                 }
@@ -671,6 +720,10 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
                 const unsigned short* yi = P.yidx + c * 2 * CUT_MAXL;
                 // (row, x) pairs times shares of the columns; a share's partial per pair
                 const int np = 2 * xn, kg = min(CUT_KG, max(1, NT / np));
+                if (kfit) {
+                    cp_async_wait_all();
+                    __syncthreads();
+                }
                 for (int q = tid; q < np * kg; q += NT) {
                     const int kk = q / np, pr = q - kk * np, row = pr / xn, il = pr - row * xn;
                     const C* er = E + (size_t)row * Ke * ldx + il;
@@ -678,8 +731,15 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
                     for (int gq = 0; gq < ne; ++gq) {
                         const C* yg = s_y + yi[gq];
                         const C* eg = er + (size_t)gq * r * ldx;
+                        int j = kk;
+                        if (gq * r < kfit) {
+                            const C* es = s_ln + ((size_t)row * kfit + gq * r) * XC + il;
+                            const int je = min(r, kfit - gq * r);
 #pragma unroll 8
-                        for (int j = kk; j < r; j += kg) cfma(s, eg[(size_t)j * ldx], yg[j]);
+                            for (; j < je; j += kg) cfma(s, es[j * XC], yg[j]);
+                        }
+#pragma unroll 8
+                        for (; j < r; j += kg) cfma(s, eg[(size_t)j * ldx], yg[j]);
                     }
                     s_up[kk * 2 * XC + row * XC + il] = s;
                 }
@@ -695,21 +755,22 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
                     nn += (float)abs2(inv0 * s);
                 }
                 nn = warp_sum(nn);
-                if (lane == 0) P.npart[e * NW + warp] = nn;
+                if (lane == 0) s_red[warp] = nn;
+                __syncthreads();
+                if (tid == 0) {
+                    float t = 0.f;
+#pragma unroll
+                    for (int w = 0; w < NW; ++w) t += s_red[w];
+                    P.npart[e] = t;
+                }
             }
             stepped = true;
             if (!(ok = bar())) break;
-            // the norm, in the same order in every block; then the tests
-            {
-                float t = 0.f;
-                for (int e = tid; e < P.nB * NW; e += NT) t += __ldcg(P.npart + e);
-                t = warp_sum(t);
-                if (lane == 0) s_red[warp] = t;
-                __syncthreads();
-                n2 = 0.f;
-#pragma unroll
-                for (int w = 0; w < NW; ++w) n2 += s_red[w];
-            }
+            // the norm, in the same order in every warp; then the tests
+            n2 = 0.f;
+#pragma unroll 5
+            for (int e = lane; e < P.nB; e += 32) n2 += __ldcg(P.npart + e);
+            n2 = warp_sum(n2);
             if (timing) { const unsigned long long t = gtime(); tC += t - t0; t0 = t; }
             first = false;
             ++it;
@@ -760,14 +821,14 @@ struct CcSmem {
 };
 HH_HD CcSmem cc_layout(const CutProb& P) {
     CcSmem s;
-    const int r = P.r, L = P.L, D = P.D, XC = P.XC;
+    const int r = P.r, L = P.L, D = P.D, XC = P.XC, Ke = 2 * L * r;
     int o = 0;
     s.xi = o; o += P.MG * P.Sx;
     s.ln = o;                       // the lines; phases B, Y and C: the rows and partial sums
     s.t = o;
     s.red = s.t + 4 * (XC + 2);
     s.up = s.red + CC_NW * 2 * L * r;
-    const int tmp = 4 * (XC + 2) + CC_NW * 2 * L * r + (CUT_KG * 2 * XC > 5 * D ? CUT_KG * 2 * XC : 5 * D);
+    const int tmp = 4 * (XC + 2) + CC_NW * 2 * L * r + (CUT_KG * 2 * XC > CC_NT ? CUT_KG * 2 * XC : CC_NT);
     o += P.MG * P.Sx > tmp ? P.MG * P.Sx : tmp;
     s.v = o; o += 4 * P.Sx;
     s.m = o; o += cut_m_elems(L, r);
@@ -775,7 +836,7 @@ HH_HD CcSmem cc_layout(const CutProb& P) {
     s.e = s.c;                      // E follows the block's C panel
     s.rs = o; o += 2 * XC;
     s.d = o; o += D;
-    s.y = o; o += D;
+    s.y = o; o += Ke;               // in the order of E's columns
     s.ya = o; o += D;
     s.own = o; o += 2 * XC;
     s.vs = o; o += 2 * XC;
@@ -808,9 +869,10 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
     using C = c64;
     constexpr int NT = CC_NT, NW = CC_NW;
     extern __shared__ __align__(16) unsigned char csm[];
-    __shared__ C s_vin[4][CUT_MGMAX], s_vout[4][CUT_MGMAX], s_sc[CUT_MGMAX];
+    __shared__ __align__(32) C s_vin[CUT_MGMAX][4], s_vout[CUT_MGMAX][4], s_sc[CUT_MGMAX];
     __shared__ float s_nrm[CC_CL][4], s_word[CC_CL];
     __shared__ unsigned short s_yi[CUT_KMAX * 2];
+    __shared__ int s_ng[2];
     __shared__ __align__(8) uint64_t s_mb[3];
     __shared__ CutProb P;
     __shared__ CutLeaf F;
@@ -828,7 +890,7 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
     // wait for `bytes` of exchange k; bounded
     auto wait = [&](int k, unsigned bytes) -> bool {
         if (tid == 0) mbar_arrive_expect_tx(&s_mb[k], bytes);
-        bool got = false;
+        bool got = warp != 0;   // one warp polls
         for (long long q = 0; q < limit && !got; ++q) {
             uint32_t d;
             asm volatile(
@@ -873,8 +935,9 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
         const int lev = cut_level(c, L), K = (lev + 1) * r, Ke = (2 * L - lev) * r;
         C* s_c = sm + lay.c;
         C* s_e = s_c + 2 * XC * K;
-        const int ng0 = has_b ? (P.leaf[c].b + MG - 1) / MG : 0, ng1 = has_b ? (P.leaf[c + 1].b + MG - 1) / MG : 0;
+        if (tid >= 64 && tid < 66) s_ng[tid - 64] = has_b ? (P.leaf[c + tid - 64].b + MG - 1) / MG : 0;
         __syncthreads();
+        const int ng0 = s_ng[0], ng1 = s_ng[1];
         const int b = F.b, nm = rank < P.nA ? max(0, min(MG, b - m0)) : 0;
         bool first = mode == 1;
         const double n0 = first ? *P.nrm : ctl->n0;
@@ -889,32 +952,23 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
             const C* V = (const C*)F.V;
             const int k = q / nm, w = q - k * nm;
             const C sc = F.sc ? ((const C*)F.sc)[m0 + w] : C{1, 0};
-            s_vout[k][w] = F.rout[k] >= 0 ? V[(size_t)F.rout[k] * b + m0 + w] : C{0, 0};
+            s_vout[w][k] = F.rout[k] >= 0 ? V[(size_t)F.rout[k] * b + m0 + w] : C{0, 0};
             const C vi = F.rin[k] >= 0 ? V[(size_t)F.rin[k] * b + m0 + w] : C{0, 0};
-            s_vin[k][w] = F.sc ? sc * vi : vi;
+            s_vin[w][k] = F.sc ? sc * vi : vi;
             if (k == 0) s_sc[w] = sc;
         }
-        C pf[2], pb[2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int w = warp + u * NW;
-            if (w < nm) {
-                const C* xi = (const C*)F.xi + (size_t)(m0 + w) * Sx;
-                for (int i = lane; i < Sx; i += 32) s_xi[w * Sx + i] = xi[i];
-                __syncwarp();
-                line_products(s_xi + w * Sx, Sx, lane, pf[u], pb[u]);
-            }
+        for (int w = warp; w < nm; w += NW) {
+            const C* xi = (const C*)F.xi + (size_t)(m0 + w) * Sx;
+            for (int i = lane; i < Sx; i += 32) cp_async_el(s_xi + w * Sx + i, xi + i);
         }
-        for (int q = tid; q < cut_m_elems(L, r); q += NT) s_m[q] = ((const C*)P.M)[q];
+        for (int q = tid; q < cut_m_elems(L, r); q += NT) cp_async_el(s_m + q, (const C*)P.M + q);
         if (has_b) {
             for (int row = 0; row < 2; ++row) {
                 const C* sc = (const C*)P.Cp + P.cp_off[c] + ((size_t)row * Sx + x0) * K;
-                for (int u = tid; u < xn * K; u += NT) s_c[row * XC * K + u] = sc[u];
+                for (int u = tid; u < xn * K; u += NT) cp_async_el(s_c + row * XC * K + u, sc + u);
                 const C* se = (const C*)P.Ep + P.ep_off[c] + (size_t)row * Ke * Sx + x0;
-                for (int u = tid; u < Ke * xn; u += NT) {
-                    const int k = u / xn, x = u - k * xn;
-                    s_e[(row * Ke + k) * XC + x] = se[(size_t)k * Sx + x];
-                }
+                for (int k = warp; k < Ke; k += NW)
+                    for (int x = lane; x < xn; x += 32) cp_async_el(s_e + (row * Ke + k) * XC + x, se + (size_t)k * Sx + x);
             }
             for (int k = tid; k < Ke; k += NT) s_yi[k] = (unsigned short)(P.yidx[c * 2 * CUT_MAXL + k / r] + k % r);
             for (int q = tid; q < 2 * xn; q += NT) {
@@ -939,6 +993,35 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
         const unsigned by3 = 4u * 4u * CC_CL + (nm > 0 ? 8u * 2u * (unsigned)Sx * ((F.rin[0] >= 0) + (F.rin[2] >= 0)) : 0u);
         unsigned long long t0 = 0, tA = 0, tB = 0, tC = 0;
         const bool timing = prof && rank == 0 && tid == 0;
+        cp_async_commit();
+        cp_async_wait_all();
+        __syncwarp();
+        LineScan<float> scan;   // of the warp's first line (its xi lines are its own copies)
+        if (warp < nm) line_scan_init(s_xi + warp * Sx, Sx, lane, scan);
+        // this thread's places in phases Y and C: an entry of d and its share of the partials, an
+        // entry of y and its share of M's row, a cut point and its share of E's columns
+        const int ke = tid >> 2;
+        int kb[4] = {-1, -1, -1, -1};
+        if (ke < D) {
+            const int p = ke / (2 * r), j = ke - p * 2 * r, kc = j >= r, jr = j - kc * r;
+            const int l = 31 - __clz(p + 1), t = p + 1 - (1 << l);
+            const int span = 1 << (L - l), ca = t * span + kc * (span / 2), own = t * span + span / 2 - 1;
+            const int nin = span / 2 - 1;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int q = (tid & 3) + 4 * u;   // at most 16 items in all
+                if (q < (nin + 1) * nch) {
+                    const int cc = q / nch, cu = cc < nin ? ca + cc : own;
+                    kb[u] = (cu * nch + q - cc * nch) * (L + 1) * r + (cc < nin ? l : l + kc) * r + jr;
+                }
+            }
+        }
+        const int ks = min(5, NT / D), msub = tid / D, me = tid - msub * D;
+        const bool mon = msub < ks;
+        int ml, mt;
+        const int mi = me % (2 * r), mo = cut_m_row(me / (2 * r) * 2 * r, L, r, ml, mt) + mi;
+        const int np = 2 * xn, kg = np ? min(CUT_KG, max(1, NT / np)) : 1;
+        const int uk = np ? tid / np : kg, upr = np ? tid - uk * np : 0, urow = upr >= xn, uil = upr - urow * xn;
         cluster.sync();   // every block's buffers are ready
         for (;;) {
             if (timing) t0 = gtime();
@@ -952,7 +1035,8 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
                     const C sc = s_sc[w];
                     for (int i = lane; i < Sx; i += 32) fs[i] = F.sc ? sc * f0[i] : f0[i];
                 } else {
-                    const C a0 = s_vin[0][w], a1 = s_vin[1][w], a2 = s_vin[2][w], a3 = s_vin[3][w];
+                    const C a0 = s_vin[w][0], a1 = s_vin[w][1], a2 = s_vin[w][2], a3 = s_vin[w][3];
+#pragma unroll 3
                     for (int i = lane; i < Sx; i += 32) {
                         C f = a0 * s_v[i];
                         cfma(f, a1, s_v[Sx + i]);
@@ -962,7 +1046,13 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
                     }
                 }
                 __syncwarp();
-                line_solve(s_xi + w * Sx, fs, Sx, lane, u ? pf[1] : pf[0], u ? pb[1] : pb[0]);
+                if (u == 0) {
+                    line_solve(s_xi + w * Sx, fs, Sx, lane, scan);
+                } else {
+                    LineScan<float> second;
+                    line_scan_init(s_xi + w * Sx, Sx, lane, second);
+                    line_solve(s_xi + w * Sx, fs, Sx, lane, second);
+                }
             }
             __syncthreads();
             // rows of the result: up (to the cut above) and down, one thread a column and pair
@@ -973,8 +1063,9 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
                     C o0 = {0, 0}, o1 = {0, 0};
                     for (int w = 0; w < nm; ++w) {
                         const C f = s_ln[w * Sx + i];
-                        cfma(o0, s_vout[2 * h][w], f);
-                        cfma(o1, s_vout[2 * h + 1][w], f);
+                        const cpair<float> vo = *(const cpair<float>*)&s_vout[w][2 * h];
+                        cfma(o0, vo.x, f);
+                        cfma(o1, vo.y, f);
                     }
                     // h = 0: rows 2, 3 of cut lf - 1; h = 1: rows 0, 1 of cut lf
                     const int cc = lf - 1 + h, row = h ? 0 : 2, grp = rank - lf * ngrp;
@@ -1060,64 +1151,59 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
             else if (tid < CC_CL) st_async(mapa(smem_u32(&s_word[rank]), tid), 0.f, mapa(mb + 8, tid));
             if (!(ok = wait(1, by2))) break;
             // ------------------------------------------------------------------ Y
-            for (int q = tid; q < D * 4; q += NT) {
-                const int e = q >> 2, sub = q & 3;
-                const int p = e / (2 * r), j = e - p * 2 * r, k = j >= r, jr = j - k * r;
-                const int l = 31 - __clz(p + 1), t = p + 1 - (1 << l);
-                const int span = 1 << (L - l), ca = t * span + k * (span / 2), own = t * span + span / 2 - 1;
-                const int nin = span / 2 - 1;
+            {
                 C s = {0, 0};
-                for (int u = sub; u < (nin + 1) * nch; u += 4) {
-                    const int cc = u / nch, cu = cc < nin ? ca + cc : own;
-                    s = s + s_bd[(cu * nch + u - cc * nch) * (L + 1) * r + (cc < nin ? l : l + k) * r + jr];
-                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (kb[u] >= 0) s = s + s_bd[kb[u]];
 #pragma unroll
                 for (int o = 1; o < 4; o <<= 1) {
-                    s.re += __shfl_xor_sync(__activemask(), s.re, o);
-                    s.im += __shfl_xor_sync(__activemask(), s.im, o);
+                    s.re += __shfl_xor_sync(0xffffffffu, s.re, o);
+                    s.im += __shfl_xor_sync(0xffffffffu, s.im, o);
                 }
-                if (sub == 0) s_d[e] = s;
+                if ((tid & 3) == 0 && ke < D) s_d[ke] = s;
             }
             __syncthreads();
             // y = M d: M transposed within a node's rows, so that the lanes' reads are
             // consecutive; a row's columns shared out over NT / D threads
-            const int ks = min(5, NT / D);
-            for (int q = tid; q < D * ks; q += NT) {
-                const int sub = q / D, e = q - sub * D;
-                const int p = e / (2 * r), i = e - p * 2 * r;
-                int l, t;
-                const int mo = cut_m_row(p * 2 * r, L, r, l, t);
+            if (mon) {
                 C s = {0, 0};
-                for (int lv = l, k0 = 0; lv < L; ++lv) {   // the subtree's columns, level by level
-                    const C* dl = s_d + ((1 << lv) - 1 + (t << (lv - l))) * 2 * r;
-                    const C* ml = s_m + mo + k0 * 2 * r + i;
-                    const int n = 2 * r << (lv - l);
+                const C* mp = s_m + mo;
+                for (int lv = ml; lv < L; ++lv) {   // the subtree's columns, level by level
+                    const C* dl = s_d + ((1 << lv) - 1 + (mt << (lv - ml))) * 2 * r;
+                    const int n = 2 * r << (lv - ml);
 #pragma unroll 4
-                    for (int k = sub; k < n; k += ks) cfma(s, ml[k * 2 * r], dl[k]);
-                    k0 += n;
+                    for (int k = msub; k < n; k += ks) cfma(s, mp[k * 2 * r], dl[k]);
+                    mp += n * 2 * r;
                 }
-                s_up[sub * D + e] = s;
+                s_up[tid] = s;
             }
             __syncthreads();
-            for (int e = tid; e < D; e += NT) {
+            // the entries of y this block's E columns take, in their order; all of them in the
+            // block that sums them
+            for (int k = has_b ? tid : Ke; k < Ke; k += NT) {
+                const int e = s_yi[k];
                 C s = s_up[e];
                 for (int u = 1; u < ks; ++u) s = s + s_up[u * D + e];
-                s_y[e] = s;
-                if (rank == 0) s_ya[e] = s_ya[e] + s;
+                s_y[k] = s;
             }
+            if (rank == 0)
+                for (int e = tid; e < D; e += NT) {
+                    C s = s_up[e];
+                    for (int u = 1; u < ks; ++u) s = s + s_up[u * D + e];
+                    s_ya[e] = s_ya[e] + s;
+                }
             __syncthreads();
             if (timing) { const unsigned long long t = gtime(); tB += t - t0; t0 = t; }
             // ------------------------------------------------------------------ C
             float nn = 0.f;
             if (has_b) {
-                const int np = 2 * xn, kg = min(CUT_KG, max(1, NT / np));
-                for (int q = tid; q < np * kg; q += NT) {
-                    const int kk = q / np, pr = q - kk * np, row = pr >= xn, il = pr - row * xn;
-                    const C* er = s_e + (size_t)row * Ke * XC + il;
+                if (uk < kg) {   // np kg <= NT
+                    const C* er = s_e + urow * Ke * XC + uil;
                     C s = {0, 0};
-#pragma unroll 4
-                    for (int k = kk; k < Ke; k += kg) cfma(s, er[k * XC], s_y[s_yi[k]]);
-                    s_up[kk * 2 * XC + row * XC + il] = s;
+#pragma unroll 8
+                    for (int k = uk; k < Ke; k += kg) cfma(s, er[k * XC], s_y[k]);
+                    s_up[uk * 2 * XC + urow * XC + uil] = s;
                 }
                 __syncthreads();
                 for (int q = tid; q < np; q += NT) {
@@ -1142,8 +1228,7 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
             nn = warp_sum(nn);
             if (warp < 4 && lane < CC_CL) st_async(mapa(smem_u32(&s_nrm[rank][warp]), lane), nn, mapa(mb + 16, lane));
             if (!(ok = wait(2, by3))) break;
-            n2 = 0.f;
-            for (int q = 0; q < CC_CL; ++q) n2 += (s_nrm[q][0] + s_nrm[q][1]) + (s_nrm[q][2] + s_nrm[q][3]);
+            n2 = warp_sum((&s_nrm[0][0])[lane] + (&s_nrm[0][0])[lane + 32]);   // alike in every warp
             if (timing) { const unsigned long long t = gtime(); tC += t - t0; t0 = t; }
             first = false;
             ++it;

@@ -73,9 +73,9 @@ __global__ void __launch_bounds__(256) k_edge_rows(const EdgeTask* __restrict__ 
                 fs[i] = f;
             }
             __syncwarp();
-            C pf, pb;
-            line_products(as, Sx, lane, pf, pb);
-            line_solve(as, fs, Sx, lane, pf, pb);
+            LineScan<T> sc;
+            line_scan_init(as, Sx, lane, sc);
+            line_solve(as, fs, Sx, lane, sc);
         }
         __syncthreads();
         for (int i = tid; i < Sx; i += 256) {

@@ -66,54 +66,82 @@ __device__ __forceinline__ void warp_line_solve(const cplx<T>* as, cplx<T>* fs, 
 }
 
 
-// The same recursions with the products of each lane's coefficients, which depend on xi
-// alone, given (line_products): 20 multiply-adds an element instead of 28.  Lane chunks are of odd
-// length, so that the lanes' strided shared-memory accesses fall in distinct banks.
+// The same recursions with everything that depends on xi alone given (line_scan_init): the
+// products of the lanes' coefficients at every stage of the two scans.  12 multiply-adds an
+// element and a scan of one value instead of 28 and two.  Lane chunks are of odd length, so
+// that the lanes' strided shared-memory accesses fall in distinct banks.
 template <typename T>
-__device__ __forceinline__ void line_products(const cplx<T>* as, int Sx, int lane, cplx<T>& pf, cplx<T>& pb) {
-    using C = cplx<T>;
-    const int L = ((Sx + 31) / 32) | 1, s = lane * L, e = min(Sx, s + L);
-    C a = {1, 0}, b = {1, 0};
-    for (int i = s; i < e; ++i) {
-        a = as[i] * a;
-        b = (i == Sx - 1 ? C{0, 0} : as[i]) * b;
-    }
-    pf = a;
-    pb = b;
+struct LineScan {
+    cplx<T> f[5], b[5];
+};
+template <typename T>
+__device__ __forceinline__ cplx<T> shfl_c(cplx<T> v, int d, bool up) {
+    cplx<T> o;
+    if (up) { o.re = __shfl_up_sync(0xffffffffu, v.re, d); o.im = __shfl_up_sync(0xffffffffu, v.im, d); }
+    else { o.re = __shfl_down_sync(0xffffffffu, v.re, d); o.im = __shfl_down_sync(0xffffffffu, v.im, d); }
+    return o;
 }
 template <typename T>
-__device__ __forceinline__ void line_solve(const cplx<T>* as, cplx<T>* fs, int Sx, int lane, cplx<T> pf, cplx<T> pb) {
+__device__ __forceinline__ void line_scan_init(const cplx<T>* as, int Sx, int lane, LineScan<T>& sc) {
+    using C = cplx<T>;
+    const int L = ((Sx + 31) / 32) | 1, s = min(Sx, lane * L), e = min(Sx, s + L);
+    C a = {1, 0};
+    for (int i = s; i < e; ++i) a = as[i] * a;
+    C f = a, b = e == Sx && s < e ? C{0, 0} : a;   // nothing enters from past the line's end
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const int d = 1 << k;
+        sc.f[k] = f;
+        sc.b[k] = b;
+        const C f2 = shfl_c(f, d, true), b2 = shfl_c(b, d, false);
+        if (lane >= d) f = f * f2;
+        if (lane + d < 32) b = b * b2;
+    }
+}
+template <typename T>
+__device__ __forceinline__ void line_solve(const cplx<T>* as, cplx<T>* fs, int Sx, int lane, const LineScan<T>& sc) {
     using C = cplx<T>;
     const int L = ((Sx + 31) / 32) | 1;
-    const int s = lane * L, e = min(Sx, s + L);
-    C A = pf, B = {0, 0};
-    for (int i = s; i < e; ++i) B = as[i] * (B + fs[i]);
-    for (int d = 1; d < 32; d <<= 1) {
-        C A2, B2;
-        affine_shfl(A, B, d, true, A2, B2);
-        if (lane >= d) { B = A * B2 + B; A = A * A2; }
+    const int s = min(Sx, lane * L), n = min(Sx - s, L);
+    const C* a = as + s;
+    C* x = fs + s;
+    C v = {0, 0};
+#pragma unroll 4
+    for (int i = 0; i < n; ++i) v = a[i] * (v + x[i]);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const C u = shfl_c(v, 1 << k, true);
+        if (lane >= (1 << k)) cfma(v, sc.f[k], u);
     }
-    C y;
-    y.re = __shfl_up_sync(0xffffffffu, B.re, 1);
-    y.im = __shfl_up_sync(0xffffffffu, B.im, 1);
-    if (lane == 0) y = {0, 0};
-    for (int i = s; i < e; ++i) { y = as[i] * (fs[i] + y); fs[i] = y; }
-    // backward over the lane's own chunk
-    A = pb;
-    B = {0, 0};
-    for (int i = e - 1; i >= s; --i) B = i == Sx - 1 ? fs[i] : as[i] * B + fs[i];
-    for (int d = 1; d < 32; d <<= 1) {
-        C A2, B2;
-        affine_shfl(A, B, d, false, A2, B2);
-        if (lane + d < 32) { B = A * B2 + B; A = A * A2; }
+    v = shfl_c(v, 1, true);
+    if (lane == 0) v = {0, 0};
+#pragma unroll 4
+    for (int i = 0; i < n; ++i) {
+        v = a[i] * (x[i] + v);
+        x[i] = v;
     }
-    C x;
-    x.re = __shfl_down_sync(0xffffffffu, B.re, 1);
-    x.im = __shfl_down_sync(0xffffffffu, B.im, 1);
-    if (lane == 31) x = {0, 0};
-    for (int i = e - 1; i >= s; --i) {
-        x = i == Sx - 1 ? fs[i] : fs[i] + as[i] * x;
-        fs[i] = x;
+    // backward over the lane's own chunk; the recursion starts from zero past the line's end,
+    // so the last element needs no case of its own
+    v = {0, 0};
+#pragma unroll 4
+    for (int i = n - 1; i >= 0; --i) {
+        C t = x[i];
+        cfma(t, a[i], v);
+        v = t;
+    }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const C u = shfl_c(v, 1 << k, false);
+        if (lane + (1 << k) < 32) cfma(v, sc.b[k], u);
+    }
+    v = shfl_c(v, 1, false);
+    if (lane == 31) v = {0, 0};
+#pragma unroll 4
+    for (int i = n - 1; i >= 0; --i) {
+        C t = x[i];
+        cfma(t, a[i], v);
+        x[i] = t;
+        v = t;
     }
     __syncwarp();
 }
