@@ -969,16 +969,17 @@ struct Solver final : SolverBase {
         d_etasks_own = a.take<EigTask>(nleaf);
         d_etask_one = a.take<EigTask>(1);
         if (mk > 0 && cut) {
-            const size_t nG = cut_ng(), nb = cut_gm_blocks((int)nG);
+            const size_t nG = cut_ng();
             cg.V = a.take<c128>(nG * (mk + 1));
             cg.alpha = a.take<c128>(mk + 1);
             cg.v1 = a.take<c128>(nG);
             cg.rG = a.take<c128>(nG);
+            cg.w = a.take<c128>(nG);
             cg.y0 = a.take<CT>(cp.D);
-            cg.part = a.take<c128>(2 * nb * 72);
+            cg.part = a.take<c128>((size_t)CUT_GM_BLOCKS * 72);
+            cg.dots = a.take<c128>(2 * 72);
             cg.scale = a.take<c128>(1);
-            cg.rho2 = a.take<double>(1);
-            cg.npart = a.take<double>(nb);
+            cg.npart = a.take<double>(CUT_GM_BLOCKS);
             cp.scale = cg.scale;
         } else if (mk > 0) {
             Vb = a.take<c128>(N * (mk + 1));
@@ -998,6 +999,7 @@ struct Solver final : SolverBase {
             gls.st = a.take<GmresState>(1);
             cg.ls = gls;
             cg.red = sizeof(T) == sizeof(float) ? 1e-4 : 1e-12;
+            cg.tol = P.tol;
         }
         d_ptrs = a.take<void*>(3 * 64);
         if (cut) {
@@ -2048,14 +2050,13 @@ struct Solver final : SolverBase {
 
     // Flexible GMRES (loop_gmres) with its Krylov space kept on the cut rows (k_cut.cu).  A
     // cycle starts from the FP64 residual of u with one step on every row, which gives S r;
-    // each further Arnoldi step is one step on the cut rows and one launch.  It ends at the
+    // it then runs in one launch, each Arnoldi step one step on the cut rows.  It ends at the
     // restart length, when the estimate is below tol / 2, or (complex64) when it has fallen by
     // as much as the steps' rounding allows; u then takes one application of M, and the FP64
-    // residual decides.
+    // residual decides.  The host reads one state a cycle.
     hh_status loop_gmres_cut(int& it, double& rel) {
         int* ctl = (int*)(dnorm + 6);
         const int nG = cut_ng(), nl = (int)lev[L].size();
-        const int* gate = (const int*)gls.st;   // GmresState.stop
         hh_status st = HH_OK;
         auto resid = [&]() {
             zero(ctl, 4 * sizeof(double) + sizeof(CutCtl));
@@ -2064,43 +2065,26 @@ struct Solver final : SolverBase {
             launch_residual_stop<T>(u, bvec, nullptr, RT, geom(0), npart, dnorm, ctl, dcounter, P.tol, stream);
             pend(PC_SPMV);
         };
-        auto step = [&](int mode, const int* g) {
-            return launch_cut_steps<T>(d_cut, 1, cut_group(), cp.cl, cut_smem, nullptr, mode, cbar, 1, derr, 0, stream, 1, g);
+        auto steps = [&](int mode, int max_steps, int gm_steps) {
+            return launch_cut_steps<T>(d_cut, 1, cut_group(), cp.cl, cut_smem, nullptr, mode, cbar, 1, derr, 0, stream,
+                                       max_steps, &cg, gm_steps);
         };
         resid();
-        for (;;) {
+        for (bool cycle = false;; cycle = true) {
             if (!read_norms(st)) return st;
+            if (cycle) {
+                if (h_gst[0].bad) return HH_ENOCONV;
+                it += h_gst[0].stop ? h_gst[0].jstop : h_gst[0].steps;
+            }
             rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;
             if (!std::isfinite(rel)) return HH_ENOCONV;
             if (rel < P.tol) return HH_OK;
             if (it >= P.max_iter) return HH_ENOCONV;
             eig_stage_prof(0, d_etasks_cin);
-            if (!step(1, nullptr)) return HH_ECUDA;
-            launch_cut_gm_start<T>(d_cut, cg, nG, stream);
-            const int nsteps = std::min(mk, P.max_iter - it);
-            int launched = 0;
-            for (int j = 0; j < nsteps; ++j) {
-                if (j >= GM_LAG) {
-                    const int sl = (j - GM_LAG) % GM_SLOTS;   // the state after step j - GM_LAG
-                    ck(cudaEventSynchronize(gm_ev[sl]), cerr);
-                    if (cerr != cudaSuccess) return HH_ECUDA;
-                    if (h_gst[sl].stop) break;
-                }
-                if (j > 0 && !step(2, gate)) return HH_ECUDA;
-                if (!launch_cut_arnoldi<T>(d_cut, cg, j, nG, P.tol, cbar, derr, stream)) return HH_ECUDA;
-                const int sl = j % GM_SLOTS;
-                ck(cudaMemcpyAsync(&h_gst[sl], gls.st, sizeof(GmresState), cudaMemcpyDeviceToHost, stream), cerr);
-                ck(cudaEventRecord(gm_ev[sl], stream), cerr);
-                ++launched;
-            }
-            const int last = (launched - 1) % GM_SLOTS;
-            if (!sync_check(st)) return st;
-            const GmresState fin = h_gst[last];   // of the last step queued: the cycle's end
-            if (fin.bad) return HH_ENOCONV;
-            const int jn = fin.stop ? fin.jstop : launched;
-            it += jn;
-            launch_cut_gm_combine<T>(d_cut, cg, jn, nG, stream);
-            if (!step(2, nullptr)) return HH_ECUDA;   // the corrections of the combined input
+            if (!steps(1, 0, std::min(mk, P.max_iter - it))) return HH_ECUDA;
+            ck(cudaMemcpyAsync(&h_gst[0], gls.st, sizeof(GmresState), cudaMemcpyDeviceToHost, stream), cerr);
+            launch_cut_gm_combine<T>(d_cut, cg, nG, stream);
+            if (!steps(2, 1, 0)) return HH_ECUDA;   // the corrections of the combined input
             launch_cut_lines<T>(d_cut, 1, nullptr, nl, b_max, Sx, stream);
             eig_stage_prof(2, d_etasks_cout);
             launch_cut_update<T>(d_upd + cut_flip, 1, Sy, Sx, stream);

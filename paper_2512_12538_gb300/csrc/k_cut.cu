@@ -313,6 +313,194 @@ __global__ void __launch_bounds__(256) k_cut_minv(const CutMinv* __restrict__ pr
     }
 }
 
+// ----------------------------------------------------------------- GMRES on the cut rows
+// Flexible GMRES's Krylov space from a residual r is spanned by r and vectors on the cut
+// rows: A M v = v - S v with S v (one step's residual) on the cut rows for any v.  A basis
+// vector is kept as (alpha, p): alpha times r off the cut rows and p on them, in FP64, with
+// the inner product conj(alpha) alpha' rho^2 + p^H p', rho = |r| off the cut rows, so the
+// Arnoldi process is that of the full vectors at 2 (2^L - 1) / S of their length.
+// S (alpha r + g) = alpha v1 + S g, v1 = S r from the cycle's first step and g = p - alpha
+// r_G on the cut rows, so every further step is one step of the iteration on g.
+//
+// One Arnoldi step inside the iteration's kernels, after phase C has left S g (the first
+// time S r) in P.v: w = V_j - S V_j, classical Gram-Schmidt twice against V_0 .. V_j, V_{j+1}
+// and the next g (into P.v), and in the first block the Givens update.  A block works on the
+// entries of its own cut items, so only the dot products cross blocks: partial sums, one
+// column a warp adds them, five barriers.  Bound by the FP64 pipe (16 multiply-adds an entry
+// and column) and the barriers; as a launch of its own, between launches of single steps
+// that load their panels again, a step took 127 us at 1023^2 where it takes 60 here.
+struct GmState {
+    c128 h[72], al[72], hc[72], sn[72];
+    double cs[72], red[32], rho2;
+};
+__device__ __forceinline__ double gm_block_sum(double x, double* red, int nw) {
+    x = warp_sum(x);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
+    __syncthreads();
+    double t = 0.0;
+    for (int k = 0; k < nw; ++k) t += red[k];
+    __syncthreads();
+    return t;
+}
+template <typename T, int NT>
+__device__ __noinline__ bool gm_arnoldi(const CutProb& P, const CutGmres& G, GmState& M, GroupBar& bar, int rank, int gsz,
+                                        int j) {
+    using C = cplx<T>;
+    constexpr int NW = NT / 32, NC8 = NT / 8;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, Sx = P.Sx, nc = j + 1;
+    const size_t nG = (size_t)2 * P.ncut * Sx;
+    C* v = (C*)P.v;
+    const double beta = sqrt(*P.nrm);
+    // this block's entries: f(entry) over its cut items
+    auto entries = [&](int t0, int step, auto&& f) {
+        for (int e = rank; e < P.nB; e += gsz) {
+            const int c = e / P.nch, x0 = (e - c * P.nch) * P.XC, xn = min(P.XC, Sx - x0);
+            for (int q = t0; q < 2 * xn; q += step) {
+                const int row = q >= xn;
+                f((size_t)(2 * c + row) * Sx + x0 + q - row * xn);
+            }
+        }
+    };
+    __syncthreads();
+    if (j == 0) {
+        const double inv = beta > 0.0 ? 1.0 / beta : 0.0;
+        double g2 = 0.0;
+        entries(tid, NT, [&](size_t o) {
+            const int c = (int)(o / (2 * (size_t)Sx));
+            const c128 r = cvt<double>(((const C*)P.rt)[(size_t)(P.mid[c] - 1) * Sx + (o - (size_t)2 * c * Sx)]);
+            G.rG[o] = r;
+            G.v1[o] = cvt<double>(v[o]);
+            G.V[o] = inv * r;
+            g2 += abs2(r);
+        });
+        g2 = gm_block_sum(g2, M.red, NW);
+        if (tid == 0) {
+            G.npart[rank] = g2;
+            M.al[0] = c128{inv, 0.0};
+            if (rank == 0) {
+                G.alpha[0] = M.al[0];
+                *G.ls.st = GmresState{0, 0, 0, 0, 0.0, 0.0};
+                G.ls.g[0] = c128{beta, 0.0};
+            }
+        }
+        if (!bar()) return false;
+        double t = 0.0;
+        for (int k = tid; k < gsz; k += NT) t += __ldcg(G.npart + k);
+        t = gm_block_sum(t, M.red, NW);
+        if (tid == 0) M.rho2 = fmax(0.0, *P.nrm - t);
+        __syncthreads();
+    }
+    const double rho2 = M.rho2;
+    c128 aw = M.al[j];                           // alpha of w: V_j's, as S V_j lies on the cut rows
+    entries(tid, NT, [&](size_t o) {
+        c128 sv = aw * G.v1[o];
+        if (j > 0) sv = sv + cvt<double>(v[o]);
+        G.w[o] = G.V[(size_t)j * nG + o] - sv;
+    });
+    for (int i = tid; i < nc; i += NT) M.hc[i] = {0, 0};
+    __syncthreads();
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int i0 = 0; i0 < nc; i0 += NC8) {
+            const int i = i0 + (tid >> 3);
+            c128 a = {0, 0};
+            if (i < nc) {
+                const c128* Vi = G.V + (size_t)i * nG;
+                entries(tid & 7, 8, [&](size_t o) { cfma_cj(a, Vi[o], G.w[o]); });
+            }
+            for (int o = 4; o > 0; o >>= 1) {
+                a.re += __shfl_xor_sync(0xffffffffu, a.re, o);
+                a.im += __shfl_xor_sync(0xffffffffu, a.im, o);
+            }
+            if (i < nc && (tid & 7) == 0) G.part[(size_t)rank * 72 + i] = a;
+        }
+        if (!bar()) return false;
+        for (int i = rank + gsz * warp; i < nc; i += gsz * NW) {
+            c128 a = {0, 0};
+            for (int k = lane; k < gsz; k += 32) a = a + ldcg(G.part + (size_t)k * 72 + i);
+            a = warp_sum(a);
+            if (lane == 0) G.dots[pass * 72 + i] = a + rho2 * (conj(M.al[i]) * aw);
+        }
+        if (!bar()) return false;
+        for (int i = tid; i < nc; i += NT) {
+            M.h[i] = ldcg(G.dots + pass * 72 + i);
+            M.hc[i] = M.hc[i] + M.h[i];
+        }
+        __syncthreads();
+        entries(tid, NT, [&](size_t o) {
+            c128 a0 = {0, 0}, a1 = {0, 0};
+            for (int i = 0; i < nc; i += 2) {
+                cfma(a0, M.h[i], G.V[(size_t)i * nG + o]);
+                if (i + 1 < nc) cfma(a1, M.h[i + 1], G.V[(size_t)(i + 1) * nG + o]);
+            }
+            G.w[o] = G.w[o] - (a0 + a1);
+        });
+        c128 da = {0, 0};
+        for (int i = lane; i < nc; i += 32) cfma(da, M.h[i], M.al[i]);
+        aw = aw - warp_sum(da);
+        __syncthreads();
+    }
+    double nn = 0.0;
+    entries(tid, NT, [&](size_t o) { nn += abs2(G.w[o]); });
+    nn = gm_block_sum(nn, M.red, NW);
+    if (tid == 0) G.npart[rank] = nn;
+    if (!bar()) return false;
+    nn = 0.0;
+    for (int k = lane; k < gsz; k += 32) nn += __ldcg(G.npart + k);
+    nn = warp_sum(nn) + rho2 * abs2(aw);          // alike in every warp
+    const double inv = nn > 0.0 ? 1.0 / sqrt(nn) : 0.0;
+    const c128 an = inv * aw;
+    entries(tid, NT, [&](size_t o) {
+        const c128 x = inv * G.w[o];
+        G.V[(size_t)(j + 1) * nG + o] = x;
+        v[o] = cvt<T>(x - an * G.rG[o]);
+    });
+    if (tid == 0) M.al[j + 1] = an;
+    if (rank != 0 || tid != 0) return true;
+    G.alpha[j + 1] = an;
+    // The Givens update of column j (k_gmres_rotate's), the chain in registers and shared
+    // memory: a column's entries back and forth through the L2 took 12 us at j = 40.
+    const GmresLs& ls = G.ls;
+    const double hn = sqrt(nn), nbv = sqrt(*P.b2);
+    c128 a = M.hc[0];
+    for (int i = 0; i < j; ++i) {
+        const c128 a1 = M.hc[i + 1];
+        ls.H[(size_t)i * ls.mk + j] = M.cs[i] * a + M.sn[i] * a1;
+        a = M.cs[i] * a1 - conj(M.sn[i]) * a;
+    }
+    const double aa = sqrt(abs2(a)), t = sqrt(abs2(a) + hn * hn);
+    double cs = 1.0;
+    c128 sn = {0.0, 0.0};
+    if (t != 0.0 && aa == 0.0) {
+        cs = 0.0;
+        sn = {1.0, 0.0};
+        a = {hn, 0.0};
+    } else if (t != 0.0) {
+        const c128 ph = (1.0 / aa) * a;
+        cs = aa / t;
+        sn = (hn / t) * ph;
+        a = t * ph;
+    }
+    ls.H[(size_t)j * ls.mk + j] = a;
+    M.cs[j] = cs;
+    M.sn[j] = sn;
+    const c128 gj = ls.g[j], gn = -(conj(sn) * gj);
+    ls.g[j + 1] = gn;
+    ls.g[j] = cs * gj;
+    GmresState* st = ls.st;
+    st->steps = j + 1;
+    const double gabs = sqrt(abs2(gn)), est = nbv > 0 ? gabs / nbv : 0.0;
+    st->est = est;
+    if (!isfinite(est)) {
+        st->bad = 1;
+        st->stop = 1;
+        st->jstop = j + 1;
+    } else if (est < 0.5 * G.tol || gabs < G.red * beta || hn == 0.0) {
+        st->stop = 1;
+        st->jstop = j + 1;
+    }
+    return true;
+}
+
 // ------------------------------------------------------------------- the iteration
 // Shared memory of a step block, in elements: the xi lines and their lane products, the
 // lines of one item, the input rows; M where every block forms y itself; the panels of the
@@ -360,8 +548,7 @@ HH_HD CutSmem cut_smem_layout(const CutProb& P, int nw) {
 template <typename T, int NT>
 __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ probs, int nprob, int gsz,
                                                   const int* modes, int mode_all, unsigned* bars, int* err,
-                                                  long long limit, int prof, int max_steps, const int* gate) {
-    if (gate && *gate) return;   // written by an earlier launch: the same for every block
+                                                  long long limit, int prof, int max_steps, CutGmres G, int gm_steps) {
     using C = cplx<T>;
     constexpr int NW = NT / 32;
     extern __shared__ __align__(16) unsigned char csm[];
@@ -371,6 +558,7 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
     // phase would fetch them from the L2 again, one dependent load after another
     __shared__ CutProb P;
     __shared__ CutLeaf F;
+    __shared__ GmState s_gm;
     const int ngroups = gridDim.x / gsz, group = blockIdx.x / gsz, rank = blockIdx.x - group * gsz;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     GroupBar bar{bars + group, (unsigned)gsz, 0u, err, limit};
@@ -765,6 +953,20 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
                 }
             }
             stepped = true;
+            if (gm_steps) {
+                // the Arnoldi step: P.v takes the next step's input
+                if (first && rank == 0)
+                    for (int e = tid; e < D; e += NT) ((C*)G.y0)[e] = s_ya[e];
+                if (!(ok = gm_arnoldi<T, NT>(P, G, s_gm, bar, rank, gsz, in_round))) break;
+                __syncthreads();
+                if (one && rank < P.nB) {
+                    const int c = rank / nch, x0 = (rank - c * nch) * XC, xn = min(XC, Sx - x0);
+                    for (int q = tid; q < 2 * xn; q += NT) {
+                        const int row = q >= xn, il = q - row * xn;
+                        s_own[row * XC + il] = v[((size_t)c * 2 + row) * Sx + x0 + il];
+                    }
+                }
+            }
             if (!(ok = bar())) break;
             // the norm, in the same order in every warp; then the tests
             n2 = 0.f;
@@ -776,7 +978,10 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
             ++it;
             ++in_round;
             reason = watch.test(n2, it, P, thr_anchor, thr_test);
-            if (!reason && ++done == max_steps) reason = CUT_LIMIT;
+            ++done;
+            // (a GMRES cycle: at its stop, written before the barrier, or its last step)
+            if (gm_steps) reason = __ldcg(&G.ls.st->stop) || done == gm_steps ? CUT_LIMIT : 0;
+            else if (!reason && done == max_steps) reason = CUT_LIMIT;
             if (reason) break;
         }
         if (ok && one && rank < P.nB) {
@@ -862,10 +1067,12 @@ __device__ __forceinline__ void st_async(uint32_t dst, float v, uint32_t mbar) {
                  : "memory");
 }
 
+// GM: with the Arnoldi steps of a GMRES cycle (apart, for its registers).
+template <bool GM>
 __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restrict__ probs, int nprob,
                                                           const int* modes, int mode_all, int* err, long long limit,
-                                                          int prof, int max_steps, const int* gate) {
-    if (gate && *gate) return;   // written by an earlier launch: the same for every block
+                                                          int prof, int max_steps, CutGmres G, int gm_steps,
+                                                          unsigned* bars) {
     using C = c64;
     constexpr int NT = CC_NT, NW = CC_NW;
     extern __shared__ __align__(16) unsigned char csm[];
@@ -886,6 +1093,7 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
     cluster.sync();
     const uint32_t mb = smem_u32(s_mb);
     unsigned phase = 0;   // steps this block has done: the mbarriers' parity
+    [[maybe_unused]] GroupBar bar{bars + group, (unsigned)CC_CL, 0u, err, 16 * limit};   // of the Arnoldi steps
     bool ok = true;
     // wait for `bytes` of exchange k; bounded
     auto wait = [&](int k, unsigned bytes) -> bool {
@@ -1214,6 +1422,28 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
                     nn += abs2(inv0 * s);
                 }
                 __syncthreads();
+            }
+            if constexpr (GM) {
+                // the Arnoldi step: S v goes through P.v, which takes the next step's input
+                C* vg = (C*)P.v;
+                for (int q = tid; q < np; q += NT) {
+                    const int row = q >= xn, il = q - row * xn;
+                    vg[((size_t)c * 2 + row) * Sx + x0 + il] = s_own[row * XC + il];
+                }
+                if (first && rank == 0)
+                    for (int e = tid; e < D; e += NT) ((C*)G.y0)[e] = s_ya[e];
+                __shared__ GmState s_gm;
+                if (!(ok = gm_arnoldi<float, NT>(P, G, s_gm, bar, rank, CC_CL, in_round))) break;
+                __syncthreads();
+                for (int q = tid; q < np; q += NT) {
+                    const int row = q >= xn, il = q - row * xn;
+                    s_own[row * XC + il] = vg[((size_t)c * 2 + row) * Sx + x0 + il];
+                }
+                __syncthreads();
+                // the first block tells the others whether the cycle ends
+                nn = rank == 0 && tid == 0 ? (float)*(volatile int*)&G.ls.st->stop : 0.f;
+            }
+            if (has_b) {
                 const int nd = ng0 + ng1;
                 for (int q = tid; q < np * nd; q += NT) {
                     const int dq = q / np, pr = q - dq * np, row = pr >= xn, il = pr - row * xn;
@@ -1235,7 +1465,9 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
             ++in_round;
             ++phase;
             reason = watch.test(n2, it, P, thr_anchor, thr_test);
-            if (!reason && ++done == max_steps) reason = CUT_LIMIT;
+            ++done;
+            if (GM) reason = s_nrm[0][0] != 0.f || done == gm_steps ? CUT_LIMIT : 0;
+            else if (!reason && done == max_steps) reason = CUT_LIMIT;
             if (reason) break;
         }
         if (ok && has_b)
@@ -1337,243 +1569,62 @@ __global__ void __launch_bounds__(256) k_cut_update(const CutUpdJob* __restrict_
     J.ut[o] = u + cvt<double>(acc);
 }
 
-// ----------------------------------------------------------------- GMRES on the cut rows
-// Flexible GMRES's Krylov space from a residual r is spanned by r and vectors on the cut
-// rows: A M v = v - S v with S v (one step's residual) on the cut rows for any v.  A basis
-// vector is kept as (alpha, p): alpha times r off the cut rows and p on them, in FP64, with
-// the inner product conj(alpha) alpha' rho^2 + p^H p', rho = |r| off the cut rows, so the
-// Arnoldi process is that of the full vectors at 2 (2^L - 1) / S of their length.
-// S (alpha r + g) = alpha v1 + S g, v1 = S r from the cycle's first step and g = p - alpha
-// r_G on the cut rows, so every further step is one step of k_cut_steps or k_cut_cluster.
-//
-// One launch per Arnoldi step j: w = V_j - S V_j, classical Gram-Schmidt twice against V_0 ..
-// V_j, V_{j+1}, the next step's input g, and in the first block the Givens update.  Each
-// block owns `eb` entries of the vectors and keeps its share of the basis in shared memory
-// for the four passes over it (FP64-pipe bound: 16 multiply-adds an entry and column).
-// (beyond 28000 entries the share is read from the L2 instead)
-static constexpr int GM_EB = 97, GM_BLOCKS = 148;
-HH_HD int gm_eb(int nG) { return nG <= GM_EB * GM_BLOCKS ? GM_EB : (nG + GM_BLOCKS - 1) / GM_BLOCKS; }
+// ----------------------------------------------------- end of a GMRES cycle (CutGmres)
+// Coefficients c = R^{-1} g (back substitution by one warp, in every block: R and the
+// reciprocals of its diagonal in shared memory first), the scale sum c_j alpha_j of r, and
+// the input sum c_j g_j on the cut rows, into P.v; its corrections and sums start from the
+// first step's, scaled, and zero.  Four threads an entry.
 template <typename T>
-__global__ void __launch_bounds__(256) k_cut_arnoldi(const CutProb* __restrict__ prob, CutGmres G, int j, int nG, int nb,
-                                                     int staged, double tol, unsigned* bars, int* err, long long limit) {
-    if (G.ls.st->stop) return;
+__global__ void __launch_bounds__(256) k_cut_gm_combine(const CutProb* __restrict__ prob, CutGmres G, int nG) {
     using C = cplx<T>;
-    extern __shared__ __align__(16) unsigned char gsm[];
-    const int EB = gm_eb(nG);
-    c128* w = (c128*)gsm;                        // [EB]
-    c128* vsm = w + EB;                          // [j + 1][EB] where it fits
-    __shared__ c128 h[72], s_al[72], hc[72], s_sn[72];
-    __shared__ double s_red[8], s_cs[72];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, blk = blockIdx.x;
-    GroupBar bar{bars, (unsigned)nb, 0u, err, limit};
-    const int e0 = blk * EB, ne = max(0, min(EB, nG - e0)), nc = j + 1;
-    const c128* vs = staged ? vsm : G.V + e0;    // entry e of V_i: vs[i * ldv + e]
-    const size_t ldv = staged ? EB : nG;
+    __shared__ c128 c[72], dinv[72], s_a;
+    extern __shared__ __align__(16) unsigned char rsm[];
+    c128* R = (c128*)rsm;                        // [jn][jn]
     const CutProb& P = *prob;
-    C* v = (C*)P.v;
-    const double beta = sqrt(*P.nrm), rho2 = *G.rho2;
-    if (staged)
-        for (int q = tid; q < nc * ne; q += 256) {
-            const int i = q / ne, e = q - i * ne;
-            vsm[i * EB + e] = G.V[(size_t)i * nG + e0 + e];
-        }
-    for (int i = tid; i < nc; i += 256) {
-        s_al[i] = G.alpha[i];
-        hc[i] = {0, 0};
-        if (blk == 0 && i < j) { s_cs[i] = G.ls.cs[i]; s_sn[i] = G.ls.sn[i]; }
+    const int tid = threadIdx.x, mk = G.ls.mk;
+    const int jn = G.ls.st->stop ? G.ls.st->jstop : G.ls.st->steps;
+    for (int q = tid; q < jn * jn; q += 256) R[q] = G.ls.H[(size_t)(q / jn) * mk + q % jn];
+    for (int i = tid; i < jn; i += 256) {
+        const c128 d = G.ls.H[(size_t)i * mk + i];
+        dinv[i] = abs2(d) > 0 ? cinv(d) : c128{0.0, 0.0};
+        c[i] = G.ls.g[i];
     }
-    __syncthreads();
-    c128 aw = s_al[j];                           // alpha of w: V_j's, as S V_j lies on the cut rows
-    for (int e = tid; e < ne; e += 256) {
-        c128 sv = s_al[j] * G.v1[e0 + e];
-        if (j > 0) sv = sv + cvt<double>(ldcg(v + e0 + e));
-        w[e] = vs[j * ldv + e] - sv;
-    }
-    __syncthreads();
-    for (int pass = 0; pass < 2; ++pass) {
-        c128* part = G.part + (size_t)pass * nb * 72;
-        for (int i0 = 0; i0 < nc; i0 += 32) {
-            const int i = i0 + (tid >> 3), sub = tid & 7;
-            c128 a = {0, 0};
-            if (i < nc)
-                for (int e = sub; e < ne; e += 8) cfma_cj(a, vs[i * ldv + e], w[e]);
-            for (int o = 4; o > 0; o >>= 1) {
-                a.re += __shfl_xor_sync(0xffffffffu, a.re, o);
-                a.im += __shfl_xor_sync(0xffffffffu, a.im, o);
-            }
-            if (i < nc && sub == 0) part[(size_t)blk * 72 + i] = a;
-        }
-        if (!bar()) return;
-        for (int i0 = 0; i0 < nc; i0 += 32) {
-            const int i = i0 + (tid >> 3), sub = tid & 7;
-            c128 a = {0, 0};
-            if (i < nc)
-                for (int k = sub; k < nb; k += 8) a = a + ldcg(part + (size_t)k * 72 + i);
-            for (int o = 4; o > 0; o >>= 1) {
-                a.re += __shfl_xor_sync(0xffffffffu, a.re, o);
-                a.im += __shfl_xor_sync(0xffffffffu, a.im, o);
-            }
-            if (i < nc && sub == 0) {
-                h[i] = a + rho2 * (conj(s_al[i]) * aw);
-                hc[i] = hc[i] + h[i];
-            }
-        }
-        __syncthreads();
-        {
-            // w -= V h, two threads an entry; alpha alike
-            const int sub = tid & 1;
-            for (int eb = 0; eb < ne; eb += 128) {
-                const int e = eb + (tid >> 1);
-                c128 a = {0, 0};
-                if (e < ne)
-                    for (int i = sub; i < nc; i += 2) cfma(a, h[i], vs[i * ldv + e]);
-                a.re += __shfl_xor_sync(0xffffffffu, a.re, 1);
-                a.im += __shfl_xor_sync(0xffffffffu, a.im, 1);
-                if (e < ne && sub == 0) w[e] = w[e] - a;
-            }
-            c128 da = {0, 0};
-            for (int i = lane; i < nc; i += 32) cfma(da, h[i], s_al[i]);
-            da = warp_sum(da);
-            aw = aw - da;
-        }
-        __syncthreads();
-    }
-    double nn = 0.0;
-    for (int e = tid; e < ne; e += 256) nn += abs2(w[e]);
-    nn = warp_sum(nn);
-    if (lane == 0) s_red[warp] = nn;
-    __syncthreads();
-    if (tid == 0) {
-        double t = 0.0;
-        for (int k = 0; k < 8; ++k) t += s_red[k];
-        G.npart[blk] = t;
-    }
-    if (!bar()) return;
-    nn = 0.0;
-    for (int k = tid; k < nb; k += 256) nn += __ldcg(G.npart + k);
-    nn = warp_sum(nn);
-    __syncthreads();
-    if (lane == 0) s_red[warp] = nn;
-    __syncthreads();
-    nn = rho2 * abs2(aw);
-    for (int k = 0; k < 8; ++k) nn += s_red[k];
-    const double inv = nn > 0.0 ? 1.0 / sqrt(nn) : 0.0;
-    const c128 an = inv * aw;
-    for (int e = tid; e < ne; e += 256) {
-        const c128 x = inv * w[e];
-        G.V[(size_t)(j + 1) * nG + e0 + e] = x;
-        v[e0 + e] = cvt<T>(x - an * G.rG[e0 + e]);
-    }
-    if (blk != 0 || tid != 0) return;
-    G.alpha[j + 1] = an;
-    // The Givens update of column j (k_gmres_rotate's), the chain in registers and shared
-    // memory: a column's entries back and forth through the L2 took 12 us at j = 40.
-    const GmresLs& ls = G.ls;
-    const double hn = sqrt(nn), nbv = sqrt(*P.b2);
-    c128 a = hc[0];
-    for (int i = 0; i < j; ++i) {
-        const c128 a1 = hc[i + 1];
-        hc[i] = s_cs[i] * a + s_sn[i] * a1;
-        a = s_cs[i] * a1 - conj(s_sn[i]) * a;
-    }
-    const double aa = sqrt(abs2(a)), t = sqrt(abs2(a) + hn * hn);
-    double cs = 1.0;
-    c128 sn = {0.0, 0.0};
-    if (t != 0.0 && aa == 0.0) {
-        cs = 0.0;
-        sn = {1.0, 0.0};
-        a = {hn, 0.0};
-    } else if (t != 0.0) {
-        const c128 ph = (1.0 / aa) * a;
-        cs = aa / t;
-        sn = (hn / t) * ph;
-        a = t * ph;
-    }
-    hc[j] = a;
-    ls.cs[j] = cs;
-    ls.sn[j] = sn;
-    const c128 gj = ls.g[j], gn = -(conj(sn) * gj);
-    ls.g[j + 1] = gn;
-    ls.g[j] = cs * gj;
-    for (int i = 0; i <= j; ++i) ls.H[(size_t)i * ls.mk + j] = hc[i];
-    GmresState* st = ls.st;
-    st->steps = j + 1;
-    const double gabs = sqrt(abs2(gn)), est = nbv > 0 ? gabs / nbv : 0.0;
-    st->est = est;
-    if (!isfinite(est)) {
-        st->bad = 1;
-        st->stop = 1;
-        st->jstop = j + 1;
-    } else if (est < 0.5 * tol || gabs < G.red * beta || hn == 0.0) {
-        st->stop = 1;
-        st->jstop = j + 1;
-    }
-}
-// Start of a cycle, after its first step: r on the cut rows, v1, rho^2, V_0 = r / |r|; one block.
-template <typename T>
-__global__ void __launch_bounds__(1024) k_cut_gm_start(const CutProb* __restrict__ prob, CutGmres G, int nG) {
-    using C = cplx<T>;
-    __shared__ double s_red[32];
-    const CutProb& P = *prob;
-    const int tid = threadIdx.x;
-    const double beta = sqrt(*P.nrm), inv = beta > 0.0 ? 1.0 / beta : 0.0;
-    double g2 = 0.0;
-    for (int e = tid; e < nG; e += 1024) {
-        const int c = e / (2 * P.Sx), q = e - c * 2 * P.Sx;
-        const c128 r = cvt<double>(((const C*)P.rt)[(size_t)(P.mid[c] - 1) * P.Sx + q]);
-        G.rG[e] = r;
-        G.v1[e] = cvt<double>(((const C*)P.v)[e]);
-        G.V[e] = inv * r;
-        g2 += abs2(r);
-    }
-    for (int d = tid; d < P.D; d += 1024) ((C*)G.y0)[d] = ((const C*)P.yacc)[d];
-    g2 = warp_sum(g2);
-    if ((tid & 31) == 0) s_red[tid >> 5] = g2;
-    __syncthreads();
-    if (tid == 0) {
-        double t = 0.0;
-        for (int k = 0; k < 32; ++k) t += s_red[k];
-        *G.rho2 = fmax(0.0, *P.nrm - t);
-        G.alpha[0] = c128{inv, 0.0};
-        *G.ls.st = GmresState{0, 0, 0, 0, 0.0, 0.0};
-        G.ls.g[0] = c128{beta, 0.0};
-    }
-}
-// End of a cycle of jn steps: coefficients c = R^{-1} g (back substitution by one warp, a
-// column at a time, in every block), the scale sum c_j alpha_j of r, the
-// input sum c_j g_j on the cut rows (into v; its corrections and sums start from scale y_0
-// and zero).
-template <typename T>
-__global__ void __launch_bounds__(256) k_cut_gm_combine(const CutProb* __restrict__ prob, CutGmres G, int jn, int nG) {
-    using C = cplx<T>;
-    __shared__ c128 c[72], s_a;
-    const CutProb& P = *prob;
-    const int tid = threadIdx.x;
-    for (int i = tid; i < jn; i += 256) c[i] = G.ls.g[i];
     __syncthreads();
     if (tid < 32)
         for (int i = jn - 1; i >= 0; --i) {
-            const c128 d = G.ls.H[(size_t)i * G.ls.mk + i];
-            const c128 y = abs2(d) > 0 ? c[i] * cinv(d) : c128{0.0, 0.0};
+            const c128 y = c[i] * dinv[i];
             __syncwarp();
             if (tid == 0) c[i] = y;
-            for (int k = tid; k < i; k += 32) c[k] = c[k] - G.ls.H[(size_t)k * G.ls.mk + i] * y;
+            for (int k = tid; k < i; k += 32) c[k] = c[k] - R[k * jn + i] * y;
             __syncwarp();
         }
     __syncthreads();
-    if (tid == 0) {
+    if (tid < 32) {
         c128 a = {0, 0};
-        for (int i = 0; i < jn; ++i) cfma(a, c[i], G.alpha[i]);
-        s_a = a;
-        if (blockIdx.x == 0) *G.scale = a;
+        for (int i = tid; i < jn; i += 32) cfma(a, c[i], G.alpha[i]);
+        a = warp_sum(a);
+        if (tid == 0) {
+            s_a = a;
+            if (blockIdx.x == 0) *G.scale = a;
+        }
     }
     __syncthreads();
     const c128 a = s_a;
-    for (int e = blockIdx.x * 256 + tid; e < nG; e += gridDim.x * 256) {
-        c128 x = -(a * G.rG[e]);
-        for (int i = 0; i < jn; ++i) cfma(x, c[i], G.V[(size_t)i * nG + e]);
-        ((C*)P.v)[e] = cvt<T>(x);
-        ((C*)P.vsum)[e] = C{0, 0};
+    const int sub = tid & 3;
+    for (int e0 = blockIdx.x * 64; e0 < nG; e0 += gridDim.x * 64) {
+        const int e = e0 + (tid >> 2);
+        c128 x = {0, 0};
+        if (e < nG)
+            for (int i = sub; i < jn; i += 4) cfma(x, c[i], G.V[(size_t)i * nG + e]);
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            x.re += __shfl_xor_sync(0xffffffffu, x.re, o);
+            x.im += __shfl_xor_sync(0xffffffffu, x.im, o);
+        }
+        if (e < nG && sub == 0) {
+            ((C*)P.v)[e] = cvt<T>(x - a * G.rG[e]);
+            ((C*)P.vsum)[e] = C{0, 0};
+        }
     }
     if (blockIdx.x == 0)
         for (int d = tid; d < P.D; d += 256) ((C*)P.yacc)[d] = cvt<T>(a * cvt<double>(((const C*)G.y0)[d]));
@@ -1615,7 +1666,7 @@ size_t cut_m_packed(int L, int r) { return (size_t)cut_m_elems(L, r); }
 //    on one cluster of sixteen (k_cut_cluster), bound by latency alone;
 //  * the others on a grid group of up to one block per SM (k_cut_steps): there the lines
 //    (FP64: the pipe, four warps fill it) and the panels' bytes want every SM.
-static constexpr int CUT_NT = 256, CUT_SMEM = 216 * 1024;
+static constexpr int CUT_NT = 256, CUT_SMEM = 212 * 1024;
 static bool cluster_form(CutProb& P, int b_max) {
     const int NL = P.ncut + 1;
     if (P.D > 128 || NL > CC_CL) return false;
@@ -1661,10 +1712,11 @@ size_t cut_plan(CutProb& P, int b_max) {
 static int cluster_count(size_t smem) {
     static std::atomic<unsigned long long> attr{0};
     if (!once_per_device(attr, [] {
-            return cudaFuncSetAttribute(k_cut_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, CUT_SMEM) ==
-                       cudaSuccess &&
-                   cudaFuncSetAttribute(k_cut_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-                       cudaSuccess;
+            for (auto fn : {k_cut_cluster<false>, k_cut_cluster<true>})
+                if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, CUT_SMEM) != cudaSuccess ||
+                    cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+                    return false;
+            return true;
         })) {
         cudaGetLastError();
         return 0;
@@ -1680,7 +1732,7 @@ static int cluster_count(size_t smem) {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_cut_cluster, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, k_cut_cluster<true>, &cfg) != cudaSuccess) {
         cudaGetLastError();
         n = 0;
     }
@@ -1690,7 +1742,8 @@ bool cut_cluster_ready(size_t smem) { return cluster_count(smem) > 0; }
 template <typename T>
 bool launch_cut_steps(const CutProb* probs, int nprob, int group, bool cl, size_t smem, const int* modes, int mode_all,
                       unsigned* bars, int max_groups, int* err, int prof, cudaStream_t s, int max_steps,
-                      const int* gate) {
+                      const CutGmres* gm, int gm_steps) {
+    const CutGmres G = gm ? *gm : CutGmres{};
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     cfg.dynamicSmemBytes = smem;
@@ -1707,9 +1760,10 @@ bool launch_cut_steps(const CutProb* probs, int nprob, int group, bool cl, size_
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         cfg.gridDim = dim3(CC_CL * std::min(nprob, nmax));
         cfg.blockDim = dim3(CC_NT);
+        if (gm_steps) cudaMemsetAsync(bars, 0, sizeof(unsigned), s);
         // (a try_wait suspends for up to microseconds: fewer of them make about a second)
-        e = cudaLaunchKernelEx(&cfg, k_cut_cluster, probs, nprob, modes, mode_all, err, std::min(polls, 1ll << 20),
-                               prof, max_steps, gate);
+        e = cudaLaunchKernelEx(&cfg, gm_steps ? k_cut_cluster<true> : k_cut_cluster<false>, probs, nprob, modes, mode_all, err, std::min(polls, 1ll << 20),
+                               prof, max_steps, G, gm_steps, bars);
     } else {
         static std::atomic<unsigned long long> attr{0};
         smem_limit_once(attr, k_cut_steps<T, CUT_NT>, CUT_SMEM);
@@ -1727,7 +1781,7 @@ bool launch_cut_steps(const CutProb* probs, int nprob, int group, bool cl, size_
         cfg.gridDim = dim3(gsz * ng);
         cfg.blockDim = dim3(CUT_NT);
         e = cudaLaunchKernelEx(&cfg, k_cut_steps<T, CUT_NT>, probs, nprob, gsz, modes, mode_all, bars, err, polls,
-                               prof, max_steps, gate);
+                               prof, max_steps, G, gm_steps);
     }
     note_launch();
     return e == cudaSuccess;
@@ -1742,39 +1796,11 @@ void launch_cut_lines(const CutProb* probs, int nprob, const int* modes, int nle
     k_cut_lines<T><<<dim3((b_max + wpb - 1) / wpb, nleaf_max, nprob), 256, per * wpb, s>>>(probs, modes, wpb);
     note_launch();
 }
-int cut_gm_blocks(int nG) { return (nG + gm_eb(nG) - 1) / gm_eb(nG); }
 template <typename T>
-void launch_cut_gm_start(const CutProb* prob, const CutGmres& G, int nG, cudaStream_t s) {
-    k_cut_gm_start<T><<<1, 1024, 0, s>>>(prob, G, nG);
-    note_launch();
-}
-template <typename T>
-bool launch_cut_arnoldi(const CutProb* prob, const CutGmres& G, int j, int nG, double tol, unsigned* bars, int* err,
-                        cudaStream_t s) {
+void launch_cut_gm_combine(const CutProb* prob, const CutGmres& G, int nG, cudaStream_t s) {
     static std::atomic<unsigned long long> attr{0};
-    smem_limit_once(attr, k_cut_arnoldi<T>, 208 * 1024);
-    const int nb = cut_gm_blocks(nG), eb = gm_eb(nG);
-    const size_t all = (size_t)(j + 2) * eb * sizeof(c128);
-    const int staged = all <= (size_t)(208 * 1024);
-    cudaMemsetAsync(bars, 0, sizeof(unsigned), s);
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    cfg.gridDim = dim3(nb);
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = staged ? all : eb * sizeof(c128);
-    cfg.stream = s;
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_cut_arnoldi<T>, prob, G, j, nG, nb, staged, tol, bars, err,
-                                             wait_polls(1ll << 24));
-    note_launch();
-    return e == cudaSuccess;
-}
-template <typename T>
-void launch_cut_gm_combine(const CutProb* prob, const CutGmres& G, int jn, int nG, cudaStream_t s) {
-    k_cut_gm_combine<T><<<std::min(152, (nG + 255) / 256), 256, 0, s>>>(prob, G, jn, nG);
+    smem_limit_once(attr, k_cut_gm_combine<T>, 64 * 64 * (int)sizeof(c128));
+    k_cut_gm_combine<T><<<std::min(152, (nG + 63) / 64), 256, sizeof(c128) * G.ls.mk * G.ls.mk, s>>>(prob, G, nG);
     note_launch();
 }
 template <typename T>
@@ -1789,11 +1815,9 @@ void launch_cut_update(const CutUpdJob* jobs, int njobs, int Sy_max, int Sx_max,
     template void launch_cut_minv<T>(const CutMinv*, int, int, int, int, const c128*, c128*, cplx<T>*, int, cudaStream_t); \
     template size_t cut_plan<T>(CutProb&, int);                                                                       \
     template bool launch_cut_steps<T>(const CutProb*, int, int, bool, size_t, const int*, int, unsigned*, int, int*, int,   \
-                                      cudaStream_t, int, const int*);                                                                  \
+                                      cudaStream_t, int, const CutGmres*, int);                                                                  \
     template void launch_cut_lines<T>(const CutProb*, int, const int*, int, int, int, cudaStream_t);                  \
-    template void launch_cut_gm_start<T>(const CutProb*, const CutGmres&, int, cudaStream_t);                         \
-    template bool launch_cut_arnoldi<T>(const CutProb*, const CutGmres&, int, int, double, unsigned*, int*, cudaStream_t); \
-    template void launch_cut_gm_combine<T>(const CutProb*, const CutGmres&, int, int, cudaStream_t);                  \
+    template void launch_cut_gm_combine<T>(const CutProb*, const CutGmres&, int, cudaStream_t);                       \
     template void launch_cut_update<T>(const CutUpdJob*, int, int, int, cudaStream_t);
 HH_CUT_INST(float)
 HH_CUT_INST(double)

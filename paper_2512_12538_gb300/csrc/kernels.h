@@ -382,35 +382,30 @@ bool cut_cluster_ready(size_t smem);
 // fills the items of P; returns the steps' shared memory, 0 if the lines do not fit
 template <typename T>
 size_t cut_plan(CutProb& P, int b_max);
+// Flexible GMRES on the cut rows: its vectors and the least-squares problem.
+struct CutGmres {
+    c128 *V, *alpha;           // [mk + 1][nG], [mk + 1]
+    c128 *v1, *rG, *w;         // [nG]: S r, r on the cut rows, the vector in work
+    void* y0;                  // [D]: the corrections of the first step
+    c128 *part, *dots, *scale; // [CUT_GM_BLOCKS][72], [2][72], [1]
+    double* npart;             // [CUT_GM_BLOCKS]
+    GmresLs ls;
+    double red, tol;           // a cycle ends when the estimate is below red |r| or tol |b| / 2
+};
+constexpr int CUT_GM_BLOCKS = 152;
 // runs every problem with a nonzero mode (1: new round, 2: go on) until its next stop, at most
-// max_steps steps (0: no limit); nothing while the device word gate is nonzero;
+// max_steps steps (0: no limit); gm_steps > 0: one problem's GMRES cycle of at most so many;
 // group: blocks per problem of a grid group (cl: one cluster); bars: a word per group; false if it cannot be launched
 template <typename T>
 bool launch_cut_steps(const CutProb* probs, int nprob, int group, bool cl, size_t smem, const int* modes, int mode_all,
                       unsigned* bars, int max_groups, int* err, int prof, cudaStream_t s, int max_steps = 0,
-                      const int* gate = nullptr);
+                      const CutGmres* gm = nullptr, int gm_steps = 0);
 template <typename T>
 void launch_cut_lines(const CutProb* probs, int nprob, const int* modes, int nleaf_max, int b_max, int Sx_max,
                       cudaStream_t s);
-// Flexible GMRES on the cut rows (k_cut.cu): its vectors, nG = 2 (2^L - 1) Sx entries each,
-// and the least-squares problem.
-struct CutGmres {
-    c128 *V, *alpha;           // [mk + 1][nG], [mk + 1]
-    c128 *v1, *rG;             // [nG]: S r, r on the cut rows
-    void* y0;                  // [D]: the corrections of the first step
-    c128 *part, *scale;        // [2][blocks][72], [1]
-    double *rho2, *npart;      // [1], [blocks]
-    GmresLs ls;
-    double red;                // a cycle ends when the estimate is below red |r|
-};
-int cut_gm_blocks(int nG);
+// end of a GMRES cycle: the combined input and its scale of r (nG = 2 (2^L - 1) Sx entries)
 template <typename T>
-void launch_cut_gm_start(const CutProb* prob, const CutGmres& G, int nG, cudaStream_t s);
-template <typename T>
-bool launch_cut_arnoldi(const CutProb* prob, const CutGmres& G, int j, int nG, double tol, unsigned* bars, int* err,
-                        cudaStream_t s);
-template <typename T>
-void launch_cut_gm_combine(const CutProb* prob, const CutGmres& G, int jn, int nG, cudaStream_t s);
+void launch_cut_gm_combine(const CutProb* prob, const CutGmres& G, int nG, cudaStream_t s);
 template <typename T>
 void launch_cut_update(const CutUpdJob* jobs, int njobs, int Sy_max, int Sx_max, cudaStream_t s);
 
