@@ -271,46 +271,50 @@ __device__ __forceinline__ int cut_m_row(int e, int L, int r, int& l, int& t) {
 }
 
 // M_ps for one pair (p, s below or equal p): Ainv_p if s = p, else
-// -Ainv_p sum_{s <= q < p} G_pq M_qs, FP64, the sum first in shared memory.
+// -Ainv_p sum_{s <= q < p} G_pq M_qs, FP64.  A block takes MINV_ROWS rows: (Ainv_p G_pq) of
+// those rows in shared memory, then its product with M_qs (bound by the latency of the FP64
+// chains; a set-up of 1023^2 at 2r = 64 took 1.4 ms longer with one block a pair).
+static constexpr int MINV_ROWS = 4;
 template <typename T>
 __global__ void __launch_bounds__(256) k_cut_minv(const CutMinv* __restrict__ prs, int D, int L, int p2,
                                                   const c128* __restrict__ G, c128* M, cplx<T>* MT, int tr) {
-    using C = cplx<T>;
-    extern __shared__ __align__(16) unsigned char msm[];
-    c128* xs = (c128*)msm;                 // [p2][p2]
+    __shared__ c128 ai[MINV_ROWS][64], xs[MINV_ROWS][64];
     const CutMinv e = prs[blockIdx.x];
     const size_t rp = (size_t)e.p * p2, cs = (size_t)e.s * p2;
+    const int i0 = blockIdx.y * MINV_ROWS, ni = min(MINV_ROWS, p2 - i0);
+    if (ni <= 0) return;
     // M in the basis precision is packed: rows of p's subtree level by level
     int l, t;
-    C* mt = MT + cut_m_row(e.p * p2, L, p2 / 2, l, t);
+    cplx<T>* mt = MT + cut_m_row(e.p * p2, L, p2 / 2, l, t);
     const int len = p2 * ((1 << (L - l)) - 1), ls = 31 - __clz(e.s + 1);
     const int k0 = p2 * ((1 << (ls - l)) - 1 + (e.s + 1 - (1 << ls)) - (t << (ls - l)));
     // (tr: the cluster form's order, transposed within the node's rows)
-    auto put = [&](int i, int j, c128 v) { mt[tr ? (size_t)(k0 + j) * p2 + i : (size_t)i * len + k0 + j] = cvt<T>(v); };
-    if (e.p == e.s) {
-        for (int q = threadIdx.x; q < p2 * p2; q += 256) {
-            const int i = q / p2, j = q - i * p2;
-            const c128 v = e.Ainv[q];
-            M[(rp + i) * D + cs + j] = v;
-            put(i, j, v);
-        }
-        return;
+    auto put = [&](int i, int j, c128 v) {
+        M[(rp + i) * D + cs + j] = v;
+        mt[tr ? (size_t)(k0 + j) * p2 + i : (size_t)i * len + k0 + j] = cvt<T>(v);
+    };
+    for (int q = threadIdx.x; q < ni * p2; q += 256) {
+        const int i = q / p2, j = q - i * p2;
+        ai[i][j] = e.Ainv[(size_t)(i0 + i) * p2 + j];
+        if (e.p == e.s) put(i0 + i, j, ai[i][j]);
     }
-    for (int t = threadIdx.x; t < p2 * p2; t += 256) {
-        const int i = t / p2, j = t - i * p2;
-        c128 a = {0, 0};
-        for (int q = e.s; q != e.p; q = (q - 1) >> 1)   // s and its ancestors below p
-            for (int k = 0; k < p2; ++k) cfma(a, G[(rp + i) * D + (size_t)q * p2 + k], M[((size_t)q * p2 + k) * D + cs + j]);
-        xs[t] = a;
+    if (e.p == e.s) return;
+    const int i = threadIdx.x >> 6, j = threadIdx.x & 63;
+    const bool on = i < ni && j < p2;
+    c128 acc = {0, 0};
+    for (int q = e.s; q != e.p; q = (q - 1) >> 1) {   // s and its ancestors below p
+        __syncthreads();
+        c128 h = {0, 0};
+        if (on)
+#pragma unroll 8
+            for (int k = 0; k < p2; ++k) cfma(h, ai[i][k], G[(rp + k) * D + (size_t)q * p2 + j]);
+        if (on) xs[i][j] = h;
+        __syncthreads();
+        if (on)
+#pragma unroll 8
+            for (int k = 0; k < p2; ++k) cfma(acc, xs[i][k], M[((size_t)q * p2 + k) * D + cs + j]);
     }
-    __syncthreads();
-    for (int t = threadIdx.x; t < p2 * p2; t += 256) {
-        const int i = t / p2, j = t - i * p2;
-        c128 a = {0, 0};
-        for (int k = 0; k < p2; ++k) cfma(a, e.Ainv[i * p2 + k], xs[k * p2 + j]);
-        M[(rp + i) * D + cs + j] = -a;
-        put(i, j, -a);
-    }
+    if (on) put(i0 + i, j, -acc);
 }
 
 // ----------------------------------------------------------------- GMRES on the cut rows
@@ -1652,9 +1656,7 @@ void launch_cut_gram(const CutGramPair* prs, int npairs, const CutGramDest* ds, 
 template <typename T>
 void launch_cut_minv(const CutMinv* prs, int n, int D, int L, int p2, const c128* G, c128* M, cplx<T>* MT, int tr,
                      cudaStream_t s) {
-    static std::atomic<unsigned long long> attr{0};
-    smem_limit_once(attr, k_cut_minv<T>, 64 * 64 * sizeof(c128));
-    k_cut_minv<T><<<n, 256, sizeof(c128) * p2 * p2, s>>>(prs, D, L, p2, G, M, MT, tr);
+    k_cut_minv<T><<<dim3(n, (p2 + MINV_ROWS - 1) / MINV_ROWS), 256, 0, s>>>(prs, D, L, p2, G, M, MT, tr);
     note_launch();
 }
 
