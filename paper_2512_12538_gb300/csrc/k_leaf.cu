@@ -5,11 +5,18 @@
 // along x), A~_leaf is block tridiagonal with b x b blocks:
 //     D_i  (tridiagonal: the y-coupling inside column i, plus the diagonal terms),
 //     L_i = U_{i-1} = -W (W = diag of the row weights w_a: 1/2 on the band edges).
-// Factorisation (Schur recursion): S_0 = D_0, S_i = D_i - W S_{i-1}^{-1} W; the kernel
-// stores X_i = S_i^{-1} (dense, explicit inverse by Gauss-Jordan with partial pivoting).
-// Solve: forward  y_0 = X_0 f_0,  y_i = X_i (f_i + W y_{i-1});
-//        backward x_{n-1} = y_{n-1}, x_i = y_i + X_i W x_{i+1}.
+// Factorisation (Schur recursion) from both ends towards the middle column m, two chains of
+// half the length that run side by side: S_0 = D_0, S_i = D_i - W X_{i-1} W left of m (the
+// mirror image right of it), S_m = D_m - W X_{m-1} W - W X_{m+1} W; the kernels store
+// X_i = S_i^{-1} (dense, explicit inverse by Gauss-Jordan with partial pivoting).
+// Solve: inwards   y_i = X_i (f_i + W y_{i-1}) (right of m: W y_{i+1}),
+//                  x_m = X_m (f_m + W y_{m-1} + W y_{m+1});
+//        outwards  x_i = y_i + X_i W x_{i+1}   (right of m: W x_{i-1}).
 // 1D leaf (Sx = 1): the same recursion with 1 x 1 blocks along the band's rows.
+#include <algorithm>
+
+#include <cooperative_groups.h>
+
 #include "k_line.cuh"
 #include "kernels.h"
 
@@ -23,6 +30,7 @@ int leaf_ldx(int b, int elem_bytes) {
 
 static constexpr uint32_t WAIT_LIMIT = 1u << 21;   // bounded mbarrier polls (~0.1-0.3 s)
 static constexpr int MAXP = 4;                       // row pieces per step in the sweep
+static constexpr int SW_SLOTS = 12;                  // pieces in flight in the sweep, at most
 
 // ------------------------------------------------------------- factorisation (2D)
 template <typename T>
@@ -89,10 +97,30 @@ __device__ void gj_invert(cplx<T>* M, int ld, int b, cplx<T>* col, cplx<T>* row,
     __syncthreads();
 }
 
+// One of the two chains' columns in order: column t of side 0 (left) or 1 (right); a chain
+// has chain_len columns, the middle one belongs to neither.
+__device__ __forceinline__ int chain_mid(int Sx) { return Sx / 2; }
+__device__ __forceinline__ int chain_len(int Sx, int side) { return side ? Sx - 1 - Sx / 2 : Sx / 2; }
+__device__ __forceinline__ int chain_col(int Sx, int side, int t) { return side ? Sx - 1 - t : t; }
+
+// Entry (r, c) of S_i without the neighbour columns' terms.
 template <typename T>
-__global__ void __launch_bounds__(256) k_factor2d(const LeafTask* __restrict__ tasks, int Sx, double kh, int* err) {
+__device__ __forceinline__ cplx<T> block_entry(int r, int c, int i, const OpGeom& g, T wi) {
+    if (r == c) {
+        const c128 d = op_diag(r, i, g);
+        return {(T)d.re, (T)d.im};
+    }
+    if (r - c == 1 || c - r == 1) return {-wi, (T)0};
+    return {(T)0, (T)0};
+}
+
+// The bands too tall for k_factor2d_reg: the block in shared memory.  mid: the middle column,
+// from the stored inverses of its neighbours; else blockIdx.y is the chain.
+template <typename T>
+__global__ void __launch_bounds__(256) k_factor2d(const LeafTask* __restrict__ tasks, int Sx, double kh, int mid,
+                                                  int* err) {
     const LeafTask tk = tasks[blockIdx.x];
-    const int b = tk.b, ldx = tk.ldx;
+    const int b = tk.b, ldx = tk.ldx, side = blockIdx.y;
     cplx<T>* X = (cplx<T>*)tk.X;
     extern __shared__ __align__(16) unsigned char smf[];
     cplx<T>* M = (cplx<T>*)smf;      // b x b, leading dimension b
@@ -101,20 +129,21 @@ __global__ void __launch_bounds__(256) k_factor2d(const LeafTask* __restrict__ t
     int* perm = (int*)(row + b);
     const OpGeom g{b, Sx, kh, tk.khr};
     const size_t step = (size_t)b * ldx;
-    for (int i = 0; i < Sx; ++i) {
-        // S_i = D_i - W X_{i-1} W, built in place over X_{i-1}
+    const int n = mid ? 1 : chain_len(Sx, side);
+    for (int t = 0; t < n; ++t) {
+        const int i = mid ? chain_mid(Sx) : chain_col(Sx, side, t);
+        // built in place over the previous column's inverse
         const T wi = (T)wcol(i, Sx);
         for (int e = threadIdx.x; e < b * b; e += blockDim.x) {
             const int r = e / b, c = e - r * b;
-            cplx<T> v = {0, 0};
-            if (i > 0) v = (-(T)(wrow(r, b) * wrow(c, b))) * M[e];
-            if (r == c) {
-                const c128 d = op_diag(r, i, g);
-                v = v + cplx<T>{(T)d.re, (T)d.im};
-            } else if (r - c == 1 || c - r == 1) {
-                v.re -= wi;
+            cplx<T> q = {0, 0};
+            if (mid) {
+                q = X[(size_t)(i - 1) * step + (size_t)r * ldx + c];
+                if (i + 1 < Sx) q = q + X[(size_t)(i + 1) * step + (size_t)r * ldx + c];
+            } else if (t > 0) {
+                q = M[e];
             }
-            M[e] = v;
+            M[e] = (-(T)(wrow(r, b) * wrow(c, b))) * q + block_entry<T>(r, c, i, g, wi);
         }
         __syncthreads();
         gj_invert(M, b, b, col, row, perm, err);
@@ -123,9 +152,130 @@ __global__ void __launch_bounds__(256) k_factor2d(const LeafTask* __restrict__ t
             const int r = e / ldx, c = e - r * ldx;
             Xi[e] = c < b ? M[r * b + c] : cplx<T>{0, 0};
         }
-        // no barrier needed: each thread rebuilds exactly the elements it owns?  Not
-        // guaranteed (different index maps), so synchronise.
         __syncthreads();
+    }
+}
+
+// The same with the block in registers: lane and slot give a thread's rows (lane + 32 rs),
+// warp and slot its columns (warp + NW cs).  Rows are not exchanged: a pivot row is marked,
+// column k of the tableau ends up as the column of the pivot row p_k, and the store puts
+// entry (p_k, c) at (k, p_c).  The chain of pivots bounds it (b columns x Sx / 2 blocks, each
+// pivot waiting for the one before): a pivot costs one barrier, its search stays in the
+// warp that owns the column, and the pivot row's entries come by shuffles.  4 bands of 37 rows
+// x 129 columns in complex64: 7.4 ms with the block in shared memory and one chain, 1.45 ms here.
+template <typename T> __device__ __forceinline__ unsigned pivot_key(T a) {
+    if constexpr (sizeof(T) == 8) return (unsigned)__double2hiint(a) + 1u;
+    else return __float_as_uint(a) + 1u;
+}
+template <typename T, int RS, int NW>
+__global__ void __launch_bounds__(NW * 32, 1) k_factor2d_reg(const LeafTask* __restrict__ tasks, int Sx, double kh,
+                                                             int mid, int* err) {
+    using C = cplx<T>;
+    constexpr int CS = (RS * 32 + NW - 1) / NW;
+    __shared__ C s_col[2][RS * 32];
+    __shared__ C s_ip[2];
+    __shared__ int s_p[RS * 32];
+    extern __shared__ __align__(16) unsigned char smf[];
+    C* sx = (C*)smf;                            // [b][b | 1]: the finished inverse
+    const LeafTask tk = tasks[blockIdx.x];
+    const int b = tk.b, ldx = tk.ldx, ld = b | 1, side = blockIdx.y;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    C* X = (C*)tk.X;
+    const OpGeom g{b, Sx, kh, tk.khr};
+    const size_t step = (size_t)b * ldx;
+    const int n = mid ? 1 : chain_len(Sx, side);
+    C m[RS][CS];
+    for (int t = 0; t < n; ++t) {
+        const int i = mid ? chain_mid(Sx) : chain_col(Sx, side, t);
+        const T wi = (T)wcol(i, Sx);
+        unsigned used = 0;                      // this lane's rows that have been pivots
+        int kk[RS];                             // and for which column
+#pragma unroll
+        for (int rs = 0; rs < RS; ++rs) {
+            const int r = lane + 32 * rs;
+            kk[rs] = 0;
+            if (r >= b) used |= 1u << rs;
+#pragma unroll
+            for (int cs = 0; cs < CS; ++cs) {
+                const int c = warp + NW * cs;
+                m[rs][cs] = C{0, 0};
+                if (r >= b || c >= b) continue;
+                C q = {0, 0};
+                if (mid) {
+                    q = X[(size_t)(i - 1) * step + (size_t)r * ldx + c];
+                    if (i + 1 < Sx) q = q + X[(size_t)(i + 1) * step + (size_t)r * ldx + c];
+                } else if (t > 0) {
+                    q = sx[r * ld + c];
+                }
+                m[rs][cs] = (-(T)(wrow(r, b) * wrow(c, b))) * q + block_entry<T>(r, c, i, g, wi);
+            }
+        }
+#pragma unroll
+        for (int cs = 0; cs < CS; ++cs)
+            for (int w = 0; w < NW; ++w) {
+                const int k = cs * NW + w;
+                if (k >= b) break;
+                const int bf = k & 1;
+                if (warp == w) {
+                    unsigned key = 0;
+                    int br = lane;
+                    C best = {(T)1, (T)0};
+#pragma unroll
+                    for (int rs = 0; rs < RS; ++rs) {
+                        s_col[bf][lane + 32 * rs] = m[rs][cs];
+                        const unsigned a = (used >> rs & 1) ? 0u : pivot_key<T>(abs2(m[rs][cs]));
+                        if (a > key) { key = a; br = lane + 32 * rs; best = m[rs][cs]; }
+                    }
+                    const unsigned kmax = __reduce_max_sync(0xffffffffu, key);
+                    const T a2 = abs2(best);
+                    const bool bad = !(a2 > (T)0) || !isfinite(a2);
+                    if (bad) best = C{(T)1, (T)0};
+                    const C ip = cinv(best);
+                    if (lane == __ffs(__ballot_sync(0xffffffffu, key == kmax)) - 1) {
+                        s_p[k] = br;
+                        s_ip[bf] = ip;
+                        if (bad) atomicExch(err, DEV_BREAKDOWN);
+                    }
+                }
+                __syncthreads();
+                const int p = s_p[k], pl = p & 31, ps = p >> 5;
+                const C ip = s_ip[bf];
+                C f[RS], fi[RS];
+#pragma unroll
+                for (int rs = 0; rs < RS; ++rs) {
+                    f[rs] = s_col[bf][lane + 32 * rs];
+                    fi[rs] = -(f[rs] * ip);
+                    if (ps == rs && lane == pl) { used |= 1u << rs; kk[rs] = k; fi[rs] = ip; }
+                }
+#pragma unroll
+                for (int c2 = 0; c2 < CS; ++c2) {
+                    C v = m[0][c2];
+#pragma unroll
+                    for (int rs = 1; rs < RS; ++rs)
+                        if (ps == rs) v = m[rs][c2];
+                    v.re = __shfl_sync(0xffffffffu, v.re, pl);
+                    v.im = __shfl_sync(0xffffffffu, v.im, pl);
+                    v = v * ip;
+                    const bool own = c2 == cs && warp == w;
+#pragma unroll
+                    for (int rs = 0; rs < RS; ++rs) {
+                        const bool pr = ps == rs && lane == pl;
+                        m[rs][c2] = own ? fi[rs] : pr ? v : m[rs][c2] - f[rs] * v;
+                    }
+                }
+            }
+#pragma unroll
+        for (int cs = 0; cs < CS; ++cs) {
+            const int c = warp + NW * cs;
+            const int pc = c < b ? s_p[c] : 0;
+#pragma unroll
+            for (int rs = 0; rs < RS; ++rs)
+                if (lane + 32 * rs < b && c < b) sx[kk[rs] * ld + pc] = m[rs][cs];
+        }
+        __syncthreads();
+        C* Xi = X + (size_t)i * step;
+        for (int r = warp; r < b; r += NW)
+            for (int c = lane; c < ldx; c += 32) Xi[(size_t)r * ldx + c] = c < b ? sx[r * ld + c] : C{0, 0};
     }
 }
 
@@ -156,6 +306,16 @@ int leaf_block_bmax(int elem_bytes) {
     return b;
 }
 
+template <typename T, int RS, int NW>
+static void factor_reg(const LeafTask* d_tasks, int ntasks, int b_max, int Sx, double kh, int* err, cudaStream_t s) {
+    const size_t sm = sizeof(cplx<T>) * (size_t)b_max * (b_max | 1);
+    cudaFuncSetAttribute(k_factor2d_reg<T, RS, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    for (int mid = 0; mid < 2; ++mid) {       // the two chains, then the middle column
+        k_factor2d_reg<T, RS, NW><<<dim3(ntasks, 2 - mid), NW * 32, sm, s>>>(d_tasks, Sx, kh, mid, err);
+        note_launch();
+    }
+}
+
 template <typename T>
 void launch_factor(const LeafTask* d_tasks, int ntasks, int b_max, int Sx, double kh, int* err, cudaStream_t s) {
     if (Sx == 1) {
@@ -163,46 +323,68 @@ void launch_factor(const LeafTask* d_tasks, int ntasks, int b_max, int Sx, doubl
         note_launch();
         return;
     }
-    const size_t sm = sizeof(cplx<T>) * ((size_t)b_max * b_max + 2 * b_max) + sizeof(int) * b_max;
-    cudaFuncSetAttribute(k_factor2d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_factor2d<T><<<ntasks, 256, sm, s>>>(d_tasks, Sx, kh, err);
-    note_launch();
+    // in registers up to 128 rows (complex64) or 96 (complex128): 32 of a thread's 64 registers
+    // (36) hold the block there, and taller blocks would spill
+    if (b_max <= 32) factor_reg<T, 1, 8>(d_tasks, ntasks, b_max, Sx, kh, err, s);
+    else if (b_max <= 64) factor_reg<T, 2, 16>(d_tasks, ntasks, b_max, Sx, kh, err, s);
+    else if (b_max <= 96) factor_reg<T, 3, 32>(d_tasks, ntasks, b_max, Sx, kh, err, s);
+    else if (sizeof(T) == 4 && b_max <= 128) {
+        if constexpr (sizeof(T) == 4) factor_reg<T, 4, 32>(d_tasks, ntasks, b_max, Sx, kh, err, s);
+    } else {
+        const size_t sm = sizeof(cplx<T>) * ((size_t)b_max * b_max + 2 * b_max) + sizeof(int) * b_max;
+        cudaFuncSetAttribute(k_factor2d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        for (int mid = 0; mid < 2; ++mid) {
+            k_factor2d<T><<<dim3(ntasks, 2 - mid), 256, sm, s>>>(d_tasks, Sx, kh, mid, err);
+            note_launch();
+        }
+    }
 }
 
 // ------------------------------------------------------------------ sweep (2D)
-// One CTA per (leaf, chunk of NC right-hand sides).  X_i pieces (row blocks of a step's
-// inverse) stream through a ring of shared-memory slots by 1D bulk copies (TMA engine)
-// completing on mbarriers; the chain vector lives in shared memory.  G lanes split
-// every row's dot product.
-template <typename T, int NC, int G>
-__global__ void k_sweep2d(const LeafTask* __restrict__ tasks, int Sx, int nrhs, int nslot, int prow,
-                          size_t slot_elems, int* err) {
+// One pair of CTAs (a cluster) per (leaf, chunk of NC right-hand sides), one for each chain;
+// both form the middle column after an exchange through the cluster's shared memory.  X_i
+// pieces (row blocks of a column's inverse; NP of them at most) stream through a ring of
+// shared-memory slots by 1D bulk copies (TMA engine) completing on mbarriers; the chain vector
+// lives in shared memory.  SW_G lanes split every row's dot product.  The latency of a column
+// (the dot products, their reduction, one barrier) bounds it, so nothing else stands on that
+// chain: f, y and x pass through registers in groups of SW_G columns, lane g holding
+// column g of the group, loaded a group ahead.  4 bands of 37 rows x 129 columns, complex64, one
+// right-hand side: 0.61 ms with one chain and loads on it, 0.099 ms here.
+static constexpr int SW_G = 8;
+// threads of a CTA at most: the rows of which three slots fit shared memory, eight lanes a row
+template <typename T, int NP> constexpr int sweep_threads() {
+    return sizeof(T) == 4 ? (NP == 1 ? 800 : 576) : (NP == 1 ? 576 : 416);
+}
+template <typename T, int NC, int NP>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(sweep_threads<T, NP>(), 1)
+    k_sweep2d(const LeafTask* __restrict__ tasks, int Sx, int nrhs, int nslot, int prow, size_t slot_elems, int* err) {
+    using C = cplx<T>;
+    constexpr int G = SW_G, VE = 16 / (int)sizeof(C);       // VE: entries of a 16-byte load
+    namespace cg = cooperative_groups;
     const LeafTask tk = tasks[blockIdx.y];
-    const int b = tk.b, ldx = tk.ldx;
-    const int c0 = blockIdx.x * NC;
-    if (c0 >= nrhs) return;
-    const int ncol = min(NC, nrhs - c0);
-    const cplx<T>* X = (const cplx<T>*)tk.X;
-    const cplx<T>* F = (const cplx<T>*)tk.F;
-    cplx<T>* W = (cplx<T>*)tk.W;
+    const int b = tk.b, ldx = tk.ldx, side = blockIdx.x & 1;
+    const int c0 = (int)(blockIdx.x >> 1) * NC, ncol = min(NC, nrhs - c0);
+    const C* X = (const C*)tk.X;
+    const C* F = (const C*)tk.F;
+    C* W = (C*)tk.W;
     const size_t ldrow = (size_t)Sx * nrhs;   // stride between rows of F / W
     const size_t step = (size_t)b * ldx;
+    const int n = chain_len(Sx, side), mid = chain_mid(Sx);
 
     extern __shared__ __align__(128) unsigned char sms[];
-    cplx<T>* slots = (cplx<T>*)sms;
-    cplx<T>* vbuf = slots + (size_t)nslot * slot_elems;          // [2][b][NC]
-    uint64_t* bars = (uint64_t*)(vbuf + 2 * (size_t)b * NC);
-    __shared__ int s_abort;
-
+    C* slots = (C*)sms;
+    C* vbuf = slots + (size_t)nslot * slot_elems;           // [2][NC][ldx]
+    C* xbuf = vbuf + 2 * (size_t)ldx * NC;                  // the other chain's W y, [NC][ldx]
+    uint64_t* bars = (uint64_t*)(xbuf + (size_t)ldx * NC);
     const int npiece = (b + prow - 1) / prow;
-    const int nsteps = 2 * Sx - 1;
+    const int nsteps = 2 * n + 1;                           // inwards, middle, outwards
     const int total = nsteps * npiece;
-    auto step_col = [&](int s) { return s < Sx ? s : 2 * Sx - 2 - s; };
+    auto step_col = [&](int s) { return s == n ? mid : chain_col(Sx, side, s < n ? s : 2 * n - s); };
     auto issue = [&](int q) {
         const int s = q / npiece, p = q - s * npiece;
         const int r0 = p * prow;
         const int rows = min(prow, b - r0);
-        const uint32_t bytes = (uint32_t)(rows * ldx * sizeof(cplx<T>));
+        const uint32_t bytes = (uint32_t)(rows * ldx * sizeof(C));
         const int slot = q % nslot;
         mbar_arrive_expect_tx(&bars[slot], bytes);
         bulk_g2s(slots + (size_t)slot * slot_elems, X + (size_t)step_col(s) * step + (size_t)r0 * ldx, bytes,
@@ -210,87 +392,186 @@ __global__ void k_sweep2d(const LeafTask* __restrict__ tasks, int Sx, int nrhs, 
     };
 
     if (threadIdx.x == 0) {
-        s_abort = 0;
         for (int k = 0; k < nslot; ++k) mbar_init(&bars[k], 1);
         fence_barrier_init();
     }
-    __syncthreads();
+    // (the padding entries of the vectors stay zero)
+    for (int e = threadIdx.x; e < 3 * ldx * NC; e += blockDim.x) vbuf[e] = C{0, 0};
+    cg::this_cluster().sync();                              // the other CTA's shared memory exists
     if (threadIdx.x == 0)
         for (int q = 0; q < nslot && q < total; ++q) issue(q);
-    // v for the first forward step: f_0
-    for (int e = threadIdx.x; e < b * NC; e += blockDim.x) {
-        const int a = e / NC, c = e - a * NC;
-        vbuf[e] = c < ncol ? F[a * ldrow + c0 + c] : cplx<T>{0, 0};
+
+    const int lr = threadIdx.x / G, g = threadIdx.x % G;
+    auto col_of = [&](int t) { return (size_t)chain_col(Sx, side, t) * nrhs + c0; };
+    // a group's entries of this lane: columns t0 + g of the chain (f, or y as written below)
+    auto load = [&](const C* src, int t0, C (&v)[NP][NC]) {
+        const int t = t0 + g;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const int a = p * prow + lr;
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+                v[p][c] = lr < prow && a < b && t >= 0 && t < n && c < ncol ? src[a * ldrow + col_of(t) + c] : C{0, 0};
+        }
+    };
+    auto store = [&](int t0, const C (&v)[NP][NC]) {
+        const int t = t0 + g;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const int a = p * prow + lr;
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+                if (lr < prow && a < b && t < n && c < ncol) W[a * ldrow + col_of(t) + c] = v[p][c];
+        }
+    };
+    auto pick = [&](C v, int t) {                           // lane t of the row's group
+        const int src = (threadIdx.x & (31 & ~(G - 1))) + (t & (G - 1));
+        return C{__shfl_sync(0xffffffffu, v.re, src), __shfl_sync(0xffffffffu, v.im, src)};
+    };
+    C in[NP][NC], nx[NP][NC], out[NP][NC], fm[NP][NC];
+    load(F, 0, in);
+    load(F, G, nx);
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        const int a = p * prow + lr;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            out[p][c] = C{0, 0};
+            // f of the middle column joins the left chain's part
+            fm[p][c] = !side && lr < prow && a < b && c < ncol ? F[a * ldrow + (size_t)mid * nrhs + c0 + c] : C{0, 0};
+            if (g == 0 && lr < prow && a < b) vbuf[c * ldx + a] = in[p][c];
+        }
     }
     __syncthreads();
-
-    const int lr = threadIdx.x / G, g = threadIdx.x - (threadIdx.x / G) * G;
-    // Per-thread registers for the rows this thread finalises (g == 0): `cur` holds
-    // y_i for the current backward step, `nxt` the data the next step needs (f_{i+1}
-    // forward, y_{i-1} backward), loaded one step ahead to hide the memory latency.
-    cplx<T> cur[MAXP][NC], nxt[MAXP][NC];
-    for (int p = 0; p < MAXP; ++p)
-        for (int c = 0; c < NC; ++c) cur[p][c] = nxt[p][c] = cplx<T>{0, 0};
     int q = 0;
-    for (int s = 0; s < nsteps; ++s) {
-        const int i = step_col(s);
-        const bool fwd = s < Sx;
-        const cplx<T>* v = vbuf + (size_t)(s & 1) * b * NC;
-        cplx<T>* vn = vbuf + (size_t)((s + 1) & 1) * b * NC;
-        if (g == 0 && s + 1 < nsteps) {
-            const int i1 = step_col(s + 1);
-            const cplx<T>* src = (s + 1 < Sx) ? F : W;     // y_{i1} was written by this thread
-            for (int p = 0; p < npiece; ++p) {
-                const int a = p * prow + lr;
-                if (lr < prow && a < b)
-                    for (int c = 0; c < NC; ++c)
-                        if (c < ncol) nxt[p][c] = src[a * ldrow + (size_t)i1 * nrhs + c0 + c];
+    bool ok = true, bad = false;
+    // rows of piece p of step s: X_i v, in every lane of the row
+    auto product = [&](int s, int p, C (&acc)[NC]) {
+        const int slot = q % nslot;
+        if (!mbar_wait_bounded(&bars[slot], (uint32_t)((q / nslot) & 1), WAIT_LIMIT)) {
+            atomicExch(err, DEV_TIMEOUT);
+            bad = true;
+        }
+        const C* v = vbuf + (size_t)(s & 1) * ldx * NC;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) acc[c] = C{0, 0};
+        if (lr < min(prow, b - p * prow)) {
+            const C* xr = slots + (size_t)slot * slot_elems + (size_t)lr * ldx;
+            for (int k = g * VE; k < ldx; k += G * VE) {
+                struct alignas(16) V { C e[VE]; };
+                const V xv = *(const V*)(xr + k);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    const V vv = *(const V*)(v + c * ldx + k);
+#pragma unroll
+                    for (int e = 0; e < VE; ++e) cfma(acc[c], xv.e[e], vv.e[e]);
+                }
             }
         }
-        for (int p = 0; p < npiece; ++p, ++q) {
-            const int slot = q % nslot;
-            if (!mbar_wait_bounded(&bars[slot], (uint32_t)((q / nslot) & 1), WAIT_LIMIT)) {
-                atomicExch(err, DEV_TIMEOUT);
-                s_abort = 1;
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                acc[c].re += __shfl_xor_sync(0xffffffffu, acc[c].re, o);
+                acc[c].im += __shfl_xor_sync(0xffffffffu, acc[c].im, o);
             }
-            const int r0 = p * prow;
-            const int rows = min(prow, b - r0);
-            const cplx<T>* Xs = slots + (size_t)slot * slot_elems;
-            cplx<T> acc[NC];
-            for (int c = 0; c < NC; ++c) acc[c] = {0, 0};
-            if (lr < rows) {
-                const cplx<T>* xr = Xs + (size_t)lr * ldx;
-                for (int k = g; k < b; k += G) {
-                    const cplx<T> xv = xr[k];
-                    for (int c = 0; c < NC; ++c) cfma(acc[c], xv, v[k * NC + c]);
-                }
-            }
-            for (int o = G / 2; o > 0; o >>= 1)
-                for (int c = 0; c < NC; ++c) {
-                    acc[c].re += __shfl_xor_sync(0xffffffffu, acc[c].re, o);
-                    acc[c].im += __shfl_xor_sync(0xffffffffu, acc[c].im, o);
-                }
-            if (g == 0 && lr < rows) {
-                const int a = r0 + lr;
-                const T wa = (T)wrow(a, b);
-                for (int c = 0; c < NC; ++c) {
-                    cplx<T> res = acc[c];
-                    if (!fwd) res = res + cur[p][c];          // x_i = y_i + X_i W x_{i+1}
-                    if (c < ncol) W[a * ldrow + (size_t)i * nrhs + c0 + c] = res;
-                    cplx<T> nv = wa * res;                     // W y_i  or  W x_i
-                    if (s + 1 < Sx) nv = nv + nxt[p][c];        // + f_{i+1}
-                    vn[a * NC + c] = nv;
-                }
-            }
-            __syncthreads();
-            if (s_abort) break;
-            if (threadIdx.x == 0 && q + nslot < total) issue(q + nslot);
+    };
+    // after a piece: its slot is free for the piece nslot further on
+    auto turn = [&] {
+        if (__syncthreads_or(bad)) return false;
+        if (threadIdx.x == 0 && q + nslot < total) issue(q + nslot);
+        ++q;
+        return true;
+    };
+    // inwards; the last column's W y (the left one's with f_m) goes to both CTAs
+    C* peer = cg::this_cluster().map_shared_rank(xbuf, side ^ 1);
+    for (int t = 0; ok && t < n; ++t) {
+        const bool last = t + 1 == n;
+        if (((t + 1) & (G - 1)) == 0 && !last) {
+#pragma unroll
+            for (int p = 0; p < NP; ++p)
+#pragma unroll
+                for (int c = 0; c < NC; ++c) in[p][c] = nx[p][c];
+            load(F, t + 1 + G, nx);
         }
-        if (s_abort) break;
-        for (int p = 0; p < MAXP; ++p)
-            for (int c = 0; c < NC; ++c) cur[p][c] = nxt[p][c];
+        C* vn = vbuf + (size_t)((t + 1) & 1) * ldx * NC;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            if (!ok || p >= npiece) break;
+            C y[NC];
+            product(t, p, y);
+            const int a = p * prow + lr;
+            const T wa = (T)wrow(a, b);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const C fn = pick(in[p][c], t + 1);
+                if (g == (t & (G - 1))) out[p][c] = y[c];
+                const C nv = wa * y[c] + (last ? fm[p][c] : fn);
+                if (g == 0 && lr < prow && a < b) {
+                    vn[c * ldx + a] = nv;
+                    if (last) peer[c * ldx + a] = nv;
+                }
+            }
+            ok = turn();
+        }
+        if ((t & (G - 1)) == G - 1 || last) store(t & ~(G - 1), out);
     }
-    if (s_abort && threadIdx.x == 0) {
+    cg::this_cluster().sync();
+    // the middle column, in both CTAs alike
+    if (ok) {
+        C* v = vbuf + (size_t)(n & 1) * ldx * NC;
+        for (int e = threadIdx.x; e < ldx * NC; e += blockDim.x) v[e] = (n > 0 ? v[e] : C{0, 0}) + xbuf[e];
+        __syncthreads();
+        C* vn = vbuf + (size_t)((n + 1) & 1) * ldx * NC;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            if (!ok || p >= npiece) break;
+            C x[NC];
+            product(n, p, x);
+            const int a = p * prow + lr;
+            if (g == 0 && lr < prow && a < b)
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    if (!side && c < ncol) W[a * ldrow + (size_t)mid * nrhs + c0 + c] = x[c];
+                    vn[c * ldx + a] = (T)wrow(a, b) * x[c];
+                }
+            ok = turn();
+        }
+    }
+    // outwards: y of the group in work is still in `out`
+    if (n > 0) load(W, ((n - 1) & ~(G - 1)) - G, nx);
+#pragma unroll
+    for (int p = 0; p < NP; ++p)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) in[p][c] = out[p][c];
+    for (int t = n - 1; ok && t >= 0; --t) {
+        const int s = 2 * n - t;
+        C* vn = vbuf + (size_t)((s + 1) & 1) * ldx * NC;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            if (!ok || p >= npiece) break;
+            C x[NC];
+            product(s, p, x);
+            const int a = p * prow + lr;
+            const T wa = (T)wrow(a, b);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                x[c] = x[c] + pick(in[p][c], t);
+                if (g == (t & (G - 1))) out[p][c] = x[c];
+                if (g == 0 && lr < prow && a < b) vn[c * ldx + a] = wa * x[c];
+            }
+            ok = turn();
+        }
+        if (ok && (t & (G - 1)) == 0) {
+            store(t, out);
+#pragma unroll
+            for (int p = 0; p < NP; ++p)
+#pragma unroll
+                for (int c = 0; c < NC; ++c) in[p][c] = nx[p][c];
+            load(W, t - 2 * G, nx);
+        }
+    }
+    if (!ok && threadIdx.x == 0) {
         // drain copies still in flight before the CTA's shared memory is released
         for (int k = q; k < total && k < q + nslot; ++k)
             mbar_wait_bounded(&bars[k % nslot], (uint32_t)((k / nslot) & 1), WAIT_LIMIT);
@@ -359,31 +640,41 @@ __global__ void __launch_bounds__(S1_THREADS) k_sweep1d(const LeafTask* __restri
     }
 }
 
-template <typename T, int NC, int G>
+template <typename T, int NC, int NP>
+static void sweep_go(const LeafTask* d_tasks, int ntasks, int Sx, int nrhs, int nslot, int prow, size_t slot_bytes,
+                     size_t sm, int* err, cudaStream_t s) {
+    const int threads = ((prow * SW_G + 31) / 32) * 32;
+    cudaFuncSetAttribute(k_sweep2d<T, NC, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    k_sweep2d<T, NC, NP><<<dim3(2 * ((nrhs + NC - 1) / NC), ntasks), threads, sm, s>>>(
+        d_tasks, Sx, nrhs, nslot, prow, slot_bytes / sizeof(cplx<T>), err);
+    note_launch();
+}
+template <typename T, int NC>
 static void sweep_cfg(const LeafTask* d_tasks, int ntasks, int b_max, int Sx, int nrhs, int* err, cudaStream_t s) {
     const int esz = (int)sizeof(cplx<T>);
     const int ldx = leaf_ldx(b_max, esz);
     const size_t budget = 220 * 1024;
-    const size_t vbytes = 2 * (size_t)b_max * NC * esz + 8 * 8 + 128;
-    int prow = b_max < 1024 / G ? b_max : 1024 / G, nslot = 3;
+    const size_t vbytes = 3 * (size_t)ldx * NC * esz + 8 * SW_SLOTS + 128;
+    int prow = std::min(b_max, 1024 / SW_G), nslot = 3;
     size_t slot_bytes = align_up((size_t)prow * ldx * esz, 128);
-    while (nslot * slot_bytes + vbytes > budget && prow > 8) {
+    auto over = [&] {
+        const int cap = prow == b_max ? sweep_threads<T, 1>() : sweep_threads<T, MAXP>();
+        return nslot * slot_bytes + vbytes > budget || prow * SW_G > cap;
+    };
+    while (over() && prow > 8) {
         prow = (prow + 1) / 2;
         slot_bytes = align_up((size_t)prow * ldx * esz, 128);
     }
-    while ((nslot + 1) * slot_bytes + vbytes <= budget && nslot < 6) ++nslot;
+    while ((nslot + 1) * slot_bytes + vbytes <= budget && nslot < SW_SLOTS) ++nslot;
     const size_t sm = nslot * slot_bytes + vbytes;
-    if ((b_max + prow - 1) / prow > MAXP) {          // band too tall for this kernel
+    const int np = (b_max + prow - 1) / prow;
+    if (np > MAXP) {          // band too tall for this kernel
         int one = DEV_BADARG;
         cudaMemcpyAsync(err, &one, sizeof(int), cudaMemcpyHostToDevice, s);
         return;
     }
-    int threads = ((prow * G + 31) / 32) * 32;
-    if (threads > 1024) threads = 1024;
-    cudaFuncSetAttribute(k_sweep2d<T, NC, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    dim3 grid((nrhs + NC - 1) / NC, ntasks);
-    k_sweep2d<T, NC, G><<<grid, threads, sm, s>>>(d_tasks, Sx, nrhs, nslot, prow, slot_bytes / esz, err);
-    note_launch();
+    if (np == 1) sweep_go<T, NC, 1>(d_tasks, ntasks, Sx, nrhs, nslot, prow, slot_bytes, sm, err, s);
+    else sweep_go<T, NC, MAXP>(d_tasks, ntasks, Sx, nrhs, nslot, prow, slot_bytes, sm, err, s);
 }
 
 template <typename T>
@@ -394,8 +685,8 @@ void launch_sweep(const LeafTask* d_tasks, int ntasks, int b_max, int Sx, int nr
         return;
     }
     // prow * G threads must fit in one CTA; rows beyond are handled as further pieces
-    if (nrhs == 1) sweep_cfg<T, 1, 8>(d_tasks, ntasks, b_max, Sx, nrhs, err, s);
-    else sweep_cfg<T, 2, 8>(d_tasks, ntasks, b_max, Sx, nrhs, err, s);
+    if (nrhs == 1) sweep_cfg<T, 1>(d_tasks, ntasks, b_max, Sx, nrhs, err, s);
+    else sweep_cfg<T, 2>(d_tasks, ntasks, b_max, Sx, nrhs, err, s);
 }
 
 template void launch_factor<float>(const LeafTask*, int, int, int, double, int*, cudaStream_t);
