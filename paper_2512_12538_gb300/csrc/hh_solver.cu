@@ -969,18 +969,7 @@ struct Solver final : SolverBase {
         d_etasks_own = a.take<EigTask>(nleaf);
         d_etask_one = a.take<EigTask>(1);
         if (mk > 0 && cut) {
-            const size_t nG = cut_ng();
-            cg.V = a.take<c128>(nG * (mk + 1));
-            cg.alpha = a.take<c128>(mk + 1);
-            cg.v1 = a.take<c128>(nG);
-            cg.rG = a.take<c128>(nG);
-            cg.w = a.take<c128>(nG);
-            cg.y0 = a.take<CT>(cp.D);
-            cg.part = a.take<c128>((size_t)CUT_GM_BLOCKS * 72);
-            cg.dots = a.take<c128>(2 * 72);
-            cg.scale = a.take<c128>(1);
-            cg.npart = a.take<double>(CUT_GM_BLOCKS);
-            cp.scale = cg.scale;
+            plan_gmres(a);
         } else if (mk > 0) {
             Vb = a.take<c128>(N * (mk + 1));
             Zb = a.take<c128>(N * mk);
@@ -990,17 +979,7 @@ struct Solver final : SolverBase {
             gdots = a.take<c128>(4 * 80);
             gy = a.take<c128>(80);
         }
-        if (mk > 0) {
-            gls.mk = mk;
-            gls.H = a.take<c128>((size_t)(mk + 1) * mk);
-            gls.cs = a.take<double>(mk);
-            gls.sn = a.take<c128>(mk);
-            gls.g = a.take<c128>(mk + 1);
-            gls.st = a.take<GmresState>(1);
-            cg.ls = gls;
-            cg.red = sizeof(T) == sizeof(float) ? 1e-4 : 1e-12;
-            cg.tol = P.tol;
-        }
+        if (mk > 0 && !cut) plan_gmres_ls(a);
         d_ptrs = a.take<void*>(3 * 64);
         if (cut) {
             size_t ncp = 0, nep = 0;
@@ -1041,6 +1020,34 @@ struct Solver final : SolverBase {
             cut_part = (c128*)a.take<unsigned char>(cut_gram_scratch((int)cut_pairs_max));
         }
         return align_up(a.off, 256);
+    }
+
+    // GMRES on the cut rows: the Krylov space, the dot products and the least-squares state
+    void plan_gmres(Arena& a) {
+        const size_t nG = cut_ng();
+        cg.V = a.take<c128>(nG * (mk + 1));
+        cg.alpha = a.take<c128>(mk + 1);
+        cg.v1 = a.take<c128>(nG);
+        cg.rG = a.take<c128>(nG);
+        cg.w = a.take<c128>(nG);
+        cg.y0 = a.take<CT>(cp.D);
+        cg.part = a.take<c128>((size_t)CUT_GM_BLOCKS * 72);
+        cg.dots = a.take<c128>(2 * 72);
+        cg.scale = a.take<c128>(1);
+        cg.npart = a.take<double>(CUT_GM_BLOCKS);
+        cp.scale = cg.scale;
+        plan_gmres_ls(a);
+    }
+    void plan_gmres_ls(Arena& a) {
+        gls.mk = mk;
+        gls.H = a.take<c128>((size_t)(mk + 1) * mk);
+        gls.cs = a.take<double>(mk);
+        gls.sn = a.take<c128>(mk);
+        gls.g = a.take<c128>(mk + 1);
+        gls.st = a.take<GmresState>(1);
+        cg.ls = gls;
+        cg.red = sizeof(T) == sizeof(float) ? 1e-4 : 1e-12;
+        cg.tol = P.tol;
     }
 
     // ------------------------------------------------------------- small helpers
@@ -1681,9 +1688,9 @@ struct Solver final : SolverBase {
         h_pin = pinned_get();
         if (!h_pin) return HH_ENOMEM;
         h_norm = (double*)h_pin;
+        h_gst = (GmresState*)((char*)h_pin + 256 + 4 * 80 * sizeof(c128));
         if (mk > 0) {
             h_dots = (c128*)((char*)h_pin + 256);
-            h_gst = (GmresState*)((char*)h_pin + 256 + 4 * 80 * sizeof(c128));
             for (auto& e : gm_ev)
                 if (!e) ck(cudaEventCreateWithFlags(&e, cudaEventDisableTiming), cerr);
         }
@@ -2264,6 +2271,33 @@ struct Solver final : SolverBase {
         return st2;
     }
 
+    // The solve by GMRES(restart) of a handle set up for the stationary iteration on the cut
+    // rows: the set-up does not depend on the outer iteration, so only the Krylov space is
+    // allocated, for the call.  (A second handle for it took 2 to 4 ms per problem, its solve 1.)
+    hh_status solve_gmres(int restart, const c128* f, const c128* g, c128* uo, hh_stats* stt) {
+        mk = restart;
+        Arena size;
+        plan_gmres(size);
+        Arena a;
+        a.base = (char*)dev_alloc(size.off, stream, hook);
+        hh_status st = HH_ENOMEM;
+        if (a.base) {
+            plan_gmres(a);
+            ck(cudaMemcpyAsync(d_cut, &cp, sizeof(cp), cudaMemcpyHostToDevice, stream), cerr);
+            st = solve(f, g, uo, stt);
+        }
+        mk = 0;
+        cg = CutGmres{};
+        gls = GmresLs{};
+        cp.scale = nullptr;
+        if (a.base) {
+            ck(cudaMemcpyAsync(d_cut, &cp, sizeof(cp), cudaMemcpyHostToDevice, stream), cerr);
+            ck(cudaStreamSynchronize(stream), cerr);
+            dev_free(a.base, size.off, stream, hook);
+        }
+        return st;
+    }
+
     hh_status residual(const c128* f, const c128* g, const c128* uu, double* rel) override {
         launch_rhs(f, g, bvec, P.dim, S, h, stream, q1());
         norm_sq(bvec, dnorm + 2);
@@ -2753,10 +2787,8 @@ static hh_status batch_solve(std::vector<Solver<T>*>& ps, const c128* const* f, 
 
 // All handles in one precision and batchable: solve them together in lockstep.  Problems
 // the stationary iteration does not converge are then solved by flexible GMRES (the
-// paper's outer solver) on handles set up for it, several at a time from host threads.
+// paper's outer solver), several at a time from host threads.
 // Handles that cannot join the lockstep batch are solved one by one.
-static hh_status setup_one(const hh_params* p, cudaStream_t s, SolverBase** out, const AllocHook& hook);
-
 static hh_status solve_many(SolverBase* const* hs, const c128* const* f, const c128* const* g, c128* const* u, int n,
                             cudaStream_t stream, hh_stats* stats) {
     std::vector<Solver<float>*> pf;
@@ -2796,20 +2828,17 @@ static hh_status solve_many(SolverBase* const* hs, const c128* const* f, const c
         }
         for (size_t i = w; i < rescue.size(); i += nw) {
             const int k = rescue[i];
-            hh_params q = hs[k]->P;
-            q.outer = HH_OUTER_GMRES;
-            if (q.restart < 1 || q.restart > 64) q.restart = 40;
-            SolverBase* g2 = nullptr;
-            rs[i] = setup_one(&q, ws, &g2, g_alloc);
-            if (rs[i] != HH_OK) continue;
+            const int restart = hs[k]->P.restart < 1 || hs[k]->P.restart > 64 ? 40 : hs[k]->P.restart;
+            const cudaStream_t own = hs[k]->stream;
             hh_stats s2{};
-            rs[i] = g2->solve(f[k], g[k], u[k], &s2);
+            hs[k]->stream = ws;
+            if (!pf.empty()) rs[i] = pf[k]->solve_gmres(restart, f[k], g[k], u[k], &s2);
+            else rs[i] = pd[k]->solve_gmres(restart, f[k], g[k], u[k], &s2);
+            hs[k]->stream = own;
             if (stats) {
                 stats[k].iters += s2.iters;
                 stats[k].rel_res = s2.rel_res;
             }
-            cudaStreamSynchronize(ws);
-            delete g2;
         }
         cudaStreamSynchronize(ws);
         cudaStreamDestroy(ws);

@@ -103,3 +103,30 @@ def test_a_handle_solves_alone_after_a_batch(hh):
     finally:
         for h in hs:
             hh.hh_destroy(h)
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+def test_a_rescued_handle_is_left_as_it_was(hh, precision):
+    """GMRES on a stationary handle (a batch's diverging member, see test_gpu_batch.py)
+    borrows the handle's set-up: the handle answers the next batch alike, to the bit, and
+    as a handle set up for GMRES does, to the accuracy both solve to."""
+    n, k = 63, 0.57 * 64
+    S = n + 2
+    ps = [hh.make_params(2, n, kk, 2, 2, 16, 8, 1, 1e-10, 400, precision, 1) for kk in (k, 20.0)]
+    hs = hh.hh_setup_batch(ps)
+    try:
+        fs = [torch.from_numpy(random_complex((S, S), 25 + i)).cuda() for i in range(2)]
+        gs = [torch.zeros((4, S), dtype=torch.complex128, device="cuda")] * 2
+        got = []
+        for _ in range(2):
+            got.append([torch.empty_like(f) for f in fs])
+            hh.hh_solve_batch(hs, fs, gs, got[-1])
+        for a, b in zip(*got):
+            assert torch.equal(a, b)
+    finally:
+        for h in hs:
+            hh.hh_destroy(h)
+    s = hh.Solver(2, n, k, 2, 2, 16, 8, tol=1e-10, max_iter=400, precision=precision, seed=1, outer="gmres", restart=40)
+    u, st = s.solve(fs[0], gs[0])
+    s.close()
+    assert ((u - got[0][0]).norm() / u.norm()).item() < 1e-8
