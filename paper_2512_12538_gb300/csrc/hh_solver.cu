@@ -1744,11 +1744,21 @@ struct Solver final : SolverBase {
         step_gate = nullptr;
     }
 
-    hh_status norm_sq(const c128* x, double* dst) {
-        const size_t N = (size_t)Sy * Sx;
-        const int nb = launch_ip_partial<double, double>(x, 1, x, 1, N, 1, 1, partial, MAX_PART_BLOCKS, stream);
-        launch_ip_reduce(partial, nb, 1, 1, (c128*)dst, nullptr, nullptr, stream);
-        return HH_OK;
+    // b and |b|^2 (dnorm[2]); with `all` also u = 0 with its residual b (squared norm into *r2),
+    // and the status, stop and control words (dnorm[4..]) cleared
+    void start(const c128* f, const c128* g, double* r2, bool all) {
+        StartOut<T> o;
+        o.b2 = dnorm + 2;
+        if (all) {
+            o.u = u;
+            if (cut || mk == 0) o.rt = RT;
+            if (!cut && mk == 0) o.res = res;
+            o.r2 = r2;
+            o.ctl = (int*)(dnorm + 6);
+            o.clear = derr;
+            o.nclear = (int)(6 * sizeof(double) + sizeof(CutCtl)) / (int)sizeof(int);
+        }
+        launch_start<T>(f, g, bvec, o, P.dim, S, h, q1(), npart, dcounter, P.tol, stream);
     }
 
     // z = M v: one coarse-corrected ORAS step from zero (v, z distinct from res and ut)
@@ -1952,10 +1962,11 @@ struct Solver final : SolverBase {
         int* ctl = (int*)(dnorm + 6);
         const int* hctl = (const int*)(h_norm + 6);
         hh_status st = HH_OK;
-        zero(ctl, 8 * sizeof(int));
-        zero(dcounter, 2 * sizeof(unsigned));   // the residual's and the root's tickets
-        gated_residual(ctl);
-        if (!read_norms(st)) return st;
+        zero(dcounter + 1, sizeof(unsigned));   // the root's ticket
+        // the first residual and its test are the start's; the host sees them with the first chunk
+        h_norm[0] = h_norm[2] = 1.0;
+        ((int*)(h_norm + 6))[0] = 0;
+        ((int*)(h_norm + 6))[1] = 1;
         double rel_prev = -1.0;
         int it_prev = 0, chunks = 0;
         for (;;) {
@@ -2011,31 +2022,31 @@ struct Solver final : SolverBase {
         int* ctl = (int*)(dnorm + 6);
         const CutCtl* hc = (const CutCtl*)(h_norm + 10);
         hh_status st = HH_OK;
-        zero(ctl, 4 * sizeof(double) + sizeof(CutCtl));   // the residual's words and the steps'
-        zero(dcounter, 2 * sizeof(unsigned));
         auto resid = [&](const c128* x) {
             pbeg(PC_SPMV, 48.0 * (double)Sy * Sx);
-            // the steps' own residuals are counted, and the first
-            if (it > 0 && prof_cat(PC_SPMV)) prof_pending.back().nl = 0;
+            // the steps' own residuals are counted, and the first (the start's)
+            if (prof_cat(PC_SPMV)) prof_pending.back().nl = 0;
             launch_residual_stop<T>(x, bvec, nullptr, RT, geom(0), npart, dnorm, ctl, dcounter, P.tol, stream);
             pend(PC_SPMV);
         };
-        resid(u);
         int mode = 1;
-        bool cand = false;   // a candidate stands in ut
-        for (;;) {
-            if (!read_norms(st)) return st;
-            it = hc->it;
-            rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;
-            if (cand && (!std::isfinite(rel) || rel < P.tol || it >= P.max_iter || hc->reason != CUT_TEST)) {
-                cut_swap();
-                mode = 1;
-            } else if (cand) {
-                mode = 2;
+        // the first round is queued without a look at b's norm
+        for (bool first = true;; first = false) {
+            if (!first) {
+                if (!read_norms(st)) return st;
+                if (start_settles(it, rel, st)) return st;
+                it = hc->it;
+                rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;
+                if (!std::isfinite(rel) || rel < P.tol || it >= P.max_iter || hc->reason != CUT_TEST) {
+                    cut_swap();   // the candidate stands in ut
+                    mode = 1;
+                } else {
+                    mode = 2;
+                }
+                if (!std::isfinite(rel)) return HH_ENOCONV;
+                if (rel < P.tol) return HH_OK;
+                if (it >= P.max_iter) return HH_ENOCONV;
             }
-            if (!std::isfinite(rel)) return HH_ENOCONV;
-            if (rel < P.tol) return HH_OK;
-            if (it >= P.max_iter) return HH_ENOCONV;
             const int nl = (int)lev[L].size();
             if (mode == 1) eig_stage_prof(0, d_etasks_cin);
             if (!launch_cut_steps<T>(d_cut, 1, cut_group(), cp.cl, cut_smem, nullptr, mode, cbar, 1, derr, prof_on, stream))
@@ -2043,10 +2054,18 @@ struct Solver final : SolverBase {
             launch_cut_lines<T>(d_cut, 1, nullptr, nl, b_max, Sx, stream);
             eig_stage_prof(2, d_etasks_cout);
             launch_cut_update<T>(d_upd + cut_flip, 1, Sy, Sx, stream);
-            it = 1;   // residual launches from here on belong to steps already counted
             resid(ut);
-            cand = true;
         }
+    }
+    // After the first read of the norms: whether the first residual, b itself (u = 0), ends the
+    // solve (b = 0, a tolerance above 1, b not finite).
+    bool start_settles(int& it, double& rel, hh_status& st) const {
+        const double r0 = h_norm[2] > 0 ? std::sqrt(h_norm[2] / h_norm[2]) : 0.0;
+        if (std::isfinite(r0) && !(r0 < P.tol)) return false;
+        it = 0;
+        rel = r0;
+        st = std::isfinite(r0) ? HH_OK : HH_ENOCONV;
+        return true;
     }
     int cut_flip = 0;   // which of the two update jobs has the current u as its source
     void cut_swap() {
@@ -2067,7 +2086,6 @@ struct Solver final : SolverBase {
         hh_status st = HH_OK;
         auto resid = [&]() {
             zero(ctl, 4 * sizeof(double) + sizeof(CutCtl));
-            zero(dcounter, 2 * sizeof(unsigned));
             pbeg(PC_SPMV, 48.0 * (double)Sy * Sx);
             launch_residual_stop<T>(u, bvec, nullptr, RT, geom(0), npart, dnorm, ctl, dcounter, P.tol, stream);
             pend(PC_SPMV);
@@ -2076,17 +2094,20 @@ struct Solver final : SolverBase {
             return launch_cut_steps<T>(d_cut, 1, cut_group(), cp.cl, cut_smem, nullptr, mode, cbar, 1, derr, 0, stream,
                                        max_steps, &cg, gm_steps);
         };
-        resid();
         for (bool cycle = false;; cycle = true) {
-            if (!read_norms(st)) return st;
             if (cycle) {
+                if (!read_norms(st)) return st;
+                if (start_settles(it, rel, st)) {
+                    zero(u, sizeof(c128) * (size_t)Sy * Sx);
+                    return st;
+                }
                 if (h_gst[0].bad) return HH_ENOCONV;
                 it += h_gst[0].stop ? h_gst[0].jstop : h_gst[0].steps;
+                rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;
+                if (!std::isfinite(rel)) return HH_ENOCONV;
+                if (rel < P.tol) return HH_OK;
+                if (it >= P.max_iter) return HH_ENOCONV;
             }
-            rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;
-            if (!std::isfinite(rel)) return HH_ENOCONV;
-            if (rel < P.tol) return HH_OK;
-            if (it >= P.max_iter) return HH_ENOCONV;
             eig_stage_prof(0, d_etasks_cin);
             if (!steps(1, 0, std::min(mk, P.max_iter - it))) return HH_ECUDA;
             ck(cudaMemcpyAsync(&h_gst[0], gls.st, sizeof(GmresState), cudaMemcpyDeviceToHost, stream), cerr);
@@ -2145,11 +2166,17 @@ struct Solver final : SolverBase {
         if (device_test_path()) return loop_oras_device_test(it, rel);
         hh_status st = HH_OK;
         for (;;) {
-            if (!true_residual(res, st, RT)) return st;
-            rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;
-            if (!std::isfinite(rel)) return HH_ENOCONV;
-            if (rel < P.tol) return HH_OK;
-            if (it >= P.max_iter) return HH_ENOCONV;
+            if (it > 0) {   // (the first residual is the start's)
+                if (!true_residual(res, st, RT)) return st;
+                if (start_settles(it, rel, st)) {
+                    zero(u, sizeof(c128) * (size_t)Sy * Sx);
+                    return st;
+                }
+                rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;
+                if (!std::isfinite(rel)) return HH_ENOCONV;
+                if (rel < P.tol) return HH_OK;
+                if (it >= P.max_iter) return HH_ENOCONV;
+            }
             via_graph(1, [&] { oras_step(u, bvec, u, true); });
             ++it;
         }
@@ -2237,14 +2264,15 @@ struct Solver final : SolverBase {
 
     hh_status solve(const c128* f, const c128* g, c128* uo, hh_stats* stt) override {
         const size_t N = (size_t)Sy * Sx;
-        zero(derr, sizeof(int) * 4);
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
         cudaEventRecord(e0, stream);
-        launch_rhs(f, g, bvec, P.dim, S, h, stream, q1());
-        norm_sq(bvec, dnorm + 2);   // dnorm[2..3] = ||b||^2 as a complex
-        zero(u, sizeof(c128) * N);
+        // (GMRES on the whole grid forms its first residual itself)
+        const bool first = cut || mk == 0;
+        if (first) pbeg(PC_SPMV, 48.0 * (double)Sy * Sx);
+        start(f, g, dnorm, true);
+        if (first) pend(PC_SPMV);
         int it = 0;
         double rel = 0.0;
         // (each loop reads the norms with its first residual and the status words with every one)
@@ -2299,8 +2327,7 @@ struct Solver final : SolverBase {
     }
 
     hh_status residual(const c128* f, const c128* g, const c128* uu, double* rel) override {
-        launch_rhs(f, g, bvec, P.dim, S, h, stream, q1());
-        norm_sq(bvec, dnorm + 2);
+        start(f, g, nullptr, false);
         int nb = 0;
         launch_apply<double, double, double>(uu, bvec, res, geom(0), 1, 1.0, npart, &nb, stream);
         launch_sum(npart, nb, dnorm, stream);
@@ -2489,7 +2516,8 @@ struct BatchEngine {
         c128* uo = nullptr;          // where the solution goes when the problem leaves
         void* tag = nullptr;
         int slot = 0, it = 0;
-        int mode = 0;                // of the next round; 0: its first residual is due
+        int mode = 1;                // of the next round
+        bool first = true;           // no round yet: u = 0, its residual is b
         double rel = 0.0;
         hh_status st = HH_OK;
     };
@@ -2578,10 +2606,8 @@ struct BatchEngine {
         q.tag = tag;
         while (used[q.slot]) ++q.slot;
         used[q.slot] = 1;
-        launch_rhs(f, g, p->bvec, p->P.dim, p->S, p->h, stream, p->q1());
-        p->norm_sq(p->bvec, p->dnorm + 2);
+        p->start(f, g, norms + q.slot, true);
         ck(cudaMemcpyAsync(p->h_norm + 2, p->dnorm + 2, sizeof(double), cudaMemcpyDeviceToHost, stream), cerr);
-        p->zero(p->u, sizeof(c128) * (size_t)p->Sy * p->Sx);
         CutProb* hp = (CutProb*)(h_up + up_bytes) + q.slot;   // read by the copy before the slot's next use
         *hp = p->cp;
         hp->nrm = norms + q.slot;
@@ -2592,13 +2618,12 @@ struct BatchEngine {
         ck(cudaMemsetAsync(d_ctl + q.slot, 0, sizeof(CutCtl), stream), cerr);
         act.push_back(q);
     }
-    // FP64 residuals of the problems sel (their u, or ut): norms[slot]
-    template <class Sel, class X> void residuals(Sel sel, X x) {
+    // FP64 residuals of the candidates (ut): norms[slot]
+    void residuals() {
         ResidBatch rb{};
         for (auto& q : act) {
-            if (!sel(q)) continue;
             ResidJob& j = rb.job[rb.njobs++];
-            j.x = x(q);
+            j.x = q.p->ut;
             j.v = q.p->bvec;
             j.yt = q.p->RT;
             j.g = q.p->geom(0);
@@ -2640,22 +2665,6 @@ struct BatchEngine {
     // (their solution already copied to uo, the copy complete).
     hh_status step(std::vector<Prob>& done) {
         if (act.empty()) return HH_OK;
-        bool fresh = false;
-        for (auto& q : act) fresh |= q.mode == 0;
-        if (fresh) {
-            residuals([](const Prob& q) { return q.mode == 0; }, [](const Prob& q) { return q.p->u; });
-            const hh_status st = read_back();
-            if (st != HH_OK) return st;
-            for (auto& q : act) {
-                if (q.mode) continue;
-                q.mode = 1;
-                q.rel = rel_of(q);
-                if (!std::isfinite(q.rel)) leave(q, HH_ENOCONV, q.p->u, done);
-                else if (q.rel < q.p->P.tol) leave(q, HH_OK, q.p->u, done);
-            }
-            settle();
-            if (act.empty()) return cerr == cudaSuccess ? HH_OK : HH_ECUDA;
-        }
         // the round's tables
         int* modes = (int*)h_up;
         CutUpdJob* jobs = (CutUpdJob*)(h_up + ((char*)d_jobs - (char*)d_modes));
@@ -2712,11 +2721,18 @@ struct BatchEngine {
         if (ngr) launch_cut_lines<T>(d_probs, top, d_modes + cap_probs, nleaf, bm, sx, stream);
         transforms(2);
         launch_cut_update<T>(d_jobs, nj, sx, sx, stream);
-        residuals([](const Prob&) { return true; }, [](const Prob& q) { return q.p->ut; });
+        residuals();
         const hh_status st = read_back();
         if (st != HH_OK) return st;
         for (auto& q : act) {
             const CutCtl& c = ctl_of(q);
+            const bool first = q.first;
+            q.first = false;
+            hh_status st0;
+            if (first && q.p->start_settles(q.it, q.rel, st0)) {
+                leave(q, st0, q.p->u, done);
+                continue;
+            }
             q.it = c.it;
             q.rel = rel_of(q);
             if (!std::isfinite(q.rel)) leave(q, HH_ENOCONV, q.p->ut, done);

@@ -355,36 +355,89 @@ __device__ c128 rhs_q1(const c128* __restrict__ f, const c128* __restrict__ g, i
     }
     return v;
 }
-__global__ void k_rhs(const c128* __restrict__ f, const c128* __restrict__ g, c128* __restrict__ b,
-                      int dim, int S, double h, int q1) {
+// The start of a solve: b, u = 0, and with u = 0 the first residual, which is b itself (rt in
+// the leaf precision, res in FP64, each if not null), its norm |b|^2 and the stopping test on
+// it, one launch.  Each block leaves a partial, the last block adds them in a fixed
+// order and clears the status and control words.  Bound by DRAM (64 B a point in the mixed
+// form); as a fill, a right-hand side, a dot product in two launches and a residual it took
+// 0.55 ms at 1023^2, 50 us at 255^2.
+template <typename T>
+__global__ void __launch_bounds__(256) k_start(const c128* __restrict__ f, const c128* __restrict__ g,
+                                               c128* __restrict__ b, StartOut<T> o, int dim, int S, double h, int q1,
+                                               double* part, unsigned* ticket, double tol) {
     const int Sx = dim == 2 ? S : 1;
     const size_t total = (size_t)S * Sx;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
-         t += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(t % Sx), j = (int)(t / Sx);
+    double acc = 0.0;
+    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
+        const int j = (int)(t / Sx), i = (int)(t - (size_t)j * Sx);
+        c128 v;
         if (q1) {
-            b[t] = rhs_q1(f, g, S, h, j, i);
-            continue;
-        }
-        const double wj = wrow(j, S), wi = wcol(i, Sx);
-        c128 v = (h * h * wi * wj) * f[t];
-        if (dim == 1) {
-            if (j == 0) v = v + h * g[0];
-            if (j == S - 1) v = v + h * g[1];
+            v = rhs_q1(f, g, S, h, j, i);
         } else {
-            if (i == 0) v = v + (h * wj) * g[0 * S + j];
-            if (i == Sx - 1) v = v + (h * wj) * g[1 * S + j];
-            if (j == 0) v = v + (h * wi) * g[2 * S + i];
-            if (j == S - 1) v = v + (h * wi) * g[3 * S + i];
+            const double wj = wrow(j, S), wi = wcol(i, Sx);
+            v = (h * h * wi * wj) * f[t];
+            if (dim == 1) {
+                if (j == 0) v = v + h * g[0];
+                if (j == S - 1) v = v + h * g[1];
+            } else {
+                if (i == 0) v = v + (h * wj) * g[0 * S + j];
+                if (i == Sx - 1) v = v + (h * wj) * g[1 * S + j];
+                if (j == 0) v = v + (h * wi) * g[2 * S + i];
+                if (j == S - 1) v = v + (h * wi) * g[3 * S + i];
+            }
         }
         b[t] = v;
+        if (o.u) o.u[t] = c128{0.0, 0.0};
+        if (o.rt) o.rt[t] = cvt<T>(v);
+        if (o.res) o.res[t] = v;
+        acc = fma(v.re, v.re, acc);
+        acc = fma(v.im, v.im, acc);
+    }
+    __shared__ double red[8];
+    __shared__ unsigned s_last;
+    acc = warp_sum(acc);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double s2 = 0.0;
+        for (int w = 0; w < 8; ++w) s2 += red[w];
+        part[blockIdx.x] = s2;
+        __threadfence();
+        s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    double a = 0.0;
+    for (unsigned i = threadIdx.x; i < gridDim.x; i += 256) a += __ldcg(part + i);
+    a = warp_sum(a);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = a;
+    for (int i = threadIdx.x; i < o.nclear; i += 256) o.clear[i] = 0;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double s2 = 0.0;
+        for (int w = 0; w < 8; ++w) s2 += red[w];
+        *ticket = 0u;
+        *o.b2 = s2;
+        if (o.r2) *o.r2 = s2;
+        if (o.ctl) {   // [0] stop, [1] tests run: as after a residual (ResidStop)
+            const double rel = s2 > 0 ? sqrt(s2 / s2) : 0.0;
+            o.ctl[0] = !isfinite(rel) ? 2 : rel < tol ? 1 : 0;
+            o.ctl[1] = 1;
+        }
     }
 }
-void launch_rhs(const c128* f, const c128* g, c128* b, int dim, int S, double h, cudaStream_t s, int q1) {
+template <typename T>
+void launch_start(const c128* f, const c128* g, c128* b, const StartOut<T>& o, int dim, int S, double h, int q1,
+                  double* part, unsigned* ticket, double tol, cudaStream_t s) {
     const size_t total = (size_t)S * (dim == 2 ? S : 1);
-    k_rhs<<<grid_for(total, 256), 256, 0, s>>>(f, g, b, dim, S, h, q1);
+    k_start<T><<<grid_for(total, 256, 152 * 4), 256, 0, s>>>(f, g, b, o, dim, S, h, q1, part, ticket, tol);
     note_launch();
 }
+template void launch_start<float>(const c128*, const c128*, c128*, const StartOut<float>&, int, int, double, int, double*,
+                                  unsigned*, double, cudaStream_t);
+template void launch_start<double>(const c128*, const c128*, c128*, const StartOut<double>&, int, int, double, int,
+                                   double*, unsigned*, double, cudaStream_t);
 
 // -------------------------------------------------------------------------- copy
 template <typename TS, typename TD>

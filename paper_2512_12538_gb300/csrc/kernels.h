@@ -54,7 +54,21 @@ void launch_residual_stop(const c128* x, const c128* v, c128* y, cplx<T>* yt, Op
 
 // b = h^2 w_i w_j f + h (w_j gx + w_i gy) for the global problem (q1: the bilinear
 // elements' load vector, h^2 M_y F M_x^T + h (edge masses) g).
-void launch_rhs(const c128* f, const c128* g, c128* b, int dim, int S, double h, cudaStream_t s, int q1 = 0);
+// the right-hand side b with |b|^2 into *b2, and as wanted (not null) u = 0, the residual b in the
+// leaf precision and in FP64, its squared norm, the stop words; nclear ints from clear are zeroed;
+// part: a double a block (608 at most), ticket: zero between launches
+template <typename T> struct StartOut {
+    c128* u = nullptr;
+    cplx<T>* rt = nullptr;
+    c128* res = nullptr;
+    double *b2 = nullptr, *r2 = nullptr;
+    int* ctl = nullptr;
+    int* clear = nullptr;
+    int nclear = 0;
+};
+template <typename T>
+void launch_start(const c128* f, const c128* g, c128* b, const StartOut<T>& o, int dim, int S, double h, int q1,
+                  double* part, unsigned* ticket, double tol, cudaStream_t s);
 
 // dst[i] (+)= (TD) src[i], i < n
 template <typename TS, typename TD>
