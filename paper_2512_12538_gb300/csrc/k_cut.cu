@@ -1054,23 +1054,6 @@ HH_HD CcSmem cc_layout(const CutProb& P) {
     s.total = o;
     return s;
 }
-__device__ __forceinline__ uint32_t mapa(uint32_t a, int rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    return r;
-}
-// 8 or 4 bytes into another block's shared memory, counted on that block's mbarrier
-__device__ __forceinline__ void st_async(uint32_t dst, c64 v, uint32_t mbar) {
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(dst),
-                 "f"(v.re), "f"(v.im), "r"(mbar)
-                 : "memory");
-}
-__device__ __forceinline__ void st_async(uint32_t dst, float v, uint32_t mbar) {
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(dst), "f"(v),
-                 "r"(mbar)
-                 : "memory");
-}
-
 // GM: with the Arnoldi steps of a GMRES cycle (apart, for its registers).
 template <bool GM>
 __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restrict__ probs, int nprob,

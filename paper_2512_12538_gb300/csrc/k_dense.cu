@@ -1670,132 +1670,161 @@ __global__ void __launch_bounds__(256) k_gj_inverse(GjBatch bt) {
         if (AT) AT[e] = cvt<float>(v);
     }
 }
-// The same elimination on a cluster of GJ_CL CTAs per matrix, each holding a slice of the
-// rows: per step every CTA proposes its best pivot row (cluster barrier), all take the
-// same pivot from the proposals (largest magnitude, then lowest row), read the pivot row
-// (and the owner of the pivot row, the old row k) from distributed shared memory, and
-// after a second barrier update their own rows.  The FP64 updates of a step spread over
-// GJ_CL SMs (FP64 issues at 2 multiply-adds per SM and clock on this GPU).
-static constexpr int GJ_CL = 8;
-template <typename R>
-__global__ void __launch_bounds__(256) k_gj_cluster(GjBatch bt) {
+// The same elimination on a cluster of CL CTAs per matrix, one warp a column (column c in warp
+// c / CL of CTA c % CL, rows lane and lane + 32 in registers), and no barrier in its steps: the
+// warp that owns column k picks the pivot among the rows that have not been one (by the
+// larger of |re|, |im|, compared as the high words' bits), and sends the column, the pivot row
+// and the pivot's reciprocal to every CTA's place for column k, counted by an mbarrier there;
+// every warp then updates its column, the next column's owner first of all what it needs to
+// send.  Rows stay in place: column k of the tableau ends as the inverse's column p_k, row
+// p_k as its row k.  The chain of pivots bounds it, and in it the FP64 issue rate (32 lanes'
+// multiply-add takes a scheduler 64 clocks): 16 CTAs, so that a warp has a scheduler to
+// itself.  With rows spread over 8 CTAs and two cluster barriers a pivot, 2r = 64 took 0.36 ms
+// and 2r = 36 0.12 ms; here 0.12 and 0.05.
+template <typename R> __device__ __forceinline__ unsigned gj_key(cplx<R> a) {
+    if constexpr (sizeof(R) == 8) {
+        const unsigned x = __double2hiint(a.re) & 0x7fffffffu, y = __double2hiint(a.im) & 0x7fffffffu;
+        return max(x, y) + 1u;
+    } else {
+        const unsigned x = __float_as_uint(a.re) & 0x7fffffffu, y = __float_as_uint(a.im) & 0x7fffffffu;
+        return max(x, y) + 1u;
+    }
+}
+static constexpr uint32_t GJ_WAIT = 1u << 21;   // bounded polls (~0.1 s)
+template <typename R, int CL>
+__global__ void __launch_bounds__(64 / CL * 32) k_gj_cluster(GjBatch bt) {
     namespace cg = cooperative_groups;
     using C = cplx<R>;
-    cg::cluster_group cluster = cg::this_cluster();
-    const int rank = (int)cluster.block_rank();
-    const int mat = blockIdx.x / GJ_CL;
-    c128* A = bt.A[mat];
-    const int n = bt.n;
-    const int rpc = (n + GJ_CL - 1) / GJ_CL;
-    const int r0 = min(n, rank * rpc), r1 = min(n, r0 + rpc), nr = r1 - r0;
     extern __shared__ __align__(16) unsigned char gjc[];
-    C* M = (C*)gjc;                 // [rpc][n] own rows
-    C* row = M + rpc * n;           // [n] the normalised pivot row
-    C* tmp = row + n;               // [n] the old row k (the pivot row's owner)
-    C* colk = tmp + n;              // [rpc] column k of the own rows, before the step
-    int* perm = (int*)(colk + rpc); // [n]
-    int* pos = perm + n;            // [n]
-    __shared__ R s_best;
-    __shared__ int s_idx, s_p;
-    __shared__ C s_ip, s_akk;
-    for (int e = threadIdx.x; e < nr * n; e += blockDim.x) M[e] = cvt<R>(A[(size_t)r0 * n + e]);
-    __syncthreads();
-    for (int k = 0; k < n; ++k) {
-        if (threadIdx.x == 0) {
-            R best = -1;
-            int bi = n;
-            for (int r = max(k, r0); r < r1; ++r) {
-                const R a = abs2(M[(r - r0) * n + k]);
-                if (a > best) { best = a; bi = r; }
-            }
-            s_best = best;
-            s_idx = bi;
-        }
-        cluster.sync();
-        if (threadIdx.x == 0) {
-            R best = -1;
-            int bi = n;
-            for (int q = 0; q < GJ_CL; ++q) {
-                const R ob = *cluster.map_shared_rank(&s_best, q);
-                const int oi = *cluster.map_shared_rank(&s_idx, q);
-                if (oi < n && (ob > best || (ob == best && oi < bi))) { best = ob; bi = oi; }
-            }
-            s_p = bi < n ? bi : k;
-            perm[k] = s_p;
-            const int ok_ = (bi < n) && (best > 0) && isfinite(best);
-            if (!ok_ && rank == 0) atomicExch(bt.err, DEV_BREAKDOWN);
-            const int ob = s_p / rpc, ok2 = k / rpc;
-            const C pk = ok_ ? cluster.map_shared_rank(M, ob)[(s_p - ob * rpc) * n + k] : C{1, 0};
-            s_ip = cinv(pk);
-            s_akk = cluster.map_shared_rank(M, ok2)[(k - ok2 * rpc) * n + k];
-        }
-        __syncthreads();
-        const int p = s_p;
-        const C ip = s_ip;
-        {
-            const int ob = p / rpc, okk = k / rpc;
-            const C* prow = cluster.map_shared_rank(M, ob) + (size_t)(p - ob * rpc) * n;
-            for (int c = threadIdx.x; c < n; c += blockDim.x) row[c] = prow[c] * ip;
-            if (p != k && p >= r0 && p < r1) {
-                const C* krow = cluster.map_shared_rank(M, okk) + (size_t)(k - okk * rpc) * n;
-                for (int c = threadIdx.x; c < n; c += blockDim.x) tmp[c] = krow[c];
-            }
-            for (int rl = threadIdx.x; rl < nr; rl += blockDim.x) colk[rl] = M[rl * n + k];
-        }
-        cluster.sync();   // every read of another CTA's rows is done before the updates
-        const C akk = s_akk;
-        for (int e = threadIdx.x; e < nr * n; e += blockDim.x) {
-            const int rl = e / n, c = e - rl * n, r = r0 + rl;
-            C v;
-            if (r == k) {
-                v = (c == k) ? ip : row[c];
-            } else {
-                const C f = (r == p) ? akk : colk[rl];
-                const C cur = (r == p) ? tmp[c] : M[e];
-                v = (c == k) ? -(f * ip) : cur - f * row[c];
-            }
-            M[e] = v;
-        }
-        __syncthreads();
+    __shared__ C s_ip[64];
+    __shared__ int s_p[64];
+    __shared__ __align__(8) uint64_t s_mb[64];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int mat = blockIdx.x / CL, n = bt.n, c = rank + CL * warp;
+    c128* A = bt.A[mat];
+    C* col = (C*)gjc;               // [n][n]: column k as its owner sent it
+    C m[2];
+    unsigned used = 0;              // this lane's rows that have been pivots, and for which column
+    int kk[2] = {0, 0};
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const int r = lane + 32 * s;
+        m[s] = r < n && c < n ? cvt<R>(A[(size_t)r * n + c]) : C{0, 0};
+        if (r >= n) used |= 1u << s;
     }
-    // unscramble columns: position c holds original column pos[c]
-    if (threadIdx.x == 0) {
-        for (int c = 0; c < n; ++c) pos[c] = c;
-        for (int k = n - 1; k >= 0; --k) {
-            const int t = pos[k]; pos[k] = pos[perm[k]]; pos[perm[k]] = t;
-        }
-    }
+    for (int k = threadIdx.x; k < n; k += blockDim.x) mbar_init(&s_mb[k], 1);
+    fence_barrier_init();
     __syncthreads();
+    for (int k = threadIdx.x; k < n; k += blockDim.x)
+        mbar_arrive_expect_tx(&s_mb[k], (uint32_t)((n + 1) * sizeof(C) + sizeof(int)));
+    cluster.sync();
+    auto send = [&] {               // this warp's column c is the next
+        const unsigned k0 = used & 1 ? 0u : gj_key<R>(m[0]), k1 = used & 2 ? 0u : gj_key<R>(m[1]);
+        const unsigned key = max(k0, k1), kmax = __reduce_max_sync(0xffffffffu, key);
+        const int src = __ffs(__ballot_sync(0xffffffffu, key == kmax)) - 1;
+        const bool hi = k1 > k0;
+        const int p = __shfl_sync(0xffffffffu, hi ? lane + 32 : lane, src);
+        C pv = hi ? m[1] : m[0];
+        pv = {__shfl_sync(0xffffffffu, pv.re, src), __shfl_sync(0xffffffffu, pv.im, src)};
+        R d = pv.re * pv.re + pv.im * pv.im;
+        if (!(d > (R)0) || !isfinite(d)) {
+            if (lane == 0) atomicExch(bt.err, DEV_BREAKDOWN);
+            pv = {1, 0};
+            d = 1;
+        }
+        const R q = (lane & 1 ? -pv.im : pv.re) / d;   // both quotients in one division
+        const C ip = {__shfl_sync(0xffffffffu, q, 0), __shfl_sync(0xffffffffu, q, 1)};
+        const uint32_t mb = smem_u32(&s_mb[c]), a0 = smem_u32(col + c * n + lane);
+#pragma unroll
+        for (int i = 0; i < CL; ++i) {                 // the next column's owner first
+            const int dst = (rank + 1 + i) & (CL - 1);
+            const uint32_t rm = mapa(mb, dst), ra = mapa(a0, dst);
+            if (lane < n) st_async(ra, m[0], rm);
+            if (lane + 32 < n) st_async(ra + 32 * (uint32_t)sizeof(C), m[1], rm);
+        }
+        if (lane < CL) {
+            const uint32_t rm = mapa(mb, lane);
+            st_async(mapa(smem_u32(&s_ip[c]), lane), ip, rm);
+            st_async(mapa(smem_u32(&s_p[c]), lane), p, rm);
+        }
+    };
+    if (c == 0) send();
+    bool ok = true;
+    for (int k = 0; ok && k < n; ++k) {
+        ok = __all_sync(0xffffffffu, mbar_wait_cluster_bounded(&s_mb[k], 0, GJ_WAIT));
+        if (!ok) break;
+        const int p = s_p[k], pl = p & 31, ps = p >> 5;
+        const C ip = s_ip[k];
+        C v = ps ? m[1] : m[0];
+        v = C{__shfl_sync(0xffffffffu, v.re, pl), __shfl_sync(0xffffffffu, v.im, pl)} * ip;
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            if (s * 32 >= n) break;
+            const int r = lane + 32 * s;
+            const C f = r < n ? col[k * n + r] : C{0, 0};
+            const bool pr = ps == s && lane == pl;
+            if (c == k) m[s] = pr ? ip : -(f * ip);
+            else m[s] = pr ? v : m[s] - f * v;
+            if (pr) {
+                used |= 1u << s;
+                kk[s] = k;
+            }
+        }
+        if (c == k + 1 && c < n) send();
+    }
+    if (!ok && lane == 0) atomicExch(bt.err, DEV_TIMEOUT);
+    cluster.sync();                 // no store to this CTA is in flight any more
+    if (!ok || c >= n) return;
     c64* AT = (c64*)bt.AT[mat];
-    for (int e = threadIdx.x; e < nr * n; e += blockDim.x) {
-        const int rl = e / n, c = e - rl * n;
-        const C v = M[rl * n + pos[c]];
-        A[(size_t)(r0 + rl) * n + c] = cvt<double>(v);
-        if (AT) AT[(size_t)(r0 + rl) * n + c] = cvt<float>(v);
+    const int pc = s_p[c];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        if (lane + 32 * s >= n) continue;
+        const size_t o = (size_t)kk[s] * n + pc;
+        A[o] = cvt<double>(m[s]);
+        if (AT) AT[o] = cvt<float>(m[s]);
     }
+}
+template <typename R, int CL>
+static bool gj_cluster(const GjBatch& bt, int count, cudaStream_t s) {
+    static std::atomic<unsigned long long> attr{0};
+    if (!once_per_device(attr, [] {
+            return cudaFuncSetAttribute(k_gj_cluster<R, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        64 * 64 * (int)sizeof(cplx<R>)) == cudaSuccess &&
+                   (CL <= 8 || cudaFuncSetAttribute(k_gj_cluster<R, CL>, cudaFuncAttributeNonPortableClusterSizeAllowed,
+                                                    1) == cudaSuccess);
+        }))
+        return false;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    cfg.gridDim = dim3(count * CL);
+    cfg.blockDim = dim3(64 / CL * 32);
+    cfg.dynamicSmemBytes = sizeof(cplx<R>) * (size_t)bt.n * bt.n;
+    cfg.stream = s;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CL;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (CL > 8) {                   // 16 is more than every device has to offer
+        int nc = 0;
+        if (cudaOccupancyMaxActiveClusters(&nc, k_gj_cluster<R, CL>, &cfg) != cudaSuccess || nc < 1) {
+            cudaGetLastError();
+            return false;
+        }
+    }
+    cudaLaunchKernelEx(&cfg, k_gj_cluster<R, CL>, bt);
+    note_launch();
+    return true;
 }
 
 void launch_gj_inverse(const GjBatch& bt, int count, bool fp32, cudaStream_t s) {
     if (count < 1) return;
     if (bt.n >= 16 && bt.n <= 64) {
-        const int n = bt.n, rpc = (n + GJ_CL - 1) / GJ_CL;
-        const size_t es = fp32 ? sizeof(c64) : sizeof(c128);
-        const size_t sm = es * ((size_t)rpc * n + 2 * n + rpc) + sizeof(int) * 2 * n;
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute at[1];
-        cfg.gridDim = dim3(count * GJ_CL);
-        cfg.blockDim = dim3(256);
-        cfg.dynamicSmemBytes = sm;
-        cfg.stream = s;
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = GJ_CL;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        if (fp32) cudaLaunchKernelEx(&cfg, k_gj_cluster<float>, bt);
-        else cudaLaunchKernelEx(&cfg, k_gj_cluster<double>, bt);
-        note_launch();
+        if (fp32) gj_cluster<float, 16>(bt, count, s) || gj_cluster<float, 8>(bt, count, s);
+        else gj_cluster<double, 16>(bt, count, s) || gj_cluster<double, 8>(bt, count, s);
         return;
     }
     const int n = bt.n;
