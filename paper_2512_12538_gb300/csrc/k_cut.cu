@@ -329,13 +329,19 @@ __global__ void __launch_bounds__(256) k_cut_minv(const CutMinv* __restrict__ pr
 // One Arnoldi step inside the iteration's kernels, after phase C has left S g (the first
 // time S r) in P.v: w = V_j - S V_j, classical Gram-Schmidt twice against V_0 .. V_j, V_{j+1}
 // and the next g (into P.v), and in the first block the Givens update.  A block works on the
-// entries of its own cut items, so only the dot products cross blocks: partial sums, one
-// column a warp adds them, five barriers.  Bound by the FP64 pipe (16 multiply-adds an entry
-// and column) and the barriers; as a launch of its own, between launches of single steps
-// that load their panels again, a step took 127 us at 1023^2 where it takes 60 here.
+// entries of its own cut item, so only the dot products cross blocks: partial sums, one
+// column a warp adds them, four barriers.  The second pass's products include |w|^2, which
+// gives |V_{j+1}| before its correction: |w - V h|^2 = |w|^2 - |h|^2.
+// What bounds it is the FP64 issue rate (a warp's multiply-add takes its scheduler 64 clocks)
+// and the loads' latency: threads share out a column's entries in the products and an
+// entry's columns in the updates, loads go four deep, scalars are left to one warp, and the
+// Givens chain keeps only its own multiply-adds.  At 500^2 (148 blocks, 48 entries each,
+// 36 columns) a step takes 26 us and the Givens update 9; with one thread an entry, w in the
+// L2 and five barriers a solve took 13.7 ms instead of 12.6.
 struct GmState {
-    c128 h[72], al[72], hc[72], sn[72];
-    double cs[72], red[32], rho2;
+    c128 h[72], al[72], hc[72], sn[72], b[72], a[72];
+    double cs[72], red[32], rho2, inv, nn, beta;
+    c128 an;
 };
 __device__ __forceinline__ double gm_block_sum(double x, double* red, int nw) {
     x = warp_sum(x);
@@ -346,30 +352,54 @@ __device__ __forceinline__ double gm_block_sum(double x, double* red, int nw) {
     __syncthreads();
     return t;
 }
+// Sum of a over groups of W lanes: the first exchange leaves the real part's sums in the group's
+// lower half and the imaginary part's in the upper, so the rest adds one number a lane.
+template <int W> __device__ __forceinline__ c128 gm_sum(c128 a) {
+    const bool up = threadIdx.x & (W / 2);
+    const double give = up ? a.re : a.im;
+    double k = (up ? a.im : a.re) + __shfl_xor_sync(0xffffffffu, give, W / 2);
+#pragma unroll
+    for (int o = W / 4; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+    const double x = __shfl_xor_sync(0xffffffffu, k, W / 2);
+    return up ? c128{x, k} : c128{k, x};
+}
+template <typename P> __device__ __forceinline__ c128* align16(P* p) { return (c128*)(((size_t)p + 15) & ~(size_t)15); }
+// scr: shared memory for cap complex numbers, free here.
 template <typename T, int NT>
 __device__ __noinline__ bool gm_arnoldi(const CutProb& P, const CutGmres& G, GmState& M, GroupBar& bar, int rank, int gsz,
-                                        int j) {
+                                        int j, c128* scr, int cap) {
     using C = cplx<T>;
-    constexpr int NW = NT / 32, NC8 = NT / 8;
+    constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, Sx = P.Sx, nc = j + 1;
     const size_t nG = (size_t)2 * P.ncut * Sx;
     C* v = (C*)P.v;
-    const double beta = sqrt(*P.nrm);
-    // this block's entries: f(entry) over its cut items
-    auto entries = [&](int t0, int step, auto&& f) {
+    // one item a block: w stays in shared memory (else in G.w), and np * kg threads share
+    // the update, partial sums behind w
+    const int xw = min(P.XC, Sx - (rank % P.nch) * P.XC);
+    const bool one = P.nB <= gsz && 2 * P.XC <= cap;
+    int kg = 1;
+    if (one && rank < P.nB) kg = max(1, min(min(8, NT / (2 * xw)), cap / (2 * P.XC) - 1));
+    c128* part = scr + 2 * P.XC;
+    // this block's items: f(entries, first column, columns, cut)
+    auto items = [&](auto&& f) {
         for (int e = rank; e < P.nB; e += gsz) {
-            const int c = e / P.nch, x0 = (e - c * P.nch) * P.XC, xn = min(P.XC, Sx - x0);
-            for (int q = t0; q < 2 * xn; q += step) {
-                const int row = q >= xn;
-                f((size_t)(2 * c + row) * Sx + x0 + q - row * xn);
-            }
+            const int c = e / P.nch, x0 = (e - c * P.nch) * P.XC;
+            f(c, x0, min(P.XC, Sx - x0));
         }
+    };
+    auto entries = [&](auto&& f) {       // f(place in w, entry)
+        items([&](int c, int x0, int xn) {
+            for (int q = tid; q < 2 * xn; q += NT) {
+                const size_t o = (size_t)(2 * c + (q >= xn)) * Sx + x0 + (q >= xn ? q - xn : q);
+                f(one ? scr + q : G.w + o, o);
+            }
+        });
     };
     __syncthreads();
     if (j == 0) {
-        const double inv = beta > 0.0 ? 1.0 / beta : 0.0;
+        const double beta = sqrt(*P.nrm), inv = beta > 0.0 ? 1.0 / beta : 0.0;
         double g2 = 0.0;
-        entries(tid, NT, [&](size_t o) {
+        entries([&](c128*, size_t o) {
             const int c = (int)(o / (2 * (size_t)Sx));
             const c128 r = cvt<double>(((const C*)P.rt)[(size_t)(P.mid[c] - 1) * Sx + (o - (size_t)2 * c * Sx)]);
             G.rG[o] = r;
@@ -381,6 +411,7 @@ __device__ __noinline__ bool gm_arnoldi(const CutProb& P, const CutGmres& G, GmS
         if (tid == 0) {
             G.npart[rank] = g2;
             M.al[0] = c128{inv, 0.0};
+            M.beta = beta;
             if (rank == 0) {
                 G.alpha[0] = M.al[0];
                 *G.ls.st = GmresState{0, 0, 0, 0, 0.0, 0.0};
@@ -396,82 +427,149 @@ __device__ __noinline__ bool gm_arnoldi(const CutProb& P, const CutGmres& G, GmS
     }
     const double rho2 = M.rho2;
     c128 aw = M.al[j];                           // alpha of w: V_j's, as S V_j lies on the cut rows
-    entries(tid, NT, [&](size_t o) {
+    entries([&](c128* w, size_t o) {
         c128 sv = aw * G.v1[o];
         if (j > 0) sv = sv + cvt<double>(v[o]);
-        G.w[o] = G.V[(size_t)j * nG + o] - sv;
+        *w = G.V[(size_t)j * nG + o] - sv;
     });
     for (int i = tid; i < nc; i += NT) M.hc[i] = {0, 0};
     __syncthreads();
     for (int pass = 0; pass < 2; ++pass) {
-        for (int i0 = 0; i0 < nc; i0 += NC8) {
-            const int i = i0 + (tid >> 3);
+        // the products: tpc threads a column; in the second pass column nc is w itself
+        const int ncp = nc + pass;
+        int tpc = 32;
+        while (tpc > 8 && NT / tpc < ncp) tpc >>= 1;
+        const int sub = tid & (tpc - 1);
+        for (int i0 = 0; i0 < ncp; i0 += NT / tpc) {
+            const int i = i0 + tid / tpc;
             c128 a = {0, 0};
-            if (i < nc) {
-                const c128* Vi = G.V + (size_t)i * nG;
-                entries(tid & 7, 8, [&](size_t o) { cfma_cj(a, Vi[o], G.w[o]); });
-            }
-            for (int o = 4; o > 0; o >>= 1) {
-                a.re += __shfl_xor_sync(0xffffffffu, a.re, o);
-                a.im += __shfl_xor_sync(0xffffffffu, a.im, o);
-            }
-            if (i < nc && (tid & 7) == 0) G.part[(size_t)rank * 72 + i] = a;
+            if (i < ncp)
+                items([&](int c, int x0, int xn) {
+                    const size_t o0 = (size_t)2 * c * Sx + x0;
+                    const c128* w = one ? scr : G.w + o0;
+                    const c128* Vi = i < nc ? G.V + (size_t)i * nG + o0 : w;
+                    const int gap = Sx - xn, wgap = one ? 0 : gap, vgap = i < nc ? gap : wgap;   // between the rows
+                    for (int q0 = sub; q0 < 2 * xn; q0 += 4 * tpc) {
+                        c128 x[4], y[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int q = q0 + u * tpc;
+                            x[u] = y[u] = c128{0, 0};
+                            if (q < 2 * xn) {
+                                x[u] = Vi[q + (q >= xn ? vgap : 0)];
+                                y[u] = w[q + (q >= xn ? wgap : 0)];
+                            }
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (q0 + u * tpc < 2 * xn) cfma_cj(a, x[u], y[u]);
+                    }
+                });
+            a = tpc == 32 ? gm_sum<32>(a) : tpc == 16 ? gm_sum<16>(a) : gm_sum<8>(a);
+            if (i < ncp && sub == 0) G.part[(size_t)rank * 72 + i] = a;
         }
         if (!bar()) return false;
-        for (int i = rank + gsz * warp; i < nc; i += gsz * NW) {
+        for (int i = rank + gsz * warp; i < ncp; i += gsz * NW) {
             c128 a = {0, 0};
+#pragma unroll 5
             for (int k = lane; k < gsz; k += 32) a = a + ldcg(G.part + (size_t)k * 72 + i);
-            a = warp_sum(a);
-            if (lane == 0) G.dots[pass * 72 + i] = a + rho2 * (conj(M.al[i]) * aw);
+            a = gm_sum<32>(a);
+            if (lane == 0) G.dots[pass * 72 + i] = a + rho2 * (conj(i < nc ? M.al[i] : aw) * aw);
         }
         if (!bar()) return false;
-        for (int i = tid; i < nc; i += NT) {
-            M.h[i] = ldcg(G.dots + pass * 72 + i);
-            M.hc[i] = M.hc[i] + M.h[i];
-        }
+        for (int i = tid; i < ncp; i += NT) M.h[i] = ldcg(G.dots + pass * 72 + i);
         __syncthreads();
-        entries(tid, NT, [&](size_t o) {
-            c128 a0 = {0, 0}, a1 = {0, 0};
-            for (int i = 0; i < nc; i += 2) {
-                cfma(a0, M.h[i], G.V[(size_t)i * nG + o]);
-                if (i + 1 < nc) cfma(a1, M.h[i + 1], G.V[(size_t)(i + 1) * nG + o]);
+        // the last warp: alpha of the new w, and after the second pass its norm
+        if (warp == NW - 1) {
+            c128 da = {0, 0};
+            double hh = 0.0;
+            for (int i = lane; i < nc; i += 32) {
+                const c128 h = M.h[i];
+                cfma(da, h, M.al[i]);
+                M.hc[i] = M.hc[i] + h;
+                if (pass) hh += abs2(h);
             }
-            G.w[o] = G.w[o] - (a0 + a1);
+            da = aw - gm_sum<32>(da);
+            if (lane == 0) M.an = da;
+            if (pass) {
+                const double nn = fmax(0.0, M.h[nc].re - warp_sum(hh)), inv = nn > 0.0 ? rsqrt(nn) : 0.0;
+                if (lane == 0) {
+                    M.nn = nn;
+                    M.inv = inv;
+                }
+            }
+        }
+        // w -= V h; after the second pass V_{j+1} and the next step's input
+        items([&](int c, int x0, int xn) {
+            const size_t o0 = (size_t)2 * c * Sx + x0;
+            const int np = 2 * xn;
+            for (int t = tid; t < np * kg; t += NT) {
+                const int kk = t / np, q = t - kk * np;
+                const c128* Vo = G.V + o0 + q + (q >= xn ? Sx - xn : 0);
+                c128 a0 = {0, 0}, a1 = {0, 0};
+                for (int i = kk; i < nc; i += 4 * kg) {
+                    c128 x[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) x[u] = i + u * kg < nc ? Vo[(size_t)(i + u * kg) * nG] : c128{0, 0};
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (i + u * kg < nc) cfma(u & 1 ? a1 : a0, M.h[i + u * kg], x[u]);
+                }
+                c128* w = one ? scr + q : G.w + (Vo - G.V);
+                if (kg > 1) part[kk * np + q] = a0 + a1;
+                else *w = *w - (a0 + a1);
+            }
         });
-        c128 da = {0, 0};
-        for (int i = lane; i < nc; i += 32) cfma(da, M.h[i], M.al[i]);
-        aw = aw - warp_sum(da);
+        __syncthreads();
+        aw = M.an;
+        const double inv = M.inv;
+        const c128 an = inv * aw;
+        if (pass || kg > 1)
+            entries([&](c128* w, size_t o) {
+                c128 x = *w;
+                if (kg > 1)
+                    for (int kk = 0; kk < kg; ++kk) x = x - part[kk * 2 * xw + (w - scr)];
+                if (!pass) {
+                    *w = x;
+                    return;
+                }
+                x = inv * x;
+                G.V[(size_t)(j + 1) * nG + o] = x;
+                v[o] = cvt<T>(x - an * G.rG[o]);
+            });
+        if (pass && tid == 0) M.al[j + 1] = an;
         __syncthreads();
     }
-    double nn = 0.0;
-    entries(tid, NT, [&](size_t o) { nn += abs2(G.w[o]); });
-    nn = gm_block_sum(nn, M.red, NW);
-    if (tid == 0) G.npart[rank] = nn;
-    if (!bar()) return false;
-    nn = 0.0;
-    for (int k = lane; k < gsz; k += 32) nn += __ldcg(G.npart + k);
-    nn = warp_sum(nn) + rho2 * abs2(aw);          // alike in every warp
-    const double inv = nn > 0.0 ? 1.0 / sqrt(nn) : 0.0;
-    const c128 an = inv * aw;
-    entries(tid, NT, [&](size_t o) {
-        const c128 x = inv * G.w[o];
-        G.V[(size_t)(j + 1) * nG + o] = x;
-        v[o] = cvt<T>(x - an * G.rG[o]);
-    });
-    if (tid == 0) M.al[j + 1] = an;
-    if (rank != 0 || tid != 0) return true;
-    G.alpha[j + 1] = an;
-    // The Givens update of column j (k_gmres_rotate's), the chain in registers and shared
-    // memory: a column's entries back and forth through the L2 took 12 us at j = 40.
+    if (rank != 0 || warp != 0) return true;
+    // The Givens update of column j (k_gmres_rotate's): with a_0 = h_0, a_{i+1} = cs_i h_{i+1} -
+    // conj(sn_i) a_i and R_i = cs_i a_i + sn_i h_{i+1}; the chain of the a alone is serial.
     const GmresLs& ls = G.ls;
-    const double hn = sqrt(nn), nbv = sqrt(*P.b2);
-    c128 a = M.hc[0];
-    for (int i = 0; i < j; ++i) {
-        const c128 a1 = M.hc[i + 1];
-        ls.H[(size_t)i * ls.mk + j] = M.cs[i] * a + M.sn[i] * a1;
-        a = M.cs[i] * a1 - conj(M.sn[i]) * a;
+    for (int i = lane; i < j; i += 32) M.b[i] = M.cs[i] * M.hc[i + 1];
+    __syncwarp();
+    if (lane == 0) {
+        c128 a = M.hc[0];
+#pragma unroll 4
+        for (int i = 0; i < j; ++i) {
+            const c128 sn = M.sn[i], b = M.b[i];
+            M.a[i] = a;
+            a = c128{fma(-sn.im, a.im, fma(-sn.re, a.re, b.re)), fma(sn.im, a.re, fma(-sn.re, a.im, b.im))};
+        }
+        M.a[j] = a;
     }
-    const double aa = sqrt(abs2(a)), t = sqrt(abs2(a) + hn * hn);
+    __syncwarp();
+    for (int i = lane; i < j; i += 32) ls.H[(size_t)i * ls.mk + j] = M.cs[i] * M.a[i] + M.sn[i] * M.hc[i + 1];
+    // the square roots and the quotients side by side in the lanes (each takes over a
+    // thousand clocks): |a|, t, |V_{j+1}|, |b|, then 1 / |a|, |a| / t, |V_{j+1}| / t
+    c128 a = M.a[j];
+    const double nn = M.nn, a2 = abs2(a);
+    const double root = sqrt(lane == 0 ? a2 : lane == 1 ? a2 + nn : lane == 2 ? nn : *P.b2);
+    const double aa = __shfl_sync(0xffffffffu, root, 0), t = __shfl_sync(0xffffffffu, root, 1),
+                 hn = __shfl_sync(0xffffffffu, root, 2), nbv = __shfl_sync(0xffffffffu, root, 3);
+    const double quo = (lane == 0 ? 1.0 : lane == 1 ? aa : hn) / (lane == 0 ? aa : t);
+    const double ia = __shfl_sync(0xffffffffu, quo, 0), at = __shfl_sync(0xffffffffu, quo, 1),
+                 ht = __shfl_sync(0xffffffffu, quo, 2);
+    if (lane != 0) return true;
+    G.alpha[j + 1] = M.al[j + 1];
     double cs = 1.0;
     c128 sn = {0.0, 0.0};
     if (t != 0.0 && aa == 0.0) {
@@ -479,9 +577,9 @@ __device__ __noinline__ bool gm_arnoldi(const CutProb& P, const CutGmres& G, GmS
         sn = {1.0, 0.0};
         a = {hn, 0.0};
     } else if (t != 0.0) {
-        const c128 ph = (1.0 / aa) * a;
-        cs = aa / t;
-        sn = (hn / t) * ph;
+        const c128 ph = ia * a;
+        cs = at;
+        sn = ht * ph;
         a = t * ph;
     }
     ls.H[(size_t)j * ls.mk + j] = a;
@@ -492,7 +590,7 @@ __device__ __noinline__ bool gm_arnoldi(const CutProb& P, const CutGmres& G, GmS
     ls.g[j] = cs * gj;
     GmresState* st = ls.st;
     st->steps = j + 1;
-    const double gabs = sqrt(abs2(gn)), est = nbv > 0 ? gabs / nbv : 0.0;
+    const double beta = M.beta, gabs = sqrt(abs2(gn)), est = nbv > 0 ? gabs / nbv : 0.0;
     st->est = est;
     if (!isfinite(est)) {
         st->bad = 1;
@@ -961,7 +1059,8 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
                 // the Arnoldi step: P.v takes the next step's input
                 if (first && rank == 0)
                     for (int e = tid; e < D; e += NT) ((C*)G.y0)[e] = s_ya[e];
-                if (!(ok = gm_arnoldi<T, NT>(P, G, s_gm, bar, rank, gsz, in_round))) break;
+                if (!(ok = gm_arnoldi<T, NT>(P, G, s_gm, bar, rank, gsz, in_round, align16(s_ln),
+                                            (int)((MG + 4) * Sx * sizeof(C) / sizeof(c128)) - 1))) break;
                 __syncthreads();
                 if (one && rank < P.nB) {
                     const int c = rank / nch, x0 = (rank - c * nch) * XC, xn = min(XC, Sx - x0);
@@ -1420,7 +1519,8 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
                 if (first && rank == 0)
                     for (int e = tid; e < D; e += NT) ((C*)G.y0)[e] = s_ya[e];
                 __shared__ GmState s_gm;
-                if (!(ok = gm_arnoldi<float, NT>(P, G, s_gm, bar, rank, CC_CL, in_round))) break;
+                if (!(ok = gm_arnoldi<float, NT>(P, G, s_gm, bar, rank, CC_CL, in_round, align16(s_ln),
+                                                P.MG * Sx / 2 - 1))) break;
                 __syncthreads();
                 for (int q = tid; q < np; q += NT) {
                     const int row = q >= xn, il = q - row * xn;
@@ -1651,7 +1751,7 @@ size_t cut_m_packed(int L, int r) { return (size_t)cut_m_elems(L, r); }
 //    on one cluster of sixteen (k_cut_cluster), bound by latency alone;
 //  * the others on a grid group of up to one block per SM (k_cut_steps): there the lines
 //    (FP64: the pipe, four warps fill it) and the panels' bytes want every SM.
-static constexpr int CUT_NT = 256, CUT_SMEM = 212 * 1024;
+static constexpr int CUT_NT = 256, CUT_SMEM = 210 * 1024;
 static bool cluster_form(CutProb& P, int b_max) {
     const int NL = P.ncut + 1;
     if (P.D > 128 || NL > CC_CL) return false;
