@@ -2053,7 +2053,7 @@ struct Solver final : SolverBase {
                 return HH_ECUDA;
             launch_cut_lines<T>(d_cut, 1, nullptr, nl, b_max, Sx, stream);
             eig_stage_prof(2, d_etasks_cout);
-            launch_cut_update<T>(d_upd + cut_flip, 1, Sy, Sx, stream);
+            launch_cut_update<T>(d_upd + cut_flip, 1, 1 << L, b_max, Sx, stream);
             resid(ut);
         }
     }
@@ -2115,7 +2115,7 @@ struct Solver final : SolverBase {
             if (!steps(2, 1, 0)) return HH_ECUDA;   // the corrections of the combined input
             launch_cut_lines<T>(d_cut, 1, nullptr, nl, b_max, Sx, stream);
             eig_stage_prof(2, d_etasks_cout);
-            launch_cut_update<T>(d_upd + cut_flip, 1, Sy, Sx, stream);
+            launch_cut_update<T>(d_upd + cut_flip, 1, 1 << L, b_max, Sx, stream);
             cut_swap();
             resid();
         }
@@ -2720,7 +2720,7 @@ struct BatchEngine {
         if (ncl) launch_cut_lines<T>(d_probs, top, d_modes, nleaf, bm, sx, stream);
         if (ngr) launch_cut_lines<T>(d_probs, top, d_modes + cap_probs, nleaf, bm, sx, stream);
         transforms(2);
-        launch_cut_update<T>(d_jobs, nj, sx, sx, stream);
+        launch_cut_update<T>(d_jobs, nj, nleaf, bm, sx, stream);
         residuals();
         const hh_status st = read_back();
         if (st != HH_OK) return st;

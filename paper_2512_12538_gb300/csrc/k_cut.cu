@@ -1624,36 +1624,54 @@ __global__ void __launch_bounds__(256) k_cut_lines(const CutProb* __restrict__ p
 
 // ut = u + w + sum over the levels of C_p y_p at every grid point (w: the composed leaf
 // solutions; y: the round's summed corrections).  HBM-bound: each level's basis read once,
-// L r values a point.  One block per row and 256 columns; rows of one leaf share the nodes.
-template <typename T>
+// L r values a point.  The rows between two cuts share the nodes and are contiguous, so a
+// block takes 256 PT points of them, whatever the columns.  1023^2, r = 32, complex64:
+// 193 us with a block per row and 256 columns, 148 here (PT = 4); 255^2 20 and 11 us (PT = 1).
+template <typename T, int PT>
 __global__ void __launch_bounds__(256) k_cut_update(const CutUpdJob* __restrict__ jobs) {
     using C = cplx<T>;
     __shared__ C sy[CUT_KMAX];
+    __shared__ const C* sc[CUT_MAXL];
+    __shared__ size_t sn[CUT_MAXL];
     const CutUpdJob& J = jobs[blockIdx.z];
     const CutProb& P = *J.prob;
-    const int Sx = P.Sx, r = P.r, L = P.L, row = blockIdx.y;
-    if (row >= J.Sy || (int)blockIdx.x * 256 >= Sx) return;
-    int lf = 0;
-    while (lf < P.ncut && row >= P.mid[lf]) ++lf;
-    for (int t = threadIdx.x; t < L * r; t += 256) {
-        const int l = t / r, j = t - l * r;
+    const int Sx = P.Sx, r = P.r, L = P.L, lf = blockIdx.y;
+    if (lf > P.ncut) return;
+    const int m0 = lf ? P.mid[lf - 1] : 0, m1 = lf < P.ncut ? P.mid[lf] : J.Sy;
+    const size_t n = (size_t)(m1 - m0) * Sx, t0 = blockIdx.x * (size_t)(256 * PT), t = t0 + threadIdx.x;
+    if (t0 >= n) return;
+    for (int q = threadIdx.x; q < L * r; q += 256) {
+        const int l = q / r, j = q - l * r;
         const int p = (1 << l) - 1 + (lf >> (L - l)), k = (lf >> (L - l - 1)) & 1;
-        sy[t] = ((const C*)P.yacc)[(size_t)p * 2 * r + k * r + j];
+        sy[q] = ((const C*)P.yacc)[(size_t)p * 2 * r + k * r + j];
+        if (j == 0) {
+            const CutNode& nd = P.node[p];
+            sn[l] = nd.N;
+            sc[l] = (const C*)nd.C + (size_t)(k * r) * nd.N + (size_t)(m0 - nd.ra) * Sx;
+        }
     }
     __syncthreads();
-    const int x = blockIdx.x * 256 + threadIdx.x;
-    if (x >= Sx) return;
-    const size_t o = (size_t)row * Sx + x;
-    C acc = ((const C*)J.w)[o];
-    for (int l = 0; l < L; ++l) {
-        const int p = (1 << l) - 1 + (lf >> (L - l)), k = (lf >> (L - l - 1)) & 1;
-        const CutNode& nd = P.node[p];
-        const C* c = (const C*)nd.C + (size_t)(k * r) * nd.N + (size_t)(row - nd.ra) * Sx + x;
-#pragma unroll 16
-        for (int j = 0; j < r; ++j) cfma(acc, c[(size_t)j * nd.N], sy[l * r + j]);
+    const size_t o = (size_t)m0 * Sx;
+    size_t ti[PT];             // (past the end: the last point again, so that no load is guarded)
+    C acc[PT];
+    c128 u[PT];
+#pragma unroll
+    for (int i = 0; i < PT; ++i) {
+        ti[i] = t + 256 * i < n ? t + 256 * i : n - 1;
+        acc[i] = ((const C*)J.w)[o + ti[i]];
+        u[i] = J.u[o + ti[i]];
     }
-    const c128 u = J.u[o];
-    J.ut[o] = u + cvt<double>(acc);
+    for (int l = 0; l < L; ++l) {
+        const C* c = sc[l];
+        const size_t N = sn[l];
+#pragma unroll 16 / PT
+        for (int j = 0; j < r; ++j, c += N)
+#pragma unroll
+            for (int i = 0; i < PT; ++i) cfma(acc[i], c[ti[i]], sy[l * r + j]);
+    }
+#pragma unroll
+    for (int i = 0; i < PT; ++i)
+        if (t + 256 * i < n) J.ut[o + ti[i]] = u[i] + cvt<double>(acc[i]);
 }
 
 // ----------------------------------------------------- end of a GMRES cycle (CutGmres)
@@ -1888,9 +1906,15 @@ void launch_cut_gm_combine(const CutProb* prob, const CutGmres& G, int nG, cudaS
     k_cut_gm_combine<T><<<std::min(152, (nG + 63) / 64), 256, sizeof(c128) * G.ls.mk * G.ls.mk, s>>>(prob, G, nG);
     note_launch();
 }
+// four points a thread once that leaves two blocks an SM
+static constexpr size_t UPD_WIDE = (size_t)152 * 2 * 1024;
 template <typename T>
-void launch_cut_update(const CutUpdJob* jobs, int njobs, int Sy_max, int Sx_max, cudaStream_t s) {
-    k_cut_update<T><<<dim3((Sx_max + 255) / 256, Sy_max, njobs), 256, 0, s>>>(jobs);
+void launch_cut_update(const CutUpdJob* jobs, int njobs, int nleaf_max, int own_max, int Sx_max, cudaStream_t s) {
+    const size_t n = (size_t)own_max * Sx_max;
+    const int pt = n * nleaf_max * njobs >= UPD_WIDE ? 4 : 1;
+    const dim3 grid((unsigned)((n + 256 * pt - 1) / (256 * pt)), nleaf_max, njobs);
+    if (pt == 4) k_cut_update<T, 4><<<grid, 256, 0, s>>>(jobs);
+    else k_cut_update<T, 1><<<grid, 256, 0, s>>>(jobs);
     note_launch();
 }
 
@@ -1903,7 +1927,7 @@ void launch_cut_update(const CutUpdJob* jobs, int njobs, int Sy_max, int Sx_max,
                                       cudaStream_t, int, const CutGmres*, int);                                                                  \
     template void launch_cut_lines<T>(const CutProb*, int, const int*, int, int, int, cudaStream_t);                  \
     template void launch_cut_gm_combine<T>(const CutProb*, const CutGmres&, int, cudaStream_t);                       \
-    template void launch_cut_update<T>(const CutUpdJob*, int, int, int, cudaStream_t);
+    template void launch_cut_update<T>(const CutUpdJob*, int, int, int, int, cudaStream_t);
 HH_CUT_INST(float)
 HH_CUT_INST(double)
 

@@ -421,7 +421,7 @@ void launch_cut_lines(const CutProb* probs, int nprob, const int* modes, int nle
 template <typename T>
 void launch_cut_gm_combine(const CutProb* prob, const CutGmres& G, int nG, cudaStream_t s);
 template <typename T>
-void launch_cut_update(const CutUpdJob* jobs, int njobs, int Sy_max, int Sx_max, cudaStream_t s);
+void launch_cut_update(const CutUpdJob* jobs, int njobs, int nleaf_max, int own_max, int Sx_max, cudaStream_t s);
 
 // ---- the set-up's sub-level solves from the interface rows (k_edge.cu) ---------------
 // A node on the path from a child's edge leaf up to the child: its basis, the child that
