@@ -23,7 +23,9 @@ namespace hh {
 // Solution rows of the edge leaves: one block per (column, child).  The modes in batches of
 // MG lines, one warp a line (xi and the lines in shared memory); after a batch each thread
 // adds the batch's share of the rows at its own grid columns.  rows: [4][Sx][nc]: the two
-// rows at the inner cut, then the trace rows.
+// rows at the inner cut, then the trace rows.  FP64-issue bound in the FP64 form, so a row
+// nobody asked for costs nothing, and a single source row's factor goes with the results'
+// (383^2, 40 columns, FP64: 656 and 644 us a call).
 template <typename T>
 __global__ void __launch_bounds__(256) k_edge_rows(const EdgeTask* __restrict__ tasks, int Sx, int nc, int adj, int MG) {
     using C = cplx<T>;
@@ -58,6 +60,11 @@ __global__ void __launch_bounds__(256) k_edge_rows(const EdgeTask* __restrict__ 
             const int a = k == 0 ? ai0 : k == 1 ? ai1 : ao[k - 2];
             C v = a >= 0 ? V[(size_t)a * b + m0 + w] : C{0, 0};
             if (k < 2 && E.sc) v = ((const C*)E.sc)[m0 + w] * v;
+            if (k >= 2 && !adj && a >= 0) {          // one source row: its factor here
+                C vi = V[(size_t)ai0 * b + m0 + w];
+                if (E.sc) vi = ((const C*)E.sc)[m0 + w] * vi;
+                v = v * vi;
+            }
             s_v[k][w] = v;
         }
         __syncthreads();
@@ -68,8 +75,11 @@ __global__ void __launch_bounds__(256) k_edge_rows(const EdgeTask* __restrict__ 
             const C v0 = s_v[0][warp], v1 = s_v[1][warp];
             for (int i = lane; i < Sx; i += 32) {
                 as[i] = xi[i];
-                C f = v0 * in[i];
-                if (adj) cfma(f, v1, in[Sx + i]);
+                C f = in[i];
+                if (adj) {
+                    f = v0 * f;
+                    cfma(f, v1, in[Sx + i]);
+                }
                 fs[i] = f;
             }
             __syncwarp();
@@ -85,7 +95,8 @@ __global__ void __launch_bounds__(256) k_edge_rows(const EdgeTask* __restrict__ 
             for (int w = 0; w < nm; ++w) {
                 const C f = ls[w * Sx + i];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) cfma(o[k], s_v[2 + k][w], f);
+                for (int k = 0; k < 4; ++k)
+                    if (ao[k] >= 0) cfma(o[k], s_v[2 + k][w], f);
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k) out[k * Sx + i] = o[k];
@@ -298,8 +309,11 @@ __global__ void __launch_bounds__(256) k_edge_lines(const EdgeTask* __restrict__
     C* fh = (C*)E.Fh + (size_t)line * Sx;
     for (int i = lane; i < Sx; i += 32) fh[i] = fs[i];
 }
+// Blocks of two warps: a chain is bound by its own latency and, in FP64, by its scheduler's issue
+// rate (64 clocks a multiply-add), so the warps go one to a scheduler over all SMs (383^2, r = 32,
+// FP64: 442 us in blocks of eight, 226 here).
 template <typename T>
-__global__ void __launch_bounds__(256) k_edge_chains(const EdgeTask* __restrict__ tasks, int Sx, int nc) {
+__global__ void __launch_bounds__(64) k_edge_chains(const EdgeTask* __restrict__ tasks, int Sx, int nc) {
     using C = cplx<T>;
     constexpr int RB = 16;
     const EdgeTask& E = tasks[blockIdx.y];
@@ -487,7 +501,7 @@ void launch_edge_path(const EdgeTask* tasks, int nchild, int Sx, int nc, int r, 
 template <typename T>
 void launch_edge_basis_lines(const EdgeTask* tasks, int nchild, int b_max, int Sx, int nc, cudaStream_t s) {
     if (!eig_line_major(nc)) {
-        k_edge_chains<T><<<dim3((b_max * ((nc + 31) / 32) + 7) / 8, nchild), 256, 0, s>>>(tasks, Sx, nc);
+        k_edge_chains<T><<<dim3((b_max * ((nc + 31) / 32) + 1) / 2, nchild), 64, 0, s>>>(tasks, Sx, nc);
     } else {
         static std::atomic<unsigned long long> attr{0};
         smem_limit_once(attr, k_edge_lines<T>, 200 * 1024);
