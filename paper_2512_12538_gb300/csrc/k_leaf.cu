@@ -249,6 +249,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_factor2d_reg(const LeafTask* __r
                 }
 #pragma unroll
                 for (int c2 = 0; c2 < CS; ++c2) {
+                    if (warp + NW * c2 >= b) break;
                     C v = m[0][c2];
 #pragma unroll
                     for (int rs = 1; rs < RS; ++rs)
@@ -349,7 +350,7 @@ void launch_factor(const LeafTask* d_tasks, int ntasks, int b_max, int Sx, doubl
 // (the dot products, their reduction, one barrier) bounds it, so nothing else stands on that
 // chain: f, y and x pass through registers in groups of SW_G columns, lane g holding
 // column g of the group, loaded a group ahead.  4 bands of 37 rows x 129 columns, complex64, one
-// right-hand side: 0.61 ms with one chain and loads on it, 0.099 ms here.
+// right-hand side: 0.61 ms with one chain and loads on it, 0.077 ms here.
 static constexpr int SW_G = 8;
 // threads of a CTA at most: the rows of which three slots fit shared memory, eight lanes a row
 template <typename T, int NP> constexpr int sweep_threads() {
@@ -380,15 +381,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(sweep_threads<T, NP>
     const int nsteps = 2 * n + 1;                           // inwards, middle, outwards
     const int total = nsteps * npiece;
     auto step_col = [&](int s) { return s == n ? mid : chain_col(Sx, side, s < n ? s : 2 * n - s); };
-    auto issue = [&](int q) {
-        const int s = q / npiece, p = q - s * npiece;
-        const int r0 = p * prow;
-        const int rows = min(prow, b - r0);
-        const uint32_t bytes = (uint32_t)(rows * ldx * sizeof(C));
-        const int slot = q % nslot;
-        mbar_arrive_expect_tx(&bars[slot], bytes);
-        bulk_g2s(slots + (size_t)slot * slot_elems, X + (size_t)step_col(s) * step + (size_t)r0 * ldx, bytes,
-                 &bars[slot]);
+    // the producer's place (thread 0): the next piece's step, piece and slot; the consumers'
+    // slot and its phase (counted on: a division a piece would stand on the chain)
+    int i_s = 0, i_p = 0, i_slot = 0, slot = 0;
+    uint32_t parity = 0;
+    auto issue = [&] {
+        const int r0 = i_p * prow;
+        const uint32_t bytes = (uint32_t)(min(prow, b - r0) * ldx * sizeof(C));
+        mbar_arrive_expect_tx(&bars[i_slot], bytes);
+        bulk_g2s(slots + (size_t)i_slot * slot_elems, X + (size_t)step_col(i_s) * step + (size_t)r0 * ldx, bytes,
+                 &bars[i_slot]);
+        if (++i_p == npiece) { i_p = 0; ++i_s; }
+        if (++i_slot == nslot) i_slot = 0;
     };
 
     if (threadIdx.x == 0) {
@@ -399,7 +403,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(sweep_threads<T, NP>
     for (int e = threadIdx.x; e < 3 * ldx * NC; e += blockDim.x) vbuf[e] = C{0, 0};
     cg::this_cluster().sync();                              // the other CTA's shared memory exists
     if (threadIdx.x == 0)
-        for (int q = 0; q < nslot && q < total; ++q) issue(q);
+        for (int q = 0; q < nslot && q < total; ++q) issue();
 
     const int lr = threadIdx.x / G, g = threadIdx.x % G;
     auto col_of = [&](int t) { return (size_t)chain_col(Sx, side, t) * nrhs + c0; };
@@ -447,8 +451,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(sweep_threads<T, NP>
     bool ok = true, bad = false;
     // rows of piece p of step s: X_i v, in every lane of the row
     auto product = [&](int s, int p, C (&acc)[NC]) {
-        const int slot = q % nslot;
-        if (!mbar_wait_bounded(&bars[slot], (uint32_t)((q / nslot) & 1), WAIT_LIMIT)) {
+        if (!mbar_wait_bounded(&bars[slot], parity, WAIT_LIMIT)) {
             atomicExch(err, DEV_TIMEOUT);
             bad = true;
         }
@@ -479,8 +482,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(sweep_threads<T, NP>
     // after a piece: its slot is free for the piece nslot further on
     auto turn = [&] {
         if (__syncthreads_or(bad)) return false;
-        if (threadIdx.x == 0 && q + nslot < total) issue(q + nslot);
+        if (threadIdx.x == 0 && q + nslot < total) issue();
         ++q;
+        if (++slot == nslot) { slot = 0; parity ^= 1; }
         return true;
     };
     // inwards; the last column's W y (the left one's with f_m) goes to both CTAs
