@@ -147,28 +147,28 @@ CATEGORY_BOUND = {
     "factor": ("latency", "k_eig_roots + k_eig_modes (eigenpairs of the column pencil, scalar Schur recursions)"),
     "sweep_in": ("tensor_tf32x3", "k_tc_transform (f^ = V^T f on the tensor cores, TF32 three-term split; "
                                   "k_eig_gemm2 on the CUDA cores where the autotuner chose it)"),
-    "sweep_recur": ("hbm", "k_eig_recur (scalar Schur recursions along the line, warp scans)"),
+    "sweep_recur": ("latency", "k_edge_rows + k_edge_chains (line recursions of the set-up's sketches and basis "
+                               "extensions, right-hand sides on the interface rows)"),
     "sweep_out": ("tensor_tf32x3", "k_tc_transform (x = V x^ on the tensor cores, TF32 three-term split; "
                                    "k_eig_gemm2 on the CUDA cores where the autotuner chose it)"),
-    "residual": ("hbm", "k_residual_cast (FP64 residual b - A u, its norm partials and complex64 copy)"),
-    "coarse_project": ("hbm", "k_coarse_batch (one-column coarse corrections: C^H r, A_c^-1, C y; "
-                              "one cooperative launch per level)"),
-    "galerkin": ("alu64", "k_galerkin_herm + k_galerkin_bdry (A_c = C^H A~ C, Hermitian-packed: the upper "
-                          "triangle by FP64 3M products of the stored basis, the impedance terms on the boundary "
-                          "points)"),
+    "residual": ("latency", "k_cut_steps / k_cut_cluster, update of the cut rows (v -= E y, its norm), and a round's "
+                            "k_residual_cast (FP64 residual b - A u)"),
+    "coarse_project": ("hbm", "k_cut_steps / k_cut_cluster, rows next to the cuts: residual, C^H r, y = M d (the basis "
+                              "rows come from shared memory and the L2; latency holds it far below either)"),
+    "galerkin": ("latency", "k_cut_gram + k_gj_cluster + k_cut_minv (FP64 coarse matrices from the cut rows, their "
+                            "inverses)"),
     "qr": ("latency", "k_qr / k_qr_cluster (sketch orthonormalisation, CGS2 in shared memory, one CTA or a cluster)"),
     "svd": ("latency", "k_heig_tri + k_heig_vec (FP64 Hermitian eigenproblem of the sketch Gram matrix)"),
-    "leaf_sweep": ("alu", "k_eig_sweep_fused (f^ = V^T f, scalar recursions, x = V x^; one cluster per leaf)"),
-    "coarse_multi": ("hbm", "k_ip_colA_rt (multi-column coarse projections of the set-up's sub-level solves)"),
+    "leaf_sweep": ("alu", "k_cut_steps / k_cut_cluster, line recursions of the leaves (inputs and results on the "
+                              "cut rows)"),
+    "coarse_multi": ("hbm", "k_edge_proj + k_coarse_updn_s (corrections of the set-up's basis extensions)"),
 }
 # FP64 peak derived from the DFMA issue rate (2 per SM per cycle, the peak ncu reports for
 # sm__sass_thread_inst_executed_op_dfma_pred_on.sum): 152 SMs x 2 x 2 flops x max SM clock.
 DFMA_PER_SM_CLK = 2
-# DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the dominant
-# kernel on this workload's shapes (mean of its three launches per step), from the ncu
-# capture summarised in profiles/coarse_batch_helm2d_n1023_k100_L3.md.  To be removed
-# whenever k_coarse_batch changes.
-TRAFFIC_BYTES_PER_LAUNCH = {"coarse_project": 491.7e6}
+# DRAM bytes per launch of a dominant category whose bound is HBM, from an ncu capture; none
+# is: the steps run on the rows next to the cuts, from shared memory and the L2.
+TRAFFIC_BYTES_PER_LAUNCH = {}
 
 
 def whole_job_rate(local_ms, units_per_rank, world, device="cuda"):
@@ -531,6 +531,8 @@ def rate(cat, ms, by, fl, pk, pk_kind):
     """Achieved rate of one category against its peak."""
     bound, kname = CATEGORY_BOUND.get(cat, ("latency", cat))
     out = {"kernel": kname, "category": cat, "bound": bound}
+    if ms <= 0:      # its work is part of another category's launches
+        bound = None
     if bound == "hbm" and by > 0:
         a = by / (ms / 1e3) / 1e9
         out.update({"achieved": a, "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": a / pk["hbm_gbs"],

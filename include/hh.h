@@ -197,9 +197,11 @@ hh_status hh_setup_batch(const hh_params* params, int count, void* stream, hh_ha
 /* Solves count set-up problems: u[k] = solution of problem h[k] for d_f[k], d_g[k]
  * (layouts as hh_solve).  When every handle uses the stationary outer iteration with
  * n_inner = 1, the eigenbasis leaf path and at least two levels, in one precision, the
- * problems iterate in lockstep: each iteration is one residual launch, one leaf-sweep
- * launch, one coarse-correction launch per hierarchy height and one for the roots, for
- * all problems together, and a problem drops out when its residual meets its own tol.
+ * problems iterate together in rounds: one launch in which every problem runs its steps on
+ * the rows next to its leaf cuts up to its own next stop, then one launch each, for all
+ * problems, of the leaf transforms, the update and the FP64 residual; a problem drops out
+ * when its residual meets its own tol.  Members whose iteration does not converge are
+ * re-solved by flexible GMRES with their set-up as it stands.
  * Otherwise the problems are solved one after another.  stats[k] (may be NULL) gets
  * problem k's iterations and residual; t_solve_ms is the time of the whole batch.
  * Synchronises.  Returns HH_OK if all converged, else the first failing status. */
@@ -350,8 +352,9 @@ hh_status hh_profile_enable(hh_handle* h, int enable);
 /* Which categories the profiler times: bit c of mask for category c (default: all).
  * Each timed category costs events on the stream, so a caller timing one kernel family
  * selects only that one.  h != NULL: that handle, from its next launch; h == NULL:
- * handles created afterwards.  Within one outer step the coarse corrections of all
- * levels run back to back and share one event pair (counted as that many launches). */
+ * handles created afterwards.  Where the steps of a solve run inside one launch (eigenbasis
+ * leaves, n_inner = 1), its phases are timed by the kernel's own clock and counted as one
+ * leaf sweep, one coarse correction per level and one residual a step. */
 hh_status hh_profile_categories(hh_handle* h, unsigned mask);
 /* total_ms: summed event time; launches: timed launches; alg_bytes / alg_flops: the
  * algorithmic memory traffic and floating-point work of those launches (formulas in the
@@ -381,7 +384,7 @@ hh_status hh_autotune_report(char* buf, size_t cap, size_t* len);
  * synchronises reports HH_ETIMEOUT with the context still usable.
  * -------------------------------------------------------------------------------- */
 /* Caps the polls of the give-up waits of the kernels launched from now on in this
- * process: the coarse corrections' cooperative grid barrier and the tensor-core
+ * process: the barriers of the cooperative kernels and the tensor-core
  * transforms' waits for their operands and MMAs.  polls = 0 makes every such wait give
  * up at once (how a test makes a wait run out without a fault); polls < 0 restores the
  * defaults (about a second).  CUDA graphs captured meanwhile keep the value of their
