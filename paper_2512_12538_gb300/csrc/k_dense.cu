@@ -1072,22 +1072,22 @@ __global__ void __launch_bounds__(512) k_qr(cplx<T>* const* Yp, int Sx, int m, i
     if (staged)
         for (size_t e = threadIdx.x; e < tot; e += blockDim.x) Yg[e] = Y[(e / m) * ld + e % m];
 }
-// The same orthogonalisation for a block too large for one CTA's shared memory: a cluster
-// of QR_CL CTAs per block, each holding a slice of the rows in shared memory.  Each dot
+// The same orthogonalisation for larger blocks: a cluster of CL CTAs per block, each holding
+// a slice of the rows in shared memory; four threads share a row's update, and in FP64, which
+// the issue rate bounds (64 clocks a warp's multiply-add), eight lanes a dot product.  Each dot
 // product and norm is a sum of the CTAs' partial sums, added in rank order from
 // distributed shared memory, so every CTA takes the same coefficients; the partial-sum
 // arrays alternate between two buffers, and the cluster barrier after each write keeps a
 // CTA from overwriting a buffer another is still reading.
-static constexpr int QR_CL = 8;
-template <typename T>
+template <typename T, int CL>
 __global__ void __launch_bounds__(512) k_qr_cluster(cplx<T>* const* Yp, int Sx, int m) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
-    cplx<T>* Yg = Yp[blockIdx.x / QR_CL];
+    cplx<T>* Yg = Yp[blockIdx.x / CL];
     extern __shared__ __align__(16) unsigned char qcs[];
     const int ld = m + 1;                       // padded rows (bank spread)
-    const int rows = (Sx + QR_CL - 1) / QR_CL;
+    const int rows = (Sx + CL - 1) / CL;
     const int r0 = min(Sx, rank * rows), r1 = min(Sx, r0 + rows), nr = r1 - r0;
     cplx<T>* Y = (cplx<T>*)qcs;                 // [rows][ld]
     __shared__ cplx<T> pd[2][128];              // partial dot products (two buffers)
@@ -1104,24 +1104,36 @@ __global__ void __launch_bounds__(512) k_qr_cluster(cplx<T>* const* Yp, int Sx, 
     int buf = 0;
     for (int j = 0; j < m; ++j) {
         for (int pass = 0; pass < 2 && j > 0; ++pass) {
-            for (int k = warp; k < j; k += nw) {
+            constexpr int G = sizeof(T) == 8 ? 8 : 32;
+            for (int k0 = warp * (32 / G); k0 < j; k0 += nw * (32 / G)) {
+                const int k = k0 + lane / G, g = lane % G;
                 cplx<T> a = {0, 0};
-                for (int x = lane; x < nr; x += 32) cfma_cj(a, Y[x * ld + k], Y[x * ld + j]);
-                a = warp_sum(a);
-                if (lane == 0) pd[buf][k] = a;
+                if (k < j)
+                    for (int x = g; x < nr; x += G) cfma_cj(a, Y[x * ld + k], Y[x * ld + j]);
+                for (int o = G / 2; o > 0; o >>= 1) {
+                    a.re += __shfl_xor_sync(0xffffffffu, a.re, o);
+                    a.im += __shfl_xor_sync(0xffffffffu, a.im, o);
+                }
+                if (k < j && g == 0) pd[buf][k] = a;
             }
             cluster.sync();
             for (int k = threadIdx.x; k < j; k += blockDim.x) {
                 cplx<T> a = {0, 0};
-                for (int r = 0; r < QR_CL; ++r) a = a + cluster.map_shared_rank(&pd[buf][0], r)[k];
+                for (int r = 0; r < CL; ++r) a = a + cluster.map_shared_rank(&pd[buf][0], r)[k];
                 dots[k] = a;
             }
             buf ^= 1;
             __syncthreads();
-            for (int x = threadIdx.x; x < nr; x += blockDim.x) {
-                cplx<T> v = Y[x * ld + j];
-                for (int k = 0; k < j; ++k) v = v - Y[x * ld + k] * dots[k];
-                Y[x * ld + j] = v;
+            for (int t0 = 0; t0 < 4 * nr; t0 += blockDim.x) {
+                const int x = (t0 + threadIdx.x) >> 2, g = threadIdx.x & 3;
+                cplx<T> v = {0, 0};
+                if (x < nr)
+                    for (int k = g; k < j; k += 4) cfma(v, Y[x * ld + k], dots[k]);
+                for (int o = 2; o > 0; o >>= 1) {
+                    v.re += __shfl_xor_sync(0xffffffffu, v.re, o);
+                    v.im += __shfl_xor_sync(0xffffffffu, v.im, o);
+                }
+                if (x < nr && g == 0) Y[x * ld + j] = Y[x * ld + j] - v;
             }
             __syncthreads();
         }
@@ -1138,7 +1150,7 @@ __global__ void __launch_bounds__(512) k_qr_cluster(cplx<T>* const* Yp, int Sx, 
         cluster.sync();
         if (threadIdx.x == 0) {
             T v = 0;
-            for (int r = 0; r < QR_CL; ++r) v += *cluster.map_shared_rank(&pn[buf], r);
+            for (int r = 0; r < CL; ++r) v += *cluster.map_shared_rank(&pn[buf], r);
             const T nrm = sqrt(v);
             s_inv = nrm > (T)0 ? (T)1 / nrm : (T)0;
         }
@@ -1156,6 +1168,32 @@ __global__ void __launch_bounds__(512) k_qr_cluster(cplx<T>* const* Yp, int Sx, 
     cluster.sync();
 }
 
+template <typename T, int CL>
+static bool qr_cluster(int nq, int Sx, int m, cplx<T>* const* ptrs, cudaStream_t s) {
+    const size_t bytes = sizeof(cplx<T>) * (size_t)((Sx + CL - 1) / CL) * (m + 1);
+    if (m > 128 || bytes > (size_t)(200 * 1024) - 4096) return false;
+    static std::atomic<unsigned long long> attr{0};
+    smem_limit_once(attr, k_qr_cluster<T, CL>, 200 * 1024);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    cfg.gridDim = dim3(nq * CL);
+    cfg.blockDim = dim3(512);
+    cfg.dynamicSmemBytes = bytes;
+    cfg.stream = s;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CL;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_qr_cluster<T, CL>, ptrs, Sx, m);
+    note_launch();
+    return true;
+}
+// One CTA holds blocks of up to 200 KB.  Four CTAs are faster in complex64 from about 16 K
+// entries on (502 x 40: 195 us a level against 278 in one CTA; 257 x 26: about 10 more than the
+// 84 in one CTA), eight in FP64, where the products bound it (385 x 40: 549 us), and where four do
+// not hold the block.
 template <typename T>
 void launch_qr(cplx<T>* const* Y, int nq, int Sx, int m, cplx<T>** dev_ptr_scratch, cudaStream_t s) {
     cudaMemcpyAsync(dev_ptr_scratch, Y, sizeof(cplx<T>*) * nq, cudaMemcpyHostToDevice, s);
@@ -1163,26 +1201,8 @@ void launch_qr(cplx<T>* const* Y, int nq, int Sx, int m, cplx<T>** dev_ptr_scrat
     smem_limit_once(attr, k_qr<T>, 200 * 1024);
     const size_t bytes = sizeof(cplx<T>) * (size_t)Sx * (m + 1);   // padded rows
     const int staged = bytes <= (size_t)(200 * 1024) - 2048;
-    const size_t cbytes = sizeof(cplx<T>) * (size_t)((Sx + QR_CL - 1) / QR_CL) * (m + 1);
-    if (!staged && m <= 128 && cbytes <= (size_t)(200 * 1024) - 4096) {
-        static std::atomic<unsigned long long> attr_c{0};
-        smem_limit_once(attr_c, k_qr_cluster<T>, 200 * 1024);
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute at[1];
-        cfg.gridDim = dim3(nq * QR_CL);
-        cfg.blockDim = dim3(512);
-        cfg.dynamicSmemBytes = cbytes;
-        cfg.stream = s;
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = QR_CL;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        cudaLaunchKernelEx(&cfg, k_qr_cluster<T>, dev_ptr_scratch, Sx, m);
-        note_launch();
-        return;
-    }
+    if (sizeof(T) == 4 && Sx * (size_t)m >= 16384 && qr_cluster<T, 4>(nq, Sx, m, dev_ptr_scratch, s)) return;
+    if (!staged && qr_cluster<T, 8>(nq, Sx, m, dev_ptr_scratch, s)) return;
     k_qr<T><<<nq, 512, staged ? bytes : 0, s>>>(dev_ptr_scratch, Sx, m, staged);
     note_launch();
 }
