@@ -2452,7 +2452,9 @@ struct Solver final : SolverBase {
         return st;
     }
 
-    c128* staging_f() override { return res; }
+    // (not a buffer that k_start writes: bilinear rows read f at a point's neighbours, which
+    // other threads may have finished; ut is written after the right-hand side on every path)
+    c128* staging_f() override { return ut; }
     c128* staging_g() override { return gbuf; }
     c128* iterate() override { return u; }
     int npoints() const override { return Sy * Sx; }
