@@ -151,6 +151,6 @@ extern "C" hh_status hh_residual_noalloc(int dim, int n, double k, const void* d
     if (cudaMemcpyAsync(out, total, sizeof(out), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return HH_ECUDA;
-    *rel_res = out[1] > 0 ? std::sqrt(out[0] / out[1]) : 0.0;
+    *rel_res = out[1] == 0.0 ? 0.0 : std::sqrt(out[0] / out[1]);
     return HH_OK;
 }

@@ -312,6 +312,12 @@ static inline cudaError_t ck(cudaError_t e, cudaError_t& first) {
     return e;
 }
 
+// |r| / |b| from the squares: 0 for b = 0, not finite (no convergence) where b or r is not.
+static double rel_norm(double r2, double b2) { return b2 == 0.0 ? 0.0 : std::sqrt(r2 / b2); }
+// What the statistics give for it: a right-hand side with a NaN has no residual, and 0 stands
+// there as for b = 0; the status tells the two apart.
+static double rel_report(double rel, double b2) { return std::isnan(b2) ? 0.0 : rel; }
+
 static const int MAX_PART_BLOCKS = 304;   // 2 x 152 SMs
 static const int COARSE_BLOCKS = 64;      // partial blocks of a one-column coarse projection
 
@@ -1970,14 +1976,14 @@ struct Solver final : SolverBase {
         double rel_prev = -1.0;
         int it_prev = 0, chunks = 0;
         for (;;) {
-            rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;   // last FP64 residual
+            rel = rel_norm(h_norm[0], h_norm[2]);   // last FP64 residual
             if (hctl[0] == 2 || !std::isfinite(rel)) return HH_ENOCONV;
             if (hctl[0] == 1) return HH_OK;
             if (it >= P.max_iter) {
                 // the FP64 residual of the last iterate, for the report
                 gated_residual(ctl);
                 if (!read_norms(st)) return st;
-                rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;
+                rel = rel_norm(h_norm[0], h_norm[2]);
                 return hctl[0] == 1 ? HH_OK : HH_ENOCONV;
             }
             // Two chunks of 8 first: the residual of the first steps may grow before it
@@ -2036,7 +2042,7 @@ struct Solver final : SolverBase {
                 if (!read_norms(st)) return st;
                 if (start_settles(it, rel, st)) return st;
                 it = hc->it;
-                rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;
+                rel = rel_norm(h_norm[0], h_norm[2]);
                 if (!std::isfinite(rel) || rel < P.tol || it >= P.max_iter || hc->reason != CUT_TEST) {
                     cut_swap();   // the candidate stands in ut
                     mode = 1;
@@ -2060,7 +2066,7 @@ struct Solver final : SolverBase {
     // After the first read of the norms: whether the first residual, b itself (u = 0), ends the
     // solve (b = 0, a tolerance above 1, b not finite).
     bool start_settles(int& it, double& rel, hh_status& st) const {
-        const double r0 = h_norm[2] > 0 ? std::sqrt(h_norm[2] / h_norm[2]) : 0.0;
+        const double r0 = rel_norm(h_norm[2], h_norm[2]);
         if (std::isfinite(r0) && !(r0 < P.tol)) return false;
         it = 0;
         rel = r0;
@@ -2103,7 +2109,7 @@ struct Solver final : SolverBase {
                 }
                 if (h_gst[0].bad) return HH_ENOCONV;
                 it += h_gst[0].stop ? h_gst[0].jstop : h_gst[0].steps;
-                rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;
+                rel = rel_norm(h_norm[0], h_norm[2]);
                 if (!std::isfinite(rel)) return HH_ENOCONV;
                 if (rel < P.tol) return HH_OK;
                 if (it >= P.max_iter) return HH_ENOCONV;
@@ -2172,7 +2178,7 @@ struct Solver final : SolverBase {
                     zero(u, sizeof(c128) * (size_t)Sy * Sx);
                     return st;
                 }
-                rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;
+                rel = rel_norm(h_norm[0], h_norm[2]);
                 if (!std::isfinite(rel)) return HH_ENOCONV;
                 if (rel < P.tol) return HH_OK;
                 if (it >= P.max_iter) return HH_ENOCONV;
@@ -2207,7 +2213,7 @@ struct Solver final : SolverBase {
             if (!true_residual(gw, st)) return st;
             const double nbv = std::sqrt(std::max(h_norm[2], 0.0));
             const double beta = std::sqrt(std::max(h_norm[0], 0.0));
-            rel = nbv > 0 ? beta / nbv : 0.0;
+            rel = nbv == 0 ? 0.0 : beta / nbv;
             if (!std::isfinite(rel)) return HH_ENOCONV;
             if (rel < P.tol) return HH_OK;
             if (it >= P.max_iter) return HH_ENOCONV;
@@ -2290,7 +2296,7 @@ struct Solver final : SolverBase {
         cudaEventDestroy(e1);
         if (stt) {
             stt->iters = it;
-            stt->rel_res = rel;
+            stt->rel_res = rel_report(rel, h_norm[2]);
             stt->t_setup_ms = t_setup_ms;
             stt->t_solve_ms = t_solve_ms;
             stt->footprint_bytes = footprint;
@@ -2334,7 +2340,7 @@ struct Solver final : SolverBase {
         ck(cudaMemcpyAsync(h_norm, dnorm, 4 * sizeof(double), cudaMemcpyDeviceToHost, stream), cerr);
         hh_status st;
         if (!sync_check(st)) return st;
-        *rel = h_norm[2] > 0 ? std::sqrt(h_norm[0] / h_norm[2]) : 0.0;
+        *rel = rel_norm(h_norm[0], h_norm[2]);
         return HH_OK;
     }
 
@@ -2648,12 +2654,13 @@ struct BatchEngine {
     const CutCtl& ctl_of(const Prob& q) const { return ((const CutCtl*)(h_dn + ((char*)d_ctl - (char*)norms)))[q.slot]; }
     double rel_of(const Prob& q) const {
         const double b2 = q.p->h_norm[2], r2 = ((const double*)h_dn)[q.slot];
-        return b2 > 0 ? std::sqrt(r2 / b2) : 0.0;
+        return rel_norm(r2, b2);
     }
     // the problem leaves with the solution in x (the copy is complete after `settle`)
     void leave(Prob& q, hh_status st, const c128* x, std::vector<Prob>& done) {
         ck(cudaMemcpyAsync(q.uo, x, sizeof(c128) * (size_t)q.p->Sy * q.p->Sx, cudaMemcpyDeviceToDevice, stream), cerr);
         q.st = st;
+        q.rel = rel_report(q.rel, q.p->h_norm[2]);
         used[q.slot] = 0;
         done.push_back(q);
         q.p = nullptr;

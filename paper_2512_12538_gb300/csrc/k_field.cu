@@ -185,7 +185,7 @@ __global__ void k_residual_cast(const c128* __restrict__ x, const c128* __restri
             stop.nrm[0] = s2;
             stop.ctl[1] += 1;
             const double b2 = stop.nrm[2];
-            const double rel = b2 > 0 ? sqrt(s2 / b2) : 0.0;
+            const double rel = b2 == 0.0 ? 0.0 : sqrt(s2 / b2);
             if (!isfinite(rel)) stop.ctl[0] = 2;
             else if (rel < stop.tol) stop.ctl[0] = 1;
         }
@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(256) k_start(const c128* __restrict__ f, const
         *o.b2 = s2;
         if (o.r2) *o.r2 = s2;
         if (o.ctl) {   // [0] stop, [1] tests run: as after a residual (ResidStop)
-            const double rel = s2 > 0 ? sqrt(s2 / s2) : 0.0;
+            const double rel = s2 == 0.0 ? 0.0 : sqrt(s2 / s2);   // (not finite: not finite)
             o.ctl[0] = !isfinite(rel) ? 2 : rel < tol ? 1 : 0;
             o.ctl[1] = 1;
         }

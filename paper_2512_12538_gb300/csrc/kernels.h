@@ -45,7 +45,7 @@ void launch_sum(const double* part, int n, double* out, cudaStream_t s);
 // launch_residual_cast with the stopping test of the stationary iteration kept on the
 // device, in the same launch.  Unless ctl[0] is already set (then nothing is done):
 // y (may be null: not stored), yt and the partials as launch_residual_cast, then
-// nrm[0] = ||y||^2 (launch_sum's order), ctl[1] += 1, and with rel = sqrt(nrm[0] / nrm[2]) (0 when nrm[2] <= 0)
+// nrm[0] = ||y||^2 (launch_sum's order), ctl[1] += 1, and with rel = sqrt(nrm[0] / nrm[2]) (0 when nrm[2] is 0)
 // ctl[0] = 2 if rel is not finite, 1 if rel < tol.  ctl[0] is the gate of the next
 // step's launches; ticket is a device counter that is zero between launches.
 template <typename T>
