@@ -252,6 +252,14 @@ __device__ __forceinline__ void st_async(uint32_t dst, int v, uint32_t mbar) {
                  "r"(mbar)
                  : "memory");
 }
+// On the way out of a kernel whose wait gave up: long enough (20 us at 2 GHz; a remote store takes
+// about one) for the stores of other CTAs that were issued before a cluster barrier, and that
+// nobody counts any more, to arrive while this CTA's shared memory is still its own.  (A cluster
+// barrier orders no asynchronous stores; __nanosleep alone may return at once.)
+__device__ __forceinline__ void settle_remote_stores() {
+    const long long t0 = clock64();
+    while (clock64() - t0 < 40000) __nanosleep(500);
+}
 // 1D bulk copy global -> shared (TMA engine), completion signalled on `bar`.
 // dst, src 16-byte aligned; bytes a multiple of 16.
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {

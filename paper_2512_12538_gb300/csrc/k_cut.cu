@@ -1108,6 +1108,7 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
             ctl->ns[2] += (double)tC;
         }
     }
+    if (!ok) cp_async_wait_all();   // the panels a barrier that gave up left on their way
 }
 
 // ------------------------------------------------- the iteration on one cluster
@@ -1582,7 +1583,7 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
     // no block leaves while another's stores may still arrive (after a wait that gave up,
     // also those nobody waited for)
     cluster.sync();
-    if (!ok) __nanosleep(20000);
+    if (!ok) settle_remote_stores();
     cluster.sync();
 }
 

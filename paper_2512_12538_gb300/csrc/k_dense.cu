@@ -1772,7 +1772,7 @@ __global__ void __launch_bounds__(64 / CL * 32) k_gj_cluster(GjBatch bt) {
     if (c == 0) send();
     bool ok = true;
     for (int k = 0; ok && k < n; ++k) {
-        ok = __all_sync(0xffffffffu, mbar_wait_cluster_bounded(&s_mb[k], 0, GJ_WAIT));
+        ok = __all_sync(0xffffffffu, mbar_wait_cluster_bounded(&s_mb[k], 0, bt.wait));
         if (!ok) break;
         const int p = s_p[k], pl = p & 31, ps = p >> 5;
         const C ip = s_ip[k];
@@ -1794,7 +1794,10 @@ __global__ void __launch_bounds__(64 / CL * 32) k_gj_cluster(GjBatch bt) {
         if (c == k + 1 && c < n) send();
     }
     if (!ok && lane == 0) atomicExch(bt.err, DEV_TIMEOUT);
-    cluster.sync();                 // no store to this CTA is in flight any more
+    // a warp that saw every column arrive has no store to this CTA in flight any more; one that
+    // gave up keeps the CTA until what the others sent before the barrier has landed
+    cluster.sync();
+    if (!ok) settle_remote_stores();
     if (!ok || c >= n) return;
     c64* AT = (c64*)bt.AT[mat];
     const int pc = s_p[c];
@@ -1840,8 +1843,9 @@ static bool gj_cluster(const GjBatch& bt, int count, cudaStream_t s) {
     return true;
 }
 
-void launch_gj_inverse(const GjBatch& bt, int count, bool fp32, cudaStream_t s) {
+void launch_gj_inverse(GjBatch bt, int count, bool fp32, cudaStream_t s) {
     if (count < 1) return;
+    bt.wait = (uint32_t)std::min<long long>(wait_polls(GJ_WAIT), GJ_WAIT);
     if (bt.n >= 16 && bt.n <= 64) {
         if (fp32) gj_cluster<float, 16>(bt, count, s) || gj_cluster<float, 8>(bt, count, s);
         else gj_cluster<double, 16>(bt, count, s) || gj_cluster<double, 8>(bt, count, s);

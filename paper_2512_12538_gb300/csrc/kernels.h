@@ -232,9 +232,10 @@ struct GjBatch {
     void* AT[GJ_MAX_BATCH];   // complex64 copies of the inverses (entries may be NULL)
     int n;
     int* err;
+    uint32_t wait;            // polls of a wait before it gives up (set by the launcher)
 };
 // fp32: eliminate in FP32 (the complex64 form), else FP64.
-void launch_gj_inverse(const GjBatch& bt, int count, bool fp32, cudaStream_t s);
+void launch_gj_inverse(GjBatch bt, int count, bool fp32, cudaStream_t s);
 
 // ---- leaf kernels (k_leaf.cu) ------------------------------------------------------
 struct LeafTask {
