@@ -414,7 +414,6 @@ __device__ __noinline__ bool gm_arnoldi(const CutProb& P, const CutGmres& G, GmS
             M.beta = beta;
             if (rank == 0) {
                 G.alpha[0] = M.al[0];
-                *G.ls.st = GmresState{0, 0, 0, 0, 0.0, 0.0};
                 G.ls.g[0] = c128{beta, 0.0};
             }
         }
@@ -665,6 +664,9 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     GroupBar bar{bars + group, (unsigned)gsz, 0u, err, limit};
     bool ok = true;
+    // (before any wait: k_cut_gm_combine takes the number of columns from it, also of a cycle
+    // whose first wait gave up)
+    if (gm_steps && rank == 0 && tid == 0) *G.ls.st = GmresState{0, 0, 0, 0, 0.0, 0.0};
     for (int pi = group; ok && pi < nprob; pi += ngroups) {
         const int mode = modes ? modes[pi] : mode_all;
         if (!mode) continue;
@@ -1177,6 +1179,7 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
         for (int k = 0; k < 3; ++k) mbar_init(&s_mb[k], 1);
         fence_barrier_init();
     }
+    if (GM && rank == 0 && tid == 0) *G.ls.st = GmresState{0, 0, 0, 0, 0.0, 0.0};   // (as k_cut_steps)
     cluster.sync();
     const uint32_t mb = smem_u32(s_mb);
     unsigned phase = 0;   // steps this block has done: the mbarriers' parity

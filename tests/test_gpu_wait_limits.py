@@ -1,8 +1,8 @@
 """Every wait that hh_debug_set_wait_limit reaches runs out as HH_ETIMEOUT and leaves the
 context and the handle usable: the grid barrier of the whole-grid coarse corrections (n_i = 2,
 block leaves), the barriers of the cut-row steps on a grid and their exchanges on a cluster,
-alone and for more problems than clusters run at once, and the column waits of the coarse
-matrices' inverse in a set-up."""
+alone, in GMRES and for more problems than clusters run at once, and the column waits of the
+coarse matrices' inverse in a set-up."""
 import numpy as np
 import pytest
 
@@ -17,7 +17,10 @@ CASES = {
     "grid_barrier_inner2_gmres": (45, 2, 6, "mixed", 2, {"outer": "gmres"}),
     "grid_barrier_block": (45, 2, 6, "fp64", 1, {"leaf_solver": "block"}),
     "cut_cluster": (63, 2, 16, "mixed", 1, {}),
+    "cut_cluster_gmres": (63, 2, 16, "mixed", 1, {"outer": "gmres"}),
+    "cut_grid_mixed": (62, 3, 16, "mixed", 1, {"outer": "gmres"}),
     "cut_grid_fp64": (63, 2, 16, "fp64", 1, {}),
+    "cut_grid_fp64_gmres": (63, 2, 16, "fp64", 1, {"outer": "gmres"}),
 }
 
 
