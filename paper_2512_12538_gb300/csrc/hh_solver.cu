@@ -2649,6 +2649,8 @@ struct BatchEngine {
         ck(cudaStreamSynchronize(stream), cerr);
         if (cerr != cudaSuccess) return HH_ECUDA;
         const int e = *(const int*)(h_dn + ((char*)berr - (char*)norms));
+        // (the engine of a server outlives this round's problems: the next ones start clear)
+        if (e != DEV_OK) ck(cudaMemsetAsync(berr, 0, sizeof(int), stream), cerr);
         return e == DEV_TIMEOUT ? HH_ETIMEOUT : e != DEV_OK ? HH_ECUDA : HH_OK;
     }
     const CutCtl& ctl_of(const Prob& q) const { return ((const CutCtl*)(h_dn + ((char*)d_ctl - (char*)norms)))[q.slot]; }

@@ -106,3 +106,35 @@ def test_a_batch_whose_wait_runs_out(hh, no_wait, count, precision):
         no_wait(False)
         for h in hs:
             hh.hh_destroy(h)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_a_server_serves_on_after_a_wait_that_ran_out(hh, no_wait, precision):
+    """The set-ups of these requests have no limited wait (ranks below the cluster inverse's,
+    transforms on CUDA cores), so it is a round of the server's engine that gives up."""
+    import time
+    n = 63
+    S = n + 2
+    p = hh.make_params(2, n, 20.0, 2, 2, 7, 6, 1, 1e-10, 400, precision, 1, flags=hh.HH_FLAG_CUDA_CORE_SWEEPS)
+    f = torch.from_numpy(random_complex((S, S), 90)).cuda()
+    g = torch.zeros((4, S), dtype=torch.complex128, device="cuda")
+    srv = hh.hh_server_create(2 << 30, 4)
+
+    def serve():
+        u = torch.empty_like(f)
+        torch.cuda.synchronize()
+        ticket, t0, res = hh.hh_server_submit(srv, p, f, g, u), time.time(), None
+        while res is None:
+            assert time.time() - t0 < 60.0
+            res = hh.hh_server_poll(srv, ticket)
+        return res[0]
+
+    try:
+        assert serve() == hh.HH_OK
+        no_wait(True)
+        assert serve() == hh.HH_ETIMEOUT
+        no_wait(False)
+        assert [serve() for _ in range(3)] == [hh.HH_OK] * 3
+    finally:
+        no_wait(False)
+        hh.hh_server_destroy(srv)
