@@ -669,14 +669,21 @@ static void sweep_cfg(const LeafTask* d_tasks, int ntasks, int b_max, int Sx, in
         prow = (prow + 1) / 2;
         slot_bytes = align_up((size_t)prow * ldx * esz, 128);
     }
+    // Halving overshoots on the tallest complex64 bands (143 rows and more: five or six pieces of
+    // about 36 rows, where four of 36 to 43 fit): take the largest pieces the kernel needs.  With
+    // that every band leaf_block_bmax accepts has a sweep (169 rows: three slots of 57 KB).
+    if ((b_max + prow - 1) / prow > MAXP) {
+        prow = (b_max + MAXP - 1) / MAXP;
+        slot_bytes = align_up((size_t)prow * ldx * esz, 128);
+        if (over()) {
+            int one = DEV_BADARG;
+            cudaMemcpyAsync(err, &one, sizeof(int), cudaMemcpyHostToDevice, s);
+            return;
+        }
+    }
     while ((nslot + 1) * slot_bytes + vbytes <= budget && nslot < SW_SLOTS) ++nslot;
     const size_t sm = nslot * slot_bytes + vbytes;
     const int np = (b_max + prow - 1) / prow;
-    if (np > MAXP) {          // band too tall for this kernel
-        int one = DEV_BADARG;
-        cudaMemcpyAsync(err, &one, sizeof(int), cudaMemcpyHostToDevice, s);
-        return;
-    }
     if (np == 1) sweep_go<T, NC, 1>(d_tasks, ntasks, Sx, nrhs, nslot, prow, slot_bytes, sm, err, s);
     else sweep_go<T, NC, MAXP>(d_tasks, ntasks, Sx, nrhs, nslot, prow, slot_bytes, sm, err, s);
 }
