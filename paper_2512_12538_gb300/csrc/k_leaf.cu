@@ -14,6 +14,7 @@
 //        outwards  x_i = y_i + X_i W x_{i+1}   (right of m: W x_{i-1}).
 // 1D leaf (Sx = 1): the same recursion with 1 x 1 blocks along the band's rows.
 #include <algorithm>
+#include <atomic>
 
 #include <cooperative_groups.h>
 
@@ -31,6 +32,7 @@ int leaf_ldx(int b, int elem_bytes) {
 static constexpr uint32_t WAIT_LIMIT = 1u << 21;   // bounded mbarrier polls (~0.1-0.3 s)
 static constexpr int MAXP = 4;                       // row pieces per step in the sweep
 static constexpr int SW_SLOTS = 12;                  // pieces in flight in the sweep, at most
+static constexpr int SW_SMEM = 220 * 1024;           // shared memory of a sweep block, at most
 
 // ------------------------------------------------------------- factorisation (2D)
 template <typename T>
@@ -310,7 +312,10 @@ int leaf_block_bmax(int elem_bytes) {
 template <typename T, int RS, int NW>
 static void factor_reg(const LeafTask* d_tasks, int ntasks, int b_max, int Sx, double kh, int* err, cudaStream_t s) {
     const size_t sm = sizeof(cplx<T>) * (size_t)b_max * (b_max | 1);
-    cudaFuncSetAttribute(k_factor2d_reg<T, RS, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    // (a kernel's limit is set once, to its own maximum: problems are set up from several host
+    // threads, and one with shorter bands must not lower another's)
+    static std::atomic<unsigned long long> attr{0};
+    smem_limit_once(attr, k_factor2d_reg<T, RS, NW>, (int)sizeof(cplx<T>) * RS * 32 * (RS * 32 | 1));
     for (int mid = 0; mid < 2; ++mid) {       // the two chains, then the middle column
         k_factor2d_reg<T, RS, NW><<<dim3(ntasks, 2 - mid), NW * 32, sm, s>>>(d_tasks, Sx, kh, mid, err);
         note_launch();
@@ -333,7 +338,9 @@ void launch_factor(const LeafTask* d_tasks, int ntasks, int b_max, int Sx, doubl
         if constexpr (sizeof(T) == 4) factor_reg<T, 4, 32>(d_tasks, ntasks, b_max, Sx, kh, err, s);
     } else {
         const size_t sm = sizeof(cplx<T>) * ((size_t)b_max * b_max + 2 * b_max) + sizeof(int) * b_max;
-        cudaFuncSetAttribute(k_factor2d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        static std::atomic<unsigned long long> attr{0};
+        const int bm = leaf_block_bmax((int)sizeof(cplx<T>));
+        smem_limit_once(attr, k_factor2d<T>, (int)sizeof(cplx<T>) * (bm * bm + 2 * bm) + (int)sizeof(int) * bm);
         for (int mid = 0; mid < 2; ++mid) {
             k_factor2d<T><<<dim3(ntasks, 2 - mid), 256, sm, s>>>(d_tasks, Sx, kh, mid, err);
             note_launch();
@@ -648,7 +655,8 @@ template <typename T, int NC, int NP>
 static void sweep_go(const LeafTask* d_tasks, int ntasks, int Sx, int nrhs, int nslot, int prow, size_t slot_bytes,
                      size_t sm, int* err, cudaStream_t s) {
     const int threads = ((prow * SW_G + 31) / 32) * 32;
-    cudaFuncSetAttribute(k_sweep2d<T, NC, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    static std::atomic<unsigned long long> attr{0};
+    smem_limit_once(attr, k_sweep2d<T, NC, NP>, SW_SMEM);
     k_sweep2d<T, NC, NP><<<dim3(2 * ((nrhs + NC - 1) / NC), ntasks), threads, sm, s>>>(
         d_tasks, Sx, nrhs, nslot, prow, slot_bytes / sizeof(cplx<T>), err);
     note_launch();
@@ -657,7 +665,7 @@ template <typename T, int NC>
 static void sweep_cfg(const LeafTask* d_tasks, int ntasks, int b_max, int Sx, int nrhs, int* err, cudaStream_t s) {
     const int esz = (int)sizeof(cplx<T>);
     const int ldx = leaf_ldx(b_max, esz);
-    const size_t budget = 220 * 1024;
+    const size_t budget = SW_SMEM;
     const size_t vbytes = 3 * (size_t)ldx * NC * esz + 8 * SW_SLOTS + 128;
     int prow = std::min(b_max, 1024 / SW_G), nslot = 3;
     size_t slot_bytes = align_up((size_t)prow * ldx * esz, 128);
