@@ -596,7 +596,8 @@ struct Solver final : SolverBase {
             cp.D = D;
             cp.q1 = q1();
             cp.kh = kh;
-            cut_smem = cut_plan<T>(cp, b_max);
+            cut_smem = cut_plan<T>(cp, b_max, true);
+            if (cp.cl && !cut_cluster_ready(cut_smem)) cut_smem = cut_plan<T>(cp, b_max, false);
             cut = cut_smem > 0;
         }
         edge = cut && edge_rows_fit<T>(Sx);

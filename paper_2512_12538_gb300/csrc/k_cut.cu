@@ -1788,12 +1788,12 @@ static bool cluster_form(CutProb& P, int b_max) {
            (2 * P.L) * P.r <= 2 * CUT_KMAX && sizeof(c64) * cc_layout(P).total <= (size_t)CUT_SMEM;
 }
 template <typename T>
-size_t cut_plan(CutProb& P, int b_max) {
+size_t cut_plan(CutProb& P, int b_max, bool cluster) {
     const size_t c = sizeof(cplx<T>), cap = CUT_SMEM;
     const int NL = P.ncut + 1;
     P.res = P.dist = 0;
     P.nbi = 1;
-    P.cl = sizeof(T) == 4 && cluster_form(P, b_max);
+    P.cl = cluster && sizeof(T) == 4 && cluster_form(P, b_max);
     if (P.cl) return c * cc_layout(P).total;
     P.XC = std::min(64, std::max(8, (P.ncut * P.Sx + 147) / 148));
     P.nch = (P.Sx + P.XC - 1) / P.XC;
@@ -1845,7 +1845,14 @@ static int cluster_count(size_t smem) {
     }
     return n;
 }
-bool cut_cluster_ready(size_t smem) { return cluster_count(smem) > 0; }
+bool cut_cluster_ready(size_t smem) {
+    int n = 0;
+    if (cudaGetDeviceCount(&n) != cudaSuccess || n < 1) {   // planning without a device (hh_footprint)
+        cudaGetLastError();
+        return true;
+    }
+    return cluster_count(smem) > 0;
+}
 template <typename T>
 bool launch_cut_steps(const CutProb* probs, int nprob, int group, bool cl, size_t smem, const int* modes, int mode_all,
                       unsigned* bars, int max_groups, int* err, int prof, cudaStream_t s, int max_steps,
@@ -1926,7 +1933,7 @@ void launch_cut_update(const CutUpdJob* jobs, int njobs, int nleaf_max, int own_
     template void launch_cut_panels<T>(const CutCpEntry*, int, const CutEpEntry*, int, int, int, OpGeom, cudaStream_t); \
     template void launch_cut_gram<T>(const CutGramPair*, int, const CutGramDest*, int, int, int, c128*, cudaStream_t); \
     template void launch_cut_minv<T>(const CutMinv*, int, int, int, int, const c128*, c128*, cplx<T>*, int, cudaStream_t); \
-    template size_t cut_plan<T>(CutProb&, int);                                                                       \
+    template size_t cut_plan<T>(CutProb&, int, bool);                                                                       \
     template bool launch_cut_steps<T>(const CutProb*, int, int, bool, size_t, const int*, int, unsigned*, int, int*, int,   \
                                       cudaStream_t, int, const CutGmres*, int);                                                                  \
     template void launch_cut_lines<T>(const CutProb*, int, const int*, int, int, int, cudaStream_t);                  \

@@ -1817,8 +1817,10 @@ static bool gj_cluster(const GjBatch& bt, int count, cudaStream_t s) {
                                         64 * 64 * (int)sizeof(cplx<R>)) == cudaSuccess &&
                    (CL <= 8 || cudaFuncSetAttribute(k_gj_cluster<R, CL>, cudaFuncAttributeNonPortableClusterSizeAllowed,
                                                     1) == cudaSuccess);
-        }))
+        })) {
+        cudaGetLastError();
         return false;
+    }
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     cfg.gridDim = dim3(count * CL);
@@ -1838,7 +1840,10 @@ static bool gj_cluster(const GjBatch& bt, int count, cudaStream_t s) {
             return false;
         }
     }
-    cudaLaunchKernelEx(&cfg, k_gj_cluster<R, CL>, bt);
+    if (cudaLaunchKernelEx(&cfg, k_gj_cluster<R, CL>, bt) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
     note_launch();
     return true;
 }
@@ -1847,9 +1852,10 @@ void launch_gj_inverse(GjBatch bt, int count, bool fp32, cudaStream_t s) {
     if (count < 1) return;
     bt.wait = (uint32_t)std::min<long long>(wait_polls(GJ_WAIT), GJ_WAIT);
     if (bt.n >= 16 && bt.n <= 64) {
-        if (fp32) gj_cluster<float, 16>(bt, count, s) || gj_cluster<float, 8>(bt, count, s);
-        else gj_cluster<double, 16>(bt, count, s) || gj_cluster<double, 8>(bt, count, s);
-        return;
+        // (one block a matrix where no cluster can be scheduled)
+        if (fp32 ? gj_cluster<float, 16>(bt, count, s) || gj_cluster<float, 8>(bt, count, s)
+                 : gj_cluster<double, 16>(bt, count, s) || gj_cluster<double, 8>(bt, count, s))
+            return;
     }
     const int n = bt.n;
     const size_t es = fp32 ? sizeof(c64) : sizeof(c128);

@@ -392,11 +392,13 @@ size_t cut_m_packed(int L, int r);
 template <typename T>
 void launch_cut_minv(const CutMinv* prs, int n, int D, int L, int p2, const c128* G, c128* M, cplx<T>* MT, int tr,
                      cudaStream_t s);
-// whether the cluster form can run with this much shared memory on the current device
+// whether the cluster form can run with this much shared memory on the current device (true
+// without one)
 bool cut_cluster_ready(size_t smem);
-// fills the items of P; returns the steps' shared memory, 0 if the lines do not fit
+// fills the items of P; returns the steps' shared memory, 0 if the lines do not fit; cluster:
+// the cluster form may be taken
 template <typename T>
-size_t cut_plan(CutProb& P, int b_max);
+size_t cut_plan(CutProb& P, int b_max, bool cluster);
 // Flexible GMRES on the cut rows: its vectors and the least-squares problem.
 struct CutGmres {
     c128 *V, *alpha;           // [mk + 1][nG], [mk + 1]
