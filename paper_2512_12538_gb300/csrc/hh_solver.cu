@@ -487,16 +487,18 @@ struct Solver final : SolverBase {
     EigTask *d_etasks_cin = nullptr, *d_etasks_cout = nullptr;   // full residual in, every row out
     std::vector<CT*> EF0;       // the round's transformed residual
     CT *cut_Cp = nullptr, *cut_Ep = nullptr, *cut_MT = nullptr;
-    c128 *cut_E64 = nullptr, *cut_G = nullptr, *cut_M64 = nullptr, *cut_part = nullptr;
+    c128 *cut_E64 = nullptr, *cut_G = nullptr, *cut_M64 = nullptr;   // (of the set-up alone)
     unsigned char* d_cut_tab = nullptr;
-    size_t cut_tab_bytes = 0, cut_pairs_max = 0;
+    size_t cut_tab_bytes = 0;
     struct CutLevel {           // the panel and product entries of one level's nodes (device)
         CutCpEntry* cpe;
         CutEpEntry* epe;
         CutGramPair* prs;
         CutGramDest* dst;
         CutMinv* minv;
-        int ncp, nep, nprs, ndst, nminv;
+        int ncp, nep, nminv;
+        struct Share { int p0, np, d0, nd; };   // pairs and destinations of one product launch
+        std::vector<Share> shares;
     };
     std::vector<CutLevel> clev;
     // the set-up's sub-level solves from the interface rows (k_edge.cu): tasks per level
@@ -506,7 +508,6 @@ struct Solver final : SolverBase {
     std::vector<std::vector<EdgeTask>> h_edge;
     std::vector<CT*> Erows, Evin, Epd;
     std::vector<c128*> Ey;
-    c128* edge_part = nullptr;
     std::vector<EigTask> h_cin, h_cout;   // host copies of the transform tasks (batched solves)
     // flexible GMRES
     int mk = 0;                                   // restart length
@@ -618,6 +619,7 @@ struct Solver final : SolverBase {
                 q.id = lf;
                 q.ra = nodes[lf].ra;
                 q.kin = q.kedge = first ? 1 : 0;
+                q.mo = cut_m_offset(lf, L, r);
                 q.C = C[lf];
                 q.N = pts(lf);
                 lf = nodes[lf].child[first ? 1 : 0];
@@ -733,7 +735,6 @@ struct Solver final : SolverBase {
         cp.leaf = (const CutLeaf*)put(lf.data(), sizeof(CutLeaf) * lf.size());
         cp.node = (const CutNode*)put(nv.data(), sizeof(CutNode) * nv.size());
         clev.assign(L, CutLevel{});
-        cut_pairs_max = 0;
         const size_t Nx = (size_t)Sx;
         for (int l = 0; l < L; ++l) {
             std::vector<CutCpEntry> ce;
@@ -798,8 +799,7 @@ struct Solver final : SolverBase {
                 if (t < (1 << l) - 1) add_e((t + 1) * span - 1, 1, 0, 1, 0);
                 mv.push_back({p, p, Ainv[p]});
             }
-            // the diagonal blocks first, then the others of the same rows (one launch each)
-            const int ndiag = (int)mv.size();
+            // the diagonal blocks, then the others of the same rows
             for (int p : lev[l])
                 for (int ls = l + 1; ls < L; ++ls)
                     for (int s2 : lev[ls])
@@ -810,8 +810,8 @@ struct Solver final : SolverBase {
                 const auto [p, kp, q, kq] = kv.first;
                 if (p == q && coarse_fp32()) continue;   // that variant's FP32 products: the full kernel
                 CutGramDest d;
-                d.out = cut_G + ((size_t)p * 2 * r + kp * r) * cp.D + (size_t)q * 2 * r + kq * r;
-                d.ld = cp.D;
+                d.ld = cut_m_len(l, L, r);
+                d.out = cut_G + cut_m_offset(p, L, r) + (size_t)(kp * r) * d.ld + cut_m_col(p, q, r) + kq * r;
                 if (p == q) {
                     d.out = Ainv[p] + (size_t)kp * r * 2 * r + kq * r;
                     d.ld = 2 * r;
@@ -828,16 +828,20 @@ struct Solver final : SolverBase {
                     pr.push_back(x);
                 }
             }
-            (void)ndiag;
             CutLevel& cl = clev[l];
-            cl.ncp = (int)ce.size(); cl.nep = (int)ee.size(); cl.nprs = (int)pr.size(); cl.ndst = (int)ds.size();
-            cl.nminv = (int)mv.size();
+            cl.ncp = (int)ce.size(); cl.nep = (int)ee.size(); cl.nminv = (int)mv.size();
+            // as many destinations a launch as the partial sums' scratch holds
+            for (int d = 0; d < (int)ds.size(); ++d) {
+                if (cl.shares.empty() || cut_gram_scratch(cl.shares.back().np + ds[d].count) > part_bytes())
+                    cl.shares.push_back({ds[d].first, 0, d, 0});
+                cl.shares.back().np += ds[d].count;
+                cl.shares.back().nd += 1;
+            }
             cl.cpe = (CutCpEntry*)put(ce.data(), sizeof(CutCpEntry) * ce.size());
             cl.epe = (CutEpEntry*)put(ee.data(), sizeof(CutEpEntry) * ee.size());
             cl.prs = (CutGramPair*)put(pr.data(), sizeof(CutGramPair) * pr.size());
             cl.dst = (CutGramDest*)put(ds.data(), sizeof(CutGramDest) * ds.size());
             cl.minv = (CutMinv*)put(mv.data(), sizeof(CutMinv) * mv.size());
-            cut_pairs_max = std::max(cut_pairs_max, pr.size());
         }
         d_edge.assign(L + 1, nullptr);
         d_edge_out.assign(L + 1, nullptr);
@@ -893,11 +897,39 @@ struct Solver final : SolverBase {
     void cut_level_products(int l) {
         const CutLevel& cl = clev[l];
         launch_cut_panels<T>(cl.cpe, cl.ncp, cl.epe, cl.nep, Sx, r, geom(0), stream);
-        if (cl.nprs) launch_cut_gram<T>(cl.prs, cl.nprs, cl.dst, cl.ndst, Sx, r, cut_part, stream);
+        for (const auto& s : cl.shares)
+            launch_cut_gram<T>(cl.prs + s.p0, s.np, s.p0, cl.dst + s.d0, s.nd, Sx, r, partial, stream);
     }
     void cut_level_minv(int l) {
         const CutLevel& cl = clev[l];
-        launch_cut_minv<T>(cl.minv, cl.nminv, cp.D, L, 2 * r, cut_G, cut_M64, cut_MT, cp.cl, stream);
+        launch_cut_minv<T>(cl.minv, cl.nminv, L, 2 * r, cut_G, cut_M64, cut_MT, cp.cl, stream);
+    }
+    // bytes of `partial`
+    static size_t part_bytes() { return (size_t)(MAX_PART_BLOCKS + 1) * 64 * 64 * sizeof(c128); }
+
+    // What a set-up on the cut rows needs and a solve does not: the FP64 rows of A C, the coarse
+    // system and its inverse (packed by subtree, as M), and, one level of the hierarchy at a
+    // time, the rows of its children's sketches.
+    void plan_cut_matrices(Arena& a, size_t nep) {
+        cut_E64 = a.take<c128>(nep);
+        cut_G = a.take<c128>(cut_m_packed(L, r));
+        cut_M64 = a.take<c128>(cut_m_packed(L, r));
+    }
+    void plan_edge_scratch(Arena& a) {
+        const size_t off = a.off;
+        size_t end = off;
+        for (int l = 1; l <= L; ++l) {
+            a.off = off;
+            for (int id : lev[l]) {
+                Erows[id] = a.take<CT>(4 * (size_t)Sx * m);
+                Evin[id] = a.take<CT>(2 * (size_t)Sx * m);
+                if (l == L) continue;   // (a leaf child has no path)
+                Epd[id] = a.take<CT>(edge_pd_elems(L - l, r, m));
+                Ey[id] = a.take<c128>((size_t)(L - l) * 2 * r * m);
+            }
+            end = std::max(end, a.off);
+        }
+        a.off = end;
     }
 
     size_t plan(char* base) override {
@@ -917,12 +949,38 @@ struct Solver final : SolverBase {
         gbuf = a.take<c128>(4 * (size_t)S);
         khr_dev = P.k_rows ? a.take<double>(S) : nullptr;
         RT = a.take<CT>(N * nmax);
+        // Vs and R, the inputs and residuals of whole-grid sub-level solves.  A set-up from the
+        // interface rows has none, so what it alone needs lies in the same storage; the calls
+        // that use them afterwards write all they read.
+        size_t ncp = 0, nep = 0, nvs = 0;
+        if (cut) cut_panel_sizes(ncp, nep);
+        Erows.assign(nn, nullptr); Evin.assign(nn, nullptr); Epd.assign(nn, nullptr); Ey.assign(nn, nullptr);
+        for (int id = 1; id < nn; ++id)
+            nvs += (nodes[id].leaf() ? 1 : 2) * align_up(sizeof(CT) * pts(id) * nmax, 256);
+        Arena sc;
+        if (edge) {
+            plan_cut_matrices(sc, nep);
+            plan_edge_scratch(sc);
+        }
+        Arena vs;
+        vs.base = (char*)a.take<unsigned char>(std::max(nvs, sc.off));
+        for (int id = 1; id < nn; ++id) {
+            Vs[id] = vs.take<CT>(pts(id) * nmax);
+            if (!nodes[id].leaf()) R[id] = vs.take<CT>(pts(id) * nmax);
+        }
+        if (edge) {
+            sc = Arena();
+            sc.base = vs.base;
+            plan_cut_matrices(sc, nep);
+            plan_edge_scratch(sc);
+        } else if (cut) {
+            plan_cut_matrices(a, nep);
+        }
         for (auto& nd : nodes) {
             const int id = nd.id;
             const size_t np = pts(id);
             if (id != 0) {
                 W[id] = a.take<CT>(np * nmax);
-                Vs[id] = a.take<CT>(np * nmax);
                 Om[id] = a.take<CT>((size_t)Sx * nmax);
                 Z[id] = a.take<CT>((size_t)Sx * nmax);
                 Vc[id] = a.take<CT>((size_t)Sx * std::max(r, 1));
@@ -931,7 +989,6 @@ struct Solver final : SolverBase {
                 lam[id] = a.take<double>(m);
             }
             if (!nd.leaf()) {
-                if (id != 0) R[id] = a.take<CT>(np * nmax);
                 C[id] = a.take<CT>(np * 2 * r);
                 Ainv[id] = a.take<c128>((size_t)4 * r * r);
                 AinvT[id] = sizeof(CT) == sizeof(c128) ? (CT*)Ainv[id] : a.take<CT>((size_t)4 * r * r);
@@ -957,7 +1014,7 @@ struct Solver final : SolverBase {
         cur_in[0] = RT;
         // per-block partial sums of up to 64 x 64 outputs, plus the block of sums that
         // launch_ip_reduce writes just past the partials
-        partial = a.take<c128>((size_t)(MAX_PART_BLOCKS + 1) * 64 * 64);
+        partial = (c128*)a.take<unsigned char>(part_bytes());
         npart = a.take<double>(2048);
         // [0] ||r||^2 (FP64 residual), [1] ||r||^2 (recursive residual), [2..4) ||b||^2,
         // [4..6) the device status words, [6..10) the device-tested loop's control words
@@ -989,15 +1046,10 @@ struct Solver final : SolverBase {
         if (mk > 0 && !cut) plan_gmres_ls(a);
         d_ptrs = a.take<void*>(3 * 64);
         if (cut) {
-            size_t ncp = 0, nep = 0;
-            cut_panel_sizes(ncp, nep);
             EF0.assign(nn, nullptr);
-            for (int id : lev[L]) EF0[id] = a.take<CT>(pts(id));
+            for (int id : lev[L]) EF0[id] = Vs[id];   // a solve's own; no call that uses Vs runs in it
             cut_Cp = a.take<CT>(ncp);
             cut_Ep = a.take<CT>(nep);
-            cut_E64 = a.take<c128>(nep);
-            cut_G = a.take<c128>((size_t)cp.D * cp.D);
-            cut_M64 = a.take<c128>((size_t)cp.D * cp.D);
             cut_MT = a.take<CT>(cut_m_packed(L, r));
             const size_t row = 2 * (size_t)cp.ncut * Sx;
             cp.v = a.take<CT>(row);
@@ -1008,23 +1060,11 @@ struct Solver final : SolverBase {
             cp.d = a.take<CT>(cp.D);
             cp.y = a.take<CT>(cp.D);
             cp.yacc = a.take<CT>(cp.D);
-            cp.npart = a.take<float>((size_t)cp.nB * 8);
+            cp.npart = a.take<float>(cp.nB);
             cbar = a.take<unsigned>(2);
-            Erows.assign(nn, nullptr); Evin.assign(nn, nullptr); Epd.assign(nn, nullptr); Ey.assign(nn, nullptr);
-            if (edge) {
-                for (int id = 1; id < nn; ++id) {
-                    const int np = L - nodes[id].level;
-                    Erows[id] = a.take<CT>(4 * (size_t)Sx * m);
-                    Evin[id] = a.take<CT>(2 * (size_t)Sx * m);
-                    Epd[id] = a.take<CT>(edge_pd_elems(np, r, m));
-                    Ey[id] = a.take<c128>((size_t)np * 2 * r * m);
-                }
-                edge_part = (c128*)a.take<unsigned char>(edge_gram_scratch(1 << L));
-            }
             d_cut = a.take<CutProb>(1);
-            if (!base) cut_tab_bytes = cut_tables(false);   // also sets cut_pairs_max
+            if (!base) cut_tab_bytes = cut_tables(false);
             d_cut_tab = a.take<unsigned char>(cut_tab_bytes);
-            cut_part = (c128*)a.take<unsigned char>(cut_gram_scratch((int)cut_pairs_max));
         }
         return align_up(a.off, 256);
     }
@@ -1455,7 +1495,7 @@ struct Solver final : SolverBase {
         pend(PC_RECUR);
         if (l < L) {
             pbeg(PC_COARSE_MC);
-            launch_edge_path<T>(d_edge[l], nch, Sx, m, r, cp.D, cut_M64, geom(0), adj, true, stream);
+            launch_edge_path<T>(d_edge[l], nch, L, Sx, m, r, cut_M64, geom(0), adj, true, stream);
             pend(PC_COARSE_MC);
         }
     }
@@ -1476,7 +1516,9 @@ struct Solver final : SolverBase {
         launch_edge_place<T>(d_edge[l], nch, Sx, m, kh, q1(), stream);
         edge_pass(l, 1);
         launch_edge_conj<T>(d_edge[l], nch, Sx, m, stream);
-        launch_edge_gram<T>(d_edge[l], nch, Sx, m, edge_part, stream);
+        const int ng = (int)(part_bytes() / edge_gram_scratch(1));   // children the scratch holds
+        for (int c0 = 0; c0 < nch; c0 += ng)
+            launch_edge_gram<T>(d_edge[l] + c0, std::min(ng, nch - c0), Sx, m, partial, stream);
         pbeg(PC_JACOBI);
         launch_heig(gs.data(), us.data(), ls.data(), nch, m, r, d_ptrs, stream);
         pend(PC_JACOBI);
@@ -1501,7 +1543,7 @@ struct Solver final : SolverBase {
         pend(PC_TOUT);
         if (l < L) {
             pbeg(PC_COARSE_MC);
-            launch_edge_path<T>(d_edge[l], nch, Sx, r, r, cp.D, cut_M64, geom(0), 0, false, stream);
+            launch_edge_path<T>(d_edge[l], nch, L, Sx, r, r, cut_M64, geom(0), 0, false, stream);
             for (auto& t : h_edge[l])
                 for (int u = 0; u < t.npath; ++u) {
                     const Node& q = nodes[t.path[u].id];
@@ -1664,7 +1706,7 @@ struct Solver final : SolverBase {
         }
         if (cut) {
             cut_tables(true);
-            zero(cut_G, sizeof(c128) * (size_t)cp.D * cp.D);
+            zero(cut_G, sizeof(c128) * cut_m_packed(L, r));
         }
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);

@@ -247,12 +247,13 @@ __global__ void __launch_bounds__(256) k_cut_gram(const CutGramPair* __restrict_
 #pragma unroll
         for (int v = 0; v < 2; ++v) o[(ti + 16 * u) * 32 + tj + 16 * v] = acc[u][v];
 }
-__global__ void __launch_bounds__(256) k_cut_gram_red(const CutGramDest* __restrict__ ds, int r, const c128* part) {
+__global__ void __launch_bounds__(256) k_cut_gram_red(const CutGramDest* __restrict__ ds, int first0, int r,
+                                                      const c128* part) {
     const CutGramDest d = ds[blockIdx.x];
     for (int t = threadIdx.x; t < r * r; t += 256) {
         const int i = t / r, j = t - i * r;
         c128 s = {0, 0};
-        for (int k = d.first * GRAM_SPLIT; k < (d.first + d.count) * GRAM_SPLIT; ++k)
+        for (int k = (d.first - first0) * GRAM_SPLIT; k < (d.first - first0 + d.count) * GRAM_SPLIT; ++k)
             s = s + part[(size_t)k * 1024 + i * 32 + j];
         d.out[(size_t)i * d.ld + j] = s;
     }
@@ -276,21 +277,19 @@ __device__ __forceinline__ int cut_m_row(int e, int L, int r, int& l, int& t) {
 // chains; a set-up of 1023^2 at 2r = 64 took 1.4 ms longer with one block a pair).
 static constexpr int MINV_ROWS = 4;
 template <typename T>
-__global__ void __launch_bounds__(256) k_cut_minv(const CutMinv* __restrict__ prs, int D, int L, int p2,
+__global__ void __launch_bounds__(256) k_cut_minv(const CutMinv* __restrict__ prs, int L, int p2,
                                                   const c128* __restrict__ G, c128* M, cplx<T>* MT, int tr) {
     __shared__ c128 ai[MINV_ROWS][64], xs[MINV_ROWS][64];
     const CutMinv e = prs[blockIdx.x];
-    const size_t rp = (size_t)e.p * p2, cs = (size_t)e.s * p2;
     const int i0 = blockIdx.y * MINV_ROWS, ni = min(MINV_ROWS, p2 - i0);
     if (ni <= 0) return;
-    // M in the basis precision is packed: rows of p's subtree level by level
-    int l, t;
-    cplx<T>* mt = MT + cut_m_row(e.p * p2, L, p2 / 2, l, t);
-    const int len = p2 * ((1 << (L - l)) - 1), ls = 31 - __clz(e.s + 1);
-    const int k0 = p2 * ((1 << (ls - l)) - 1 + (e.s + 1 - (1 << ls)) - (t << (ls - l)));
+    // all packed by subtree; this pair's first entry in p's rows
+    const int r = p2 / 2, len = cut_m_len(cut_level_of(e.p), L, r), k0 = cut_m_col(e.p, e.s, r);
+    const size_t op = cut_m_offset(e.p, L, r);
+    cplx<T>* mt = MT + op;
     // (tr: the cluster form's order, transposed within the node's rows)
     auto put = [&](int i, int j, c128 v) {
-        M[(rp + i) * D + cs + j] = v;
+        M[op + (size_t)i * len + k0 + j] = v;
         mt[tr ? (size_t)(k0 + j) * p2 + i : (size_t)i * len + k0 + j] = cvt<T>(v);
     };
     for (int q = threadIdx.x; q < ni * p2; q += 256) {
@@ -303,16 +302,19 @@ __global__ void __launch_bounds__(256) k_cut_minv(const CutMinv* __restrict__ pr
     const bool on = i < ni && j < p2;
     c128 acc = {0, 0};
     for (int q = e.s; q != e.p; q = (q - 1) >> 1) {   // s and its ancestors below p
+        const int lenq = cut_m_len(cut_level_of(q), L, r);
+        const c128* gq = G + op + cut_m_col(e.p, q, r) + j;
+        const c128* mq = M + cut_m_offset(q, L, r) + cut_m_col(q, e.s, r) + j;
         __syncthreads();
         c128 h = {0, 0};
         if (on)
 #pragma unroll 8
-            for (int k = 0; k < p2; ++k) cfma(h, ai[i][k], G[(rp + k) * D + (size_t)q * p2 + j]);
+            for (int k = 0; k < p2; ++k) cfma(h, ai[i][k], gq[(size_t)k * len]);
         if (on) xs[i][j] = h;
         __syncthreads();
         if (on)
 #pragma unroll 8
-            for (int k = 0; k < p2; ++k) cfma(acc, xs[i][k], M[((size_t)q * p2 + k) * D + cs + j]);
+            for (int k = 0; k < p2; ++k) cfma(acc, xs[i][k], mq[(size_t)k * lenq]);
     }
     if (on) put(i0 + i, j, -acc);
 }
@@ -1751,17 +1753,17 @@ void launch_cut_panels(const CutCpEntry* cp, int ncp, const CutEpEntry* ep, int 
 }
 size_t cut_gram_scratch(int npairs) { return (size_t)npairs * GRAM_SPLIT * 1024 * sizeof(c128); }
 template <typename T>
-void launch_cut_gram(const CutGramPair* prs, int npairs, const CutGramDest* ds, int ndest, int Sx, int r, c128* part,
-                     cudaStream_t s) {
+void launch_cut_gram(const CutGramPair* prs, int npairs, int first0, const CutGramDest* ds, int ndest, int Sx, int r,
+                     c128* part, cudaStream_t s) {
     k_cut_gram<T><<<dim3(npairs, GRAM_SPLIT), 256, 0, s>>>(prs, Sx, r, part);
     note_launch();
-    k_cut_gram_red<<<ndest, 256, 0, s>>>(ds, r, part);
+    k_cut_gram_red<<<ndest, 256, 0, s>>>(ds, first0, r, part);
     note_launch();
 }
 template <typename T>
-void launch_cut_minv(const CutMinv* prs, int n, int D, int L, int p2, const c128* G, c128* M, cplx<T>* MT, int tr,
+void launch_cut_minv(const CutMinv* prs, int n, int L, int p2, const c128* G, c128* M, cplx<T>* MT, int tr,
                      cudaStream_t s) {
-    k_cut_minv<T><<<dim3(n, (p2 + MINV_ROWS - 1) / MINV_ROWS), 256, 0, s>>>(prs, D, L, p2, G, M, MT, tr);
+    k_cut_minv<T><<<dim3(n, (p2 + MINV_ROWS - 1) / MINV_ROWS), 256, 0, s>>>(prs, L, p2, G, M, MT, tr);
     note_launch();
 }
 
@@ -1931,8 +1933,8 @@ void launch_cut_update(const CutUpdJob* jobs, int njobs, int nleaf_max, int own_
 
 #define HH_CUT_INST(T)                                                                                             \
     template void launch_cut_panels<T>(const CutCpEntry*, int, const CutEpEntry*, int, int, int, OpGeom, cudaStream_t); \
-    template void launch_cut_gram<T>(const CutGramPair*, int, const CutGramDest*, int, int, int, c128*, cudaStream_t); \
-    template void launch_cut_minv<T>(const CutMinv*, int, int, int, int, const c128*, c128*, cplx<T>*, int, cudaStream_t); \
+    template void launch_cut_gram<T>(const CutGramPair*, int, int, const CutGramDest*, int, int, int, c128*, cudaStream_t); \
+    template void launch_cut_minv<T>(const CutMinv*, int, int, int, const c128*, c128*, cplx<T>*, int, cudaStream_t); \
     template size_t cut_plan<T>(CutProb&, int, bool);                                                                       \
     template bool launch_cut_steps<T>(const CutProb*, int, int, bool, size_t, const int*, int, unsigned*, int, int*, int,   \
                                       cudaStream_t, int, const CutGmres*, int);                                                                  \

@@ -190,10 +190,10 @@ __global__ void __launch_bounds__(256) k_edge_proj(const EdgeTask* __restrict__ 
 }
 
 // The path's corrections of one column (block) of one child, FP64: d from the partials, then
-// y_q = sum over the path below and at q of M_qs d_s (M: the full inverse, [D][D]).
+// y_q = sum over the path below and at q of M_qs d_s (M packed by subtree, cut_m_offset).
 // y: [npath][2r][nc], the node nearest the leaf first.
 template <typename T>
-__global__ void __launch_bounds__(256) k_edge_y(const EdgeTask* __restrict__ tasks, int nc, int r, int D,
+__global__ void __launch_bounds__(256) k_edge_y(const EdgeTask* __restrict__ tasks, int L, int nc, int r,
                                                 const c128* __restrict__ M) {
     using C = cplx<T>;
     __shared__ EdgeTask E;
@@ -216,12 +216,14 @@ __global__ void __launch_bounds__(256) k_edge_y(const EdgeTask* __restrict__ tas
         c128 a = {0, 0};
         if (e < E.npath * p2) {
             const int u = e / p2, i = e - u * p2;      // path node u (0: own), its row i
-            const c128* mr = M + ((size_t)E.path[u].id * p2 + i) * D;
-            for (int s = sub; s < p2; s += 8) cfma(a, mr[(size_t)E.path[0].id * p2 + s], d[na * r + s]);
+            const int pu = E.path[u].id;               // of level L - 1 - u
+            const c128* mr = M + E.path[u].mo + (size_t)i * cut_m_len(L - 1 - u, L, r);
+            const c128* m0 = mr + cut_m_col(pu, E.path[0].id, r);
+            for (int s = sub; s < p2; s += 8) cfma(a, m0[s], d[na * r + s]);
             // ancestors below and at u: their columns of the child that holds the cut
             for (int w = 1; w <= u; ++w) {
-                const size_t col = (size_t)E.path[w].id * p2 + E.path[w].kin * r;
-                for (int s = sub; s < r; s += 8) cfma(a, mr[col + s], d[(na - w) * r + s]);
+                const c128* mw = mr + cut_m_col(pu, E.path[w].id, r) + E.path[w].kin * r;
+                for (int s = sub; s < r; s += 8) cfma(a, mw[s], d[(na - w) * r + s]);
             }
         }
         for (int o = 4; o > 0; o >>= 1) {
@@ -487,12 +489,12 @@ void launch_edge_rows(const EdgeTask* tasks, int nchild, int Sx, int nc, int adj
 }
 // the path's corrections of nc columns from the leaf rows: y, and (rows_out) the trace rows
 template <typename T>
-void launch_edge_path(const EdgeTask* tasks, int nchild, int Sx, int nc, int r, int D, const c128* M, OpGeom g, int adj,
+void launch_edge_path(const EdgeTask* tasks, int nchild, int L, int Sx, int nc, int r, const c128* M, OpGeom g, int adj,
                       bool rows_out, cudaStream_t s) {
     g.b = 3;
     k_edge_proj<T><<<dim3(EDGE_CH, nchild, ((CUT_MAXL + 1) * r + 63) / 64), 256, 0, s>>>(tasks, Sx, nc, r, g);
     note_launch();
-    k_edge_y<T><<<dim3(nc, nchild), 256, sizeof(c128) * (size_t)(CUT_MAXL + 1) * r, s>>>(tasks, nc, r, D, M);
+    k_edge_y<T><<<dim3(nc, nchild), 256, sizeof(c128) * (size_t)(CUT_MAXL + 1) * r, s>>>(tasks, L, nc, r, M);
     note_launch();
     if (!rows_out) return;
     k_edge_out<T><<<dim3((Sx + 31) / 32, adj ? 1 : 2, nchild), 256, 0, s>>>(tasks, Sx, nc, r, adj);

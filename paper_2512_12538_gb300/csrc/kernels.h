@@ -366,7 +366,7 @@ struct CutProb {
     const void* rt;                   // [Sy][Sx] the round's residual
     void *v, *vsum, *res0;            // [ncut][2][Sx]
     void *prow, *pd, *d, *y, *yacc;   // [nA][4][Sx], [nB][(L + 1) r], [D] each
-    float* npart;                     // [nB][8] partial |v|^2
+    float* npart;                     // [nB] partial |v|^2
     const double *nrm, *b2;           // |r|^2 and |b|^2 (FP64)
     const c128* scale;                // of the round's residual in k_cut_lines (null: 1)
     CutCtl* ctl;
@@ -382,15 +382,36 @@ template <typename T>
 void launch_cut_panels(const CutCpEntry* cp, int ncp, const CutEpEntry* ep, int nep, int Sx, int r, OpGeom g,
                        cudaStream_t s);
 size_t cut_gram_scratch(int npairs);
-// sums of C_p^H E_q per pair into the destinations (pairs [first, first + count) each)
+// sums of C_p^H E_q per pair into the destinations (pairs [first, first + count) each, prs[0]
+// being pair `first0`)
 template <typename T>
-void launch_cut_gram(const CutGramPair* prs, int npairs, const CutGramDest* ds, int ndest, int Sx, int r, c128* part,
-                     cudaStream_t s);
+void launch_cut_gram(const CutGramPair* prs, int npairs, int first0, const CutGramDest* ds, int ndest, int Sx, int r,
+                     c128* part, cudaStream_t s);
 // blocks of the inverse of the corrections' triangular system (children before parents);
-// MT: packed (cut_m_packed entries), row-major or (tr) transposed within a node's rows
+// G, M and MT packed: a node's 2 r rows hold the corrections of its subtree level by level
+// (cut_m_packed entries in all; full matrices took 16 D^2 bytes each, 260 MB at D = 4032 against
+// 21).  cut_m_offset: the node's first entry; cut_m_len: entries of a row of a node of level l;
+// cut_m_col: first column of node s at or below p.  MT: row-major or (tr) transposed within a
+// node's rows
+HH_HD int cut_level_of(int p) {
+    int l = 0;
+    while ((2 << l) <= p + 1) ++l;
+    return l;
+}
+HH_HD int cut_m_len(int l, int L, int r) { return 2 * r * ((1 << (L - l)) - 1); }
+HH_HD size_t cut_m_offset(int p, int L, int r) {
+    const int l = cut_level_of(p);
+    size_t o = 0;
+    for (int q = 0; q < l; ++q) o += ((size_t)1 << q) * 2 * r * cut_m_len(q, L, r);
+    return o + (size_t)(p + 1 - (1 << l)) * 2 * r * cut_m_len(l, L, r);
+}
+HH_HD int cut_m_col(int p, int s, int r) {
+    const int l = cut_level_of(p), d = cut_level_of(s) - l;
+    return 2 * r * ((1 << d) - 1 + (s + 1 - (1 << (l + d))) - ((p + 1 - (1 << l)) << d));
+}
 size_t cut_m_packed(int L, int r);
 template <typename T>
-void launch_cut_minv(const CutMinv* prs, int n, int D, int L, int p2, const c128* G, c128* M, cplx<T>* MT, int tr,
+void launch_cut_minv(const CutMinv* prs, int n, int L, int p2, const c128* G, c128* M, cplx<T>* MT, int tr,
                      cudaStream_t s);
 // whether the cluster form can run with this much shared memory on the current device (true
 // without one)
@@ -432,7 +453,7 @@ void launch_cut_update(const CutUpdJob* jobs, int njobs, int nleaf_max, int own_
 struct EdgePath {
     int id, ra, kin, kedge;
     const void* C;
-    size_t N;
+    size_t N, mo;                     // points; first entry of its rows of M
 };
 struct EdgeTask {
     const void *V, *xi, *sc;          // edge leaf, as EigTask
@@ -463,7 +484,7 @@ size_t edge_gram_scratch(int nchild);
 template <typename T>
 void launch_edge_rows(const EdgeTask* tasks, int nchild, int Sx, int nc, int adj, cudaStream_t s);
 template <typename T>
-void launch_edge_path(const EdgeTask* tasks, int nchild, int Sx, int nc, int r, int D, const c128* M, OpGeom g, int adj,
+void launch_edge_path(const EdgeTask* tasks, int nchild, int L, int Sx, int nc, int r, const c128* M, OpGeom g, int adj,
                       bool rows_out, cudaStream_t s);
 // recursions of the basis extension (into Fh, transformed layout of nc right-hand sides)
 template <typename T>
