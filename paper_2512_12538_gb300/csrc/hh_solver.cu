@@ -2905,7 +2905,8 @@ static hh_status solve_many(SolverBase* const* hs, const c128* const* f, const c
             if (!pf.empty()) rs[i] = pf[k]->solve_gmres(restart, f[k], g[k], u[k], &s2);
             else rs[i] = pd[k]->solve_gmres(restart, f[k], g[k], u[k], &s2);
             hs[k]->stream = own;
-            if (stats) {
+            // (without memory for it nothing ran: the stationary run's figures and iterate stand)
+            if (stats && rs[i] != HH_ENOMEM) {
                 stats[k].iters += s2.iters;
                 stats[k].rel_res = s2.rel_res;
             }
