@@ -200,8 +200,9 @@ hh_status hh_setup_batch(const hh_params* params, int count, void* stream, hh_ha
  * problems iterate together in rounds: one launch in which every problem runs its steps on
  * the rows next to its leaf cuts up to its own next stop, then one launch each, for all
  * problems, of the leaf transforms, the update and the FP64 residual; a problem drops out
- * when its residual meets its own tol.  Members whose iteration does not converge are
- * re-solved by flexible GMRES with their set-up as it stands.
+ * when its residual meets its own tol.  (Hierarchies too large for those rows' launch are
+ * solved one after another.)  Members whose iteration does not converge are re-solved by
+ * flexible GMRES with their set-up as it stands, or, of those hierarchies, on a second one.
  * Otherwise the problems are solved one after another.  stats[k] (may be NULL) gets
  * problem k's iterations and residual; t_solve_ms is the time of the whole batch.
  * Synchronises.  Returns HH_OK if all converged, else the first failing status. */

@@ -418,6 +418,10 @@ struct SolverBase {
         prof_on = on;
         prof_mask = mask;
     }
+    // The caller re-solves by GMRES what does not converge: a stationary solve on the whole grid
+    // then ends (HH_ENOCONV) once its residual is a hundred times its smallest, or fell less than
+    // tenfold over 25 steps (the steps on the cut rows have this test in the kernel, StepWatch).
+    bool early = false;
     virtual size_t plan(char* base) = 0;
     virtual hh_status setup() = 0;
     virtual hh_status solve(const c128* f, const c128* g, c128* u, hh_stats* st) = 0;
@@ -2016,12 +2020,20 @@ struct Solver final : SolverBase {
         h_norm[0] = h_norm[2] = 1.0;
         ((int*)(h_norm + 6))[0] = 0;
         ((int*)(h_norm + 6))[1] = 1;
-        double rel_prev = -1.0;
-        int it_prev = 0, chunks = 0;
+        double rel_prev = -1.0, best = 1.0, chk = 1.0;
+        int it_prev = 0, chunks = 0, chk_it = 0;
         for (;;) {
-            rel = rel_norm(h_norm[0], h_norm[2]);   // last FP64 residual
+            rel = rel_norm(h_norm[0], h_norm[2]);   // last FP64 residual (of b: 1)
             if (hctl[0] == 2 || !std::isfinite(rel)) return HH_ENOCONV;
             if (hctl[0] == 1) return HH_OK;
+            best = std::min(best, rel);
+            bool slow = rel > 100.0 * best;
+            if (it - chk_it >= 25) {
+                slow = slow || rel > 0.1 * chk;
+                chk = rel;
+                chk_it = it;
+            }
+            if (early && slow) return HH_ENOCONV;
             if (it >= P.max_iter) {
                 // the FP64 residual of the last iterate, for the report
                 gated_residual(ctl);
@@ -2545,12 +2557,17 @@ static hh_status setup_one(const hh_params* p, cudaStream_t s, SolverBase** out,
 }
 
 // ------------------------------------------------------------------ batched solves
-// Several set-up problems solved together (the batching form).  Requires the stationary
-// iteration on the cut rows (n_i = 1, eigenbasis leaves) of the 5-point rows with leaves that
-// fit the one-launch sweep, for every problem, in one precision.
+// Several set-up problems solved together (the batching form), all in one precision, by the
+// stationary iteration (n_i = 1) on the 5-point rows with eigenbasis leaves that fit the
+// one-launch sweep; a member that does not converge is re-solved by GMRES.  BatchEngine takes
+// those on the cut rows, the few hierarchies these do not take (cut_plan) go one by one.
+template <typename T>
+static bool member(const Solver<T>* p) {
+    return p->eig && p->eig_fused && p->pre_direct && p->P.n_inner == 1 && p->P.outer == HH_OUTER_ORAS && !p->q1();
+}
 template <typename T>
 static bool batchable(const Solver<T>* p) {
-    return p->cut && p->eig_fused && p->pre_direct && p->P.outer == HH_OUTER_ORAS && !p->q1();
+    return p->cut && member(p);
 }
 
 // Iteration of several set-up problems together: the engine of the batching and serving
@@ -2855,30 +2872,76 @@ static hh_status batch_solve(std::vector<Solver<T>*>& ps, const c128* const* f, 
     return HH_OK;
 }
 
-// All handles in one precision and batchable: solve them together in lockstep.  Problems
-// the stationary iteration does not converge are then solved by flexible GMRES (the
-// paper's outer solver), several at a time from host threads.
-// Handles that cannot join the lockstep batch are solved one by one.
+// The stationary runs of a batch's members (`member`); per[k]: member k's status.
+template <typename T>
+static hh_status run_members(std::vector<Solver<T>*>& ps, const c128* const* f, const c128* const* g, c128* const* u,
+                             cudaStream_t stream, hh_stats* stats, std::vector<hh_status>& per) {
+    const int n = (int)ps.size();
+    std::vector<int> in, alone;
+    for (int k = 0; k < n; ++k) (ps[k]->cut ? in : alone).push_back(k);
+    if (alone.empty()) {
+        const hh_status st = batch_solve<T>(ps, f, g, u, stream, stats, per);
+        if (st != HH_ENOTIMPL) return st;
+        alone.swap(in);
+    }
+    per.assign(n, HH_OK);
+    if (!in.empty()) {
+        std::vector<Solver<T>*> p2;
+        std::vector<const c128*> f2, g2;
+        std::vector<c128*> u2;
+        std::vector<hh_stats> s2;
+        std::vector<hh_status> per2;
+        for (int k : in) {
+            p2.push_back(ps[k]);
+            f2.push_back(f[k]);
+            g2.push_back(g[k]);
+            u2.push_back(u[k]);
+            s2.push_back(stats ? stats[k] : hh_stats{});
+        }
+        const hh_status st = batch_solve<T>(p2, f2.data(), g2.data(), u2.data(), stream, s2.data(), per2);
+        if (st == HH_ENOTIMPL) alone.insert(alone.end(), in.begin(), in.end());
+        else if (st != HH_OK && st != HH_ENOCONV) return st;
+        else
+            for (size_t i = 0; i < in.size(); ++i) {
+                per[in[i]] = per2[i];
+                if (stats) stats[in[i]] = s2[i];
+            }
+    }
+    hh_status st = HH_OK;
+    for (int k : alone) {
+        ps[k]->stream = stream;
+        ps[k]->early = true;
+        per[k] = ps[k]->solve(f[k], g[k], u[k], stats ? stats + k : nullptr);
+        ps[k]->early = false;
+        if (per[k] != HH_OK && per[k] != HH_ENOCONV) return per[k];
+    }
+    for (auto s1 : per)
+        if (s1 != HH_OK) st = s1;
+    return st;
+}
+
+// All handles in one precision and members: run them together.  Problems the stationary
+// iteration does not converge are then solved by flexible GMRES (the paper's outer solver),
+// several at a time from host threads.  Other lists are solved one by one.
 static hh_status solve_many(SolverBase* const* hs, const c128* const* f, const c128* const* g, c128* const* u, int n,
                             cudaStream_t stream, hh_stats* stats) {
     std::vector<Solver<float>*> pf;
     std::vector<Solver<double>*> pd;
     for (int k = 0; k < n; ++k) {
-        if (auto* a = dynamic_cast<Solver<float>*>(hs[k])) { if (batchable(a)) pf.push_back(a); }
-        else if (auto* b = dynamic_cast<Solver<double>*>(hs[k])) { if (batchable(b)) pd.push_back(b); }
+        if (auto* a = dynamic_cast<Solver<float>*>(hs[k])) { if (member(a)) pf.push_back(a); }
+        else if (auto* b = dynamic_cast<Solver<double>*>(hs[k])) { if (member(b)) pd.push_back(b); }
     }
     std::vector<hh_status> per;
-    hh_status st = HH_ENOTIMPL;
-    if ((int)pf.size() == n) st = batch_solve<float>(pf, f, g, u, stream, stats, per);
-    else if ((int)pd.size() == n) st = batch_solve<double>(pd, f, g, u, stream, stats, per);
-    if (st == HH_ENOTIMPL) {
-        hh_status first = HH_OK;
+    hh_status st = HH_OK;
+    if ((int)pf.size() == n) st = run_members<float>(pf, f, g, u, stream, stats, per);
+    else if ((int)pd.size() == n) st = run_members<double>(pd, f, g, u, stream, stats, per);
+    else {
         for (int k = 0; k < n; ++k) {
             hs[k]->stream = stream;
             const hh_status s1 = hs[k]->solve(f[k], g[k], u[k], stats ? stats + k : nullptr);
-            if (s1 != HH_OK && first == HH_OK) first = s1;
+            if (s1 != HH_OK && st == HH_OK) st = s1;
         }
-        return first;
+        return st;
     }
     if (st != HH_OK && st != HH_ENOCONV) return st;
     std::vector<int> rescue;
@@ -2899,14 +2962,29 @@ static hh_status solve_many(SolverBase* const* hs, const c128* const* f, const c
         for (size_t i = w; i < rescue.size(); i += nw) {
             const int k = rescue[i];
             const int restart = hs[k]->P.restart < 1 || hs[k]->P.restart > 64 ? 40 : hs[k]->P.restart;
-            const cudaStream_t own = hs[k]->stream;
             hh_stats s2{};
-            hs[k]->stream = ws;
-            if (!pf.empty()) rs[i] = pf[k]->solve_gmres(restart, f[k], g[k], u[k], &s2);
-            else rs[i] = pd[k]->solve_gmres(restart, f[k], g[k], u[k], &s2);
-            hs[k]->stream = own;
-            // (without memory for it nothing ran: the stationary run's figures and iterate stand)
-            if (stats && rs[i] != HH_ENOMEM) {
+            bool ran = true;
+            if (pf.empty() ? pd[k]->cut : pf[k]->cut) {
+                const cudaStream_t own = hs[k]->stream;
+                hs[k]->stream = ws;
+                if (!pf.empty()) rs[i] = pf[k]->solve_gmres(restart, f[k], g[k], u[k], &s2);
+                else rs[i] = pd[k]->solve_gmres(restart, f[k], g[k], u[k], &s2);
+                hs[k]->stream = own;
+                ran = rs[i] != HH_ENOMEM;
+            } else {
+                // on the whole grid GMRES's vectors are part of the plan: a handle of its own
+                hh_params q = hs[k]->P;
+                q.outer = HH_OUTER_GMRES;
+                q.restart = restart;
+                SolverBase* g2 = nullptr;
+                rs[i] = setup_one(&q, ws, &g2, g_alloc);
+                ran = rs[i] == HH_OK;
+                if (ran) rs[i] = g2->solve(f[k], g[k], u[k], &s2);
+                cudaStreamSynchronize(ws);
+                delete g2;
+            }
+            // (where it could not run, the stationary run's figures and iterate stand)
+            if (stats && ran) {
                 stats[k].iters += s2.iters;
                 stats[k].rel_res = s2.rel_res;
             }
@@ -3026,8 +3104,8 @@ struct Server {
             r->stats.t_setup_ms = sb->t_setup_ms;
             r->stats.footprint_bytes = sb->footprint;
             bool lock = false;
-            if (auto* a = dynamic_cast<Solver<float>*>(sb)) lock = batchable(a);
-            else if (auto* b = dynamic_cast<Solver<double>*>(sb)) lock = batchable(b);
+            if (auto* a = dynamic_cast<Solver<float>*>(sb)) { lock = batchable(a); sb->early = member(a); }
+            else if (auto* b = dynamic_cast<Solver<double>*>(sb)) { lock = batchable(b); sb->early = member(b); }
             if (lock) {
                 cudaStreamSynchronize(ws);
                 std::lock_guard<std::mutex> lk(mu);
