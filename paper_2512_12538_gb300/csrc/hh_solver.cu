@@ -22,6 +22,7 @@
 #include <chrono>
 #include <cmath>
 #include <condition_variable>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <deque>
@@ -2146,14 +2147,16 @@ struct Solver final : SolverBase {
         const int nG = cut_ng(), nl = (int)lev[L].size();
         hh_status st = HH_OK;
         auto resid = [&]() {
-            zero(ctl, 4 * sizeof(double) + sizeof(CutCtl));
+            // (the profiled phases add up over the cycles)
+            zero(ctl, 4 * sizeof(double) + offsetof(CutCtl, ns));
             pbeg(PC_SPMV, 48.0 * (double)Sy * Sx);
+            if (prof_cat(PC_SPMV)) prof_pending.back().nl = 0;   // (counted by the steps, as in loop_cut)
             launch_residual_stop<T>(u, bvec, nullptr, RT, geom(0), npart, dnorm, ctl, dcounter, P.tol, stream);
             pend(PC_SPMV);
         };
         auto steps = [&](int mode, int max_steps, int gm_steps) {
-            return launch_cut_steps<T>(d_cut, 1, cut_group(), cp.cl, cut_smem, nullptr, mode, cbar, 1, derr, 0, stream,
-                                       max_steps, &cg, gm_steps);
+            return launch_cut_steps<T>(d_cut, 1, cut_group(), cp.cl, cut_smem, nullptr, mode, cbar, 1, derr,
+                                       prof_on && gm_steps, stream, max_steps, &cg, gm_steps);
         };
         for (bool cycle = false;; cycle = true) {
             if (cycle) {
@@ -2254,7 +2257,11 @@ struct Solver final : SolverBase {
     // update reads (g and H up to the stopping column).  Convergence is confirmed on the
     // true residual at every restart.
     hh_status loop_gmres(int& it, double& rel) {
-        if (cut) return loop_gmres_cut(it, rel);
+        if (cut) {
+            const hh_status cs = loop_gmres_cut(it, rel);
+            if (prof_on) cut_prof(it);
+            return cs;
+        }
         const size_t N = (size_t)Sy * Sx;
         const int ld = mk + 1;
         hh_status st = HH_OK;

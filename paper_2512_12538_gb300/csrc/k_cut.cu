@@ -1060,6 +1060,7 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
             }
             stepped = true;
             if (gm_steps) {
+                if (timing) tC += gtime() - t0;   // (the Arnoldi step is no phase of the iteration)
                 // the Arnoldi step: P.v takes the next step's input
                 if (first && rank == 0)
                     for (int e = tid; e < D; e += NT) ((C*)G.y0)[e] = s_ya[e];
@@ -1080,7 +1081,7 @@ __global__ void __launch_bounds__(NT) k_cut_steps(const CutProb* __restrict__ pr
 #pragma unroll 5
             for (int e = lane; e < P.nB; e += 32) n2 += __ldcg(P.npart + e);
             n2 = warp_sum(n2);
-            if (timing) { const unsigned long long t = gtime(); tC += t - t0; t0 = t; }
+            if (timing && !gm_steps) tC += gtime() - t0;
             first = false;
             ++it;
             ++in_round;
@@ -1516,6 +1517,7 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
                 __syncthreads();
             }
             if constexpr (GM) {
+                if (timing) tC += gtime() - t0;
                 // the Arnoldi step: S v goes through P.v, which takes the next step's input
                 C* vg = (C*)P.v;
                 for (int q = tid; q < np; q += NT) {
@@ -1552,7 +1554,7 @@ __global__ void __launch_bounds__(CC_NT, 1) k_cut_cluster(const CutProb* __restr
             if (warp < 4 && lane < CC_CL) st_async(mapa(smem_u32(&s_nrm[rank][warp]), lane), nn, mapa(mb + 16, lane));
             if (!(ok = wait(2, by3))) break;
             n2 = warp_sum((&s_nrm[0][0])[lane] + (&s_nrm[0][0])[lane + 32]);   // alike in every warp
-            if (timing) { const unsigned long long t = gtime(); tC += t - t0; t0 = t; }
+            if (timing && !GM) tC += gtime() - t0;
             first = false;
             ++it;
             ++in_round;
