@@ -128,12 +128,15 @@ typedef enum {
 
 typedef enum {
     HH_OUTER_ORAS = 0,    /* stationary iteration u <- u + M (b - A u) (Eqs. (2)-(3))          */
-    HH_OUTER_GMRES = 1    /* flexible GMRES right-preconditioned by M (Sec. 3), FP64 Arnoldi   */
+    HH_OUTER_GMRES = 1    /* flexible GMRES right-preconditioned by M (Sec. 3), FP64 Arnoldi;  */
+                          /* with the cut rows (eigenbasis leaves, n_inner = 1) A M v is taken */
+                          /* in the leaf precision and refined by each cycle's FP64 residual   */
 } hh_outer;
 
 typedef struct {
     int iters;            /* outer iterations taken                                      */
-    double rel_res;       /* final ||b - A u|| / ||b|| (FP64)                            */
+    double rel_res;       /* final ||b - A u|| / ||b|| (FP64); 0 for b = 0, and beside    */
+                          /* HH_ENOCONV for a right-hand side with a NaN                  */
     double t_setup_ms;    /* device time of hh_setup (CUDA events)                       */
     double t_solve_ms;    /* device time of the last hh_solve                            */
     size_t footprint_bytes;
@@ -385,7 +388,8 @@ hh_status hh_autotune_report(char* buf, size_t cap, size_t* len);
  * synchronises reports HH_ETIMEOUT with the context still usable.
  * -------------------------------------------------------------------------------- */
 /* Caps the polls of the give-up waits of the kernels launched from now on in this
- * process: the barriers of the cooperative kernels and the tensor-core
+ * process: the barriers of the cooperative kernels, the exchanges of the cluster
+ * kernels (cut-row steps, inverse of the coarse matrices) and the tensor-core
  * transforms' waits for their operands and MMAs.  polls = 0 makes every such wait give
  * up at once (how a test makes a wait run out without a fault); polls < 0 restores the
  * defaults (about a second).  CUDA graphs captured meanwhile keep the value of their

@@ -1977,10 +1977,12 @@ struct Solver final : SolverBase {
         return ok;
     }
 
-    // The launches of one stationary step on the fast path (n_i = 1, fused eigenbasis
-    // leaf sweeps writing into the parents, L >= 2) are the leaf sweep and the batched
-    // coarse corrections: all of them, and the residual that follows, take a gate.
-    // (the one-launch sweep and the three-stage one both take the stop word)
+    // The launches of one stationary step with eigenbasis leaves that write into the parents
+    // (n_i = 1, L >= 2) are the leaf sweep and the batched coarse corrections: all of them,
+    // and the residual that follows, take a gate.  (The one-launch sweep and the three-stage
+    // one both take the stop word.)  Hierarchies too large for the cut rows come here (cut_plan: in
+    // FP64 six levels with r >= 24, or five with r = 32 from 541 points a side); the others with n_i = 1
+    // iterate on those rows.
     bool device_test_path() const {
         return eig && pre_direct && P.n_inner == 1 && L >= 2 && P.outer == HH_OUTER_ORAS;
     }
@@ -2136,7 +2138,9 @@ struct Solver final : SolverBase {
     }
     int cut_ng() const { return 2 * cp.ncut * Sx; }   // entries on the cut rows
 
-    // Flexible GMRES (loop_gmres) with its Krylov space kept on the cut rows (k_cut.cu).  A
+    // Flexible GMRES (loop_gmres) with its Krylov space kept on the cut rows (k_cut.cu): the
+    // vectors and the orthogonalisation in FP64, the steps S v in the leaf precision (complex64
+    // in the mixed form, where the FP64 residual that starts a cycle refines them).  A
     // cycle starts from the FP64 residual of u with one step on every row, which gives S r;
     // it then runs in one launch, each Arnoldi step one step on the cut rows.  It ends at the
     // restart length, when the estimate is below tol / 2, or (complex64) when it has fallen by

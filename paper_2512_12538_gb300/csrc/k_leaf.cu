@@ -163,7 +163,8 @@ __global__ void __launch_bounds__(256) k_factor2d(const LeafTask* __restrict__ t
 // column k of the tableau ends up as the column of the pivot row p_k, and the store puts
 // entry (p_k, c) at (k, p_c).  The chain of pivots bounds it (b columns x Sx / 2 blocks, each
 // pivot waiting for the one before): a pivot costs one barrier, its search stays in the
-// warp that owns the column, and the pivot row's entries come by shuffles.  4 bands of 37 rows
+// warp that owns the column (by the high word of |a|^2: within 1e-6 of the largest), and the pivot
+// row's entries come by shuffles.  4 bands of 37 rows
 // x 129 columns in complex64: 7.4 ms with the block in shared memory and one chain, 1.45 ms here.
 template <typename T> __device__ __forceinline__ unsigned pivot_key(T a) {
     if constexpr (sizeof(T) == 8) return (unsigned)__double2hiint(a) + 1u;
